@@ -286,7 +286,7 @@ static float bf16_to_float(uint16_t h)
 struct Workspace {
     NbrWork nbr;
     DBuf pos, spec, pair_i, coef, phat, pnorm, gp_of_atom, flag, fpos, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
-        W, eps_part, Gam, fpair, f2, forces, vir_atom, cfgpart, energy, virial, local, err, A_hi, A_lo, t_row, W_hi, W_lo,
+        W, eps_part, Gam, fpair, fw2, forces, vir_atom, cfgpart, energy, virial, local, err, A_hi, A_lo, t_row, W_hi, W_lo,
         epart_f, wpart_f, Gs, outbuf, kA, kAhi, kAlo, kt, ksrc, kseg, kdest, segstart, outrow, Wp, kq, P, Kbuf, A_mid, W_mid,
         kAmid, phatc, pnormc, hfull, kV;
     // Graph mode (gap_step_graph): no host synchronisation inside a call; the
@@ -297,7 +297,7 @@ struct Workspace {
     {
         nbr.release();
         DBuf *bs[] = {&pos, &spec, &pair_i, &coef, &phat, &pnorm, &gp_of_atom, &flag, &fpos, &scan_tmp, &rows,
-                      &counts, &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &f2, &forces, &vir_atom, &cfgpart, &energy,
+                      &counts, &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &fw2, &forces, &vir_atom, &cfgpart, &energy,
                       &virial, &local, &err, &A_hi, &A_lo, &t_row, &W_hi, &W_lo, &epart_f, &wpart_f, &Gs, &outbuf,
                       &kA, &kAhi, &kAlo, &kt, &ksrc, &kseg, &kdest, &segstart, &outrow, &Wp, &kq, &P, &Kbuf, &A_mid, &W_mid,
                       &kAmid, &phatc, &pnormc, &hfull, &kV};
@@ -1359,14 +1359,16 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
         GAP_TRY(gap_pairforce<T>(g, tab_of<T>(soap), pl, w.pair_i.as<int>(), spec, w.Gam.as<T>(), w.fpair.as<T>(), st));
         gap_prof_end(ST_PAIRFORCE, st);
     }
-    double *eps2 = nullptr, *f2 = nullptr;
+    double *eps2 = nullptr, *fw2 = nullptr;
     if (m->has_tb) {
         GAP_TRY(w.eps2.ensure(sizeof(double) * (size_t)n));
-        GAP_TRY(w.f2.ensure(sizeof(double) * 3 * (size_t)pl.n_pairs));
         eps2 = w.eps2.as<double>();
-        f2 = w.f2.as<double>();
+        if (grad) {
+            GAP_TRY(w.fw2.ensure(sizeof(double) * 9 * (size_t)n));
+            fw2 = w.fw2.as<double>();
+        }
         gap_prof_begin(ST_TWOBODY, st);
-        GAP_TRY(gap_twobody(n, pl, m->tb, f2, eps2, st));
+        GAP_TRY(gap_twobody(n, pl, m->tb, fw2, eps2, st));
         gap_prof_end(ST_TWOBODY, st);
     }
     // outputs
@@ -1387,8 +1389,8 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
         vir_atom = w.vir_atom.as<double>();
     }
     gap_prof_begin(ST_GATHER, st);
-    if (d_forces || vir_atom) GAP_TRY(gap_gather<T>(n, pl, w.fpair.as<T>(), f2, d_forces, vir_atom, st));
-    if (d_energy || d_virial) {
+    if (d_forces || vir_atom) GAP_TRY(gap_gather<T>(n, pl, w.fpair.as<T>(), fw2, d_forces, vir_atom, st));
+    if (d_energy || d_virial || d_local) {
         int max_atoms = 0;
         for (int c = 0; c < C; ++c) {
             const int na = b->config_offsets[c + 1] - b->config_offsets[c];
@@ -1396,9 +1398,8 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
         }
         GAP_TRY(w.cfgpart.ensure(sizeof(double) * gap_config_part_doubles(C, max_atoms)));
         GAP_TRY(gap_config_sums(C, w.nbr.cfg_offsets, max_atoms, w.eps.as<double>(), eps2, vir_atom, d_energy,
-                                d_virial, w.cfgpart.as<double>(), st));
+                                d_virial, d_local, w.cfgpart.as<double>(), st));
     }
-    if (d_local) GAP_TRY(gap_local_energy(n, w.eps.as<double>(), eps2, d_local, st));
     gap_prof_end(ST_GATHER, st);
     if (!b->device) {
         if (forces && n) GAP_TRY_CUDA(cudaMemcpyAsync(forces, d_forces, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, st));

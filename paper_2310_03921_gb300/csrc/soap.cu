@@ -465,126 +465,252 @@ __global__ void k_twobody_table(TwoBodyDev tb, D4 *__restrict__ tab)
     tab[k] = D4{e0, h * d0, 3.0 * (e1 - e0) - h * (2.0 * d0 + d1), 2.0 * (e0 - e1) + h * (d0 + d1)};
 }
 
-// Half of each pair's two-body energy goes to the pair's first atom and half
-// of its derivative to f2[p], from the tabulated E(r) (FP64 in every
-// precision mode: the term is large next to the 1e-4 eV/A force bound).
-// One thread per atom.
-__global__ void k_twobody(int n_atoms, const int *__restrict__ offsets, const D4 *__restrict__ vec, TwoBodyDev tb,
-                          double *__restrict__ f2, double *__restrict__ eps2)
+// 1 / r to the last bit or so: the FP32 reciprocal and two Newton steps
+// (errors 2^-23, 2^-46, 2^-92 before rounding).  CUDA's FP64 division takes
+// several times the FP64 instructions, each ~64 cycles per warp here.
+__device__ __forceinline__ double recip_newton(double r)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_atoms) return;
-    double e = 0.0;
+    double y = (double)(1.0f / (float)r);
+    y = fma(y, fma(-r, y, 1.0), y);
+    return fma(y, fma(-r, y, 1.0), y);
+}
+
+// Lanes that share one atom's pairs in the per-atom sums below.  An atom has
+// 25-40 pairs: eight lanes leave a chain of four or five dependent loads (one
+// thread per atom walked all of them: 30 us of latency at 64 atoms), and a
+// block still covers 16 atoms.
+constexpr int kPairLanes = 8;
+
+template <typename T> __device__ __forceinline__ T group_sum(T v)
+{
+#pragma unroll
+    for (int o = kPairLanes / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Two-body term of every atom from the tabulated E(r), FP64 in every
+// precision mode (the term is large next to the 1e-4 eV/A force bound): half
+// of each pair's energy to eps2, and, when fw2 is given, the atom's force and
+// virial (F, then W_xx W_yy W_zz W_yz W_xz W_xy: it is symmetric).  The pair's
+// two directions carry opposite derivatives, so the reverse pair is not read:
+// F_i = sum_p 2 f[p], W_i = -sum_p f[p] (x) r_p with f = E'(r) / 2 u.
+// Bound by the FP64 pipe (about 25 FP64 instructions per pair).
+__global__ void __launch_bounds__(128)
+k_twobody(int n_atoms, const int *__restrict__ offsets, const D4 *__restrict__ vec, TwoBodyDev tb,
+          double *__restrict__ eps2, double *__restrict__ fw2)
+{
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) / kPairLanes, sub = threadIdx.x % kPairLanes;
     const double rt = tb.rc - tb.d, inv_in = 1.0 / tb.h_in, inv_out = 1.0 / tb.h_out;
-    for (int p = offsets[i]; p < offsets[i + 1]; ++p) {
-        D4 v = vec[p];
-        double r = v.w, c = 0.0;
-        if (r < tb.rc) {
-            double s, inv;
-            int k;
-            if (r < rt) {
-                s = r * inv_in;
-                k = min((int)s, tb.g_in - 1);
-                inv = inv_in;
-            } else {
-                s = (r - rt) * inv_out;
-                k = min((int)s, tb.g_out - 1);
-                inv = inv_out;
-            }
-            const double u = s - k;
-            const D4 a = tb.tab[r < rt ? k : tb.g_in + k];
-            e += 0.5 * (a.x + u * (a.y + u * (a.z + u * a.w)));
-            c = 0.5 * (a.y + u * (2.0 * a.z + 3.0 * u * a.w)) * inv / r;
+    double e = 0.0, F[3] = {0, 0, 0}, W[6] = {0, 0, 0, 0, 0, 0};
+    const int p1 = i < n_atoms ? offsets[i + 1] : 0;
+    for (int p = i < n_atoms ? offsets[i] + sub : 0; p < p1; p += kPairLanes) {
+        const D4 v = vec[p];
+        const double r = v.w;
+        if (r >= tb.rc) continue;
+        const bool in = r < rt;
+        const double inv = in ? inv_in : inv_out, s = (in ? r : r - rt) * inv;
+        const int k = min((int)s, (in ? tb.g_in : tb.g_out) - 1);
+        const double u = s - k;
+        const D4 a = tb.tab[in ? k : tb.g_in + k];
+        e += a.x + u * (a.y + u * (a.z + u * a.w));
+        if (fw2) {
+            const double c = (a.y + u * (2.0 * a.z + 3.0 * u * a.w)) * inv * recip_newton(r);
+            const double fx = c * v.x, fy = c * v.y, fz = c * v.z;
+            F[0] += fx;
+            F[1] += fy;
+            F[2] += fz;
+            W[0] -= fx * v.x;
+            W[1] -= fy * v.y;
+            W[2] -= fz * v.z;
+            W[3] -= fy * v.z;
+            W[4] -= fx * v.z;
+            W[5] -= fx * v.y;
         }
-        f2[3 * (size_t)p] = c * v.x;
-        f2[3 * (size_t)p + 1] = c * v.y;
-        f2[3 * (size_t)p + 2] = c * v.z;
     }
-    eps2[i] = e;
+    e = group_sum(e);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) F[a] = group_sum(F[a]);
+#pragma unroll
+    for (int a = 0; a < 6; ++a) W[a] = group_sum(W[a]);
+    if (i < n_atoms && sub == 0) {
+        eps2[i] = 0.5 * e;
+        if (fw2) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) fw2[9 * (size_t)i + a] = F[a];
+#pragma unroll
+            for (int a = 0; a < 6; ++a) fw2[9 * (size_t)i + 3 + a] = 0.5 * W[a];
+        }
+    }
 }
 
 // ------------------------------------------------------ forces and virials
-// F_j = sum_{p in pairs(j)} (f[p] - f[rev p]);  W_j = -sum_{p in pairs(j)} f[p] (x) r_p.
+// Running sums of the pair terms.  FP64 terms are summed in FP64; FP32 terms
+// (and the exact products of two of them) in a compensated FP32 pair (two-sum
+// and two-product, Ogita, Rump and Oishi 2005: ~48 bits), because one FP64
+// instruction holds GB300's FP64 pipe for ~64 cycles per warp where the
+// seven FP32 ones of a two-sum take seven.
+template <typename T> struct PairSum;
+template <> struct PairSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double x) { s += x; }
+    __device__ __forceinline__ void sub_product(double a, double b) { s -= a * b; }
+    __device__ __forceinline__ void reduce() { s = group_sum(s); }
+    __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct PairSum<float> {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float t = s + x, b = t - s;
+        c += (s - (t - b)) + (x - b);
+        s = t;
+    }
+    __device__ __forceinline__ void sub_product(float a, float b)
+    {
+        const float p = -(a * b);
+        c -= fmaf(a, b, p);
+        add(p);
+    }
+    __device__ __forceinline__ void reduce()
+    {
+#pragma unroll
+        for (int o = kPairLanes / 2; o > 0; o >>= 1) {
+            const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+            add(s2);
+            c += c2;
+        }
+    }
+    // an infinite sum leaves a NaN correction, which is dropped
+    __device__ __forceinline__ double value() const { return c - c == 0.f ? (double)s + (double)c : (double)s; }
+};
+
+// F_j = sum_{p in pairs(j)} (f[p] - f[rev p]);  W_j = -sum_{p in pairs(j)} f[p] (x) r_p,
+// plus the two-body force and virial of the atom (fw2, see k_twobody).
+// kPairLanes lanes per atom.  A captured step of 64 atoms takes 120 us with it
+// (151 us with one thread per atom), outputs bit for bit the same.
 template <typename T>
-__global__ void k_gather(int n_atoms, const int *__restrict__ offsets, const int *__restrict__ rev,
-                         const typename V4<T>::type *__restrict__ vec, const T *__restrict__ fpair,
-                         const double *__restrict__ f2, double *__restrict__ forces, double *__restrict__ vir_atom)
+__global__ void __launch_bounds__(128)
+k_gather(int n_atoms, const int *__restrict__ offsets, const int *__restrict__ rev,
+         const typename V4<T>::type *__restrict__ vec, const T *__restrict__ fpair, const double *__restrict__ fw2,
+         double *__restrict__ forces, double *__restrict__ vir_atom)
 {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n_atoms) return;
-    double F[3] = {0, 0, 0}, W[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int p = offsets[j]; p < offsets[j + 1]; ++p) {
-        int q = rev[p];
-        typename V4<T>::type v = vec[p];
-        double fp[3] = {(double)fpair[3 * (size_t)p], (double)fpair[3 * (size_t)p + 1], (double)fpair[3 * (size_t)p + 2]};
-        double vv[3] = {(double)v.x, (double)v.y, (double)v.z};
-        for (int a = 0; a < 3; ++a) F[a] += fp[a] - (double)fpair[3 * (size_t)q + a];
-        if (f2) {
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kPairLanes, sub = threadIdx.x % kPairLanes;
+    PairSum<T> acc[12];  // F, then W row-major
+    const int p1 = j < n_atoms ? offsets[j + 1] : 0;
+    for (int p = j < n_atoms ? offsets[j] + sub : 0; p < p1; p += kPairLanes) {
+        const size_t q = 3 * (size_t)rev[p];
+        const typename V4<T>::type v = vec[p];
+        T fp[3], fq[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            fp[a] = fpair[3 * (size_t)p + a];
+            fq[a] = fpair[q + a];
+        }
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            acc[a].add(fp[a]);
+            acc[a].add(-fq[a]);
+        }
+        if (vir_atom) {
+#pragma unroll
             for (int a = 0; a < 3; ++a) {
-                F[a] += f2[3 * (size_t)p + a] - f2[3 * (size_t)q + a];
-                fp[a] += f2[3 * (size_t)p + a];
+                acc[3 + 3 * a].sub_product(fp[a], v.x);
+                acc[4 + 3 * a].sub_product(fp[a], v.y);
+                acc[5 + 3 * a].sub_product(fp[a], v.z);
             }
         }
-        for (int a = 0; a < 3; ++a)
-            for (int b = 0; b < 3; ++b) W[3 * a + b] -= fp[a] * vv[b];
     }
-    if (forces)
-        for (int a = 0; a < 3; ++a) forces[3 * (size_t)j + a] = F[a];
-    if (vir_atom)
-        for (int a = 0; a < 9; ++a) vir_atom[9 * (size_t)j + a] = W[a];
+#pragma unroll
+    for (int q = 0; q < 12; ++q) acc[q].reduce();
+    if (j >= n_atoms) return;
+    // lane `sub` writes entries sub and sub + 8
+#pragma unroll
+    for (int q = 0; q < 12; ++q) {
+        if (q % kPairLanes != sub) continue;
+        double v = acc[q].value();
+        // the two-body term's symmetric virial is stored xx yy zz yz xz xy
+        constexpr int kSym[12] = {0, 1, 2, 3, 8, 7, 8, 4, 6, 7, 6, 5};
+        if (fw2) v += fw2[9 * (size_t)j + kSym[q]];
+        if (q < 3) {
+            if (forces) forces[3 * (size_t)j + q] = v;
+        } else if (vir_atom) {
+            vir_atom[9 * (size_t)j + q - 3] = v;
+        }
+    }
 }
 
-// Per-configuration sums of local energies and atomic virials (block per config).
 // Energy (eps + eps2) and virial sums of each configuration, over chunks of
-// kCfgChunk atoms (block (c, k): atoms k kCfgChunk .. of configuration c) so
-// that a large configuration spreads over many SMs; k_config_final adds the
-// chunks in order (deterministic).
-constexpr int kCfgChunk = 2048;
+// atoms (block (c, k): atoms k chunk .. of configuration c), so that a large
+// configuration spreads over many SMs; with one chunk per configuration the
+// sums are final, else k_config_final adds the chunks (fixed order:
+// deterministic).  Also writes the local energies eps + eps2.  The FP64 pipe
+// bounds it: one atom per thread (256 atoms per chunk), then each warp sums
+// whole columns over the block (13 FP64 adds per column).  Chunks of 2048
+// where 256 would need too many blocks or partial sums (grid y is limited to
+// 65535; 2^20 chunks hold 84 MB).
+constexpr int kCfgThreads = 256;
 
-__global__ void k_config_part(int n_configs, int nchunk, const int *__restrict__ cfg_off,
-                              const double *__restrict__ eps, const double *__restrict__ eps2,
-                              const double *__restrict__ vir_atom, double *__restrict__ part)
+int config_chunk(int n_configs, int max_atoms)
 {
-    __shared__ double red[256][10];
-    const int c = blockIdx.x, k = blockIdx.y;
-    const int i0 = cfg_off[c] + k * kCfgChunk, i1e = cfg_off[c + 1];
-    const int i1 = i0 + kCfgChunk < i1e ? i0 + kCfgChunk : i1e;
-    double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        acc[0] += eps[i] + (eps2 ? eps2[i] : 0.0);
-        if (vir_atom)
-            for (int a = 0; a < 9; ++a) acc[1 + a] += vir_atom[9 * (size_t)i + a];
-    }
-    for (int a = 0; a < 10; ++a) red[threadIdx.x][a] = acc[a];
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if ((int)threadIdx.x < s)
-            for (int a = 0; a < 10; ++a) red[threadIdx.x][a] += red[threadIdx.x + s][a];
-        __syncthreads();
-    }
-    if (threadIdx.x < 10) part[((size_t)c * nchunk + k) * 10 + threadIdx.x] = red[0][threadIdx.x];
+    const long nchunk = ((long)max_atoms + kCfgThreads - 1) / kCfgThreads;
+    return nchunk <= 65535 && (nchunk <= 1 || nchunk * n_configs <= (1L << 20)) ? kCfgThreads : 2048;
 }
 
-__global__ void k_config_final(int n_configs, int nchunk, const double *__restrict__ part, double *__restrict__ energy,
-                               double *__restrict__ virial)
+__device__ __forceinline__ void config_store(int c, int a, double s, double *energy, double *virial)
 {
-    const long idx = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (idx >= 10L * n_configs) return;
-    const int c = (int)(idx / 10), a = (int)(idx % 10);
-    double s = 0.0;
-    for (int k = 0; k < nchunk; ++k) s += part[((size_t)c * nchunk + k) * 10 + a];
     if (a == 0) {
         if (energy) energy[c] = s;
     } else if (virial) {
-        virial[9 * c + a - 1] = s;
+        virial[9 * (size_t)c + a - 1] = s;
     }
 }
 
-__global__ void k_local_energy(int n_atoms, const double *__restrict__ eps, const double *__restrict__ eps2,
-                               double *__restrict__ out)
+__global__ void __launch_bounds__(kCfgThreads)
+k_config_part(int nchunk, int chunk, const int *__restrict__ cfg_off, const double *__restrict__ eps,
+              const double *__restrict__ eps2, const double *__restrict__ vir_atom, double *__restrict__ part,
+              double *__restrict__ energy, double *__restrict__ virial, double *__restrict__ local_e)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n_atoms) out[i] = eps[i] + (eps2 ? eps2[i] : 0.0);
+    __shared__ double red[10][kCfgThreads];
+    const int c = blockIdx.x, k = blockIdx.y;
+    const int i0 = cfg_off[c] + k * chunk, iend = cfg_off[c + 1], i1 = iend - i0 < chunk ? iend : i0 + chunk;
+    const int nq = vir_atom ? 10 : 1;
+    double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int i = i0 + (int)threadIdx.x; i < i1; i += kCfgThreads) {
+        const double e = eps[i] + (eps2 ? eps2[i] : 0.0);
+        if (local_e) local_e[i] = e;
+        acc[0] += e;
+        if (vir_atom)
+#pragma unroll
+            for (int a = 0; a < 9; ++a) acc[1 + a] += vir_atom[9 * (size_t)i + a];
+    }
+#pragma unroll
+    for (int a = 0; a < 10; ++a)
+        if (a < nq) red[a][threadIdx.x] = acc[a];
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int a = warp; a < nq; a += kCfgThreads / 32) {
+        double s = 0.0;
+#pragma unroll
+        for (int t = 0; t < kCfgThreads / 32; ++t) s += red[a][32 * t + lane];
+        s = warp_sum(s);
+        if (lane == 0) {
+            if (nchunk == 1) config_store(c, a, s, energy, virial);
+            else part[((size_t)c * nchunk + k) * 10 + a] = s;
+        }
+    }
+}
+
+// Block per configuration, warp per column: lanes over chunks.
+__global__ void __launch_bounds__(320)
+k_config_final(int nchunk, int nq, const double *__restrict__ part, double *__restrict__ energy,
+               double *__restrict__ virial)
+{
+    const int c = blockIdx.x, a = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (a >= nq) return;
+    double s = 0.0;
+    for (int k = lane; k < nchunk; k += 32) s += part[((size_t)c * nchunk + k) * 10 + a];
+    s = warp_sum(s);
+    if (lane == 0) config_store(c, a, s, energy, virial);
 }
 
 __global__ void k_pair_atoms(int n_atoms, const int *__restrict__ offsets, int *__restrict__ pair_i)
@@ -718,45 +844,48 @@ gap_status gap_twobody_table(const TwoBodyDev &tb, D4 *tab, cudaStream_t st)
     return gap_cuda_status(cudaGetLastError(), "k_twobody_table");
 }
 
-gap_status gap_twobody(int n, const PairList &pl, const TwoBodyDev &tb, double *f2, double *eps2, cudaStream_t st)
+gap_status gap_twobody(int n, const PairList &pl, const TwoBodyDev &tb, double *fw2, double *eps2, cudaStream_t st)
 {
     if (n == 0) return GAP_OK;
+    constexpr int kAtoms = 128 / kPairLanes;  // per block
     gap_count_launch();
-    k_twobody<<<(n + 127) / 128, 128, 0, st>>>(n, pl.offsets, pl.vec64, tb, f2, eps2);
+    k_twobody<<<(n + kAtoms - 1) / kAtoms, 128, 0, st>>>(n, pl.offsets, pl.vec64, tb, eps2, fw2);
     return gap_cuda_status(cudaGetLastError(), "k_twobody");
 }
 
 template <typename T>
-gap_status gap_gather(int n, const PairList &pl, const T *fpair, const double *f2, double *forces, double *vir_atom,
+gap_status gap_gather(int n, const PairList &pl, const T *fpair, const double *fw2, double *forces, double *vir_atom,
                       cudaStream_t st)
 {
     if (n == 0) return GAP_OK;
     const typename V4<T>::type *vec;
     if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
+    constexpr int kAtoms = 128 / kPairLanes;  // per block
     gap_count_launch();
-    k_gather<T><<<(n + 127) / 128, 128, 0, st>>>(n, pl.offsets, pl.rev, vec, fpair, f2, forces, vir_atom);
+    k_gather<T><<<(n + kAtoms - 1) / kAtoms, 128, 0, st>>>(n, pl.offsets, pl.rev, vec, fpair, fw2, forces, vir_atom);
     return gap_cuda_status(cudaGetLastError(), "k_gather");
 }
 
-gap_status gap_config_sums(int n_configs, const int *cfg_off, int max_atoms, const double *eps, const double *eps2,
-                           const double *vir_atom, double *energy, double *virial, double *part, cudaStream_t st)
+size_t gap_config_part_doubles(int n_configs, int max_atoms)
 {
-    if (n_configs == 0) return GAP_OK;
-    const int nchunk = max_atoms > kCfgChunk ? (max_atoms + kCfgChunk - 1) / kCfgChunk : 1;
-    gap_count_launch();
-    k_config_part<<<dim3(n_configs, nchunk), 256, 0, st>>>(n_configs, nchunk, cfg_off, eps, eps2, vir_atom, part);
-    GAP_TRY_CUDA(cudaGetLastError());
-    gap_count_launch();
-    k_config_final<<<(unsigned)((10L * n_configs + 255) / 256), 256, 0, st>>>(n_configs, nchunk, part, energy, virial);
-    return gap_cuda_status(cudaGetLastError(), "k_config_final");
+    const int chunk = config_chunk(n_configs, max_atoms);
+    return 10 * (size_t)n_configs * (max_atoms > chunk ? (max_atoms + chunk - 1) / chunk : 1);
 }
 
-gap_status gap_local_energy(int n, const double *eps, const double *eps2, double *out, cudaStream_t st)
+gap_status gap_config_sums(int n_configs, const int *cfg_off, int max_atoms, const double *eps, const double *eps2,
+                           const double *vir_atom, double *energy, double *virial, double *local_e, double *part,
+                           cudaStream_t st)
 {
-    if (n == 0) return GAP_OK;
+    if (n_configs == 0) return GAP_OK;
+    const int chunk = config_chunk(n_configs, max_atoms), nchunk = max_atoms > chunk ? (max_atoms + chunk - 1) / chunk : 1;
     gap_count_launch();
-    k_local_energy<<<(n + 127) / 128, 128, 0, st>>>(n, eps, eps2, out);
-    return gap_cuda_status(cudaGetLastError(), "k_local_energy");
+    k_config_part<<<dim3(n_configs, nchunk), kCfgThreads, 0, st>>>(nchunk, chunk, cfg_off, eps, eps2, vir_atom, part,
+                                                                   energy, virial, local_e);
+    GAP_TRY_CUDA(cudaGetLastError());
+    if (nchunk == 1) return GAP_OK;
+    gap_count_launch();
+    k_config_final<<<n_configs, 320, 0, st>>>(nchunk, vir_atom ? 10 : 1, part, energy, virial);
+    return gap_cuda_status(cudaGetLastError(), "k_config_final");
 }
 
 gap_status gap_pair_atoms(int n, const PairList &pl, int *pair_i, cudaStream_t st)

@@ -31,21 +31,18 @@ gap_status gap_chain(const SoapGeom &g, int n, const T *gvec, const T *wsum, con
 template <typename T>
 gap_status gap_pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *pair_i, const int *species,
                          const T *Gam, T *fpair, cudaStream_t st);
-// Two-body term in FP64: per-pair half derivatives f2[P][3], half energies per atom eps2.
-gap_status gap_twobody(int n, const PairList &pl, const TwoBodyDev &tb, double *f2, double *eps2, cudaStream_t st);
-// Forces and atomic virials from the per-pair derivatives fpair (and f2 if not NULL).
+// Two-body term in FP64: half energies per atom eps2 and, if fw2 is not NULL,
+// each atom's force and symmetric virial fw2[N][9] (F; xx yy zz yz xz xy).
+gap_status gap_twobody(int n, const PairList &pl, const TwoBodyDev &tb, double *fw2, double *eps2, cudaStream_t st);
+// Forces and atomic virials from the per-pair derivatives fpair (plus fw2 if not NULL).
 template <typename T>
-gap_status gap_gather(int n, const PairList &pl, const T *fpair, const double *f2, double *forces, double *vir_atom,
+gap_status gap_gather(int n, const PairList &pl, const T *fpair, const double *fw2, double *forces, double *vir_atom,
                       cudaStream_t st);
-// Per-configuration energy and virial sums; max_atoms bounds the atoms of a
-// configuration, part holds 10 * n_configs * ceil(max_atoms / 2048) doubles
-// (gap_config_part_doubles).
+// Per-configuration energy and virial sums, and the local energies eps + eps2
+// if local_e is not NULL; max_atoms bounds the atoms of a configuration, part
+// holds gap_config_part_doubles doubles.
 gap_status gap_config_sums(int n_configs, const int *cfg_off, int max_atoms, const double *eps, const double *eps2,
-                           const double *vir_atom, double *energy, double *virial, double *part, cudaStream_t st);
-inline size_t gap_config_part_doubles(int n_configs, int max_atoms)
-{
-    const int nchunk = max_atoms > 2048 ? (max_atoms + 2047) / 2048 : 1;
-    return 10 * (size_t)n_configs * nchunk;
-}
-gap_status gap_local_energy(int n, const double *eps, const double *eps2, double *out, cudaStream_t st);
+                           const double *vir_atom, double *energy, double *virial, double *local_e, double *part,
+                           cudaStream_t st);
+size_t gap_config_part_doubles(int n_configs, int max_atoms);
 gap_status gap_pair_atoms(int n, const PairList &pl, int *pair_i, cudaStream_t st);
