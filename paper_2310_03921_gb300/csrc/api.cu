@@ -285,7 +285,7 @@ static float bf16_to_float(uint16_t h)
 
 struct Workspace {
     NbrWork nbr;
-    DBuf pos, spec, pair_i, coef, phat, pnorm, gp_of_atom, flag, fpos, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
+    DBuf pos, spec, coef, phat, pnorm, gp_of_atom, flag, fpos, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
         W, eps_part, Gam, fpair, fw2, forces, vir_atom, cfgpart, energy, virial, local, err, A_hi, A_lo, t_row, W_hi, W_lo,
         epart_f, wpart_f, Gs, outbuf, kA, kAhi, kAlo, kt, ksrc, kseg, kdest, segstart, outrow, Wp, kq, P, Kbuf, A_mid, W_mid,
         kAmid, phatc, pnormc, hfull, kV;
@@ -296,7 +296,7 @@ struct Workspace {
     void release()
     {
         nbr.release();
-        DBuf *bs[] = {&pos, &spec, &pair_i, &coef, &phat, &pnorm, &gp_of_atom, &flag, &fpos, &scan_tmp, &rows,
+        DBuf *bs[] = {&pos, &spec, &coef, &phat, &pnorm, &gp_of_atom, &flag, &fpos, &scan_tmp, &rows,
                       &counts, &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &fw2, &forces, &vir_atom, &cfgpart, &energy,
                       &virial, &local, &err, &A_hi, &A_lo, &t_row, &W_hi, &W_lo, &epart_f, &wpart_f, &Gs, &outbuf,
                       &kA, &kAhi, &kAlo, &kt, &ksrc, &kseg, &kdest, &segstart, &outrow, &Wp, &kq, &P, &Kbuf, &A_mid, &W_mid,
@@ -800,8 +800,6 @@ static gap_status run_descriptor(gap_soap *soap, Workspace &w, const gap_batch *
     GAP_TRY(stage_inputs(w, b, g.S, &pos, &spec, st));
     GAP_TRY(gap_neighbours(w.nbr, b, pos, g.rc, st));
     const PairList &pl = w.nbr.pairs;
-    GAP_TRY(w.pair_i.ensure(sizeof(int) * (size_t)pl.n_pairs));
-    GAP_TRY(gap_pair_atoms(n, pl, w.pair_i.as<int>(), st));
     gap_prof_end(ST_NEIGHBOURS, st);
     GAP_TRY(w.coef.ensure(sizeof(T) * (size_t)n * g.GA * g.N * g.LM));
     GAP_TRY(w.phat.ensure(sizeof(T) * (size_t)n * g.D));
@@ -1356,7 +1354,7 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
         gap_prof_end(ST_CHAIN, st);
         GAP_TRY(w.fpair.ensure(sizeof(T) * 3 * (size_t)pl.n_pairs));
         gap_prof_begin(ST_PAIRFORCE, st);
-        GAP_TRY(gap_pairforce<T>(g, tab_of<T>(soap), pl, w.pair_i.as<int>(), spec, w.Gam.as<T>(), w.fpair.as<T>(), st));
+        GAP_TRY(gap_pairforce<T>(g, tab_of<T>(soap), pl, spec, w.Gam.as<T>(), w.fpair.as<T>(), st));
         gap_prof_end(ST_PAIRFORCE, st);
     }
     double *eps2 = nullptr, *fw2 = nullptr;

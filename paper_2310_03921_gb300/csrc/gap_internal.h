@@ -88,7 +88,7 @@ struct PairList {
     int n_pairs;      // host: pairs the arrays hold (a capacity in graph mode)
     const int *count; // device: pairs of the current build (<= n_pairs)
     int *offsets;     // [N+1]
-    int *j;           // [P]
+    int *i, *j;       // [P] the pair's two atoms
     int *rev;         // [P] index of the reverse pair (j -> i, -shift)
     D4 *vec64;        // [P] (dx, dy, dz, r)
     float4 *vec32;    // [P]

@@ -19,11 +19,14 @@ namespace {
 
 constexpr int kShiftBias = 128;
 
-__device__ __forceinline__ long long pair_key(int j, int sx, int sy, int sz)
+// A lattice shift packed into 24 bits, ordered as (sx, sy, sz).
+__device__ __forceinline__ int shift_code(int sx, int sy, int sz)
 {
-    return ((long long)j << 24) | ((long long)(sx + kShiftBias) << 16) | ((long long)(sy + kShiftBias) << 8) |
-           (long long)(sz + kShiftBias);
+    return ((sx + kShiftBias) << 16) | ((sy + kShiftBias) << 8) | (sz + kShiftBias);
 }
+constexpr int kNoShift = (kShiftBias << 16) | (kShiftBias << 8) | kShiftBias;
+
+__device__ __forceinline__ long long pair_key(int j, int code) { return ((long long)j << 24) | (long long)code; }
 
 __device__ __forceinline__ int config_of(const int *offsets, int n_configs, int i)
 {
@@ -37,7 +40,7 @@ __device__ __forceinline__ int config_of(const int *offsets, int n_configs, int 
 }
 
 __global__ void k_bin(int n, const double *__restrict__ pos, const int *__restrict__ offsets, int n_configs,
-                      const CellGeom *__restrict__ geo, double *__restrict__ frac, float4 *__restrict__ frac32,
+                      const CellGeom *__restrict__ geo, D4 *__restrict__ cart, float4 *__restrict__ cart32,
                       int *__restrict__ atom_cfg, int *__restrict__ atom_bin, int *__restrict__ bin_count)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -46,6 +49,7 @@ __global__ void k_bin(int n, const double *__restrict__ pos, const int *__restri
     const CellGeom &g = geo[c];
     double p[3] = {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]};
     int b[3];
+    double fr[3];
     for (int k = 0; k < 3; ++k) {
         double s = p[0] * g.inv[k] + p[1] * g.inv[3 + k] + p[2] * g.inv[6 + k];
         if (g.pbc[k]) {
@@ -54,14 +58,18 @@ __global__ void k_bin(int n, const double *__restrict__ pos, const int *__restri
         }
         int bk = (int)floor(s * g.nb[k]);
         bk = bk < 0 ? 0 : (bk >= g.nb[k] ? g.nb[k] - 1 : bk);
-        frac[3 * i + k] = s;
+        fr[k] = s;
         b[k] = bk;
     }
     int gb = g.bin0 + (b[0] * g.nb[1] + b[1]) * g.nb[2] + b[2];
-    // w = 1 marks coordinates within [-4, 4] (always so along periodic
-    // directions), where the FP32 copy is close enough for the prefilter
-    const bool near = fabs(frac[3 * i]) <= 4.0 && fabs(frac[3 * i + 1]) <= 4.0 && fabs(frac[3 * i + 2]) <= 4.0;
-    frac32[i] = make_float4((float)frac[3 * i], (float)frac[3 * i + 1], (float)frac[3 * i + 2], near ? 1.f : 0.f);
+    // the wrapped atom in Cartesian coordinates; w = 1 marks fractional
+    // coordinates within [-4, 4] (always so along periodic directions), where
+    // the FP32 copy is close enough for the prefilter
+    const bool near = fabs(fr[0]) <= 4.0 && fabs(fr[1]) <= 4.0 && fabs(fr[2]) <= 4.0;
+    double x[3];
+    for (int a = 0; a < 3; ++a) x[a] = fr[0] * g.cell[a] + fr[1] * g.cell[3 + a] + fr[2] * g.cell[6 + a];
+    cart[i] = D4{x[0], x[1], x[2], near ? 1.0 : 0.0};
+    cart32[i] = make_float4((float)x[0], (float)x[1], (float)x[2], near ? 1.f : 0.f);
     atom_cfg[i] = c;
     atom_bin[i] = gb;
     atomicAdd(&bin_count[gb], 1);
@@ -77,84 +85,111 @@ __global__ void k_scatter(int n, const int *__restrict__ atom_bin, const int *__
     bin_atoms[bin_start[gb] + slot] = i;
 }
 
+// floor(a / n) for n > 0.
+__device__ __forceinline__ int floor_div(int a, int n) { return a >= 0 ? a / n : -((n - 1 - a) / n); }
+
+// sqrt(x) to the last bit or so for 0 < x < rc^2: the FP32 reciprocal square
+// root and two Newton steps on the root (errors 2^-22, 2^-43, 2^-64 before
+// rounding); CUDA's FP64 square root takes about three times the FP64
+// instructions.
+__device__ __forceinline__ double sqrt_newton(double x)
+{
+    if (!(x > 1e-30)) return sqrt(x);
+    const double y = (double)rsqrtf((float)x), h = 0.5 * y;
+    double r = x * y;
+    r = fma(fma(-r, r, x), h, r);
+    return fma(fma(-r, r, x), h, r);
+}
+
+// Per warp: the non-empty bins of the current chunk of 32 bins around the
+// atom (their lattice shifts in FP64 and FP32, the offset taking a candidate's
+// number to its slot of bin_atoms, the packed shift) and the candidates that
+// wait for the exact test.
+constexpr int kNbrQueue = 64;
+struct NbrScan {
+    double T[32][3];
+    float4 T32[32];
+    int first[32], code[32];
+    int2 queue[kNbrQueue];  // (atom, bin slot)
+};
+
 // Visits every candidate (j, shift) of atom i, one warp per atom, 32 at a
-// time; f(hit, j, sx, sy, sz, v, r2) is called by every lane with uniform
-// control flow (it may use warp votes), hit marking a pair within the
-// cutoff.  The bins around the atom ((2R+1)^3, 32 at a time: lane b resolves
-// bin b's periodic shift and atom range) are flattened into one run of
-// candidates, which the lanes take 32 at a time through an FP32 prefilter:
-// the cutoff widened by 5 10^-4 rc + 10^-5 of the cell's edge lengths, far
-// beyond the error of the FP32 fractional coordinates (|s| <= 4: ~5 10^-7
-// of the edges; atoms outside that range, beyond the box of a non-periodic
-// direction, skip it).  The survivors (~15%) queue in shared memory and
-// take the exact FP64 test 32 at a time, so that every FP64 instruction works
-// on a full warp (GB300's FP64 pipe takes about 64 cycles per warp
-// instruction, whatever the active lanes).  The pair set is the FP64 one.
+// time; f(hit, j, code, v, r2) is called by every lane with uniform control
+// flow (it may use warp votes), hit marking a pair within the cutoff.  The
+// bins around the atom ((2R+1)^3, 32 at a time: lane b resolves bin b's
+// periodic shift and atom range) are flattened into one run of candidates,
+// which the lanes take 32 at a time through an FP32 prefilter: the cutoff
+// widened by 5 10^-4 rc + 3 10^-5 of the cell's edge lengths, beyond the error
+// of the FP32 coordinates and shifts (~4 10^-6 of the edges at 60 images;
+// atoms far outside the box of a non-periodic direction skip it).  The
+// survivors (~15%) queue in shared memory and take the exact FP64 test 32 at
+// a time.  GB300's FP64 pipe takes about 64 cycles per warp instruction
+// whatever the active lanes, and bounded this scan: so every FP64 instruction
+// works on a full warp, the exact test is r = (x_j - x_i) + T on wrapped
+// Cartesian coordinates (six additions; the reverse pair gets exactly the
+// negative), the shifts T are formed once per bin (not at all for an atom
+// whose bins need none), and bin wrapping is integer arithmetic.  The pair
+// set is the FP64 one.  (With FP64 fractional coordinates, divisions and
+// square roots a step of 32768 atoms took 0.13 ms longer, 512 four-species
+// boxes 0.4 ms.)
 // SURE (counting only): a candidate whose FP32 distance is below the cutoff
 // narrowed by the same margin is inside for FP64 too; it is counted in
 // sure_hits without the exact test, which then sees only the thin shell
 // between the two bounds.
-constexpr int kNbrQueue = 64;
-
 template <bool SURE, typename F>
-__device__ __forceinline__ void warp_candidates(int i, int lane, const double *__restrict__ frac,
-                                                const float4 *__restrict__ frac32, const int *__restrict__ atom_cfg,
-                                                const CellGeom *__restrict__ geo, const int *__restrict__ bin_start,
-                                                const int *__restrict__ bin_atoms, int2 *__restrict__ queue, F &&f,
-                                                int &sure_hits)
+__device__ __forceinline__ void warp_candidates(int i, int lane, const D4 *__restrict__ cart,
+                                                const float4 *__restrict__ cart32, const int *__restrict__ atom_cfg,
+                                                const int *__restrict__ atom_bin, const CellGeom *__restrict__ geo,
+                                                const int *__restrict__ bin_start,
+                                                const int *__restrict__ bin_atoms, NbrScan &sc, F &&f, int &sure_hits)
 {
     const CellGeom &g = geo[atom_cfg[i]];
-    const double si0 = frac[3 * i], si1 = frac[3 * i + 1], si2 = frac[3 * i + 2];
-    const float4 s32 = frac32[i];
-    int b[3];
-    const double si[3] = {si0, si1, si2};
-    for (int k = 0; k < 3; ++k) {
-        int bk = (int)floor(si[k] * g.nb[k]);
-        b[k] = bk < 0 ? 0 : (bk >= g.nb[k] ? g.nb[k] - 1 : bk);
-    }
+    const D4 xi = cart[i];
+    const float4 xi32 = cart32[i];
+    const int nb0 = g.nb[0], nb1 = g.nb[1], nb2 = g.nb[2], ib = atom_bin[i] - g.bin0;
+    const int b2 = ib % nb2, b1 = (ib / nb2) % nb1, b0 = ib / (nb2 * nb1);
+    const double rc2 = g.rc2;
+    const float loose = g.rc2_loose, tight = g.rc2_tight;
     const unsigned lt = (1u << lane) - 1u;
     int qn = 0;  // queued candidates
     // the exact test of queue[0 .. cnt) (cnt <= 32), one per lane
     auto drain = [&](int cnt) {
         bool hit = false;
-        int j = -1, sx = 0, sy = 0, sz = 0;
+        int j = -1, code = 0;
         double v[3] = {0.0, 0.0, 0.0}, r2 = 0.0;
         if (lane < cnt) {
-            const int2 e = queue[lane];
+            const int2 e = sc.queue[lane];
             j = e.x;
-            sx = ((e.y >> 16) & 0xff) - 128;
-            sy = ((e.y >> 8) & 0xff) - 128;
-            sz = (e.y & 0xff) - 128;
-            const double ds0 = frac[3 * j] + sx - si0, ds1 = frac[3 * j + 1] + sy - si1, ds2 = frac[3 * j + 2] + sz - si2;
-            for (int a = 0; a < 3; ++a) v[a] = ds0 * g.cell[a] + ds1 * g.cell[3 + a] + ds2 * g.cell[6 + a];
+            code = sc.code[e.y];
+            const D4 xj = cart[j];
+            v[0] = (xj.x - xi.x) + sc.T[e.y][0];
+            v[1] = (xj.y - xi.y) + sc.T[e.y][1];
+            v[2] = (xj.z - xi.z) + sc.T[e.y][2];
             r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
-            hit = r2 < g.rc2;
+            hit = r2 < rc2;
         }
-        f(hit, j, sx, sy, sz, v, r2);
+        f(hit, j, code, v, r2);
     };
     const int wx = 2 * g.R[0] + 1, wy = 2 * g.R[1] + 1, wz = 2 * g.R[2] + 1, nbins = wx * wy * wz;
-    for (int b0 = 0; b0 < nbins; b0 += 32) {
-        int st = 0, cnt = 0, shift = 0;
-        const int bb = b0 + lane;
+    for (int c0b = 0; c0b < nbins; c0b += 32) {
+        int st = 0, cnt = 0, sx = 0, sy = 0, sz = 0;
+        const int bb = c0b + lane;
         if (bb < nbins) {
-            const int dz = bb % wz - g.R[2], dy = (bb / wz) % wy - g.R[1], dx = bb / (wz * wy) - g.R[0];
-            int nx = b[0] + dx, ny = b[1] + dy, nz = b[2] + dz, sxl = 0, syl = 0, szl = 0;
+            int nz = b2 + bb % wz - g.R[2], ny = b1 + (bb / wz) % wy - g.R[1], nx = b0 + bb / (wz * wy) - g.R[0];
             bool ok = true;
-            if (g.pbc[0]) { sxl = (int)floor((double)nx / g.nb[0]); nx -= sxl * g.nb[0]; }
-            else ok = ok && nx >= 0 && nx < g.nb[0];
-            if (g.pbc[1]) { syl = (int)floor((double)ny / g.nb[1]); ny -= syl * g.nb[1]; }
-            else ok = ok && ny >= 0 && ny < g.nb[1];
-            if (g.pbc[2]) { szl = (int)floor((double)nz / g.nb[2]); nz -= szl * g.nb[2]; }
-            else ok = ok && nz >= 0 && nz < g.nb[2];
+            if (g.pbc[0]) { sx = floor_div(nx, nb0); nx -= sx * nb0; }
+            else ok = ok && nx >= 0 && nx < nb0;
+            if (g.pbc[1]) { sy = floor_div(ny, nb1); ny -= sy * nb1; }
+            else ok = ok && ny >= 0 && ny < nb1;
+            if (g.pbc[2]) { sz = floor_div(nz, nb2); nz -= sz * nb2; }
+            else ok = ok && nz >= 0 && nz < nb2;
             if (ok) {
-                const int gb = g.bin0 + (nx * g.nb[1] + ny) * g.nb[2] + nz;
+                const int gb = g.bin0 + (nx * nb1 + ny) * nb2 + nz;
                 st = bin_start[gb];
                 cnt = bin_start[gb + 1] - st;
             }
-            shift = ((sxl + 128) << 16) | ((syl + 128) << 8) | (szl + 128);
         }
-        // exclusive prefix of the bin sizes: candidate c of this chunk lies in
-        // the last bin whose prefix is <= c
+        // exclusive prefix of the bin sizes
         int pre = cnt;
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, pre, o);
@@ -162,34 +197,42 @@ __device__ __forceinline__ void warp_candidates(int i, int lane, const double *_
         }
         const int total = __shfl_sync(0xffffffffu, pre, 31);
         pre -= cnt;
+        const unsigned full = __ballot_sync(0xffffffffu, cnt > 0);
+        const int code = shift_code(sx, sy, sz);
+        const bool shifted = __ballot_sync(0xffffffffu, cnt > 0 && code != kNoShift) != 0;
+        __syncwarp();  // the previous chunk's drain has read the tables
+        if (cnt > 0) {
+            const int slot = __popc(full & lt);
+            double T[3] = {0.0, 0.0, 0.0};
+            if (shifted)
+                for (int a = 0; a < 3; ++a)
+                    T[a] = (double)sx * g.cell[a] + (double)sy * g.cell[3 + a] + (double)sz * g.cell[6 + a];
+            for (int a = 0; a < 3; ++a) sc.T[slot][a] = T[a];
+            sc.T32[slot] = make_float4((float)T[0], (float)T[1], (float)T[2], 0.f);
+            sc.first[slot] = st - pre;
+            sc.code[slot] = code;
+        }
+        __syncwarp();
         for (int c0 = 0; c0 < total; c0 += 32) {
             const int c = c0 + lane;
-            int lo = 0;  // binary search for the bin of c
-            for (int step = 16; step; step >>= 1) {
-                const int p = __shfl_sync(0xffffffffu, pre, lo + step);
-                if (c >= p && lo + step < 32) lo += step;
-            }
-            const int bst = __shfl_sync(0xffffffffu, st, lo), bpre = __shfl_sync(0xffffffffu, pre, lo);
-            const int bsh = __shfl_sync(0xffffffffu, shift, lo);
+            // the bin of candidate c: bins that start at or before it, from
+            // the starts in this window and the number before it
+            const unsigned heads =
+                __reduce_or_sync(0xffffffffu, cnt > 0 && pre >= c0 && pre < c0 + 32 ? 1u << (pre - c0) : 0u);
+            const int slot = __popc(__ballot_sync(0xffffffffu, cnt > 0 && pre < c0)) +
+                             __popc(heads & (lt | (1u << lane))) - 1;
             bool pass = false, sure = false;
             int j = -1;
             if (c < total) {
-                j = bin_atoms[bst + (c - bpre)];
-                const int sx = ((bsh >> 16) & 0xff) - 128, sy = ((bsh >> 8) & 0xff) - 128, sz = (bsh & 0xff) - 128;
-                if (!(j == i && sx == 0 && sy == 0 && sz == 0)) {
+                j = bin_atoms[sc.first[slot] + c];
+                if (!(j == i && sc.code[slot] == kNoShift)) {
                     pass = true;
-                    const float4 f32 = frac32[j];
-                    if (s32.w != 0.f && f32.w != 0.f) {
-                        const float d0 = (f32.x - s32.x) + (float)sx, d1 = (f32.y - s32.y) + (float)sy,
-                                    d2 = (f32.z - s32.z) + (float)sz;
-                        float r2f = 0.f;
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            const float va = d0 * g.cell32[a] + d1 * g.cell32[3 + a] + d2 * g.cell32[6 + a];
-                            r2f += va * va;
-                        }
-                        pass = r2f < g.rc2_loose;
-                        if (SURE && r2f < g.rc2_tight) {
+                    const float4 xj = cart32[j], T = sc.T32[slot];
+                    if (xi32.w != 0.f && xj.w != 0.f) {
+                        const float d0 = (xj.x - xi32.x) + T.x, d1 = (xj.y - xi32.y) + T.y, d2 = (xj.z - xi32.z) + T.z;
+                        const float r2f = d0 * d0 + d1 * d1 + d2 * d2;
+                        pass = r2f < loose;
+                        if (SURE && r2f < tight) {
                             sure = true;
                             pass = false;
                         }
@@ -198,35 +241,38 @@ __device__ __forceinline__ void warp_candidates(int i, int lane, const double *_
             }
             if (SURE) sure_hits += __popc(__ballot_sync(0xffffffffu, sure));
             const unsigned pm = __ballot_sync(0xffffffffu, pass);
-            if (pass) queue[qn + __popc(pm & lt)] = make_int2(j, bsh);
+            if (pass) sc.queue[qn + __popc(pm & lt)] = make_int2(j, slot);
             qn += __popc(pm);
             __syncwarp();
             if (qn >= 32) {
                 drain(32);
                 __syncwarp();
                 qn -= 32;
-                if (lane < qn) queue[lane] = queue[32 + lane];
+                if (lane < qn) sc.queue[lane] = sc.queue[32 + lane];
                 __syncwarp();
             }
         }
+        if (qn > 0) {  // before the next chunk's tables
+            drain(qn);
+            qn = 0;
+        }
     }
-    if (qn > 0) drain(qn);
 }
 
 constexpr int kNbrWarps = 4;   // warps (atoms) per block
 constexpr int kNbrSort = 128;   // pairs per atom sorted in shared memory
 
 __global__ void __launch_bounds__(32 * kNbrWarps)
-k_count_warp(int n, const double *__restrict__ frac, const float4 *__restrict__ frac32,
-             const int *__restrict__ atom_cfg, const CellGeom *__restrict__ geo, const int *__restrict__ bin_start,
-             const int *__restrict__ bin_atoms, int *__restrict__ counts)
+k_count_warp(int n, const D4 *__restrict__ cart, const float4 *__restrict__ cart32,
+             const int *__restrict__ atom_cfg, const int *__restrict__ atom_bin, const CellGeom *__restrict__ geo,
+             const int *__restrict__ bin_start, const int *__restrict__ bin_atoms, int *__restrict__ counts)
 {
-    __shared__ int2 queue[kNbrWarps][kNbrQueue];
+    __shared__ NbrScan scan[kNbrWarps];
     const int i = blockIdx.x * kNbrWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (i >= n) return;
     int c = 0, sure = 0;
-    warp_candidates<true>(i, lane, frac, frac32, atom_cfg, geo, bin_start, bin_atoms, queue[threadIdx.x >> 5],
-                          [&](bool hit, int, int, int, int, const double *, double) {
+    warp_candidates<true>(i, lane, cart, cart32, atom_cfg, atom_bin, geo, bin_start, bin_atoms, scan[threadIdx.x >> 5],
+                          [&](bool hit, int, int, const double *, double) {
                               c += __popc(__ballot_sync(0xffffffffu, hit));
                           },
                           sure);
@@ -237,15 +283,15 @@ k_count_warp(int n, const double *__restrict__ frac, const float4 *__restrict__ 
 // placed by rank (keys are distinct), or, beyond kNbrSort pairs, written in
 // scan order and insertion-sorted by one lane.
 __global__ void __launch_bounds__(32 * kNbrWarps)
-k_fill_warp(int n, const double *__restrict__ frac, const float4 *__restrict__ frac32,
-            const int *__restrict__ atom_cfg, const CellGeom *__restrict__ geo, const int *__restrict__ bin_start,
-            const int *__restrict__ bin_atoms, const int *__restrict__ offsets, int cap,
-            long long *__restrict__ keys, int *__restrict__ nbr_j, D4 *__restrict__ vec64,
-            float4 *__restrict__ vec32, int *__restrict__ err)
+k_fill_warp(int n, const D4 *__restrict__ cart, const float4 *__restrict__ cart32,
+            const int *__restrict__ atom_cfg, const int *__restrict__ atom_bin, const CellGeom *__restrict__ geo,
+            const int *__restrict__ bin_start, const int *__restrict__ bin_atoms, const int *__restrict__ offsets,
+            int cap, long long *__restrict__ keys, int *__restrict__ pair_i, int *__restrict__ nbr_j,
+            D4 *__restrict__ vec64, float4 *__restrict__ vec32, int *__restrict__ err)
 {
-    __shared__ long long skey[kNbrWarps][kNbrSort];
+    __shared__ __align__(16) long long skey[kNbrWarps][kNbrSort];
     __shared__ D4 svec[kNbrWarps][kNbrSort];
-    __shared__ int2 queue[kNbrWarps][kNbrQueue];
+    __shared__ NbrScan scan[kNbrWarps];
     const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int i = blockIdx.x * kNbrWarps + wi;
     if (i >= n) return;
@@ -257,14 +303,14 @@ k_fill_warp(int n, const double *__restrict__ frac, const float4 *__restrict__ f
     const bool local = np <= kNbrSort;
     int w = 0;  // pairs found so far
     int no_sure = 0;
-    warp_candidates<false>(i, lane, frac, frac32, atom_cfg, geo, bin_start, bin_atoms, queue[wi],
-                    [&](bool hit, int j, int sx, int sy, int sz, const double *v, double r2) {
+    warp_candidates<false>(i, lane, cart, cart32, atom_cfg, atom_bin, geo, bin_start, bin_atoms, scan[wi],
+                    [&](bool hit, int j, int code, const double *v, double r2) {
                         const unsigned m = __ballot_sync(0xffffffffu, hit);
                         if (hit) {
                             const int pos = w + __popc(m & ((1u << lane) - 1u));
                             if (pos < np) {
-                                const long long key = pair_key(j, sx, sy, sz);
-                                const D4 d{v[0], v[1], v[2], sqrt(r2)};
+                                const long long key = pair_key(j, code);
+                                const D4 d{v[0], v[1], v[2], sqrt_newton(r2)};
                                 if (local) {
                                     skey[wi][pos] = key;
                                     svec[wi][pos] = d;
@@ -285,11 +331,16 @@ k_fill_warp(int n, const double *__restrict__ frac, const float4 *__restrict__ f
         __syncwarp();
         for (int e = lane; e < np; e += 32) {
             const long long k = skey[wi][e];
-            int rank = 0;
-            for (int e2 = 0; e2 < np; ++e2) rank += skey[wi][e2] < k ? 1 : 0;
+            int rank = 0, e2 = 0;
+            for (; e2 + 2 <= np; e2 += 2) {  // two keys per 16-byte load
+                const longlong2 k2 = *reinterpret_cast<const longlong2 *>(&skey[wi][e2]);
+                rank += (k2.x < k ? 1 : 0) + (k2.y < k ? 1 : 0);
+            }
+            if (e2 < np) rank += skey[wi][e2] < k ? 1 : 0;
             const D4 d = svec[wi][e];
             keys[p0 + rank] = k;
             vec64[p0 + rank] = d;
+            pair_i[p0 + rank] = i;
             nbr_j[p0 + rank] = (int)(k >> 24);
             vec32[p0 + rank] = make_float4((float)d.x, (float)d.y, (float)d.z, (float)d.w);
         }
@@ -312,6 +363,7 @@ k_fill_warp(int n, const double *__restrict__ frac, const float4 *__restrict__ f
     }
     __syncwarp();
     for (int a = p0 + lane; a < p1; a += 32) {
+        pair_i[a] = i;
         nbr_j[a] = (int)(keys[a] >> 24);
         const D4 v = vec64[a];
         vec32[a] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
@@ -345,7 +397,7 @@ __global__ void k_reverse(int n, const int *__restrict__ offsets, const long lon
         int j = (int)(k >> 24);
         int sx = (int)((k >> 16) & 255) - kShiftBias, sy = (int)((k >> 8) & 255) - kShiftBias,
             sz = (int)(k & 255) - kShiftBias;
-        long long want = pair_key(i, -sx, -sy, -sz);
+        long long want = pair_key(i, shift_code(-sx, -sy, -sz));
         int lo = offsets[j], hi = offsets[j + 1] - 1, found = -1;
         while (lo <= hi) {
             int mid = (lo + hi) >> 1;
@@ -476,14 +528,13 @@ gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom
         for (int k = 0; k < 9; ++k) {
             g.cell[k] = m[k];
             g.inv[k] = inv[k];
-            g.cell32[k] = (float)m[k];
         }
         g.rc2 = rc * rc;
-        // FP32 fractional coordinates carry ~1.2e-7 of the cell per component:
-        // a bound well above that error in Cartesian length
+        // FP32 coordinates and shifts carry ~6e-8 of their size, up to 60 cell
+        // edges, per component: a bound above that error
         double span = 0.0;
         for (int k = 0; k < 3; ++k) span += std::sqrt(m[3 * k] * m[3 * k] + m[3 * k + 1] * m[3 * k + 1] + m[3 * k + 2] * m[3 * k + 2]);
-        const double rl = rc * (1.0 + 5e-4) + 1e-5 * span, rt = rc * (1.0 - 5e-4) - 1e-5 * span;
+        const double rl = rc * (1.0 + 5e-4) + 3e-5 * span, rt = rc * (1.0 - 5e-4) - 3e-5 * span;
         g.rc2_loose = (float)(rl * rl);
         g.rc2_tight = rt > 0.0 ? (float)(rt * rt) : 0.f;
         g.bin0 = n_bins;
@@ -515,7 +566,7 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, d
     int gridN = (n + T - 1) / T;
     if (n > 0) {
         gap_count_launch();
-        k_bin<<<gridN, T, 0, st>>>(n, d_pos, w.cfg_offsets, b->n_configs, w.geo, w.frac, w.frac32, w.atom_cfg,
+        k_bin<<<gridN, T, 0, st>>>(n, d_pos, w.cfg_offsets, b->n_configs, w.geo, w.cart, w.cart32, w.atom_cfg,
                                    w.atom_bin, w.bin_count);
         GAP_TRY_CUDA(cudaGetLastError());
     }
@@ -526,8 +577,8 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, d
         GAP_TRY_CUDA(cudaGetLastError());
         gap_count_launch();
         const int gridW = (n + kNbrWarps - 1) / kNbrWarps;
-        k_count_warp<<<gridW, 32 * kNbrWarps, 0, st>>>(n, w.frac, w.frac32, w.atom_cfg, w.geo, w.bin_start,
-                                                       w.bin_atoms, w.counts);
+        k_count_warp<<<gridW, 32 * kNbrWarps, 0, st>>>(n, w.cart, w.cart32, w.atom_cfg, w.atom_bin, w.geo,
+                                                       w.bin_start, w.bin_atoms, w.counts);
         GAP_TRY_CUDA(cudaGetLastError());
     }
     GAP_TRY(gap_scan(w.counts, n, w.pairs.offsets, w.scan_tmp, w.total, st));
@@ -549,8 +600,8 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, d
     if (n > 0) {
         gap_count_launch();
         k_fill_warp<<<(n + kNbrWarps - 1) / kNbrWarps, 32 * kNbrWarps, 0, st>>>(
-            n, w.frac, w.frac32, w.atom_cfg, w.geo, w.bin_start, w.bin_atoms, w.pairs.offsets, P, w.keys, w.pairs.j,
-            w.pairs.vec64, w.pairs.vec32, w.err);
+            n, w.cart, w.cart32, w.atom_cfg, w.atom_bin, w.geo, w.bin_start, w.bin_atoms, w.pairs.offsets, P, w.keys,
+            w.pairs.i, w.pairs.j, w.pairs.vec64, w.pairs.vec32, w.err);
         GAP_TRY_CUDA(cudaGetLastError());
         gap_count_launch();
         k_reverse<<<n, 64, 0, st>>>(n, w.pairs.offsets, w.keys, w.pairs.rev, w.err);
@@ -598,8 +649,8 @@ gap_status NbrWork::reserve_atoms(int n, int n_configs, int n_bins)
 {
     GAP_TRY(grow((void **)&geo, cap_geo, sizeof(CellGeom) * (n_configs + 1)));
     GAP_TRY(grow((void **)&cfg_offsets, cap_cfg, sizeof(int) * (n_configs + 2)));
-    GAP_TRY(grow((void **)&frac, cap_frac, sizeof(double) * 3 * (size_t)(n + 1)));
-    GAP_TRY(grow((void **)&frac32, cap_f32, sizeof(float4) * (size_t)(n + 1)));
+    GAP_TRY(grow((void **)&cart, cap_cart, sizeof(D4) * (size_t)(n + 1)));
+    GAP_TRY(grow((void **)&cart32, cap_c32, sizeof(float4) * (size_t)(n + 1)));
     GAP_TRY(grow((void **)&atom_cfg, cap_acfg, sizeof(int) * (size_t)(n + 1)));
     GAP_TRY(grow((void **)&atom_bin, cap_abin, sizeof(int) * (size_t)(n + 1)));
     GAP_TRY(grow((void **)&bin_atoms, cap_batoms, sizeof(int) * (size_t)(n + 1)));
@@ -619,6 +670,7 @@ gap_status NbrWork::reserve_pairs(int P)
 {
     size_t p = (size_t)(P > 0 ? P : 1);
     GAP_TRY(grow((void **)&keys, cap_keys, sizeof(long long) * p));
+    GAP_TRY(grow((void **)&pairs.i, cap_i, sizeof(int) * p));
     GAP_TRY(grow((void **)&pairs.j, cap_j, sizeof(int) * p));
     GAP_TRY(grow((void **)&pairs.rev, cap_rev, sizeof(int) * p));
     GAP_TRY(grow((void **)&pairs.vec64, cap_v64, sizeof(D4) * p));
@@ -628,8 +680,8 @@ gap_status NbrWork::reserve_pairs(int P)
 
 void NbrWork::release()
 {
-    void *ps[] = {geo, cfg_offsets, frac, frac32, atom_cfg, atom_bin, bin_atoms, counts, pairs.offsets, bin_count,
-                  bin_fill, bin_start, scan_tmp, total, keys, pairs.j, pairs.rev, pairs.vec64, pairs.vec32};
+    void *ps[] = {geo, cfg_offsets, cart, cart32, atom_cfg, atom_bin, bin_atoms, counts, pairs.offsets, bin_count,
+                  bin_fill, bin_start, scan_tmp, total, keys, pairs.i, pairs.j, pairs.rev, pairs.vec64, pairs.vec32};
     for (void *p : ps)
         if (p) cudaFree(p);
     *this = NbrWork();

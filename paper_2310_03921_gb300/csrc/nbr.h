@@ -8,8 +8,7 @@
 struct CellGeom {
     double cell[9], inv[9];
     double rc2;
-    float cell32[9];
-    float rc2_loose;  // squared cutoff widened past the FP32 rounding of frac32: the prefilter bound
+    float rc2_loose;  // squared cutoff widened past the FP32 rounding of cart32: the prefilter bound
     float rc2_tight;  // squared cutoff narrowed by the same margin: below it a pair is surely inside
     int nb[3], R[3], pbc[3];
     int bin0;
@@ -18,8 +17,8 @@ struct CellGeom {
 struct NbrWork {
     CellGeom *geo = nullptr;
     int *cfg_offsets = nullptr;
-    double *frac = nullptr;
-    float4 *frac32 = nullptr;  // FP32 copy of frac (prefilter of the candidate scans)
+    D4 *cart = nullptr;        // wrapped atoms, Cartesian (x, y, z, near)
+    float4 *cart32 = nullptr;  // FP32 copy of cart (prefilter of the candidate scans)
     int *atom_cfg = nullptr, *atom_bin = nullptr, *bin_atoms = nullptr, *counts = nullptr;
     int *bin_count = nullptr, *bin_fill = nullptr, *bin_start = nullptr;
     int *scan_tmp = nullptr, *total = nullptr, *err = nullptr;
@@ -31,9 +30,9 @@ struct NbrWork {
     // exceed the capacity leaves every atom without pairs and sets err bit 1.
     bool graph = false;
     int pair_cap = 0;
-    size_t cap_geo = 0, cap_cfg = 0, cap_frac = 0, cap_acfg = 0, cap_abin = 0, cap_batoms = 0, cap_counts = 0,
+    size_t cap_geo = 0, cap_cfg = 0, cap_cart = 0, cap_acfg = 0, cap_abin = 0, cap_batoms = 0, cap_counts = 0,
            cap_offsets = 0, cap_bcount = 0, cap_bfill = 0, cap_bstart = 0, cap_scan = 0, cap_total = 0,
-           cap_keys = 0, cap_j = 0, cap_rev = 0, cap_v64 = 0, cap_v32 = 0, cap_f32 = 0;
+           cap_keys = 0, cap_i = 0, cap_j = 0, cap_rev = 0, cap_v64 = 0, cap_v32 = 0, cap_c32 = 0;
 
     gap_status reserve_atoms(int n, int n_configs, int n_bins);
     gap_status reserve_pairs(int P);

@@ -713,13 +713,6 @@ k_config_final(int nchunk, int nq, const double *__restrict__ part, double *__re
     if (lane == 0) config_store(c, a, s, energy, virial);
 }
 
-__global__ void k_pair_atoms(int n_atoms, const int *__restrict__ offsets, int *__restrict__ pair_i)
-{
-    int i = blockIdx.x;
-    if (i >= n_atoms) return;
-    for (int p = offsets[i] + threadIdx.x; p < offsets[i + 1]; p += blockDim.x) pair_i[p] = i;
-}
-
 // ----------------------------------------------------------- dispatching
 constexpr size_t kMaxSmem = 227 * 1024;  // opt-in dynamic shared memory per block
 
@@ -760,14 +753,14 @@ template <typename T> struct Launch {
         return gap_cuda_status(cudaGetLastError(), "k_chain");
     }
     template <int N, int L, int GA>
-    static gap_status pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *pair_i,
-                                const int *species, const T *Gam, T *fpair, cudaStream_t st)
+    static gap_status pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *species,
+                                const T *Gam, T *fpair, cudaStream_t st)
     {
         if (pl.n_pairs == 0) return GAP_OK;
         const typename V4<T>::type *vec;
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();
-        k_pairforce<N, L, T><<<(pl.n_pairs + 127) / 128, 128, 0, st>>>(g, tab, pl.n_pairs, pl.count, pair_i, pl.j,
+        k_pairforce<N, L, T><<<(pl.n_pairs + 127) / 128, 128, 0, st>>>(g, tab, pl.n_pairs, pl.count, pl.i, pl.j,
                                                                        vec, species, Gam, fpair);
         return gap_cuda_status(cudaGetLastError(), "k_pairforce");
     }
@@ -825,11 +818,11 @@ gap_status gap_chain(const SoapGeom &g, int n, const T *gvec, const T *wsum, con
 }
 
 template <typename T>
-gap_status gap_pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *pair_i, const int *species,
-                         const T *Gam, T *fpair, cudaStream_t st)
+gap_status gap_pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *species, const T *Gam,
+                         T *fpair, cudaStream_t st)
 {
 #define X(nn, ll, ga) \
-    if (g.N == nn && g.L == ll) return Launch<T>::template pairforce<nn, ll, 1>(g, tab, pl, pair_i, species, Gam, fpair, st);
+    if (g.N == nn && g.L == ll) return Launch<T>::template pairforce<nn, ll, 1>(g, tab, pl, species, Gam, fpair, st);
     GAP_SHAPES(X)
 #undef X
     gap_set_error("unsupported (n_max, l_max)");
@@ -888,21 +881,13 @@ gap_status gap_config_sums(int n_configs, const int *cfg_off, int max_atoms, con
     return gap_cuda_status(cudaGetLastError(), "k_config_final");
 }
 
-gap_status gap_pair_atoms(int n, const PairList &pl, int *pair_i, cudaStream_t st)
-{
-    if (n == 0) return GAP_OK;
-    gap_count_launch();
-    k_pair_atoms<<<n, 64, 0, st>>>(n, pl.offsets, pair_i);
-    return gap_cuda_status(cudaGetLastError(), "k_pair_atoms");
-}
-
 #define INST(T)                                                                                                      \
     template gap_status gap_expand<T>(const SoapGeom &, const T *, int, const PairList &, const int *, T *, T *, T *, \
                                       cudaStream_t);                                                                 \
     template gap_status gap_chain<T>(const SoapGeom &, int, const T *, const T *, const T *, const int *, const T *,  \
                                      const T *, const T *, T *, cudaStream_t);                                       \
-    template gap_status gap_pairforce<T>(const SoapGeom &, const T *, const PairList &, const int *, const int *,     \
-                                         const T *, T *, cudaStream_t);                                              \
+    template gap_status gap_pairforce<T>(const SoapGeom &, const T *, const PairList &, const int *, const T *, T *,    \
+                                         cudaStream_t);                                                              \
     template gap_status gap_gather<T>(int, const PairList &, const T *, const double *, double *, double *,          \
                                       cudaStream_t);
 INST(double)

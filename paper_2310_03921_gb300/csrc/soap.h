@@ -29,7 +29,7 @@ template <typename T>
 gap_status gap_chain(const SoapGeom &g, int n, const T *gvec, const T *wsum, const T *mu, const int *gp_of_atom,
                      const T *phat, const T *pnorm, const T *coef, T *Gam, cudaStream_t st);
 template <typename T>
-gap_status gap_pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *pair_i, const int *species,
+gap_status gap_pairforce(const SoapGeom &g, const T *tab, const PairList &pl, const int *species,
                          const T *Gam, T *fpair, cudaStream_t st);
 // Two-body term in FP64: half energies per atom eps2 and, if fw2 is not NULL,
 // each atom's force and symmetric virial fw2[N][9] (F; xx yy zz yz xz xy).
@@ -45,4 +45,3 @@ gap_status gap_config_sums(int n_configs, const int *cfg_off, int max_atoms, con
                            const double *vir_atom, double *energy, double *virial, double *local_e, double *part,
                            cudaStream_t st);
 size_t gap_config_part_doubles(int n_configs, int max_atoms);
-gap_status gap_pair_atoms(int n, const PairList &pl, int *pair_i, cudaStream_t st);
