@@ -1289,7 +1289,7 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
         if (R == 0 || gp.M == 0) continue;
         const int *rows = w.rows.as<int>() + (size_t)s * n;
         if (!tc) {
-            int nt = (gp.M + 63) / 64;
+            const int nt = gap_contract_simt_parts(gp.M);
             GAP_TRY(w.W.ensure(sizeof(T) * (size_t)R * gp.M));
             GAP_TRY(w.eps_part.ensure(sizeof(double) * (size_t)R * nt));
             GAP_TRY(gap_contract_simt<T>(phg, Dg, Dg16, rows, w.counts.as<int>() + s, R, gp_X<T>(gp),

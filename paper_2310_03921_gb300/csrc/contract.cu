@@ -123,15 +123,127 @@ k_simt_G(const T *__restrict__ W, int ldw, const int *__restrict__ rows, const i
     }
 }
 
-template <typename T>
-__global__ void k_eps_rows(const int *__restrict__ rows, const int *__restrict__ nrows_p,
-                           const double *__restrict__ eps_part, int n_tiles, double *__restrict__ eps)
+// eps of each row from its column tiles' partial energies: a warp per row.
+__global__ void __launch_bounds__(128)
+k_eps_rows(const int *__restrict__ rows, const int *__restrict__ nrows_p, const double *__restrict__ eps_part,
+           int n_tiles, double *__restrict__ eps)
 {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
+    const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= *nrows_p) return;
     double e = 0.0;
-    for (int t = 0; t < n_tiles; ++t) e += eps_part[(size_t)r * n_tiles + t];
-    eps[rows[r]] = e;
+    for (int t = lane; t < n_tiles; t += 32) e += eps_part[(size_t)r * n_tiles + t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0) eps[rows[r]] = e;
+}
+
+// ------------------------------------------------ the same on small tiles
+// 8 x 8 outputs per block, the K sum split four ways over its 256 threads and
+// the four partial sums added in a fixed order.  The 64 x 64 tiles above keep
+// a small product on few SMs (64 atoms x 100 points: two blocks, a serial
+// chain over K of 134 us); these spread it over R M / 64 blocks.  In FP64
+// they are the better tile at every size: GB300's FP64 pipe holds a warp
+// instruction for ~64 cycles, which covers two shared-memory reads and the
+// tile loads per FMA.  In FP32 the reads bound them, so they serve only
+// products whose 64 x 64 tiles would leave most SMs idle (small_tiles).
+// Whole predictions with 64 x 64 and 8 x 8 tiles, n_max 8, l_max 6: FP64 215
+// atoms x 4000 points 5371 and 1216 us, 4095 x 2000 9089 and 8392 us; FP32 215
+// x 4000 (252 tiles and 16) 905 and 461 us.
+constexpr int kST = 8, kSK = 64, kSplit = 4;
+
+// acc = sum over this thread's quarter of K of A(r, k) B(k, c); load(e, kk, rr)
+// fills the staged operands.
+template <typename T, typename LoadA, typename LoadB>
+__device__ __forceinline__ T small_tile_sum(int K, T (&As)[kSK][kST + 1], T (&Bs)[kSK][kST + 1],
+                                            T (&red)[kSplit][kST * kST], LoadA &&la, LoadB &&lb)
+{
+    const int cell = threadIdx.x & 63, split = threadIdx.x >> 6, r = cell >> 3, c = cell & 7;
+    T acc = T(0);
+    for (int k0 = 0; k0 < K; k0 += kSK) {
+#pragma unroll
+        for (int u = 0; u < kSK * kST / 256; ++u) {
+            la(k0, (int)threadIdx.x + 256 * u);
+            lb(k0, (int)threadIdx.x + 256 * u);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < kSK / kSplit; ++kk) acc += As[split * (kSK / kSplit) + kk][r] * Bs[split * (kSK / kSplit) + kk][c];
+        __syncthreads();
+    }
+    red[split][cell] = acc;
+    __syncthreads();
+    return (red[0][cell] + red[1][cell]) + (red[2][cell] + red[3][cell]);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_small_qW(const T *__restrict__ phat, int D, const int *__restrict__ rows, const int *__restrict__ nrows_p,
+           const T *__restrict__ X, const T *__restrict__ alpha, int M, T d2, int zeta, T *__restrict__ W, int ldw,
+           double *__restrict__ eps_part, int n_tiles)
+{
+    __shared__ T As[kSK][kST + 1], Bs[kSK][kST + 1];
+    __shared__ T red[kSplit][kST * kST];
+    __shared__ int atom[kST];
+    const int nrows = *nrows_p;
+    const int r0 = blockIdx.y * kST, m0 = blockIdx.x * kST;
+    if (r0 >= nrows) return;
+    if (threadIdx.x < kST) atom[threadIdx.x] = r0 + (int)threadIdx.x < nrows ? rows[r0 + threadIdx.x] : -1;
+    __syncthreads();
+    const T q = small_tile_sum<T>(
+        D, As, Bs, red,
+        [&](int k0, int e) {
+            const int kk = e % kSK, rr = e / kSK, k = k0 + kk;
+            As[kk][rr] = (atom[rr] >= 0 && k < D) ? phat[(size_t)atom[rr] * D + k] : T(0);
+        },
+        [&](int k0, int e) {
+            const int kk = e % kSK, rr = e / kSK, k = k0 + kk, m = m0 + rr;
+            Bs[kk][rr] = (m < M && k < D) ? X[(size_t)m * D + k] : T(0);
+        });
+    if (threadIdx.x >= kST * kST) return;
+    const int r = r0 + (threadIdx.x >> 3), m = m0 + (threadIdx.x & 7);
+    double e = 0.0;
+    if (r < nrows && m < M) {
+        T qz = T(1);
+        for (int z = 1; z < zeta; ++z) qz *= q;
+        const T a = d2 * alpha[m];
+        e = (double)(a * qz * q);
+        W[(size_t)r * ldw + m] = T(zeta) * a * qz;
+    }
+#pragma unroll
+    for (int o = kST / 2; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if ((threadIdx.x & 7) == 0 && r < nrows) eps_part[(size_t)r * n_tiles + blockIdx.x] = e;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_small_G(const T *__restrict__ W, int ldw, const int *__restrict__ rows, const int *__restrict__ nrows_p,
+          const T *__restrict__ X, int M, int D, T *__restrict__ g, int ldg)
+{
+    __shared__ T As[kSK][kST + 1], Bs[kSK][kST + 1];
+    __shared__ T red[kSplit][kST * kST];
+    const int nrows = *nrows_p;
+    const int r0 = blockIdx.y * kST, d0 = blockIdx.x * kST;
+    if (r0 >= nrows) return;
+    const T v = small_tile_sum<T>(
+        M, As, Bs, red,
+        [&](int k0, int e) {
+            const int kk = e % kSK, rr = e / kSK, k = k0 + kk;
+            As[kk][rr] = (r0 + rr < nrows && k < M) ? W[(size_t)(r0 + rr) * ldw + k] : T(0);
+        },
+        [&](int k0, int e) {
+            const int dd = e % kST, kk = e / kST, k = k0 + kk;
+            Bs[kk][dd] = (k < M && d0 + dd < D) ? X[(size_t)k * D + d0 + dd] : T(0);
+        });
+    if (threadIdx.x >= kST * kST) return;
+    const int r = r0 + (threadIdx.x >> 3), d = d0 + (threadIdx.x & 7);
+    if (r < nrows && d < D) g[(size_t)rows[r] * ldg + d] = v;
+}
+
+// Whether the small tiles serve a product of rows x cols outputs.
+template <typename T> bool small_tiles(int rows, int cols)
+{
+    if (sizeof(T) == 8) return (rows + kST - 1) / kST <= 65535;  // grid y
+    return (long)((rows + TM - 1) / TM) * ((cols + TN - 1) / TN) <= 48;
 }
 
 // ---------------------------------------------------------------- rows
@@ -226,22 +338,31 @@ gap_status gap_contract_simt(const T *phat, int D, int D16, const int *rows, con
 {
     if (max_rows <= 0 || M <= 0) return GAP_OK;
     int n_tiles = (M + TN - 1) / TN;
-    dim3 g1(n_tiles, (max_rows + TM - 1) / TM);
     gap_prof_begin(ST_GEMM_Q, st);
     gap_count_launch();
-    k_simt_qW<T><<<g1, 256, 0, st>>>(phat, D, rows, nrows_dev, X, alpha, M, (T)(delta * delta), zeta, W, M, eps_part,
-                                      n_tiles);
+    if (small_tiles<T>(max_rows, M)) {
+        n_tiles = (M + kST - 1) / kST;
+        k_small_qW<T><<<dim3(n_tiles, (max_rows + kST - 1) / kST), 256, 0, st>>>(
+            phat, D, rows, nrows_dev, X, alpha, M, (T)(delta * delta), zeta, W, M, eps_part, n_tiles);
+    } else {
+        k_simt_qW<T><<<dim3(n_tiles, (max_rows + TM - 1) / TM), 256, 0, st>>>(
+            phat, D, rows, nrows_dev, X, alpha, M, (T)(delta * delta), zeta, W, M, eps_part, n_tiles);
+    }
     GAP_TRY_CUDA(cudaGetLastError());
     gap_prof_end(ST_GEMM_Q, st);
-    dim3 g2((D + TN - 1) / TN, (max_rows + TM - 1) / TM);
     gap_prof_begin(ST_GEMM_G, st);
     if (g) {
         gap_count_launch();
-        k_simt_G<T><<<g2, 256, 0, st>>>(W, M, rows, nrows_dev, X, M, D, g, D16);
+        if (small_tiles<T>(max_rows, D))
+            k_small_G<T><<<dim3((D + kST - 1) / kST, (max_rows + kST - 1) / kST), 256, 0, st>>>(W, M, rows, nrows_dev,
+                                                                                                X, M, D, g, D16);
+        else
+            k_simt_G<T><<<dim3((D + TN - 1) / TN, (max_rows + TM - 1) / TM), 256, 0, st>>>(W, M, rows, nrows_dev, X, M,
+                                                                                           D, g, D16);
         GAP_TRY_CUDA(cudaGetLastError());
     }
     gap_count_launch();
-    k_eps_rows<T><<<(max_rows + 127) / 128, 128, 0, st>>>(rows, nrows_dev, eps_part, n_tiles, eps);
+    k_eps_rows<<<(max_rows + 3) / 4, 128, 0, st>>>(rows, nrows_dev, eps_part, n_tiles, eps);
     GAP_TRY_CUDA(cudaGetLastError());
     gap_prof_end(ST_GEMM_G, st);
     return GAP_OK;
@@ -255,6 +376,7 @@ template gap_status gap_contract_simt<float>(const float *, int, int, const int 
                                              cudaStream_t);
 
 int gap_contract_simt_tiles(int M) { return M > 0 ? (M + TN - 1) / TN : 0; }
+int gap_contract_simt_parts(int M) { return M > 0 ? (M + kST - 1) / kST : 0; }
 
 // The same two GEMMs as gap_contract_simt<double> on the identity row list,
 // launched without stage profiling (used by the allocation-free entry point).
@@ -274,7 +396,7 @@ gap_status gap_contract_simt_fixed(const double *phat, int D, int ldg, const int
     k_simt_G<double><<<g2, 256, 0, st>>>(W, M, rows, nrows_dev, X, M, D, g, ldg);
     GAP_TRY_CUDA(cudaGetLastError());
     gap_count_launch();
-    k_eps_rows<double><<<(n_rows + 127) / 128, 128, 0, st>>>(rows, nrows_dev, eps_part, n_tiles, eps);
+    k_eps_rows<<<(n_rows + 3) / 4, 128, 0, st>>>(rows, nrows_dev, eps_part, n_tiles, eps);
     return gap_cuda_status(cudaGetLastError(), "k_eps_rows");
 }
 

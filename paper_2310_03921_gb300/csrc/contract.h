@@ -35,8 +35,10 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
                            double delta, int zeta, int nsplit, TcScratch &sc, double *eps, float *wsum, float *g,
                            int *err, cudaStream_t st);
 
-// Column tiles of the FP64/FP32 contraction for M sparse points: the row
-// stride of its per-tile partial energies (eps_part holds n_rows x tiles).
+// Capacity per row of gap_contract_simt's partial energies (eps_part).
+int gap_contract_simt_parts(int M);
+// Column tiles of gap_contract_simt_fixed for M sparse points: the row stride
+// of its partial energies (eps_part holds n_rows x tiles).
 int gap_contract_simt_tiles(int M);
 // The same contraction for several GPs (a batch's central species) with one
 // persistent launch per GEMM stage: rows[q], nrows[q] and sc[q] per GP.
