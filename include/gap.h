@@ -411,10 +411,9 @@ long gap_launch_count(void);
  * tile shapes picked per workload).  The first call of a shape class on a
  * device (epilogue, split, K, columns, ceil(log2 rows)) outside stream
  * capture times each tile variant on its own operands - 128 x 256 with two
- * TMA stages, 128 x 128 with two, 128 x 128 with three, and for the K_NM
- * force rows (K <= 256), the kernel-energy and the gradient contractions
- * 128 x 192 with twelve epilogue warps - and keeps
- * the fastest; captured calls reuse the choice (128 x 256 with two stages
+ * TMA stages, 128 x 128 with two, 128 x 128 with three, and for the
+ * kernel-energy and the gradient contractions 128 x 192 with twelve epilogue
+ * warps - and keeps the fastest; captured calls reuse the choice (128 x 256 with two stages
  * for a class not yet tuned).  gap_tile_tuning_count gives
  * the number of tuned classes; entry k: fields[8] = (epilogue, planes, K,
  * columns, ceil(log2 rows), chosen column tile, chosen stages, device) and

@@ -13,6 +13,7 @@
 #include "crt_gemm.h"
 #include "gap_internal.h"
 #include "knm.h"
+#include "knm_gemm.h"
 #include "nbr.h"
 #include "radial.h"
 #include "solve.h"
@@ -287,8 +288,8 @@ struct Workspace {
     NbrWork nbr;
     DBuf pos, spec, coef, phat, pnorm, gp_of_atom, flag, fpos, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
         W, eps_part, Gam, fpair, fw2, forces, vir_atom, cfgpart, energy, virial, local, err, A_hi, A_lo, t_row, W_hi, W_lo,
-        epart_f, wpart_f, Gs, outbuf, kA, kAhi, kAlo, kt, ksrc, kseg, kdest, segstart, outrow, Wp, kq, P, Kbuf, A_mid, W_mid,
-        kAmid, phatc, pnormc, hfull, kV;
+        epart_f, wpart_f, Gs, outbuf, kA, kAhi, kAlo, ksrc, kseg, kdest, kmeta, kslot, kfirst, kcount, kbounds, rank, segstart, outrow, Wp, kq, P,
+        Kbuf, A_mid, W_mid, kAmid, phatc, pnormc, hfull, kV;
     // Graph mode (gap_step_graph): no host synchronisation inside a call; the
     // rows of each GP are those of the last ordinary call (species are fixed).
     bool graph = false;
@@ -299,8 +300,8 @@ struct Workspace {
         DBuf *bs[] = {&pos, &spec, &coef, &phat, &pnorm, &gp_of_atom, &flag, &fpos, &scan_tmp, &rows,
                       &counts, &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &fw2, &forces, &vir_atom, &cfgpart, &energy,
                       &virial, &local, &err, &A_hi, &A_lo, &t_row, &W_hi, &W_lo, &epart_f, &wpart_f, &Gs, &outbuf,
-                      &kA, &kAhi, &kAlo, &kt, &ksrc, &kseg, &kdest, &segstart, &outrow, &Wp, &kq, &P, &Kbuf, &A_mid, &W_mid,
-                      &kAmid, &phatc, &pnormc, &hfull, &kV};
+                      &kA, &kAhi, &kAlo, &ksrc, &kseg, &kdest, &kmeta, &kslot, &kfirst, &kcount, &kbounds, &rank, &segstart,
+                      &outrow, &Wp, &kq, &P, &Kbuf, &A_mid, &W_mid, &kAmid, &phatc, &pnormc, &hfull, &kV};
         for (DBuf *b : bs) b->release();
     }
 };
@@ -1171,6 +1172,7 @@ static gap_status gp_rows_all(gap_model *m, Workspace &w, int n, const int *spec
 {
     int G = m->n_gp;
     GAP_TRY(w.gp_of_atom.ensure(sizeof(int) * (size_t)n));
+    GAP_TRY(w.rank.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.flag.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.fpos.ensure(sizeof(int) * (size_t)(n + 1)));
     GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_scan_tmp_ints(n)));
@@ -1179,7 +1181,7 @@ static gap_status gp_rows_all(gap_model *m, Workspace &w, int n, const int *spec
     GAP_TRY(gap_fill_int(w.gp_of_atom.as<int>(), n, -1, st));
     for (int s = 0; s < G; ++s)
         GAP_TRY(gap_gp_rows(n, spec, s, w.flag.as<int>(), w.fpos.as<int>(), w.scan_tmp.as<int>(),
-                            w.rows.as<int>() + (size_t)s * n, w.counts.as<int>() + s, w.gp_of_atom.as<int>(), st));
+                            w.rows.as<int>() + (size_t)s * n, w.counts.as<int>() + s, w.gp_of_atom.as<int>(), w.rank.as<int>(), st));
     if (w.graph) {
         counts = w.counts_fixed;
         return GAP_OK;
@@ -1573,10 +1575,137 @@ extern "C" gap_status gap_step_graph_destroy(gap_step_graph *G)
     GAP_API_END
 }
 
-// knm == NULL keeps K_NM in the workspace (w.Kbuf) whatever the batch's
-// memory: the fused fit reads it there.
+// K_NM on the tensor cores: W' and k of every GP's atoms (one launch over the
+// GPs), the Jacobian triples, the force rows of all GPs in one launch, the
+// energy rows.  K [C + 3 n][Mt]; the descriptor has been run.
+static gap_status knm_tc(gap_model *m, Workspace &w, const gap_batch *b, int nsplit, const int *spec,
+                         const std::vector<int> &counts, double *K, int Mt, cudaStream_t st)
+{
+    gap_soap *soap = m->soap;
+    const SoapGeom &g = soap->geo;
+    const bool cmp = soap->comp != 0, three = nsplit == 3;
+    const int Dg16 = soap->Dg16;
+    const int Dw = cmp && Dg16 > g.D16 ? Dg16 : g.D16;  // width of the row planes
+    const int n = b->n_atoms, C = b->n_configs, G = m->n_gp;
+    const PairList &pl = w.nbr.pairs;
+    const long nt = (long)n + pl.n_pairs;  // triples, at most (species without a GP have none)
+    if (G > kKnmMaxGPs || 3 * nt > 2147483647L || (long)G * n > 2147483646L) {
+        gap_set_error("K_NM: too many Jacobian rows for one call");
+        return GAP_EUNSUPPORTED;
+    }
+    gap_prof_begin(ST_KNM_ROWS, st);
+    GAP_TRY(w.kslot.ensure(sizeof(int) * (size_t)pl.n_pairs));
+    GAP_TRY(w.kcount.ensure(sizeof(int) * (size_t)G * n));
+    GAP_TRY(w.kfirst.ensure(sizeof(int) * ((size_t)G * n + 1)));
+    GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_scan_tmp_ints(G * n)));
+    GAP_TRY(w.kAhi.ensure(2 * 3 * (size_t)nt * Dw));
+    GAP_TRY(w.kAlo.ensure(2 * 3 * (size_t)nt * Dw));
+    if (three) GAP_TRY(w.kAmid.ensure(2 * 3 * (size_t)nt * Dw));
+    GAP_TRY(w.kmeta.ensure(sizeof(float4) * (size_t)nt));
+    GAP_TRY(w.kdest.ensure(sizeof(int) * (size_t)nt));
+    if (cmp) GAP_TRY(w.ksrc.ensure(sizeof(int) * (size_t)nt));
+    GAP_TRY(w.kbounds.ensure(sizeof(int) * gap_knm_bounds_ints(G)));
+    KnmRows rows{};
+    rows.tri = KnmTriples{w.kAhi.as<__nv_bfloat16>(), w.kAlo.as<__nv_bfloat16>(),
+                          three ? w.kAmid.as<__nv_bfloat16>() : nullptr, w.kmeta.as<float4>(), w.kdest.as<int>(),
+                          cmp ? w.ksrc.as<int>() : nullptr, w.kfirst.as<int>(), w.kslot.as<int>(), w.rank.as<int>(),
+                          w.nbr.atom_cfg};
+    if (n > 0) {
+        GAP_TRY(gap_knm_slots(n, G, pl.offsets, pl.j, w.gp_of_atom.as<int>(), w.kslot.as<int>(), w.kcount.as<int>(), st));
+        GAP_TRY(gap_scan(w.kcount.as<int>(), G * n, w.kfirst.as<int>(), w.scan_tmp.as<int>(), nullptr, st));
+        if (cmp) GAP_TRY_CUDA(cudaMemsetAsync(w.ksrc.p, 0xff, sizeof(int) * (size_t)nt, st));
+        gap_prof_begin(ST_KNM_JACOBIAN, st);
+        GAP_TRY((gap_jacobian_rows<float, true>(g, tab_of<float>(soap), n, pl, spec, w.coef.as<float>(),
+                                                w.phat.as<float>(), w.pnorm.as<float>(), w.gp_of_atom.as<int>(),
+                                                cmp ? nullptr : m->mu_all.as<float>(), rows, st)));
+        if (cmp) {
+            // V = J Q^T on the tensor cores (J's planes against Q's), then
+            // J~ into the same planes (J is consumed by then), Dg16 wide
+            GAP_TRY(w.kV.ensure(4 * 3 * (size_t)nt * Dg16));
+            TcOperands opq{w.kAhi.as<__nv_bfloat16>(), w.kAlo.as<__nv_bfloat16>(),
+                           soap->Qhi.as<__nv_bfloat16>(), (three ? soap->Qlo3 : soap->Qlo).as<__nv_bfloat16>(),
+                           (int)(3 * nt), soap->Dg, g.D16, g.D16, g.D16, nsplit,
+                           three ? w.kAmid.as<__nv_bfloat16>() : nullptr,
+                           three ? soap->Qmid.as<__nv_bfloat16>() : nullptr};
+            TcEpilogue eq{};
+            eq.C = w.kV.as<float>();
+            eq.ldc = Dg16;
+            GAP_TRY(gap_tc_gemm(opq, eq, EPI_STORE, w.err.as<int>() + 2, st));
+            GAP_TRY((gap_jacobian_compress<float, true>(3 * nt, soap->Dg, Dg16, w.kV.as<float>(), Dg16, nullptr,
+                                                        w.gp_of_atom.as<int>(), w.phatc.as<float>(),
+                                                        w.pnorm.as<float>(), w.pnormc.as<float>(),
+                                                        m->mu_all.as<float>(), rows, st)));
+        }
+        gap_prof_end(ST_KNM_JACOBIAN, st);
+    }
+    gap_prof_end(ST_KNM_ROWS, st);
+    // W' and k of each GP's atoms, rows in the GP's order
+    size_t ra = 0, rw = 0, rr = 0;
+    int n_active = 0;
+    for (int s = 0; s < G; ++s) {
+        const size_t R = m->gp[s].M > 0 ? counts[s] : 0;
+        ra += R * Dg16;
+        rw += R * m->gp[s].M_pad;
+        rr += R;
+        n_active += R > 0;
+    }
+    GAP_TRY(w.A_hi.ensure(2 * ra));
+    GAP_TRY(w.A_lo.ensure(2 * ra));
+    if (three) GAP_TRY(w.A_mid.ensure(2 * ra));
+    GAP_TRY(w.t_row.ensure(4 * rr));
+    GAP_TRY(w.Wp.ensure(sizeof(float) * rw));
+    GAP_TRY(w.kq.ensure(sizeof(float) * rw));
+    KnmGP kg[kKnmMaxGPs];
+    TcOperands ops[kKnmMaxGPs];
+    TcEpilogue eps[kKnmMaxGPs];
+    gap_prof_begin(ST_KNM_GEMM, st);
+    size_t oa = 0, ow = 0, orr = 0;
+    int col = 0, k = 0;
+    for (int s = 0; s < G; ++s) {
+        const GPData &gp = m->gp[s];
+        const int R = gp.M > 0 ? counts[s] : 0;
+        const int *grow = w.rows.as<int>() + (size_t)s * n;
+        const __nv_bfloat16 *Blo = (three ? gp.Blo3 : gp.Blo).as<__nv_bfloat16>();
+        kg[s] = KnmGP{gp.M, gp.M_pad, R, gp.Bhi.as<__nv_bfloat16>(), Blo, gp.Bmid.as<__nv_bfloat16>(),
+                      w.Wp.as<float>() + ow, w.kq.as<float>() + ow, grow, col};
+        col += gp.M;
+        if (R == 0) continue;
+        __nv_bfloat16 *Ah = w.A_hi.as<__nv_bfloat16>() + oa, *Al = w.A_lo.as<__nv_bfloat16>() + oa,
+                      *Am = three ? w.A_mid.as<__nv_bfloat16>() + oa : nullptr;
+        float *tr = w.t_row.as<float>() + orr;
+        GAP_TRY(gap_split_rows(gp_phat<float>(soap, w), soap->Dg, Dg16, grow, R,
+                               m->mu_all.as<float>() + (size_t)s * Dg16, Ah, Al, Am, tr, st));
+        ops[k] = TcOperands{Ah, Al, kg[s].B_hi, Blo, R, gp.M, Dg16, Dg16, Dg16, nsplit, Am,
+                            three ? kg[s].B_mid : nullptr};
+        eps[k] = TcEpilogue{};
+        eps[k].s_col = gp.s_col.as<float>();
+        eps[k].t_row = tr;
+        eps[k].d2 = (float)(m->delta * m->delta);
+        eps[k].zeta = m->zeta;
+        eps[k].Wp = w.Wp.as<float>() + ow;
+        eps[k].kq = w.kq.as<float>() + ow;
+        eps[k].ldwp = gp.M_pad;
+        ++k;
+        oa += (size_t)R * Dg16;
+        ow += (size_t)R * gp.M_pad;
+        orr += R;
+    }
+    if (n_active == 1) GAP_TRY(gap_tc_gemm(ops[0], eps[0], EPI_QPOW, w.err.as<int>() + 2, st));
+    else if (n_active > 1) GAP_TRY(gap_tc_gemm_grouped(ops, eps, k, EPI_QPOW, w.err.as<int>() + 2, st));
+    if (n > 0)
+        GAP_TRY(gap_knm_force_tc(rows.tri, nt, n, Dg16, nsplit, kg, G, w.kbounds.as<int>(), K, Mt,
+                                 w.err.as<int>() + 2, st));
+    gap_prof_end(ST_KNM_GEMM, st);
+    gap_prof_begin(ST_KNM_REDUCE, st);
+    GAP_TRY(gap_knm_energy_tc(C, w.nbr.cfg_offsets, kg, G, K, Mt, st));
+    gap_prof_end(ST_KNM_REDUCE, st);
+    return GAP_OK;
+}
+
+// K_NM on the CUDA cores (FP64 or FP32), as knm_tc.
 template <typename T>
-static gap_status knm_impl(gap_model *m, const gap_batch *b, gap_precision prec, double *knm, cudaStream_t st)
+static gap_status knm_simt(gap_model *m, Workspace &w, const gap_batch *b, const int *spec,
+                           const std::vector<int> &counts, double *K, int Mt, cudaStream_t st)
 {
     gap_soap *soap = m->soap;
     const SoapGeom &g = soap->geo;
@@ -1584,28 +1713,8 @@ static gap_status knm_impl(gap_model *m, const gap_batch *b, gap_precision prec,
     // Jacobian rows are those of p_hat mapped by gap_jacobian_compress
     const bool cmp = soap->comp != 0;
     const int Dg = soap->Dg, Dg16 = soap->Dg16;
-    const int Dw = cmp && Dg16 > g.D16 ? Dg16 : g.D16;  // width of the row planes
-    Workspace &w = m->ws;
     const int n = b->n_atoms, C = b->n_configs;
-    const bool tc = prec == GAP_BF16X3 || prec == GAP_BF16X6;
-    const int nsplit = prec == GAP_BF16X6 ? 3 : 2;
-    const bool three = nsplit == 3;
-    int Mt = 0;
-    std::vector<int> col_off(m->n_gp + 1, 0);
-    for (int s = 0; s < m->n_gp; ++s) col_off[s + 1] = col_off[s] + m->gp[s].M;
-    Mt = col_off[m->n_gp];
-    const size_t krows = (size_t)C + 3 * (size_t)n;
-    double *K = knm;
-    if (!b->device || !knm) {
-        GAP_TRY(w.Kbuf.ensure(sizeof(double) * krows * (Mt > 0 ? Mt : 1)));
-        K = w.Kbuf.as<double>();
-    }
-    if (krows * Mt) GAP_TRY_CUDA(cudaMemsetAsync(K, 0, sizeof(double) * krows * Mt, st));
-    const int *spec;
-    GAP_TRY(run_descriptor<T>(soap, w, b, &spec, st));
     const PairList &pl = w.nbr.pairs;
-    std::vector<int> counts;
-    GAP_TRY(gp_rows_all(m, w, n, spec, counts, st));
     const size_t nrow = 3 * ((size_t)n + pl.n_pairs);
     const int nseg = 3 * n;
     GAP_TRY(w.segstart.ensure(sizeof(int) * (nseg + 1)));
@@ -1617,75 +1726,29 @@ static gap_status knm_impl(gap_model *m, const gap_batch *b, gap_precision prec,
     KnmRows rows{};
     rows.src_sign = w.ksrc.as<int>();
     rows.seg = w.kseg.as<int>();
-    if (tc) {
-        if constexpr (sizeof(T) == 4) {
-            GAP_TRY(w.kAhi.ensure(2 * nrow * Dw));
-            GAP_TRY(w.kAlo.ensure(2 * nrow * Dw));
-            GAP_TRY(w.kt.ensure(4 * nrow));
-            rows.A_hi = w.kAhi.as<__nv_bfloat16>();
-            rows.A_lo = w.kAlo.as<__nv_bfloat16>();
-            if (three) {
-                GAP_TRY(w.kAmid.ensure(2 * nrow * Dw));
-                rows.A_mid = w.kAmid.as<__nv_bfloat16>();
-            }
-            rows.t_row = w.kt.as<float>();
-            gap_prof_begin(ST_KNM_JACOBIAN, st);
-            GAP_TRY((gap_jacobian_rows<float, true>(g, tab_of<float>(soap), n, pl, spec, w.coef.as<float>(),
-                                                    w.phat.as<float>(), w.pnorm.as<float>(), w.gp_of_atom.as<int>(),
-                                                    cmp ? nullptr : m->mu_all.as<float>(), rows, st)));
-            if (cmp && nrow) {
-                // V = J Q^T on the tensor cores (J's planes against Q's), then
-                // J~ into the same planes (J is consumed by then), Dg16 wide
-                GAP_TRY(w.kV.ensure(4 * nrow * Dg16));
-                TcOperands opq{w.kAhi.as<__nv_bfloat16>(), w.kAlo.as<__nv_bfloat16>(),
-                               soap->Qhi.as<__nv_bfloat16>(), (three ? soap->Qlo3 : soap->Qlo).as<__nv_bfloat16>(),
-                               (int)nrow, Dg, g.D16, g.D16, g.D16, nsplit,
-                               three ? w.kAmid.as<__nv_bfloat16>() : nullptr,
-                               three ? soap->Qmid.as<__nv_bfloat16>() : nullptr};
-                TcEpilogue eq{};
-                eq.C = w.kV.as<float>();
-                eq.ldc = Dg16;
-                GAP_TRY(gap_tc_gemm(opq, eq, EPI_STORE, w.err.as<int>() + 2, st));
-                GAP_TRY((gap_jacobian_compress<float, true>((long)nrow, Dg, Dg16, w.kV.as<float>(), Dg16,
-                                                            w.ksrc.as<int>(), w.gp_of_atom.as<int>(),
-                                                            w.phatc.as<float>(), w.pnorm.as<float>(),
-                                                            w.pnormc.as<float>(), m->mu_all.as<float>(), rows, st)));
-            }
-            gap_prof_end(ST_KNM_JACOBIAN, st);
-        }
-    } else {
-        GAP_TRY(w.kA.ensure(sizeof(T) * nrow * g.D16));
-        rows.A = w.kA.p;
-        gap_prof_begin(ST_KNM_JACOBIAN, st);
-        GAP_TRY((gap_jacobian_rows<T, false>(g, tab_of<T>(soap), n, pl, spec, w.coef.as<T>(), w.phat.as<T>(),
-                                             w.pnorm.as<T>(), w.gp_of_atom.as<int>(), m->mu_all.as<float>(), rows,
-                                             st)));
-        if (cmp && nrow) {
-            // V = J Q^T, then J~ in place: the force GEMM reads kV [nrow][Dg16]
-            GAP_TRY(w.kV.ensure(sizeof(T) * nrow * Dg16));
-            GAP_TRY(gap_rows_times_qt<T>((long)nrow, g.D, w.kA.as<T>(), g.D16, Dg, q_of<T>(soap), w.kV.as<T>(), Dg16,
-                                         st));
-            rows.A = w.kV.p;
-            GAP_TRY((gap_jacobian_compress<T, false>((long)nrow, Dg, Dg16, w.kV.as<T>(), Dg16, w.ksrc.as<int>(),
-                                                     w.gp_of_atom.as<int>(), w.phatc.as<T>(), w.pnorm.as<T>(),
-                                                     w.pnormc.as<T>(), nullptr, rows, st)));
-        }
-        gap_prof_end(ST_KNM_JACOBIAN, st);
+    GAP_TRY(w.kA.ensure(sizeof(T) * nrow * g.D16));
+    rows.A = w.kA.p;
+    gap_prof_begin(ST_KNM_JACOBIAN, st);
+    GAP_TRY((gap_jacobian_rows<T, false>(g, tab_of<T>(soap), n, pl, spec, w.coef.as<T>(), w.phat.as<T>(),
+                                         w.pnorm.as<T>(), w.gp_of_atom.as<int>(), m->mu_all.as<float>(), rows, st)));
+    if (cmp && nrow) {
+        // V = J Q^T, then J~ in place: the force GEMM reads kV [nrow][Dg16]
+        GAP_TRY(w.kV.ensure(sizeof(T) * nrow * Dg16));
+        GAP_TRY(gap_rows_times_qt<T>((long)nrow, g.D, w.kA.as<T>(), g.D16, Dg, q_of<T>(soap), w.kV.as<T>(), Dg16, st));
+        rows.A = w.kV.p;
+        GAP_TRY((gap_jacobian_compress<T, false>((long)nrow, Dg, Dg16, w.kV.as<T>(), Dg16, w.ksrc.as<int>(),
+                                                 w.gp_of_atom.as<int>(), w.phatc.as<T>(), w.pnorm.as<T>(),
+                                                 w.pnormc.as<T>(), nullptr, rows, st)));
     }
-    if (tc) {  // destinations of the tensor-core epilogue's segment sums (all GPs)
-        GAP_TRY(w.kdest.ensure(sizeof(int) * (nrow > 0 ? nrow : 1)));
-        GAP_TRY(gap_knm_dest((long)nrow, w.kseg.as<int>(), w.segstart.as<int>(), w.outrow.as<int>(),
-                             w.kdest.as<int>(), st));
-    }
+    gap_prof_end(ST_KNM_JACOBIAN, st);
     gap_prof_end(ST_KNM_ROWS, st);
+    int col = 0;
     for (int s = 0; s < m->n_gp; ++s) {
         const GPData &gp = m->gp[s];
         if (gp.M == 0) continue;
-        const int R = counts[s];
         const int *grow = w.rows.as<int>() + (size_t)s * n;
-        const int ld = tc ? gp.M_pad : gp.M;
-        const __nv_bfloat16 *Blo = (three ? gp.Blo3 : gp.Blo).as<__nv_bfloat16>();
-        const size_t wbytes = (tc ? sizeof(float) : sizeof(T)) * (size_t)n * ld;
+        const int ld = gp.M;
+        const size_t wbytes = sizeof(T) * (size_t)n * ld;
         GAP_TRY(w.Wp.ensure(wbytes));
         GAP_TRY(w.kq.ensure(wbytes));
         if (n) {
@@ -1693,72 +1756,51 @@ static gap_status knm_impl(gap_model *m, const gap_batch *b, gap_precision prec,
             GAP_TRY_CUDA(cudaMemsetAsync(w.kq.p, 0, wbytes, st));
         }
         gap_prof_begin(ST_KNM_GEMM, st);
-        if (tc) {
-            if constexpr (sizeof(T) == 4) {
-                if (R > 0) {
-                    GAP_TRY(w.A_hi.ensure(2 * (size_t)R * Dg16));
-                    GAP_TRY(w.A_lo.ensure(2 * (size_t)R * Dg16));
-                    GAP_TRY(w.t_row.ensure(4 * (size_t)R));
-                    if (three) GAP_TRY(w.A_mid.ensure(2 * (size_t)R * Dg16));
-                    GAP_TRY(gap_split_rows(gp_phat<float>(soap, w), Dg, Dg16, grow, R,
-                                           m->mu_all.as<float>() + (size_t)s * Dg16, w.A_hi.as<__nv_bfloat16>(),
-                                           w.A_lo.as<__nv_bfloat16>(), three ? w.A_mid.as<__nv_bfloat16>() : nullptr,
-                                           w.t_row.as<float>(), st));
-                    TcOperands op1{w.A_hi.as<__nv_bfloat16>(), w.A_lo.as<__nv_bfloat16>(), gp.Bhi.as<__nv_bfloat16>(),
-                                   Blo, R, gp.M, Dg16, Dg16, Dg16, nsplit,
-                                   three ? w.A_mid.as<__nv_bfloat16>() : nullptr,
-                                   three ? gp.Bmid.as<__nv_bfloat16>() : nullptr};
-                    TcEpilogue e1{};
-                    e1.s_col = gp.s_col.as<float>();
-                    e1.t_row = w.t_row.as<float>();
-                    e1.d2 = (float)(m->delta * m->delta);
-                    e1.zeta = m->zeta;
-                    e1.row_map = grow;
-                    e1.Wp = w.Wp.as<float>();
-                    e1.kq = w.kq.as<float>();
-                    e1.ldwp = ld;
-                    GAP_TRY(gap_tc_gemm(op1, e1, EPI_QPOW, w.err.as<int>() + 2, st));
-                }
-                const int tiles = (int)((nrow + 127) / 128);
-                GAP_TRY(w.P.ensure(sizeof(float) * (size_t)tiles * 2 * ld));
-                TcOperands op2{w.kAhi.as<__nv_bfloat16>(), w.kAlo.as<__nv_bfloat16>(), gp.Bhi.as<__nv_bfloat16>(),
-                               Blo, (int)nrow, gp.M, Dg16, Dg16, Dg16, nsplit,
-                               three ? w.kAmid.as<__nv_bfloat16>() : nullptr,
-                               three ? gp.Bmid.as<__nv_bfloat16>() : nullptr};
-                TcEpilogue e2{};
-                e2.t_row = w.kt.as<float>();
-                e2.Wp = w.Wp.as<float>();
-                e2.ldwp = ld;
-                e2.src_sign = w.ksrc.as<int>();
-                e2.seg = w.kseg.as<int>();
-                e2.seg_start = w.segstart.as<int>();
-                e2.out_row = w.outrow.as<int>();
-                e2.dest = w.kdest.as<int>();
-                e2.K = K;
-                e2.ldk = Mt;
-                e2.col_out0 = col_off[s];
-                e2.P = w.P.as<float>();
-                e2.ldp = ld;
-                GAP_TRY(gap_tc_gemm(op2, e2, EPI_KNM, w.err.as<int>() + 2, st));
-                gap_prof_end(ST_KNM_GEMM, st);
-                gap_prof_begin(ST_KNM_REDUCE, st);
-                GAP_TRY(gap_knm_fixup((long)nrow, w.kseg.as<int>(), w.segstart.as<int>(), w.outrow.as<int>(),
-                                      w.P.as<float>(), ld, gp.M, K, Mt, col_off[s], st));
-                GAP_TRY(gap_knm_energy<float>(C, w.nbr.cfg_offsets, w.kq.as<float>(), ld, gp.M, K, Mt, col_off[s], st));
-                gap_prof_end(ST_KNM_REDUCE, st);
-            }
-        } else {
-            GAP_TRY(gap_knm_qpow_simt<T>(gp_phat<T>(soap, w), Dg, grow, R, gp_X<T>(gp), gp.M, m->delta, m->zeta, w.Wp.as<T>(),
-                                         w.kq.as<T>(), ld, st));
-            GAP_TRY(w.P.ensure(sizeof(T) * ((nrow + 63) / 64) * 2 * (size_t)ld));
-            GAP_TRY(gap_knm_force_simt<T>(reinterpret_cast<const T *>(rows.A), Dg, Dg16, (long)nrow, w.kseg.as<int>(), nseg,
-                                          w.segstart.as<int>(), w.outrow.as<int>(), w.ksrc.as<int>(), gp_X<T>(gp), gp.M,
-                                          w.Wp.as<T>(), ld, K, Mt, col_off[s], w.P.as<T>(), ld, st));
-            gap_prof_end(ST_KNM_GEMM, st);
-            gap_prof_begin(ST_KNM_REDUCE, st);
-            GAP_TRY(gap_knm_energy<T>(C, w.nbr.cfg_offsets, w.kq.as<T>(), ld, gp.M, K, Mt, col_off[s], st));
-            gap_prof_end(ST_KNM_REDUCE, st);
+        GAP_TRY(gap_knm_qpow_simt<T>(gp_phat<T>(soap, w), Dg, grow, counts[s], gp_X<T>(gp), gp.M, m->delta, m->zeta,
+                                     w.Wp.as<T>(), w.kq.as<T>(), ld, st));
+        GAP_TRY(w.P.ensure(sizeof(T) * ((nrow + 63) / 64) * 2 * (size_t)ld));
+        GAP_TRY(gap_knm_force_simt<T>(reinterpret_cast<const T *>(rows.A), Dg, Dg16, (long)nrow, w.kseg.as<int>(), nseg,
+                                      w.segstart.as<int>(), w.outrow.as<int>(), w.ksrc.as<int>(), gp_X<T>(gp), gp.M,
+                                      w.Wp.as<T>(), ld, K, Mt, col, w.P.as<T>(), ld, st));
+        gap_prof_end(ST_KNM_GEMM, st);
+        gap_prof_begin(ST_KNM_REDUCE, st);
+        GAP_TRY(gap_knm_energy<T>(C, w.nbr.cfg_offsets, w.kq.as<T>(), ld, gp.M, K, Mt, col, st));
+        gap_prof_end(ST_KNM_REDUCE, st);
+        col += gp.M;
+    }
+    return GAP_OK;
+}
+
+// knm == NULL keeps K_NM in the workspace (w.Kbuf) whatever the batch's
+// memory: the fused fit reads it there.
+template <typename T>
+static gap_status knm_impl(gap_model *m, const gap_batch *b, gap_precision prec, double *knm, cudaStream_t st)
+{
+    Workspace &w = m->ws;
+    const int n = b->n_atoms, C = b->n_configs;
+    const bool tc = prec == GAP_BF16X3 || prec == GAP_BF16X6;
+    int Mt = 0;
+    for (const GPData &gp : m->gp) Mt += gp.M;
+    const size_t krows = (size_t)C + 3 * (size_t)n;
+    double *K = knm;
+    if (!b->device || !knm) {
+        GAP_TRY(w.Kbuf.ensure(sizeof(double) * krows * (Mt > 0 ? Mt : 1)));
+        K = w.Kbuf.as<double>();
+    }
+    // With one species and its GP the tensor-core form writes every entry;
+    // else a target may have no triple of some GP.
+    if (krows * Mt && !(tc && m->soap->geo.S == 1 && m->n_gp == 1))
+        GAP_TRY_CUDA(cudaMemsetAsync(K, 0, sizeof(double) * krows * Mt, st));
+    const int *spec;
+    GAP_TRY(run_descriptor<T>(m->soap, w, b, &spec, st));
+    std::vector<int> counts;
+    GAP_TRY(gp_rows_all(m, w, n, spec, counts, st));
+    if (tc) {
+        if constexpr (sizeof(T) == 4) {
+            if (Mt > 0) GAP_TRY(knm_tc(m, w, b, prec == GAP_BF16X6 ? 3 : 2, spec, counts, K, Mt, st));
         }
+    } else {
+        GAP_TRY(knm_simt<T>(m, w, b, spec, counts, K, Mt, st));
     }
     if (!b->device && knm && krows * Mt)
         GAP_TRY_CUDA(cudaMemcpyAsync(knm, K, sizeof(double) * krows * Mt, cudaMemcpyDeviceToHost, st));

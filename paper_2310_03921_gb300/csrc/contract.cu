@@ -254,11 +254,12 @@ __global__ void k_gp_flags(int n, const int *__restrict__ species, int s, int *_
 }
 
 __global__ void k_gp_compact(int n, const int *__restrict__ flag, const int *__restrict__ pos, int *__restrict__ rows,
-                             int *__restrict__ gp_of_atom, int s)
+                             int *__restrict__ gp_of_atom, int *__restrict__ rank, int s)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n && flag[i]) {
         rows[pos[i]] = i;
+        rank[i] = pos[i];
         gp_of_atom[i] = s;
     }
 }
@@ -401,7 +402,7 @@ gap_status gap_contract_simt_fixed(const double *phat, int D, int ldg, const int
 }
 
 gap_status gap_gp_rows(int n, const int *species, int s, int *flag, int *pos, int *scan_tmp, int *rows, int *count,
-                       int *gp_of_atom, cudaStream_t st)
+                       int *gp_of_atom, int *rank, cudaStream_t st)
 {
     if (n == 0) {
         GAP_TRY_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
@@ -412,7 +413,7 @@ gap_status gap_gp_rows(int n, const int *species, int s, int *flag, int *pos, in
     GAP_TRY_CUDA(cudaGetLastError());
     GAP_TRY(gap_scan(flag, n, pos, scan_tmp, count, st));
     gap_count_launch();
-    k_gp_compact<<<(n + 255) / 256, 256, 0, st>>>(n, flag, pos, rows, gp_of_atom, s);
+    k_gp_compact<<<(n + 255) / 256, 256, 0, st>>>(n, flag, pos, rows, gp_of_atom, rank, s);
     return gap_cuda_status(cudaGetLastError(), "k_gp_compact");
 }
 

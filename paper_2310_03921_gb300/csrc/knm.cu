@@ -8,7 +8,9 @@
 // S_j = sum_{p of j} J_p (scaled by +W'_j) and one "incoming" row per pair
 // q = (i -> j) (scaled by -W'_i): 1 + n_j rows per (j, a), laid out
 // contiguously (target-major), so every K_F entry is a segmented row sum of
-// one GEMM [3 (N + P)] x D x M against the sparse points.
+// one GEMM [3 (N + P)] x D x M against the sparse points.  The tensor-core
+// form (knm_gemm.cu) keeps its own row order and GEMM; the CUDA-core forms
+// are here.
 #include "gap_internal.h"
 #include "knm.h"
 
@@ -54,8 +56,9 @@ __global__ void k_seg_tables(int n, const int *__restrict__ offsets, const int *
 // Jacobian rows: one warp per source atom i.  For each pair p = (i -> j)
 // the warp builds d c / d r_ij, d p / d r_ij and J_p = (dp - p_hat (p_hat . dp)) / |p|
 // and writes its three rows into target j's segments; the sum S_i of all J_p
-// becomes atom i's own rows.  SPLIT: rows as BF16 hi + lo and t_row = J . mu
-// (mu of atom i's GP); otherwise rows in T.
+// becomes atom i's own rows.  SPLIT: triples of the tensor-core form
+// (KnmTriples: BF16 planes and J . mu with mu of atom i's GP); otherwise rows
+// in T.
 // Shared memory of k_jacobian_rows, in elements: A/B ([channels][l] quads)
 // and the coefficients, rounded to whole quads; then Y_lm, its gradient,
 // R_nl, dR_nl, Q_l^m and (C_m, S_m), rounded to whole quads (the rows after
@@ -77,9 +80,9 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
                 const typename V4<T>::type *__restrict__ vec, const int *__restrict__ species,
                 const T *__restrict__ coef, const T *__restrict__ phat, const T *__restrict__ pnorm,
                 const int *__restrict__ gp_of_atom, const float *__restrict__ mu_all, T *__restrict__ A,
-                __nv_bfloat16 *__restrict__ Ahi, __nv_bfloat16 *__restrict__ Alo, __nv_bfloat16 *__restrict__ Amid,
-                float *__restrict__ t_row, int *__restrict__ src_sign, int *__restrict__ seg)
+                KnmTriples tr, int *__restrict__ src_sign, int *__restrict__ seg)
 {
+    __nv_bfloat16 *Ahi = tr.hi, *Alo = tr.lo, *Amid = tr.mid;
     constexpr int LM = (L + 1) * (L + 1), NL = N * (L + 1), NC = GA * N * LM;
     typedef typename V4<T>::type V4T;
     extern __shared__ __align__(32) unsigned char smem_raw[];
@@ -127,13 +130,18 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
     for (int k = 0; k < SK; ++k) sreg[k][0] = sreg[k][1] = sreg[k][2] = T(0);
     const T inv_norm = T(1) / pnorm[i];
     const int gp = gp_of_atom ? gp_of_atom[i] : -1;
-    const float *mu = (SPLIT && gp >= 0) ? mu_all + (size_t)gp * D16 : nullptr;
+    if (SPLIT && gp < 0) return;  // no sparse points of this species: no column of K_NM reads its rows
+    const float *mu = (SPLIT && mu_all) ? mu_all + (size_t)gp * D16 : nullptr;
+    const int *tfirst = SPLIT ? tr.first + (size_t)gp * n_atoms : nullptr;
     const int p0 = offsets[i], p1 = offsets[i + 1];
     const T rc = (T)geo.rc, dw = (T)geo.d, inv_h = T(1) / (T)geo.h;
     __syncwarp();
 
     auto write_rows = [&](const T *Jv, int row_base, int stride, int sgn, int seg0) {
-        // three rows row_base + a * stride, a = 0..2
+        // three rows row_base + a * stride, a = 0..2; SPLIT: a triple, negated
+        // for an incoming pair (sgn < 0)
+        float tv[3];
+#pragma unroll
         for (int a = 0; a < 3; ++a) {
             size_t row = (size_t)row_base + (size_t)a * stride;
             float t = 0.f;
@@ -151,7 +159,7 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
 #pragma unroll
                         for (int k = 0; k < 2; ++k) {
                             const int d = d0 + u + k;
-                            const float f = (float)jv[u + k];
+                            const float f = sgn > 0 ? (float)jv[u + k] : -(float)jv[u + k];
                             const __nv_bfloat16 hb = __float2bfloat16_rn(f);
                             float rest = f - __bfloat162float(hb);
                             f2[k] = __bfloat162float(hb);
@@ -180,14 +188,17 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
             } else {
                 for (int d = lane; d < D16; d += 32) A[row * D16 + d] = Jv[a * D16 + d];
             }
-            if (SPLIT) {
-                t = warp_sum(t);
-                if (lane == 0) t_row[row] = t;
-            }
-            if (lane == 0) {
+            tv[a] = SPLIT ? warp_sum(t) : t;
+            if (!SPLIT && lane == 0) {
                 src_sign[row] = sgn;
                 seg[row] = seg0 + a;
             }
+        }
+        if (SPLIT && lane == 0) {
+            const int q = row_base / 3, j = seg0 / 3;
+            tr.meta[q] = make_float4(tv[0], tv[1], tv[2], __int_as_float(tr.rank[i]));
+            tr.dest[q] = q + 1 == tfirst[j + 1] ? tr.atom_cfg[j] + 1 + 3 * j : -1;
+            if (tr.src) tr.src[q] = i;
         }
     };
 
@@ -334,9 +345,14 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
             }
         }
         __syncwarp();
-        const int nj = offsets[j + 1] - offsets[j];
-        const int slot = rev[p] - offsets[j];
-        write_rows(Jsm, 3 * (j + offsets[j]) + 1 + slot, 1 + nj, -(i + 1), 3 * j);
+        if (SPLIT) {
+            const int rv = rev[p];
+            write_rows(Jsm, 3 * (tfirst[j] + tr.slot[rv >= 0 ? rv : 0]), 1, -(i + 1), 3 * j);
+        } else {
+            const int nj = offsets[j + 1] - offsets[j];
+            const int slot = rev[p] - offsets[j];
+            write_rows(Jsm, 3 * (j + offsets[j]) + 1 + slot, 1 + nj, -(i + 1), 3 * j);
+        }
         __syncwarp();
     }
     if constexpr (SREG) {
@@ -348,10 +364,10 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
             if (d < D) { Jsm[d] = sreg[k][0]; Jsm[D16 + d] = sreg[k][1]; Jsm[2 * D16 + d] = sreg[k][2]; }
         }
         __syncwarp();
-        write_rows(Jsm, 3 * (i + offsets[i]), 1 + (p1 - p0), i + 1, 3 * i);
-    } else {
-        write_rows(Ssm, 3 * (i + offsets[i]), 1 + (p1 - p0), i + 1, 3 * i);
     }
+    const T *own = SREG ? Jsm : Ssm;
+    if (SPLIT) write_rows(own, 3 * tfirst[i], 1, i + 1, 3 * i);
+    else write_rows(own, 3 * (i + offsets[i]), 1 + (p1 - p0), i + 1, 3 * i);
 }
 
 // ----------------------------------------------------- CUDA-core forms
@@ -523,27 +539,6 @@ __global__ void k_knm_fixup(int n_seg, const int *__restrict__ seg_start, const 
 
 }  // namespace
 
-namespace {
-__global__ void k_knm_dest(long nrow, const int *__restrict__ seg, const int *__restrict__ seg_start,
-                           const int *__restrict__ out_row, int *__restrict__ dest)
-{
-    const long r = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (r >= nrow) return;
-    const long t0 = r - r % 128;
-    const int sg = seg[r];
-    dest[r] = (seg_start[sg] >= t0 && seg_start[sg + 1] <= t0 + 128) ? out_row[sg] : -1 - (r == t0 ? 0 : 1);
-}
-}  // namespace
-
-gap_status gap_knm_dest(long nrow, const int *seg, const int *seg_start, const int *out_row, int *dest,
-                        cudaStream_t st)
-{
-    if (nrow <= 0) return GAP_OK;
-    gap_count_launch();
-    k_knm_dest<<<(unsigned)((nrow + 255) / 256), 256, 0, st>>>(nrow, seg, seg_start, out_row, dest);
-    return gap_cuda_status(cudaGetLastError(), "k_knm_dest");
-}
-
 gap_status gap_knm_segments(int n, const int *offsets, const int *atom_cfg, int *seg_start, int *out_row,
                             cudaStream_t st)
 {
@@ -577,8 +572,7 @@ struct JacLaunch {
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();
         kern<<<n, 32, shm, st>>>(g, tab, n, pl.offsets, pl.j, pl.rev, vec, species, coef, phat, pnorm, gp_of_atom,
-                                 mu_all, reinterpret_cast<T *>(out.A), out.A_hi, out.A_lo, out.A_mid, out.t_row,
-                                 out.src_sign, out.seg);
+                                 mu_all, reinterpret_cast<T *>(out.A), out.tri, out.src_sign, out.seg);
         return gap_cuda_status(cudaGetLastError(), "k_jacobian_rows");
     }
 };
@@ -662,70 +656,6 @@ gap_status gap_knm_energy(int n_configs, const int *cfg_off, const T *kq, int ld
     return gap_cuda_status(cudaGetLastError(), "k_knm_energy");
 }
 
-namespace {
-// Cut segments of the 128-row tensor-core tiles: a tile originates at most
-// one, its last segment when that runs past the tile's end (slot 0 of P if
-// it starts at the tile's first row, else slot 1); every later tile it
-// covers holds its next partial in slot 0.
-// A block takes kFixTiles tiles and 128 columns: its first threads decode the
-// tiles' last segments at once, then every thread sums the cut ones.
-constexpr int kFixTiles = 64;
-__global__ void __launch_bounds__(128) k_knm_fixup_tiles(long nrow, const int *__restrict__ seg,
-                                                         const int *__restrict__ seg_start,
-                                                         const int *__restrict__ out_row, const float *__restrict__ P,
-                                                         int ldp, int M, double *__restrict__ K, int ldk,
-                                                         int col_out0)
-{
-    __shared__ int cut_sg[kFixTiles];  // segment originated and cut by the tile, or -1
-    __shared__ long cut_end[kFixTiles];
-    __shared__ unsigned char cut_slot[kFixTiles];
-    const long tiles = (nrow + 127) / 128;
-    const long tb = (long)blockIdx.x * kFixTiles;
-    if (threadIdx.x < kFixTiles) {
-        const long t = tb + threadIdx.x;
-        int sgc = -1;
-        if (t < tiles) {
-            const long t0 = t * 128, t1 = t0 + 128;
-            const long last = (t1 < nrow ? t1 : nrow) - 1;
-            const int sg = seg[last];
-            const long g0 = seg_start[sg], g1 = seg_start[sg + 1];
-            if (g1 > t1 && g0 >= t0) {  // runs past this tile and starts in it
-                sgc = sg;
-                cut_end[threadIdx.x] = g1;
-                cut_slot[threadIdx.x] = g0 == t0 ? 0 : 1;
-            }
-        }
-        cut_sg[threadIdx.x] = sgc;
-    }
-    __syncthreads();
-    const int m = blockIdx.y * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    for (int k = 0; k < kFixTiles; ++k) {
-        const int sg = cut_sg[k];
-        if (sg < 0) continue;
-        const long t = tb + k, g1 = cut_end[k];
-        double s = (double)P[((size_t)t * 2 + cut_slot[k]) * ldp + m];
-        for (long u = t + 1; u * 128 < g1; ++u) s += (double)P[((size_t)u * 2) * ldp + m];
-        K[(size_t)out_row[sg] * ldk + col_out0 + m] = s;
-    }
-}
-}  // namespace
-
-gap_status gap_knm_fixup(long nrow, const int *seg, const int *seg_start, const int *out_row, const float *P, int ldp,
-                         int M, double *K, int ldk, int col_out0, cudaStream_t st)
-{
-    if (nrow <= 0 || M <= 0) return GAP_OK;
-    const long tiles = (nrow + 127) / 128;
-    if (tiles > 2147483647L) {
-        gap_set_error("K_NM fix-up: too many tiles");
-        return GAP_EUNSUPPORTED;
-    }
-    dim3 grid((unsigned)((tiles + kFixTiles - 1) / kFixTiles), (M + 127) / 128);
-    gap_count_launch();
-    k_knm_fixup_tiles<<<grid, 128, 0, st>>>(nrow, seg, seg_start, out_row, P, ldp, M, K, ldk, col_out0);
-    return gap_cuda_status(cudaGetLastError(), "k_knm_fixup_tiles");
-}
-
 #define INSTK(T)                                                                                                     \
     template gap_status gap_knm_qpow_simt<T>(const T *, int, const int *, int, const T *, int, double, int, T *, T *, \
                                              int, cudaStream_t);                                                    \
@@ -802,18 +732,18 @@ __global__ void __launch_bounds__(256) k_rows_qt(long nrow, int D, const T *__re
 // its entries before the reduction and writes the same entries after it.
 template <typename T, bool SPLIT>
 __global__ void __launch_bounds__(256) k_jac_project(long nrow, int Dg, int Dg16, const T *V, int ldv,
-                                                     const int *__restrict__ src_sign,
+                                                     const int *__restrict__ src_sign, KnmTriples tr,
                                                      const int *__restrict__ gp_of_atom, const T *__restrict__ phatc,
                                                      const T *__restrict__ pnorm, const T *__restrict__ pnormc,
-                                                     const float *__restrict__ mu_all, T *A,
-                                                     __nv_bfloat16 *__restrict__ Ahi, __nv_bfloat16 *__restrict__ Alo,
-                                                     __nv_bfloat16 *__restrict__ Amid, float *__restrict__ t_row)
+                                                     const float *__restrict__ mu_all, T *A)
 {
+    __nv_bfloat16 *Ahi = tr.hi, *Alo = tr.lo, *Amid = tr.mid;
     const long row = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (row >= nrow) return;
-    const int sg = src_sign[row];
+    const int sg = SPLIT ? tr.src[row / 3] + 1 : src_sign[row];
     const int i = (sg > 0 ? sg : -sg) - 1;
+    if (SPLIT && i < 0) return;  // a triple of no GP
     const T *v = V + row * ldv;
     const T *ph = phatc + (size_t)i * Dg;
     T c = T(0);
@@ -843,7 +773,7 @@ __global__ void __launch_bounds__(256) k_jac_project(long nrow, int Dg, int Dg16
     }
     if constexpr (SPLIT) {
         t = warp_sum(t);
-        if (lane == 0) t_row[row] = t;
+        if (lane == 0) reinterpret_cast<float *>(tr.meta + row / 3)[row % 3] = t;
     }
 }
 }  // namespace
@@ -876,9 +806,8 @@ gap_status gap_jacobian_compress(long nrow, int Dg, int Dg16, const T *V, int ld
         return GAP_EUNSUPPORTED;
     }
     gap_count_launch();
-    k_jac_project<T, SPLIT><<<(unsigned)blocks, 256, 0, st>>>(nrow, Dg, Dg16, V, ldv, src_sign, gp_of_atom, phatc,
-                                                              pnorm, pnormc, mu_all, reinterpret_cast<T *>(out.A),
-                                                              out.A_hi, out.A_lo, out.A_mid, out.t_row);
+    k_jac_project<T, SPLIT><<<(unsigned)blocks, 256, 0, st>>>(nrow, Dg, Dg16, V, ldv, src_sign, out.tri, gp_of_atom, phatc,
+                                                              pnorm, pnormc, mu_all, reinterpret_cast<T *>(out.A));
     return gap_cuda_status(cudaGetLastError(), "k_jac_project");
 }
 

@@ -20,10 +20,6 @@
 //                BF16 hi/lo, per-tile partial sums of delta^2 alpha q^zeta and of W
 //   EPI_QPOW     per atom and sparse point, W' = zeta delta^2 q^(zeta-1) and
 //                delta^2 q^zeta (FP32) for the K_NM rows
-//   EPI_KNM      K_NM force rows: each Jacobian row scaled by +-W'[source atom],
-//                rows summed per (target atom, direction) segment, cut segments
-//                left as per-tile partials (EPI_KNM1: the form for K <= 256,
-//                accumulator kept in TMEM)
 //   EPI_STORE    FP32 store of C
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -55,103 +51,7 @@ struct SharedTail {
     uint64_t acc_empty[2];   // epilogue -> MMA (all epilogue threads arrive)
     uint32_t tmem_base;
     int abort;
-    unsigned seg_mask[4][4];  // per column group of the epilogue, per lane quadrant
 };
-
-// K_NM force rows: scale row r by sign * W'[src][col], then sum the rows of
-// each (target atom, xyz) segment of this 128-row tile.  Segments that are
-// wholly inside the tile go to K; a segment cut by a tile edge leaves a
-// partial sum in P[tile][slot] (slot 0: the tile's first segment) for the
-// fix-up pass.  Runs on the 128 threads of one column half.
-template <int BN>
-__device__ __forceinline__ void epilogue_knm(const TcEpilogue &ep, const float (&acc)[BN / 2],
-                                             unsigned char *stage_smem, SharedTail *tail, int quad, int lane,
-                                             int half, int row0, int col0, int rows, int ncol, int rt)
-{
-    constexpr int HC = BN / 2;
-    // [128 rows][32 columns] per half, column index XOR-swizzled by the row
-    // so that row-wise stores and column-wise sums are both conflict-free;
-    // then each row's signed source atom.
-    float *buf = reinterpret_cast<float *>(stage_smem) + half * (128 * 32);
-    int *rsrc = reinterpret_cast<int *>(reinterpret_cast<float *>(stage_smem) + 2 * 128 * 32) + half * 128;
-    const int rl = quad * 32 + lane;  // row within tile
-    const int r = row0 + rl;
-    const int nvalid = rows - row0 < 128 ? rows - row0 : 128;
-    int seg = -1;
-    float trow = 0.f;
-    rsrc[rl] = 0;
-    if (rl < nvalid) {
-        rsrc[rl] = ep.src_sign[r];
-        seg = ep.seg[r];
-        trow = ep.t_row[r];
-    }
-    bool start = rl < nvalid && (rl == 0 || ep.seg[r - 1] != seg);
-    unsigned m = __ballot_sync(0xffffffffu, start);
-    if (lane == 0) tail->seg_mask[half][quad] = m;
-    named_barrier(1 + half, 128);
-    unsigned masks[4] = {tail->seg_mask[half][0], tail->seg_mask[half][1], tail->seg_mask[half][2],
-                         tail->seg_mask[half][3]};
-    int nseg = __popc(masks[0]) + __popc(masks[1]) + __popc(masks[2]) + __popc(masks[3]);
-#pragma unroll
-    for (int ch = 0; ch < HC / 32; ++ch) {
-        int cbase = half * HC + ch * 32;
-        if (cbase < ncol) {
-            int c0 = col0 + cbase;
-#pragma unroll
-            for (int k = 0; k < 32; ++k) buf[rl * 32 + (k ^ lane)] = acc[ch * 32 + k] + trow;
-            named_barrier(1 + half, 128);
-            // warp `quad` sums segments quad, quad + 4, ...; lane = column.
-            // Each row is scaled by +-W'[source][column] here, where the
-            // loads of W' are one coalesced 128-byte row segment per row.
-            for (int sgi = quad; sgi < nseg; sgi += 4) {
-                int b = sgi, q = 0;
-                while (b >= __popc(masks[q])) { b -= __popc(masks[q]); ++q; }
-                unsigned mm = masks[q];
-                for (int t = 0; t < b; ++t) mm &= mm - 1;
-                int s0 = q * 32 + __ffs(mm) - 1;
-                int s1 = nvalid;
-                {
-                    unsigned rest = mm & (mm - 1);
-                    if (rest) s1 = q * 32 + __ffs(rest) - 1;
-                    else
-                        for (int q2 = q + 1; q2 < 4; ++q2)
-                            if (masks[q2]) { s1 = q2 * 32 + __ffs(masks[q2]) - 1; break; }
-                }
-                // the segment's destination, loaded ahead of the sums
-                const int dest = ep.dest[row0 + s0];
-                // eight rows at a time: eight W' loads in flight before the sums
-                float sum = 0.f;
-                int rr = s0;
-                for (; rr + 8 <= s1; rr += 8) {
-                    float wv[8];
-                    int sv[8];
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        sv[u] = rsrc[rr + u];
-                        wv[u] = __ldg(ep.Wp + (size_t)((sv[u] > 0 ? sv[u] : -sv[u]) - 1) * ep.ldwp + c0 + lane);
-                    }
-#pragma unroll
-                    for (int u = 0; u < 8; ++u) {
-                        const float v = buf[(rr + u) * 32 + (lane ^ ((rr + u) & 31))];
-                        sum = fmaf(sv[u] > 0 ? wv[u] : -wv[u], v, sum);
-                    }
-                }
-                for (; rr < s1; ++rr) {
-                    const int sv = rsrc[rr];
-                    const float w = __ldg(ep.Wp + (size_t)((sv > 0 ? sv : -sv) - 1) * ep.ldwp + c0 + lane);
-                    const float v = buf[rr * 32 + (lane ^ (rr & 31))];
-                    sum = fmaf(sv > 0 ? w : -w, v, sum);
-                }
-                int col = c0 + lane;
-                if (cbase + lane < ncol) {
-                    if (dest >= 0) ep.K[(size_t)dest * ep.ldk + ep.col_out0 + col] = (double)sum;
-                    else ep.P[((size_t)rt * 2 + (-1 - dest)) * ep.ldp + col] = sum;
-                }
-            }
-            named_barrier(1 + half, 128);
-        }
-    }
-}
 
 // q^e for 0 <= e < 64 by square-and-multiply over the six bits of e: fully
 // unrolled (e is the same for every thread), so the epilogue's element loops
@@ -165,131 +65,6 @@ __device__ __forceinline__ float powi_small(float q, int e)
         b *= b;
     }
     return r;
-}
-
-// EPI_KNM with a single K chunk (K <= 256): the accumulator stays in TMEM and
-// is read one 32-column slice at a time.  Each warp loads the W' slices of
-// its 32 rows cooperatively (eight lanes per 128-byte row segment, the next
-// slice's loads in flight during this slice's sums) into the staging rows;
-// each thread then scales its row's accumulator slice by +-W' in place, so
-// the segment sums read shared memory only.  Segment bounds and destinations
-// are decoded once per tile.
-constexpr int EPI_KNM1 = 4;
-constexpr int kKnmStartBytes = 136;  // per group: up to 128 segment starts and the end
-// Named barriers of the single-chunk K_NM epilogue's column groups (8 ..):
-// clear of 3 and 4, which the kernel uses across all epilogue warps.
-constexpr int kKnmGroupBar = 8;
-
-// Lane L of a warp loads W' for rows 4 i + L / 8 (i < 8) of the warp's 32
-// rows, columns c + 4 (L % 8) ... + 3; wsrc[i] is that row's source atom (-1:
-// a row past the end of the GEMM, zeros).  c is a multiple of 32 inside the
-// padded rows of W' (a multiple of 256 columns); c < 0 loads nothing.
-__device__ __forceinline__ void knm_w_rows(const float *__restrict__ Wp, int ldwp, const int (&wsrc)[8], int c,
-                                           int lane, float4 (&wq)[8])
-{
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        wq[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c >= 0 && wsrc[i] >= 0)
-            wq[i] = __ldg(reinterpret_cast<const float4 *>(Wp + (size_t)wsrc[i] * ldwp + c) + (lane & 7));
-    }
-}
-
-template <int BN, int NG>
-__device__ __forceinline__ void epilogue_knm1(const TcEpilogue &ep, uint32_t tacc, unsigned char *stage_smem,
-                                              SharedTail *tail, int quad, int lane, int half, int row0, int col0,
-                                              int rows, int ncol, int rt, const int (&wsrc)[8], float sgn,
-                                              float4 (&wq)[8])
-{
-    // `half` is the warp's column group (NG groups of BN / NG columns, four
-    // warps each, one per TMEM lane quadrant)
-    constexpr int HC = BN / NG;
-    // [128 rows][32 columns] per half; the 16-byte column group g of row R
-    // sits at group g ^ (R & 7), so that 16-byte row accesses (a thread per
-    // row, or eight lanes per row) and column reads (a lane per column) are
-    // all free of bank conflicts.  Then per half the segments' destinations
-    // and their start rows.
-    float *buf = reinterpret_cast<float *>(stage_smem) + half * (128 * 32);
-    int *sdest = reinterpret_cast<int *>(reinterpret_cast<float *>(stage_smem) + NG * 128 * 32);
-    unsigned char *sstart = reinterpret_cast<unsigned char *>(sdest + NG * 128) + half * kKnmStartBytes;
-    sdest += half * 128;
-    const int rl = quad * 32 + lane;  // row within tile
-    const int r = row0 + rl;
-    const int nvalid = rows - row0 < 128 ? rows - row0 : 128;
-    int seg = -1;
-    float trow = 0.f;
-    if (rl < nvalid) {
-        seg = ep.seg[r];
-        trow = ep.t_row[r];
-    }
-    const bool start = rl < nvalid && (rl == 0 || ep.seg[r - 1] != seg);
-    const unsigned m = __ballot_sync(0xffffffffu, start);
-    if (lane == 0) tail->seg_mask[half][quad] = m;
-    named_barrier(kKnmGroupBar + half, 128);
-    int before = 0, nseg = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int c = __popc(tail->seg_mask[half][q]);
-        before += q < quad ? c : 0;
-        nseg += c;
-    }
-    // segment k covers rows [sstart[k], sstart[k + 1]); visible to the half
-    // after the first slice's barrier
-    if (start) {
-        const int k = before + __popc(m & ((1u << lane) - 1u));
-        sstart[k] = (unsigned char)rl;
-        sdest[k] = ep.dest[r];
-    }
-    if (rl == 0) sstart[nseg] = (unsigned char)nvalid;
-    float *wrows = buf + quad * 32 * 32;  // this warp's 32 rows
-    float *myrow = buf + rl * 32;
-    for (int ch = 0; ch < HC / 32; ++ch) {
-        const int cbase = half * HC + ch * 32;
-        if (cbase >= ncol) break;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int rho = 4 * i + (lane >> 3);
-            *reinterpret_cast<float4 *>(wrows + rho * 32 + 4 * ((lane & 7) ^ (rho & 7))) = wq[i];
-        }
-        __syncwarp();
-        {
-            float v[32];
-            tmem_ld32(tacc + (uint32_t)cbase, v);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                float4 *p = reinterpret_cast<float4 *>(myrow + 4 * (j ^ (lane & 7)));
-                float4 w = *p;
-                w.x = (sgn * w.x) * (v[4 * j] + trow);
-                w.y = (sgn * w.y) * (v[4 * j + 1] + trow);
-                w.z = (sgn * w.z) * (v[4 * j + 2] + trow);
-                w.w = (sgn * w.w) * (v[4 * j + 3] + trow);
-                *p = w;
-            }
-        }
-        knm_w_rows(ep.Wp, ep.ldwp, wsrc, ch + 1 < HC / 32 && cbase + 32 < ncol ? col0 + cbase + 32 : -1, lane, wq);
-        named_barrier(kKnmGroupBar + half, 128);
-        // warp `quad` sums segments quad, quad + 4, ...; lane = column
-        const int col = col0 + cbase + lane;
-        const int cg = lane >> 2, cw = lane & 3;
-        for (int sgi = quad; sgi < nseg; sgi += 4) {
-            const int s0 = sstart[sgi], s1 = sstart[sgi + 1];
-            const int dest = sdest[sgi];
-            float sum = 0.f;
-            int rr = s0;
-            for (; rr + 8 <= s1; rr += 8) {
-                float a[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) a[u] = buf[(rr + u) * 32 + 4 * (cg ^ ((rr + u) & 7)) + cw];
-                sum += ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
-            }
-            for (; rr < s1; ++rr) sum += buf[rr * 32 + 4 * (cg ^ (rr & 7)) + cw];
-            if (cbase + lane < ncol) {
-                if (dest >= 0) ep.K[(size_t)dest * ep.ldk + ep.col_out0 + col] = (double)sum;
-                else ep.P[((size_t)rt * 2 + (-1 - dest)) * ep.ldp + col] = sum;
-            }
-        }
-        named_barrier(kKnmGroupBar + half, 128);
-    }
 }
 
 // One GEMM problem of a launch: its operand maps (A hi / mid-or-lo / lo, B
@@ -306,23 +81,18 @@ template <int G> struct TcProblems {
     TcProblem p[G];
 };
 
-// The single-chunk K_NM instantiation (EPI_KNM1) returns to the tile loop
-// before the register-accumulator path, which is unreachable there.
-#pragma nv_diag_suppress 128
-
 // NS = number of BF16 planes per operand: 2 (hi, lo: three MMAs per K step)
 // or 3 (hi, mid, lo: the six products with plane-index sum <= 2, an
 // FP32-grade product).
-// EW = epilogue warps: 8 (two column groups), or 12 (three, the K_NM
-// single-chunk epilogue on 192-column tiles).
+// EW = epilogue warps: 8 (two column groups), or 12 (three, on 192-column
+// tiles).
 template <int BN, int STAGES, int EPI, int NS, int G, int EW>
 __global__ void __launch_bounds__(32 * (2 + EW), 1)
 k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
 {
     static_assert(BN == 128 || BN == 192 || BN == 256, "tile width");
     static_assert(NS == 2 || NS == 3, "planes");
-    static_assert(EW == 8 || (EW == 12 && (EPI == EPI_KNM1 || EPI == EPI_KERNEL || EPI == EPI_STORE) && BN == 192),
-                  "epilogue warps");
+    static_assert(EW == 8 || (EW == 12 && (EPI == EPI_KERNEL || EPI == EPI_STORE) && BN == 192), "epilogue warps");
     constexpr int kThreads = 32 * (2 + EW);  // this instantiation's block
     constexpr int NG = EW / 4;               // epilogue column groups
     constexpr uint32_t TMEM_COLS = 2 * BN <= 256 ? 256 : 512;  // two accumulators, a power of two
@@ -502,38 +272,6 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                 }
                 named_barrier(3, kThreads - 64);
             }
-            if constexpr (EPI == EPI_KNM1) {
-                // one K chunk: the epilogue reads the accumulator in TMEM and
-                // releases the buffer when it is done
-                const int buf = gc & 1, use = gc >> 1;
-                // this row's sign and the source atoms of the rows whose W'
-                // slices this lane loads; the first slice's loads are in
-                // flight while the accumulator completes
-                const int sv = r < rows ? ep.src_sign[r] : 0;
-                int wsrc[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int ri = row0 + quad * 32 + 4 * i + (lane >> 3);
-                    const int si = ri < rows ? ep.src_sign[ri] : 0;
-                    wsrc[i] = si != 0 ? (si > 0 ? si : -si) - 1 : -1;
-                }
-                float4 wq[8];
-                knm_w_rows(ep.Wp, ep.ldwp, wsrc, half * HC < ncol ? col0 + half * HC : -1, lane, wq);
-                bool ok1 = mbar_wait(&tail->acc_full[buf], use & 1, abort_flag, wlim);
-                if (!ok1) {
-                    *abort_flag = 1;
-                    atomicOr(err, 4);
-                }
-                tc_fence_after();
-                ok1 = bar_and(4, kThreads - 64, ok1);
-                if (!ok1) break;
-                epilogue_knm1<BN, NG>(ep, tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * BN), scratch, tail,
-                                  quad, lane, half, row0, col0, rows, ncol, rt, wsrc, sv > 0 ? 1.f : -1.f, wq);
-                tc_fence_before();
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tail->acc_empty[buf]))
-                             : "memory");
-                continue;
-            }
             // promoted accumulation of the chunk results
             float acc[HC];
 #pragma unroll
@@ -566,9 +304,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
             // named barriers), so a wait that expired in one warp stops them all
             ok = bar_and(4, kThreads - 64, ok);
             if (!ok) break;
-            if constexpr (EPI == EPI_KNM) {
-                epilogue_knm<BN>(ep, acc, scratch, tail, quad, lane, half, row0, col0, rows, ncol, rt);
-            } else {
+            {
                 float esum = 0.f, wsum = 0.f;
                 const int zeta = ep.zeta;
 #pragma unroll
@@ -591,7 +327,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                         }
                     } else if (EPI == EPI_QPOW) {
                         const float tr = ep.t_row[r];
-                        int orow = ep.row_map[r];
+                        const int orow = ep.row_map ? ep.row_map[r] : r;
                         float *pw = ep.Wp + (size_t)orow * ep.ldwp + c0, *pk = ep.kq + (size_t)orow * ep.ldwp + c0;
 #pragma unroll
                         for (int k = 0; k < 32; k += 4) {
@@ -756,11 +492,7 @@ gap_status launch_g(const TcOperands *ops, const TcEpilogue *eps, int n, int *er
         return GAP_EUNSUPPORTED;
     }
     P.n_tiles = (int)tiles;
-    constexpr int NG = EW / 4;  // epilogue column groups
-    const size_t scratch = EPI == EPI_KNM ? 2 * 128 * 32 * sizeof(float) + 2 * 128 * sizeof(int)
-                           : EPI == EPI_KNM1
-                               ? NG * (128 * 32 * sizeof(float) + 128 * sizeof(int) + kKnmStartBytes)
-                               : 2 * BN * sizeof(float);
+    const size_t scratch = 2 * BN * sizeof(float);
     size_t shm = (size_t)STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + ((sizeof(SharedTail) + 127) & ~size_t(127)) +
                  scratch + 1024;
     auto kern = k_tc_gemm<BN, STAGES, EPI, NS, G, EW>;
@@ -785,25 +517,25 @@ gap_status launch_grouped(const TcOperands *ops, const TcEpilogue *eps, int n, i
     constexpr int BN = NS == 3 ? 128 : 256;
     if (epi == EPI_KERNEL) return launch_g<BN, 2, EPI_KERNEL, NS, kMaxGroups>(ops, eps, n, err, st);
     if (epi == EPI_STORE) return launch_g<BN, 2, EPI_STORE, NS, kMaxGroups>(ops, eps, n, err, st);
-    gap_set_error("grouped tensor-core GEMM: energy and store epilogues only");
+    if (epi == EPI_QPOW) return launch_g<BN, 2, EPI_QPOW, NS, kMaxGroups>(ops, eps, n, err, st);
+    gap_set_error("grouped tensor-core GEMM: bad epilogue");
     return GAP_EINVAL;
 }
 
 // Tile variants of the two-plane split: (column tile, TMA stages, epilogue
 // warps).  The three-plane split has one (128, 2): its 96 KB stages leave
 // room for two.  The last variant (192 columns, twelve epilogue warps in
-// three column groups) exists for the K_NM single-chunk epilogue only.
+// three column groups) exists for the kernel-energy and store epilogues.
 struct TileVariant {
     int bn, stages, ew;
 };
 constexpr TileVariant kVariants2[] = {{256, 2, 8}, {128, 2, 8}, {128, 3, 8}, {192, 2, 12}};
 constexpr int kNumVariants2 = 4;
-constexpr int kVariantKnmWide = 3;
+constexpr int kVariantWide = 3;
 
 bool variant_applies(int v, const TcOperands &op, int epi)
 {
-    return v < kVariantKnmWide ||
-           (op.nsplit == 2 && ((epi == EPI_KNM && op.K <= 4 * BK) || epi == EPI_KERNEL || epi == EPI_STORE));
+    return v < kVariantWide || (op.nsplit == 2 && (epi == EPI_KERNEL || epi == EPI_STORE));
 }
 
 template <int BN, int ST, int NS>
@@ -811,22 +543,19 @@ gap_status launch_bn(const TcOperands &op, const TcEpilogue &ep, int epi, int *e
 {
     if (epi == EPI_KERNEL) return launch<BN, ST, EPI_KERNEL, NS>(op, ep, err, st);
     if (epi == EPI_QPOW) return launch<BN, ST, EPI_QPOW, NS>(op, ep, err, st);
-    if (epi == EPI_KNM)  // one K chunk of KC blocks: the TMEM-resident epilogue
-        return op.K <= 4 * BK ? launch<BN, ST, EPI_KNM1, NS>(op, ep, err, st) : launch<BN, ST, EPI_KNM, NS>(op, ep, err, st);
     return launch<BN, ST, EPI_STORE, NS>(op, ep, err, st);
 }
 
 gap_status launch_variant(const TcOperands &op, const TcEpilogue &ep, int epi, int v, int *err, cudaStream_t st)
 {
     if (op.nsplit == 3) return launch_bn<128, 2, 3>(op, ep, epi, err, st);
-    if (v == kVariantKnmWide) {
+    if (v == kVariantWide) {
         if (!variant_applies(v, op, epi)) {
-            gap_set_error("tile variant for the K_NM and kernel-energy epilogues only");
+            gap_set_error("tile variant for the kernel-energy and store epilogues only");
             return GAP_EINVAL;
         }
         if (epi == EPI_KERNEL) return launch_g<192, 2, EPI_KERNEL, 2, 1, 12>(&op, &ep, 1, err, st);
-        if (epi == EPI_STORE) return launch_g<192, 2, EPI_STORE, 2, 1, 12>(&op, &ep, 1, err, st);
-        return launch_g<192, 2, EPI_KNM1, 2, 1, 12>(&op, &ep, 1, err, st);
+        return launch_g<192, 2, EPI_STORE, 2, 1, 12>(&op, &ep, 1, err, st);
     }
 
     switch (v) {
@@ -880,6 +609,13 @@ TcEpilogue with_parts(const TcEpilogue &ep, int epi, const TcOperands &op, const
 }
 
 }  // namespace
+
+int gap_tc_sm_count() { return sm_count(); }
+
+gap_status gap_tc_make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows)
+{
+    return make_map(m, ptr, rows, cols, ld, box_rows);
+}
 
 int gap_tc_max_parts(int cols)
 {

@@ -1,9 +1,11 @@
 // Split-precision BF16 tensor-core GEMM (internal).
 #pragma once
 
+#include <cuda.h>
+
 #include "gap_internal.h"
 
-enum { EPI_STORE = 0, EPI_KERNEL = 1, EPI_QPOW = 2, EPI_KNM = 3 };
+enum { EPI_STORE = 0, EPI_KERNEL = 1, EPI_QPOW = 2 };
 
 // A: [rows][K] (leading dimension lda elements), B: [cols][K] (ldb), both BF16
 // K-major, hi and lo parts.  K must be a multiple of 16; lda, ldb multiples of 8.
@@ -27,20 +29,9 @@ struct TcEpilogue {
     int ldw;
     float *eps_part, *wsum_part;  // [rows][n_part]
     int n_part;                   // 2 * number of column tiles
-    // EPI_QPOW: Wp[row_map[r]][c] = zeta d2 q^(zeta-1), kq[row_map[r]][c] = d2 q^zeta
+    // EPI_QPOW (row_map: optional): Wp[row][c] = zeta d2 q^(zeta-1), kq[row][c] = d2 q^zeta
     float *Wp, *kq;
     int ldwp;
-    // EPI_KNM (also uses t_row, Wp, ldwp)
-    const int *src_sign;   // [rows] +(atom+1) own row, -(atom+1) incoming row
-    const int *seg;        // [rows] segment (3 * target + xyz) of each row
-    const int *seg_start;  // [segments + 1]
-    const int *out_row;    // [segments] row of K
-    const int *dest;       // [rows] where a segment starting at this row (or a tile's first row)
-                           // goes: its K row, or -1 - slot of P[tile][slot] (gap_knm_dest)
-    double *K;
-    int ldk, col_out0;
-    float *P;              // [row tiles][2][ldp] partial sums of cut segments
-    int ldp;
     // Bounded waits: limit of each mbarrier wait in ns (0: the default 2 s).
     unsigned long long wait_ns;
     // Test of the timeout path: the producer issues no copies (so no MMA is
@@ -60,16 +51,19 @@ int gap_tc_plan(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, c
 // The tuner's record, in the order the shape classes were tuned: fields =
 // (epilogue, planes, K, columns, ceil(log2 rows), column tile, stages,
 // device), ms[4] = best time of each variant (256/2, 128/2, 128/3, and
-// 192/2 with twelve epilogue warps for the K_NM single-chunk epilogue; -1
-// where a variant is not a candidate).
+// 192/2 with twelve epilogue warps; -1 where a variant is not a candidate).
 int gap_tc_tuned_count();
 // Test hook: every later two-plane call where variant v applies uses it (v < 0: the tuner).
 void gap_tc_force_variant(int v);
 bool gap_tc_tuned_entry(int k, int *fields, float *ms);
+// SMs of the current device, and the tensor map of a BF16 operand
+// [rows][ld] (cols of them valid) loaded in boxes of box_rows x 64.
+int gap_tc_sm_count();
+gap_status gap_tc_make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows);
 // *err (device int) receives a nonzero code if a bounded wait expired.
 gap_status gap_tc_gemm(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, cudaStream_t st);
 // Several problems (the GEMMs of a batch's GPs: same planes, epilogue
-// EPI_KERNEL or EPI_STORE) in one persistent launch per four problems, tiles
+// EPI_KERNEL, EPI_QPOW or EPI_STORE) in one persistent launch per four problems, tiles
 // numbered problem after problem; the default tile variant, whose column tile
 // gap_tc_grouped_col_tile gives (EPI_KERNEL's n_part must be 2 ceil(cols / it)).
 int gap_tc_grouped_col_tile(int nsplit);

@@ -537,7 +537,7 @@ def launch_count() -> int:
     return int(lib().gap_launch_count())
 
 
-EPILOGUES = {0: "store", 1: "kernel", 2: "qpow", 3: "knm"}
+EPILOGUES = {0: "store", 1: "kernel", 2: "qpow"}
 
 
 def tile_tuning() -> list:
