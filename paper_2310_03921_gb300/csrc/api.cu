@@ -335,7 +335,7 @@ struct gap_soap {
     double *tab64 = nullptr;   // knot values and derivatives (FP64)
     double *coef64 = nullptr;  // per-interval cubic coefficients
     float *coef32 = nullptr;
-    int4 *dtab = nullptr;      // geo.dtab
+    int4 *dtab = nullptr;      // geo.dtab and, after it, geo.etab
     // Compression (gap_soap_set_compression): the GP sees p~ / |p~| with
     // p~ = Q p, Q [Dg][D] (FP64 and FP32 copies, and the BF16 planes
     // [Dg16][D16] of the FP32 copy for the tensor-core K_NM rows: hi, lo of
@@ -435,16 +435,26 @@ extern "C" gap_status gap_soap_create(const gap_soap_params *p, gap_soap **out)
                                               (g2 * g.N + n2) * g.LM + l * l, l | ((a != ap ? 1 : 0) << 8)));
                     }
             }
-        gap_status ts = gap_cuda_status(cudaMalloc((void **)&s->dtab, sizeof(int4) * t.size()), "cudaMalloc");
+        std::vector<unsigned> et(g.D);
+        for (const int4 &e : t) {
+            const int l = e.w & 0xff, c1 = (e.y - l * l) / g.LM, c2 = (e.z - l * l) / g.LM;
+            et[e.x] = (unsigned)(c1 * (g.L + 1) + l) | (unsigned)(c2 * (g.L + 1) + l) << 8 | (unsigned)(e.w >> 8) << 16;
+        }
+        gap_status ts = gap_cuda_status(
+            cudaMalloc((void **)&s->dtab, sizeof(int4) * t.size() + sizeof(unsigned) * et.size()), "cudaMalloc");
         if (ts == GAP_OK)
             ts = gap_cuda_status(cudaMemcpy(s->dtab, t.data(), sizeof(int4) * t.size(), cudaMemcpyHostToDevice),
                                  "cudaMemcpy");
+        if (ts == GAP_OK)
+            ts = gap_cuda_status(cudaMemcpy(s->dtab + t.size(), et.data(), sizeof(unsigned) * et.size(),
+                                            cudaMemcpyHostToDevice), "cudaMemcpy");
         if (ts != GAP_OK) {
             if (s->dtab) cudaFree(s->dtab);
             delete s;
             return ts;
         }
         g.dtab = s->dtab;
+        g.etab = reinterpret_cast<const unsigned *>(s->dtab + t.size());
     }
     gap_status st = gap_radial_table(g, &s->tab64, &s->coef64, &s->coef32);
     if (st != GAP_OK) {
@@ -1615,9 +1625,9 @@ static gap_status knm_tc(gap_model *m, Workspace &w, const gap_batch *b, int nsp
         GAP_TRY(gap_scan(w.kcount.as<int>(), G * n, w.kfirst.as<int>(), w.scan_tmp.as<int>(), nullptr, st));
         if (cmp) GAP_TRY_CUDA(cudaMemsetAsync(w.ksrc.p, 0xff, sizeof(int) * (size_t)nt, st));
         gap_prof_begin(ST_KNM_JACOBIAN, st);
-        GAP_TRY((gap_jacobian_rows<float, true>(g, tab_of<float>(soap), n, pl, spec, w.coef.as<float>(),
-                                                w.phat.as<float>(), w.pnorm.as<float>(), w.gp_of_atom.as<int>(),
-                                                cmp ? nullptr : m->mu_all.as<float>(), rows, st)));
+        GAP_TRY(gap_jacobian_triples(g, tab_of<float>(soap), n, pl, spec, w.coef.as<float>(), w.phat.as<float>(),
+                                     w.pnorm.as<float>(), w.gp_of_atom.as<int>(),
+                                     cmp ? nullptr : m->mu_all.as<float>(), rows.tri, st));
         if (cmp) {
             // V = J Q^T on the tensor cores (J's planes against Q's), then
             // J~ into the same planes (J is consumed by then), Dg16 wide
@@ -1729,8 +1739,8 @@ static gap_status knm_simt(gap_model *m, Workspace &w, const gap_batch *b, const
     GAP_TRY(w.kA.ensure(sizeof(T) * nrow * g.D16));
     rows.A = w.kA.p;
     gap_prof_begin(ST_KNM_JACOBIAN, st);
-    GAP_TRY((gap_jacobian_rows<T, false>(g, tab_of<T>(soap), n, pl, spec, w.coef.as<T>(), w.phat.as<T>(),
-                                         w.pnorm.as<T>(), w.gp_of_atom.as<int>(), m->mu_all.as<float>(), rows, st)));
+    GAP_TRY(gap_jacobian_rows<T>(g, tab_of<T>(soap), n, pl, spec, w.coef.as<T>(), w.phat.as<T>(), w.pnorm.as<T>(),
+                                 rows, st));
     if (cmp && nrow) {
         // V = J Q^T, then J~ in place: the force GEMM reads kV [nrow][Dg16]
         GAP_TRY(w.kV.ensure(sizeof(T) * nrow * Dg16));

@@ -71,6 +71,10 @@ struct SoapGeom {
     // coupled channels' (n, l, m = -l) coefficients, so that consecutive
     // entries share their m-range.
     const int4 *dtab;
+    // Device table of the entries in descriptor order: the two channels'
+    // (channel (L + 1) + l) places in bytes 0 and 1, bit 16 set when they
+    // differ (0xff.. places are not used: shapes without K_NM rows).
+    const unsigned *etab;
 };
 
 // 32-byte aligned (dx, dy, dz, r) of a pair in FP64.

@@ -56,9 +56,7 @@ __global__ void k_seg_tables(int n, const int *__restrict__ offsets, const int *
 // Jacobian rows: one warp per source atom i.  For each pair p = (i -> j)
 // the warp builds d c / d r_ij, d p / d r_ij and J_p = (dp - p_hat (p_hat . dp)) / |p|
 // and writes its three rows into target j's segments; the sum S_i of all J_p
-// becomes atom i's own rows.  SPLIT: triples of the tensor-core form
-// (KnmTriples: BF16 planes and J . mu with mu of atom i's GP); otherwise rows
-// in T.
+// becomes atom i's own rows.
 // Shared memory of k_jacobian_rows, in elements: A/B ([channels][l] quads)
 // and the coefficients, rounded to whole quads; then Y_lm, its gradient,
 // R_nl, dR_nl, Q_l^m and (C_m, S_m), rounded to whole quads (the rows after
@@ -73,16 +71,14 @@ __host__ __device__ constexpr int jac_head_words(int N, int L, int GA)
            4 * 4;
 }
 
-template <int N, int L, int GA, typename T, bool SPLIT>
+template <int N, int L, int GA, typename T>
 __global__ void __launch_bounds__(32)
 k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int *__restrict__ offsets,
                 const int *__restrict__ nbr_j, const int *__restrict__ rev,
                 const typename V4<T>::type *__restrict__ vec, const int *__restrict__ species,
                 const T *__restrict__ coef, const T *__restrict__ phat, const T *__restrict__ pnorm,
-                const int *__restrict__ gp_of_atom, const float *__restrict__ mu_all, T *__restrict__ A,
-                KnmTriples tr, int *__restrict__ src_sign, int *__restrict__ seg)
+                T *__restrict__ A, int *__restrict__ src_sign, int *__restrict__ seg)
 {
-    __nv_bfloat16 *Ahi = tr.hi, *Alo = tr.lo, *Amid = tr.mid;
     constexpr int LM = (L + 1) * (L + 1), NL = N * (L + 1), NC = GA * N * LM;
     typedef typename V4<T>::type V4T;
     extern __shared__ __align__(32) unsigned char smem_raw[];
@@ -129,76 +125,19 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
 #pragma unroll
     for (int k = 0; k < SK; ++k) sreg[k][0] = sreg[k][1] = sreg[k][2] = T(0);
     const T inv_norm = T(1) / pnorm[i];
-    const int gp = gp_of_atom ? gp_of_atom[i] : -1;
-    if (SPLIT && gp < 0) return;  // no sparse points of this species: no column of K_NM reads its rows
-    const float *mu = (SPLIT && mu_all) ? mu_all + (size_t)gp * D16 : nullptr;
-    const int *tfirst = SPLIT ? tr.first + (size_t)gp * n_atoms : nullptr;
     const int p0 = offsets[i], p1 = offsets[i + 1];
     const T rc = (T)geo.rc, dw = (T)geo.d, inv_h = T(1) / (T)geo.h;
     __syncwarp();
 
     auto write_rows = [&](const T *Jv, int row_base, int stride, int sgn, int seg0) {
-        // three rows row_base + a * stride, a = 0..2; SPLIT: a triple, negated
-        // for an incoming pair (sgn < 0)
-        float tv[3];
-#pragma unroll
+        // three rows row_base + a * stride, a = 0..2
         for (int a = 0; a < 3; ++a) {
-            size_t row = (size_t)row_base + (size_t)a * stride;
-            float t = 0.f;
-            if constexpr (SPLIT) {
-                // eight entries per lane: one 16-byte store per plane (D16 is
-                // a multiple of 16, so every chunk is aligned and in the row)
-                for (int d0 = 8 * lane; d0 < D16; d0 += 256) {
-                    T jv[8];
-                    *reinterpret_cast<float4 *>(jv) = *reinterpret_cast<const float4 *>(Jv + a * D16 + d0);
-                    *reinterpret_cast<float4 *>(jv + 4) = *reinterpret_cast<const float4 *>(Jv + a * D16 + d0 + 4);
-                    uint32_t hi[4], mid[4], lo[4];
-#pragma unroll
-                    for (int u = 0; u < 8; u += 2) {
-                        float f2[2], r2[2], m2[2];
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            const int d = d0 + u + k;
-                            const float f = sgn > 0 ? (float)jv[u + k] : -(float)jv[u + k];
-                            const __nv_bfloat16 hb = __float2bfloat16_rn(f);
-                            float rest = f - __bfloat162float(hb);
-                            f2[k] = __bfloat162float(hb);
-                            if (Amid) {
-                                const __nv_bfloat16 mb = __float2bfloat16_rn(rest);
-                                m2[k] = __bfloat162float(mb);
-                                rest -= m2[k];
-                            } else {
-                                m2[k] = 0.f;
-                            }
-                            r2[k] = rest;
-                            if (mu) t += f * mu[d];
-                        }
-                        __nv_bfloat162 h = __floats2bfloat162_rn(f2[0], f2[1]);
-                        __nv_bfloat162 mm = __floats2bfloat162_rn(m2[0], m2[1]);
-                        __nv_bfloat162 l2 = __floats2bfloat162_rn(r2[0], r2[1]);
-                        hi[u / 2] = *reinterpret_cast<uint32_t *>(&h);
-                        mid[u / 2] = *reinterpret_cast<uint32_t *>(&mm);
-                        lo[u / 2] = *reinterpret_cast<uint32_t *>(&l2);
-                    }
-                    *reinterpret_cast<uint4 *>(Ahi + row * D16 + d0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-                    *reinterpret_cast<uint4 *>(Alo + row * D16 + d0) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-                    if (Amid)
-                        *reinterpret_cast<uint4 *>(Amid + row * D16 + d0) = make_uint4(mid[0], mid[1], mid[2], mid[3]);
-                }
-            } else {
-                for (int d = lane; d < D16; d += 32) A[row * D16 + d] = Jv[a * D16 + d];
-            }
-            tv[a] = SPLIT ? warp_sum(t) : t;
-            if (!SPLIT && lane == 0) {
+            const size_t row = (size_t)row_base + (size_t)a * stride;
+            for (int d = lane; d < D16; d += 32) A[row * D16 + d] = Jv[a * D16 + d];
+            if (lane == 0) {
                 src_sign[row] = sgn;
                 seg[row] = seg0 + a;
             }
-        }
-        if (SPLIT && lane == 0) {
-            const int q = row_base / 3, j = seg0 / 3;
-            tr.meta[q] = make_float4(tv[0], tv[1], tv[2], __int_as_float(tr.rank[i]));
-            tr.dest[q] = q + 1 == tfirst[j + 1] ? tr.atom_cfg[j] + 1 + 3 * j : -1;
-            if (tr.src) tr.src[q] = i;
         }
     };
 
@@ -345,14 +284,9 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
             }
         }
         __syncwarp();
-        if (SPLIT) {
-            const int rv = rev[p];
-            write_rows(Jsm, 3 * (tfirst[j] + tr.slot[rv >= 0 ? rv : 0]), 1, -(i + 1), 3 * j);
-        } else {
-            const int nj = offsets[j + 1] - offsets[j];
-            const int slot = rev[p] - offsets[j];
-            write_rows(Jsm, 3 * (j + offsets[j]) + 1 + slot, 1 + nj, -(i + 1), 3 * j);
-        }
+        const int nj = offsets[j + 1] - offsets[j];
+        const int slot = rev[p] - offsets[j];
+        write_rows(Jsm, 3 * (j + offsets[j]) + 1 + slot, 1 + nj, -(i + 1), 3 * j);
         __syncwarp();
     }
     if constexpr (SREG) {
@@ -366,8 +300,337 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
         __syncwarp();
     }
     const T *own = SREG ? Jsm : Ssm;
-    if (SPLIT) write_rows(own, 3 * tfirst[i], 1, i + 1, 3 * i);
-    else write_rows(own, 3 * (i + offsets[i]), 1 + (p1 - p0), i + 1, 3 * i);
+    write_rows(own, 3 * (i + offsets[i]), 1 + (p1 - p0), i + 1, 3 * i);
+}
+
+// ------------------------------------------ tensor-core form: BF16 triples
+// Jacobian triples of every pair and atom (KnmTriples), one block per source
+// atom, FP32.  Pairs are taken kTriBatch at a time, every phase with its
+// lanes over (pair, task): radial functions, Legendre columns, Y_lm and
+// gradients, then A and B per (l, pair, channel) so that a warp's lanes run
+// one m-range.  Each lane owns descriptor entries 64 k + 2 lane, + 1 of its
+// warp's KW groups, so the rows go out as full 128-byte stores of BF16 pairs,
+// the own row accumulates in registers and nothing is staged.  J is
+// projected with pd = p_hat . dp, and J . mu = (dp . mu - pd p_hat . mu) / |p|
+// comes from the same pass.  Descriptors beyond 256 entries use several warps
+// per atom (MULTI), which form pd in a first pass over the batch.  Latency
+// bound: 18 warps per SM.  K_NM of 200 silicon cells takes 0.73 ms less than
+// with a warp walking one pair after another through staged rows, of 24
+// four-species boxes (D = 1008, 1067 atoms) 0.78 ms less of 1.74.
+constexpr int kTriBatch = 4;
+
+struct TriPair {  // one pair of the batch
+    float ux, uy, uz, ir, r, f, df, u;
+    int k, j, z, q;
+};
+
+template <int N, int L, int GA> struct TriShape {
+    static constexpr int LM = (L + 1) * (L + 1), NL = N * (L + 1), NAB = GA * NL, NC = GA * N * LM;
+    static constexpr int G64 = GA == 1 ? ((N * (N + 1) / 2 * (L + 1) + 15) / 16 * 16 + 63) / 64 : 0;  // groups of 64 entries
+    static constexpr int W = (G64 + 3) / 4;                                                      // warps (GA == 1)
+    static constexpr int KW = GA == 1 ? (G64 + W - 1) / (W > 0 ? W : 1) : 4;                      // groups per warp
+    // block sizes: registers for 18 warps per SM with one channel group
+    static constexpr int kThreads = GA == 1 ? 32 * (W > 0 ? W : 1) : GA >= 5 ? 544 : 512;
+    static constexpr int kBlocks = GA == 1 ? 18 / (W > 0 ? W : 1) : 1;
+    // per pair, in floats: (A, B) quads, reused from the Legendre columns; (w R, w dR); (Y, grad Y)
+    static constexpr int PAIR = 4 * NAB + 2 * NAB + 4 * LM;
+    static_assert((L + 2) * (L + 2) + 2 * (L + 1) <= 4 * NAB, "Legendre columns fit the A/B area");
+    static_assert(NAB <= 256, "entry table bytes");
+};
+
+// Five unmixed groups (D = 4100) take 17 warps, the other shapes at most 16.
+template <int N, int L, int GA, bool MULTI>
+__global__ void __launch_bounds__(MULTI ? TriShape<N, L, GA>::kThreads : 32, MULTI ? TriShape<N, L, GA>::kBlocks : 18)
+k_jacobian_triples(SoapGeom geo, const float *__restrict__ tab, int n_atoms,
+                                   const int *__restrict__ offsets, const int *__restrict__ nbr_j,
+                                   const int *__restrict__ rev, const float4 *__restrict__ vec,
+                                   const int *__restrict__ species, const float *__restrict__ coef,
+                                   const float *__restrict__ phat, const float *__restrict__ pnorm,
+                                   const int *__restrict__ gp_of_atom, const float *__restrict__ mu_all, KnmTriples tr)
+{
+    using S = TriShape<N, L, GA>;
+    constexpr int LM = S::LM, NL = S::NL, NAB = S::NAB, NC = S::NC, KW = S::KW, QS = L + 2;
+    extern __shared__ __align__(16) float tri_smem[];
+    // [kTriBatch][NAB] quads; [kTriBatch][NAB] pairs; [kTriBatch][LM] quads; pair data; partial sums; coefficients
+    float4 *AB = reinterpret_cast<float4 *>(tri_smem);
+    float4 *Y4 = AB + kTriBatch * NAB;
+    float2 *RW = reinterpret_cast<float2 *>(Y4 + kTriBatch * LM);
+    TriPair *pr = reinterpret_cast<TriPair *>(RW + kTriBatch * NAB);
+    float *part = reinterpret_cast<float *>(pr + kTriBatch);  // MULTI: [warps][kTriBatch][6]
+    const int warps = blockDim.x >> 5;
+    float *csm = part + (MULTI ? warps * kTriBatch * 6 : 0);
+    const int tid = threadIdx.x, nthr = blockDim.x, warp = tid >> 5, lane = tid & 31;
+    const int i = blockIdx.x;
+    const int gp = gp_of_atom[i];
+    if (gp < 0) return;  // no sparse points of this species: no column of K_NM reads its rows
+    const int D = geo.D, D16 = geo.D16;
+    const int *tfirst = tr.first + (size_t)gp * n_atoms;
+    const float *mu = mu_all ? mu_all + (size_t)gp * D16 : nullptr;
+    auto sync = [&]() {
+        if constexpr (MULTI) __syncthreads();
+        else __syncwarp();
+    };
+    for (int q = tid; q < NC; q += nthr) csm[q] = coef[(size_t)i * NC + q];
+    // this lane's entries: packed channel offsets, p_hat, mu, own-row sums
+    unsigned et[KW][2];
+    float ph[KW][2], me[KW][2], own[KW][2][3];
+    float pm = 0.f;  // p_hat . mu
+#pragma unroll
+    for (int k = 0; k < KW; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int e = 64 * (warp * KW + k) + 2 * lane + h;
+            et[k][h] = e < D ? geo.etab[e] : 0u;
+            ph[k][h] = e < D ? phat[(size_t)i * D + e] : 0.f;
+            me[k][h] = (e < D && mu) ? mu[e] : 0.f;
+            pm += ph[k][h] * me[k][h];
+            own[k][h][0] = own[k][h][1] = own[k][h][2] = 0.f;
+        }
+    pm = warp_sum(pm);
+    if constexpr (MULTI) {
+        if (lane == 0) part[warp] = pm;
+        __syncthreads();
+        pm = 0.f;
+        for (int w = 0; w < warps; ++w) pm += part[w];
+        __syncthreads();
+    }
+    const float inv_norm = 1.f / pnorm[i];
+    const float rc = (float)geo.rc, dw = (float)geo.d, inv_h = 1.f / (float)geo.h;
+    const int p0 = offsets[i], p1 = offsets[i + 1], rank = tr.rank[i];
+
+    // dp / d r of one entry for the pair b of the batch
+    auto entry = [&](int b, unsigned e, float (&s)[3]) {
+        const int i1 = e & 0xff, i2 = (e >> 8) & 0xff;
+        const float4 a1 = AB[b * NAB + i1], a2 = AB[b * NAB + i2];
+        const float2 r1 = RW[b * NAB + i1], r2 = RW[b * NAB + i2];
+        const float cu = r1.y * a2.x + r2.y * a1.x;
+        const float sc = (e >> 16) ? 1.41421356237309504880f : 1.f;
+        s[0] = sc * (cu * pr[b].ux + r1.x * a2.y + r2.x * a1.y);
+        s[1] = sc * (cu * pr[b].uy + r1.x * a2.z + r2.x * a1.z);
+        s[2] = sc * (cu * pr[b].uz + r1.x * a2.w + r2.x * a1.w);
+    };
+    // two neighbouring entries of row `row` as BF16 planes
+    auto put = [&](size_t row, int e, float a, float b) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+        const float2 hf = __bfloat1622float2(h);
+        float ra = a - hf.x, rb = b - hf.y;
+        *reinterpret_cast<__nv_bfloat162 *>(tr.hi + row * D16 + e) = h;
+        if (tr.mid) {
+            const __nv_bfloat162 m = __floats2bfloat162_rn(ra, rb);
+            const float2 mf = __bfloat1622float2(m);
+            *reinterpret_cast<__nv_bfloat162 *>(tr.mid + row * D16 + e) = m;
+            ra -= mf.x;
+            rb -= mf.y;
+        }
+        *reinterpret_cast<__nv_bfloat162 *>(tr.lo + row * D16 + e) = __floats2bfloat162_rn(ra, rb);
+    };
+    auto put_meta = [&](int q, int j, const float (&t)[3]) {
+        tr.meta[q] = make_float4(t[0], t[1], t[2], __int_as_float(rank));
+        tr.dest[q] = q + 1 == tfirst[j + 1] ? tr.atom_cfg[j] + 1 + 3 * j : -1;
+        if (tr.src) tr.src[q] = i;
+    };
+
+    for (int pb = p0; pb < p1; pb += kTriBatch) {
+        const int nb = p1 - pb < kTriBatch ? p1 - pb : kTriBatch;
+        if (tid < nb) {
+            const int p = pb + tid, j = nbr_j[p], zr = species[j], rv = rev[p];
+            const float4 v = vec[p];
+            TriPair t;
+            t.r = v.w;
+            t.ir = 1.f / v.w;
+            t.ux = v.x * t.ir;
+            t.uy = v.y * t.ir;
+            t.uz = v.z * t.ir;
+            t.f = fcut_dev<float>(v.w, rc, dw, &t.df);
+            const RadialPos<float> rp = radial_pos<float>(v.w, inv_h, geo.G);
+            t.k = rp.k;
+            t.u = rp.u;
+            t.j = j;
+            t.z = zr >= 0 && zr < geo.S ? zr : 0;  // out of range: the call fails
+            t.q = tfirst[j] + tr.slot[rv >= 0 ? rv : 0];
+            pr[tid] = t;
+        }
+        sync();
+        // Legendre columns Q_l^m and (x + i y)^m: a thread per (pair, m), in the A/B area
+        for (int t = tid; t < nb * (L + 1); t += nthr) {
+            const int b = t / (L + 1), m = t - b * (L + 1);
+            float *Q = reinterpret_cast<float *>(AB + b * NAB), *CS = Q + QS * QS;
+            const float ux = pr[b].ux, uy = pr[b].uy, uz = pr[b].uz;
+            float C = 1.f, Sn = 0.f;
+            for (int k = 0; k < m; ++k) {
+                const float c2 = ux * C - uy * Sn;
+                Sn = ux * Sn + uy * C;
+                C = c2;
+            }
+            CS[2 * m] = C;
+            CS[2 * m + 1] = Sn;
+            float q2 = 0.f, q1 = 1.f;  // Q_m^m = (2m-1)!!
+            for (int k = 1; k <= m; ++k) q1 *= (float)(2 * k - 1);
+            for (int l = 0; l < m; ++l) Q[l * QS + m] = 0.f;
+            Q[m * QS + m] = q1;
+            if (m == L)
+                for (int l = 0; l <= L; ++l) Q[l * QS + L + 1] = 0.f;
+            if (m + 1 <= L) {
+                const float qq = (float)(2 * m + 1) * uz * q1;
+                Q[(m + 1) * QS + m] = qq;
+                q2 = q1;
+                q1 = qq;
+#pragma unroll
+                for (int k = 2; k <= L; ++k) {
+                    if (k <= L - m) {
+                        const int l = m + k;
+                        const float qn = ((float)(2 * l - 1) * uz * q1 - (float)(l + m - 1) * q2) * (1.f / (float)k);
+                        Q[l * QS + m] = qn;
+                        q2 = q1;
+                        q1 = qn;
+                    }
+                }
+            }
+        }
+        // w_g (f R, d(f R)/dr): a thread per (pair, n, l)
+        for (int t = tid; t < nb * NL; t += nthr) {
+            const int b = t / NL, q = t - b * NL;
+            float I, dI;
+            radial_eval<float>(tab, NL, q, RadialPos<float>{pr[b].k, pr[b].u}, inv_h, I, dI);
+            const float R = pr[b].f * I, dR = pr[b].df * I + pr[b].f * dI;
+#pragma unroll
+            for (int g = 0; g < GA; ++g) {
+                const float w = waccT<float>(geo, g, pr[b].z);
+                RW[b * NAB + g * NL + q] = make_float2(w * R, w * dR);
+            }
+        }
+        sync();
+        // (Y_lm, its gradient): a thread per (pair, lm)
+        for (int t = tid; t < nb * LM; t += nthr) {
+            const int b = t / LM, lm = t - b * LM;
+            const int l = (int)sqrtf((float)lm + 0.5f);  // floor(sqrt(lm)), lm < 121
+            const int m = lm - l * l - l, am = m < 0 ? -m : m;
+            const float *Q = reinterpret_cast<const float *>(AB + b * NAB), *CS = Q + QS * QS;
+            const float k = ylm_k<float>(geo, l, am), qv = k * Q[l * QS + am], qd = k * Q[l * QS + am + 1];
+            float y, gx, gy, gz;
+            if (am == 0) {
+                y = qv; gx = 0.f; gy = 0.f; gz = qd;
+            } else {
+                const float C = CS[2 * am], Sn = CS[2 * am + 1], Cm = (float)am * CS[2 * am - 2], Sm = (float)am * CS[2 * am - 1];
+                if (m > 0) {
+                    y = qv * C; gx = qv * Cm; gy = -qv * Sm; gz = qd * C;
+                } else {
+                    y = qv * Sn; gx = qv * Sm; gy = qv * Cm; gz = qd * Sn;
+                }
+            }
+            const float ux = pr[b].ux, uy = pr[b].uy, uz = pr[b].uz, ir = pr[b].ir, ud = ux * gx + uy * gy + uz * gz;
+            Y4[b * LM + lm] = make_float4(y, (gx - ud * ux) * ir, (gy - ud * uy) * ir, (gz - ud * uz) * ir);
+        }
+        sync();
+        // A = sum_m Y c, B = sum_m grad Y c: a thread per (l, pair, channel), l slowest
+        for (int t = tid; t < nb * NAB; t += nthr) {
+            const int per = nb * GA * N, l = t / per, bc = t - l * per, b = bc / (GA * N), ch = bc - b * (GA * N);
+            const float *cc = csm + ch * LM + l * l;
+            const float4 *yy = Y4 + b * LM + l * l;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int m = 0; m <= 2 * l; ++m) {
+                const float c = cc[m];
+                const float4 y = yy[m];
+                v.x += y.x * c;
+                v.y += y.y * c;
+                v.z += y.z * c;
+                v.w += y.w * c;
+            }
+            AB[b * NAB + ch * (L + 1) + l] = v;
+        }
+        sync();
+        if constexpr (MULTI) {
+            for (int b = 0; b < nb; ++b) {
+                float a6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k < KW; ++k)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        float s[3];
+                        entry(b, et[k][h], s);
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            a6[a] += ph[k][h] * s[a];
+                            a6[3 + a] += me[k][h] * s[a];
+                        }
+                    }
+#pragma unroll
+                for (int a = 0; a < 6; ++a) a6[a] = warp_sum(a6[a]);
+                if (lane == 0)
+                    for (int a = 0; a < 6; ++a) part[(warp * kTriBatch + b) * 6 + a] = a6[a];
+            }
+            __syncthreads();
+        }
+        for (int b = 0; b < nb; ++b) {
+            float J[KW][2][3], a6[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < KW; ++k)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    entry(b, et[k][h], J[k][h]);
+                    if constexpr (!MULTI) {
+#pragma unroll
+                        for (int a = 0; a < 3; ++a) {
+                            a6[a] += ph[k][h] * J[k][h][a];
+                            a6[3 + a] += me[k][h] * J[k][h][a];
+                        }
+                    }
+                }
+            if constexpr (MULTI) {
+                for (int w = 0; w < warps; ++w)
+#pragma unroll
+                    for (int a = 0; a < 6; ++a) a6[a] += part[(w * kTriBatch + b) * 6 + a];
+            } else {
+#pragma unroll
+                for (int a = 0; a < 6; ++a) a6[a] = warp_sum(a6[a]);
+            }
+            const int q = pr[b].q;
+#pragma unroll
+            for (int k = 0; k < KW; ++k) {
+                const int e = 64 * (warp * KW + k) + 2 * lane;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        J[k][h][a] = (J[k][h][a] - ph[k][h] * a6[a]) * inv_norm;
+                        own[k][h][a] += J[k][h][a];
+                    }
+                    // incoming triples are negated
+                    if (e < D16) put(3 * (size_t)q + a, e, e < D ? -J[k][0][a] : 0.f, e + 1 < D ? -J[k][1][a] : 0.f);
+                }
+            }
+            if (tid == 0) {
+                float t[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) t[a] = (a6[a] * pm - a6[3 + a]) * inv_norm;
+                put_meta(q, pr[b].j, t);
+            }
+        }
+        sync();
+    }
+    // the own triple
+    const int q = tfirst[i];
+    float t[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < KW; ++k) {
+        const int e = 64 * (warp * KW + k) + 2 * lane;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (e < D16) put(3 * (size_t)q + a, e, e < D ? own[k][0][a] : 0.f, e + 1 < D ? own[k][1][a] : 0.f);
+            t[a] += own[k][0][a] * me[k][0] + own[k][1][a] * me[k][1];
+        }
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a) t[a] = warp_sum(t[a]);
+    if constexpr (MULTI) {
+        if (lane == 0)
+            for (int a = 0; a < 3; ++a) part[warp * 3 + a] = t[a];
+        __syncthreads();
+        if (tid == 0)
+            for (int w = 1; w < warps; ++w)
+                for (int a = 0; a < 3; ++a) t[a] += part[w * 3 + a];
+    }
+    if (tid == 0) put_meta(q, i, t);
 }
 
 // ----------------------------------------------------- CUDA-core forms
@@ -548,12 +811,11 @@ gap_status gap_knm_segments(int n, const int *offsets, const int *atom_cfg, int 
     return gap_cuda_status(cudaGetLastError(), "k_seg_tables");
 }
 
-template <typename T, bool SPLIT>
+template <typename T>
 struct JacLaunch {
     template <int N, int L, int GA>
     static gap_status run(const SoapGeom &g, const T *tab, int n, const PairList &pl, const int *species,
-                          const T *coef, const T *phat, const T *pnorm, const int *gp_of_atom, const float *mu_all,
-                          KnmRows &out, cudaStream_t st)
+                          const T *coef, const T *phat, const T *pnorm, KnmRows &out, cudaStream_t st)
     {
         constexpr bool SREG = GA == 1 && N * (N + 1) / 2 * (L + 1) <= 256;  // as in the kernel
         if (SREG && g.D != N * (N + 1) / 2 * (L + 1)) {
@@ -566,16 +828,41 @@ struct JacLaunch {
             gap_set_error("descriptor too large for the Jacobian-row kernel's shared memory");
             return GAP_EUNSUPPORTED;
         }
-        auto kern = k_jacobian_rows<N, L, GA, T, SPLIT>;
+        auto kern = k_jacobian_rows<N, L, GA, T>;
         GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
         const typename V4<T>::type *vec;
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();
-        kern<<<n, 32, shm, st>>>(g, tab, n, pl.offsets, pl.j, pl.rev, vec, species, coef, phat, pnorm, gp_of_atom,
-                                 mu_all, reinterpret_cast<T *>(out.A), out.tri, out.src_sign, out.seg);
+        kern<<<n, 32, shm, st>>>(g, tab, n, pl.offsets, pl.j, pl.rev, vec, species, coef, phat, pnorm,
+                                 reinterpret_cast<T *>(out.A), out.src_sign, out.seg);
         return gap_cuda_status(cudaGetLastError(), "k_jacobian_rows");
     }
 };
+
+template <int N, int L, int GA>
+static gap_status launch_triples(const SoapGeom &g, const float *tab, int n, const PairList &pl, const int *species,
+                                 const float *coef, const float *phat, const float *pnorm, const int *gp_of_atom,
+                                 const float *mu_all, const KnmTriples &tr, cudaStream_t st)
+{
+    using S = TriShape<N, L, GA>;
+    // warps per atom: each owns up to KW groups of 64 entries
+    const int groups = (g.D16 + 63) / 64, warps = (groups + S::KW - 1) / S::KW;
+    const size_t shm = sizeof(float) * ((size_t)kTriBatch * S::PAIR + S::NC + (warps > 1 ? warps * kTriBatch * 6 : 0)) +
+                       kTriBatch * sizeof(TriPair);
+    auto kern = k_jacobian_triples<N, L, GA, (GA > 1 || S::W > 1)>;
+    if constexpr (GA > 1)
+        if (warps == 1) kern = k_jacobian_triples<N, L, GA, false>;
+    if ((GA == 1 && warps != S::W) || warps > (GA >= 5 ? 17 : 16)) {
+        gap_set_error("Jacobian rows: descriptor size does not match its shape");
+        return GAP_EINVAL;
+    }
+    if (shm > 48 * 1024)
+        GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+    gap_count_launch();
+    kern<<<n, 32 * warps, shm, st>>>(g, tab, n, pl.offsets, pl.j, pl.rev, pl.vec32, species, coef, phat, pnorm,
+                                     gp_of_atom, mu_all, tr);
+    return gap_cuda_status(cudaGetLastError(), "k_jacobian_triples");
+}
 
 #define GAP_KNM_SHAPES(X) \
     X(2, 1, 1)            \
@@ -591,30 +878,38 @@ struct JacLaunch {
     X(8, 8, 1)            \
     X(10, 8, 1)
 
-template <typename T, bool SPLIT>
+template <typename T>
 gap_status gap_jacobian_rows(const SoapGeom &g, const T *tab, int n, const PairList &pl, const int *species,
-                             const T *coef, const T *phat, const T *pnorm, const int *gp_of_atom, const float *mu_all,
-                             KnmRows &out, cudaStream_t st)
+                             const T *coef, const T *phat, const T *pnorm, KnmRows &out, cudaStream_t st)
 {
     if (n == 0) return GAP_OK;
 #define X(nn, ll, ga) \
     if (g.N == nn && g.L == ll && g.GA == ga) \
-        return JacLaunch<T, SPLIT>::template run<nn, ll, ga>(g, tab, n, pl, species, coef, phat, pnorm, gp_of_atom, mu_all, out, st);
+        return JacLaunch<T>::template run<nn, ll, ga>(g, tab, n, pl, species, coef, phat, pnorm, out, st);
     GAP_KNM_SHAPES(X)
 #undef X
     gap_set_error("unsupported (n_max, l_max, groups) for K_NM rows");
     return GAP_EUNSUPPORTED;
 }
 
-template gap_status gap_jacobian_rows<double, false>(const SoapGeom &, const double *, int, const PairList &,
-                                                     const int *, const double *, const double *, const double *,
-                                                     const int *, const float *, KnmRows &, cudaStream_t);
-template gap_status gap_jacobian_rows<float, false>(const SoapGeom &, const float *, int, const PairList &,
-                                                    const int *, const float *, const float *, const float *,
-                                                    const int *, const float *, KnmRows &, cudaStream_t);
-template gap_status gap_jacobian_rows<float, true>(const SoapGeom &, const float *, int, const PairList &,
-                                                   const int *, const float *, const float *, const float *,
-                                                   const int *, const float *, KnmRows &, cudaStream_t);
+template gap_status gap_jacobian_rows<double>(const SoapGeom &, const double *, int, const PairList &, const int *,
+                                              const double *, const double *, const double *, KnmRows &, cudaStream_t);
+template gap_status gap_jacobian_rows<float>(const SoapGeom &, const float *, int, const PairList &, const int *,
+                                             const float *, const float *, const float *, KnmRows &, cudaStream_t);
+
+gap_status gap_jacobian_triples(const SoapGeom &g, const float *tab, int n, const PairList &pl, const int *species,
+                                const float *coef, const float *phat, const float *pnorm, const int *gp_of_atom,
+                                const float *mu_all, const KnmTriples &tr, cudaStream_t st)
+{
+    if (n == 0) return GAP_OK;
+#define X(nn, ll, ga) \
+    if (g.N == nn && g.L == ll && g.GA == ga) \
+        return launch_triples<nn, ll, ga>(g, tab, n, pl, species, coef, phat, pnorm, gp_of_atom, mu_all, tr, st);
+    GAP_KNM_SHAPES(X)
+#undef X
+    gap_set_error("unsupported (n_max, l_max, groups) for K_NM rows");
+    return GAP_EUNSUPPORTED;
+}
 
 template <typename T>
 gap_status gap_knm_qpow_simt(const T *phat, int D, const int *rows, int nrows, const T *X, int M, double delta,

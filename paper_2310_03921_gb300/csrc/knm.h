@@ -15,10 +15,13 @@ struct KnmRows {
 
 gap_status gap_knm_segments(int n, const int *offsets, const int *atom_cfg, int *seg_start, int *out_row,
                             cudaStream_t st);
-template <typename T, bool SPLIT>
+template <typename T>
 gap_status gap_jacobian_rows(const SoapGeom &g, const T *tab, int n, const PairList &pl, const int *species,
-                             const T *coef, const T *phat, const T *pnorm, const int *gp_of_atom, const float *mu_all,
-                             KnmRows &out, cudaStream_t st);
+                             const T *coef, const T *phat, const T *pnorm, KnmRows &out, cudaStream_t st);
+// The tensor-core form's triples (mu_all NULL: J . mu written as 0).
+gap_status gap_jacobian_triples(const SoapGeom &g, const float *tab, int n, const PairList &pl, const int *species,
+                                const float *coef, const float *phat, const float *pnorm, const int *gp_of_atom,
+                                const float *mu_all, const KnmTriples &tr, cudaStream_t st);
 // Compressed descriptors (p~ = Q p renormalised): V = J Q^T for rows J
 // [nrow][ldj] in T and Q [Dg][D] (CUDA-core forms; V [nrow][ldv], columns
 // Dg .. ldv - 1 untouched) ...

@@ -40,3 +40,33 @@ def test_contraction_edges(G, atoms, M, prec, tol):
     assert np.abs(out["forces"].cpu().numpy() - F).max() <= tol
     assert abs(float(out["energy"][0]) - E) <= tol * atoms
     assert np.abs(out["virial"][0].cpu().numpy() - V).max() <= 10 * tol * max(1.0, np.abs(V).max())
+
+
+@pytest.mark.parametrize("prec,rel", [("bf16x3", 5e-5), ("bf16x6", 2e-5)])
+@pytest.mark.parametrize("M", [1, 127, 129])
+def test_knm_edges_one_species(G, M, prec, rel):
+    """Force rows at the edges of the point tiles and of the groups of 16 triples: an isolated atom, few and many
+    triples per target, D = 105 and 252."""
+    for index, cells in ((0, [_cluster(9), S.displaced_diamond(0, 3, (2, 2, 2), 0.1), _cluster(1)]),
+                         (1, [S.displaced_diamond(1, 3, (1, 1, 2), 0.1), _cluster(17)])):
+        soap_o, model_o, sparse, alpha = oracle_model(index, M, n_cells=1 if M <= 64 else 3)
+        w = S.workload(index)
+        ref = np.concatenate([O.knm(soap_o, model_o, c) for c in cells])
+        model = G.Model(G.Soap.from_spec(w.soap), sparse, alpha, w.delta, w.zeta)
+        K = model.assemble_knm(G.Batch.from_synth(S.make_batch(cells), device="cuda"), precision=prec).cpu().numpy()
+        assert np.abs(K - ref).max() <= rel * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("prec,rel", [("bf16x3", 5e-5), ("bf16x6", 2e-5)])
+def test_knm_edges_four_species(G, prec, rel):
+    """Four GPs in one launch, targets without a source of some species (their columns are zero)."""
+    soap_o, model_o, sparse, alpha = oracle_model(3, 33, n_max=4, l_max=3, n_cells=1)
+    w = S.workload(3)
+    lone = S.Structure(np.zeros((1, 3)), np.array([2], np.int32), np.eye(3) * 30.0, np.zeros(3, np.int32))
+    cells = [S.random_packing(3, 5, 8, 0.05, 1.8, n_species=2), lone, S.random_packing(3, 6, 40, 0.05, 1.8, n_species=4)]
+    ref = np.concatenate([O.knm(soap_o, model_o, c) for c in cells])
+    soap = G.Soap(4, 3, w.soap.rc, w.soap.sigma, w.soap.d, w.soap.central_weight, 4, 4, w.soap.mix_w)
+    model = G.Model(soap, sparse, alpha, w.delta, w.zeta)
+    K = model.assemble_knm(G.Batch.from_synth(S.make_batch(cells), device="cuda"), precision=prec).cpu().numpy()
+    assert np.abs(K - ref).max() <= rel * np.abs(ref).max()
+    assert np.all(K[ref == 0.0] == 0.0)
