@@ -286,7 +286,7 @@ static float bf16_to_float(uint16_t h)
 
 struct Workspace {
     NbrWork nbr;
-    DBuf pos, spec, coef, phat, pnorm, gp_of_atom, flag, fpos, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
+    DBuf pos, spec, coef, phat, pnorm, gp_of_atom, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
         W, eps_part, Gam, fpair, fw2, forces, vir_atom, cfgpart, energy, virial, local, err, A_hi, A_lo, t_row, W_hi, W_lo,
         epart_f, wpart_f, Gs, outbuf, kA, kAhi, kAlo, ksrc, kseg, kdest, kmeta, kslot, kfirst, kcount, kbounds, rank, segstart, outrow, Wp, kq, P,
         Kbuf, A_mid, W_mid, kAmid, phatc, pnormc, hfull, kV;
@@ -297,7 +297,7 @@ struct Workspace {
     void release()
     {
         nbr.release();
-        DBuf *bs[] = {&pos, &spec, &coef, &phat, &pnorm, &gp_of_atom, &flag, &fpos, &scan_tmp, &rows,
+        DBuf *bs[] = {&pos, &spec, &coef, &phat, &pnorm, &gp_of_atom, &scan_tmp, &rows,
                       &counts, &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &fw2, &forces, &vir_atom, &cfgpart, &energy,
                       &virial, &local, &err, &A_hi, &A_lo, &t_row, &W_hi, &W_lo, &epart_f, &wpart_f, &Gs, &outbuf,
                       &kA, &kAhi, &kAlo, &ksrc, &kseg, &kdest, &kmeta, &kslot, &kfirst, &kcount, &kbounds, &rank, &segstart,
@@ -544,12 +544,6 @@ static gap_status check_batch(const gap_batch *b)
     return GAP_OK;
 }
 
-__global__ void k_check_species(int n, const int *__restrict__ spec, int S, int *__restrict__ err)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && (spec[i] < 0 || spec[i] >= S)) atomicOr(err, 1);
-}
-
 // Device copies of positions and species (staged from host if needed).
 static gap_status stage_inputs(Workspace &w, const gap_batch *b, int S, const double **pos, const int **spec,
                                cudaStream_t st)
@@ -559,12 +553,7 @@ static gap_status stage_inputs(Workspace &w, const gap_batch *b, int S, const do
     GAP_TRY_CUDA(cudaMemsetAsync(w.err.p, 0, 16 * sizeof(int), st));
     if (b->device) {
         *pos = b->pos;
-        *spec = b->species;
-        if (n > 0) {
-            gap_count_launch();
-            k_check_species<<<(n + 255) / 256, 256, 0, st>>>(n, b->species, S, w.err.as<int>() + 1);
-            GAP_TRY_CUDA(cudaGetLastError());
-        }
+        *spec = b->species;  // checked by the neighbour build
         return GAP_OK;
     }
     for (int i = 0; i < n; ++i)
@@ -593,8 +582,7 @@ static gap_status check_device_errors(Workspace &w, cudaStream_t st)
         gap_set_error("tensor-core GEMM wait expired (code " + std::to_string(e[2]) + ")");
         return GAP_ETIMEOUT;
     }
-    GAP_TRY(gap_neighbours_check(w.nbr, st));
-    return GAP_OK;
+    return gap_neighbours_status(w.nbr, e[kNbrErr]);
 }
 
 extern "C" gap_status gap_soap_set_compression(gap_soap *s, const gap_compression *c)
@@ -809,7 +797,7 @@ static gap_status run_descriptor(gap_soap *soap, Workspace &w, const gap_batch *
     const int *spec;
     gap_prof_begin(ST_NEIGHBOURS, st);
     GAP_TRY(stage_inputs(w, b, g.S, &pos, &spec, st));
-    GAP_TRY(gap_neighbours(w.nbr, b, pos, g.rc, st));
+    GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, g.S, g.rc, w.err.as<int>(), st));
     const PairList &pl = w.nbr.pairs;
     gap_prof_end(ST_NEIGHBOURS, st);
     GAP_TRY(w.coef.ensure(sizeof(T) * (size_t)n * g.GA * g.N * g.LM));
@@ -851,7 +839,7 @@ extern "C" gap_status gap_descriptor_sizes(gap_soap *soap, const gap_batch *b, l
     const double *pos;
     const int *spec;
     GAP_TRY(stage_inputs(w, b, soap->geo.S, &pos, &spec, st));
-    GAP_TRY(gap_neighbours(w.nbr, b, pos, soap->geo.rc, st));
+    GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, soap->geo.S, soap->geo.rc, w.err.as<int>(), st));
     GAP_TRY(check_device_errors(w, st));
     if (n_desc) *n_desc = b->n_atoms;
     if (n_pairs) *n_pairs = w.nbr.pairs.n_pairs;
@@ -1183,15 +1171,11 @@ static gap_status gp_rows_all(gap_model *m, Workspace &w, int n, const int *spec
     int G = m->n_gp;
     GAP_TRY(w.gp_of_atom.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.rank.ensure(sizeof(int) * (size_t)n));
-    GAP_TRY(w.flag.ensure(sizeof(int) * (size_t)n));
-    GAP_TRY(w.fpos.ensure(sizeof(int) * (size_t)(n + 1)));
-    GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_scan_tmp_ints(n)));
+    GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_gp_rows_tmp_ints(n, G)));
     GAP_TRY(w.rows.ensure(sizeof(int) * (size_t)(G > 0 ? G : 1) * n));
     GAP_TRY(w.counts.ensure(sizeof(int) * (size_t)(G + 1)));
-    GAP_TRY(gap_fill_int(w.gp_of_atom.as<int>(), n, -1, st));
-    for (int s = 0; s < G; ++s)
-        GAP_TRY(gap_gp_rows(n, spec, s, w.flag.as<int>(), w.fpos.as<int>(), w.scan_tmp.as<int>(),
-                            w.rows.as<int>() + (size_t)s * n, w.counts.as<int>() + s, w.gp_of_atom.as<int>(), w.rank.as<int>(), st));
+    GAP_TRY(gap_gp_rows(n, G, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.counts.as<int>(),
+                        w.gp_of_atom.as<int>(), w.rank.as<int>(), st));
     if (w.graph) {
         counts = w.counts_fixed;
         return GAP_OK;
@@ -1228,7 +1212,10 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
     GAP_TRY(w.eps.ensure(sizeof(double) * (size_t)n));
     GAP_TRY(w.wsum.ensure(sizeof(float) * (size_t)n));
     T *gvec = grad ? w.gvec.as<T>() : nullptr;
-    if (n > 0) {
+    // with a GP of sparse points for every species each atom's are written
+    bool covered = m->n_gp == g.S;
+    for (const GPData &gp : m->gp) covered = covered && gp.M > 0;
+    if (n > 0 && !covered) {
         if (grad) GAP_TRY_CUDA(cudaMemsetAsync(w.gvec.p, 0, sizeof(T) * (size_t)n * Dg16, st));
         GAP_TRY_CUDA(cudaMemsetAsync(w.eps.p, 0, sizeof(double) * (size_t)n, st));
         GAP_TRY_CUDA(cudaMemsetAsync(w.wsum.p, 0, sizeof(float) * (size_t)n, st));

@@ -247,27 +247,95 @@ template <typename T> bool small_tiles(int rows, int cols)
 }
 
 // ---------------------------------------------------------------- rows
-__global__ void k_gp_flags(int n, const int *__restrict__ species, int s, int *__restrict__ flag)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) flag[i] = species[i] == s ? 1 : 0;
-}
+constexpr int kRowsOne = 8192, kRowsTile = 1024;  // atoms of the one-block form; per block else
+constexpr int kMaxGPs = 8;
 
-__global__ void k_gp_compact(int n, const int *__restrict__ flag, const int *__restrict__ pos, int *__restrict__ rows,
-                             int *__restrict__ gp_of_atom, int *__restrict__ rank, int s)
+// Atoms of each GP (species below n_gp) in kRowsTile consecutive atoms.
+__global__ void __launch_bounds__(kRowsTile)
+k_gp_counts(int n, int n_gp, const int *__restrict__ species, int *__restrict__ block_counts)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n && flag[i]) {
-        rows[pos[i]] = i;
-        rank[i] = pos[i];
-        gp_of_atom[i] = s;
+    __shared__ int cnt[kMaxGPs];
+    if (threadIdx.x < kMaxGPs) cnt[threadIdx.x] = 0;
+    __syncthreads();
+    const int i = blockIdx.x * kRowsTile + threadIdx.x;
+    const int z = i < n ? species[i] : -1;
+    for (int s = 0; s < n_gp; ++s) {
+        const unsigned m = __ballot_sync(0xffffffffu, z == s);
+        if ((threadIdx.x & 31) == 0 && m) atomicAdd(&cnt[s], __popc(m));
     }
+    __syncthreads();
+    if (threadIdx.x < n_gp) block_counts[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
 }
 
-__global__ void k_fill_int(int *__restrict__ a, int n, int v)
+// rows[s][.] = the atoms of GP s in index order, rank = an atom's place among
+// them, gp_of_atom (-1 without a GP), counts[s].  One block over all atoms
+// (block_counts NULL, tiles in turn), or a block per tile after
+// k_gp_counts, whose counts of the tiles before it each block adds up.  One
+// or two launches for all GPs; a flag, scan and compaction per GP were six.
+__global__ void __launch_bounds__(kRowsTile)
+k_gp_rows(int n, int n_gp, const int *__restrict__ species, const int *__restrict__ block_counts,
+          int *__restrict__ rows, int *__restrict__ counts, int *__restrict__ gp_of_atom, int *__restrict__ rank)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) a[i] = v;
+    __shared__ int wcnt[kMaxGPs][33], base[kMaxGPs];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (threadIdx.x < kMaxGPs) base[threadIdx.x] = 0;
+    if (block_counts) {
+        if (w < n_gp) {
+            int sum = 0, all = 0;
+            for (int b = lane; b < (int)gridDim.x; b += 32) {
+                const int c = block_counts[(size_t)w * gridDim.x + b];
+                all += c;
+                if (b < (int)blockIdx.x) sum += c;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                all += __shfl_xor_sync(0xffffffffu, all, o);
+            }
+            if (lane == 0) {
+                base[w] = sum;
+                if (blockIdx.x == 0) counts[w] = all;
+            }
+        }
+    }
+    __syncthreads();
+    const int t0 = block_counts ? blockIdx.x : 0, t1 = block_counts ? blockIdx.x + 1 : (n + kRowsTile - 1) / kRowsTile;
+    for (int t = t0; t < t1; ++t) {
+        const int i = t * kRowsTile + threadIdx.x;
+        const int z = i < n ? species[i] : -1;
+        int before = 0;
+        for (int s = 0; s < n_gp; ++s) {
+            const unsigned m = __ballot_sync(0xffffffffu, z == s);
+            if (lane == 0) wcnt[s][w] = __popc(m);
+            if (z == s) before = __popc(m & ((1u << lane) - 1u));
+        }
+        __syncthreads();
+        if (w < n_gp) {  // exclusive prefix over the 32 warps
+            const int c = wcnt[w][lane];
+            int x = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x, o);
+                if (lane >= o) x += y;
+            }
+            wcnt[w][lane] = base[w] + x - c;
+            if (lane == 31) wcnt[w][32] = base[w] + x;
+        }
+        __syncthreads();
+        if (i < n) {
+            const bool in = z >= 0 && z < n_gp;
+            gp_of_atom[i] = in ? z : -1;
+            if (in) {
+                const int r = wcnt[z][w] + before;
+                rows[(size_t)z * n + r] = i;
+                rank[i] = r;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < n_gp) base[threadIdx.x] = wcnt[threadIdx.x][32];
+        __syncthreads();
+    }
+    if (!block_counts && threadIdx.x < n_gp) counts[threadIdx.x] = base[threadIdx.x];
 }
 
 // -------------------------------------------------- tensor-core operands
@@ -401,20 +469,34 @@ gap_status gap_contract_simt_fixed(const double *phat, int D, int ldg, const int
     return gap_cuda_status(cudaGetLastError(), "k_eps_rows");
 }
 
-gap_status gap_gp_rows(int n, const int *species, int s, int *flag, int *pos, int *scan_tmp, int *rows, int *count,
-                       int *gp_of_atom, int *rank, cudaStream_t st)
+gap_status gap_gp_rows(int n, int n_gp, const int *species, int *tmp, int *rows, int *counts, int *gp_of_atom,
+                       int *rank, cudaStream_t st)
 {
+    if (n_gp > kMaxGPs) {
+        gap_set_error("too many GPs");
+        return GAP_EINVAL;
+    }
     if (n == 0) {
-        GAP_TRY_CUDA(cudaMemsetAsync(count, 0, sizeof(int), st));
+        if (n_gp > 0) GAP_TRY_CUDA(cudaMemsetAsync(counts, 0, sizeof(int) * n_gp, st));
         return GAP_OK;
     }
+    if (n <= kRowsOne) {
+        gap_count_launch();
+        k_gp_rows<<<1, kRowsTile, 0, st>>>(n, n_gp, species, nullptr, rows, counts, gp_of_atom, rank);
+        return gap_cuda_status(cudaGetLastError(), "k_gp_rows");
+    }
+    const int nb = (n + kRowsTile - 1) / kRowsTile;
     gap_count_launch();
-    k_gp_flags<<<(n + 255) / 256, 256, 0, st>>>(n, species, s, flag);
+    k_gp_counts<<<nb, kRowsTile, 0, st>>>(n, n_gp, species, tmp);
     GAP_TRY_CUDA(cudaGetLastError());
-    GAP_TRY(gap_scan(flag, n, pos, scan_tmp, count, st));
     gap_count_launch();
-    k_gp_compact<<<(n + 255) / 256, 256, 0, st>>>(n, flag, pos, rows, gp_of_atom, rank, s);
-    return gap_cuda_status(cudaGetLastError(), "k_gp_compact");
+    k_gp_rows<<<nb, kRowsTile, 0, st>>>(n, n_gp, species, tmp, rows, counts, gp_of_atom, rank);
+    return gap_cuda_status(cudaGetLastError(), "k_gp_rows");
+}
+
+size_t gap_gp_rows_tmp_ints(int n, int n_gp)
+{
+    return ((size_t)n + kRowsTile - 1) / kRowsTile * (n_gp > 0 ? n_gp : 1) + 1;
 }
 
 gap_status gap_split_rows(const float *phat, int D, int D16, const int *rows, int nrows, const float *mu,
@@ -424,14 +506,6 @@ gap_status gap_split_rows(const float *phat, int D, int D16, const int *rows, in
     gap_count_launch();
     k_split_rows<<<(nrows + 3) / 4, 128, 0, st>>>(phat, D, D16, rows, nrows, mu, Ahi, Alo, Amid, t_row);
     return gap_cuda_status(cudaGetLastError(), "k_split_rows");
-}
-
-gap_status gap_fill_int(int *a, int n, int v, cudaStream_t st)
-{
-    if (n <= 0) return GAP_OK;
-    gap_count_launch();
-    k_fill_int<<<(n + 255) / 256, 256, 0, st>>>(a, n, v);
-    return gap_cuda_status(cudaGetLastError(), "k_fill_int");
 }
 
 gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, int nrows, const TcModelGP &gp,

@@ -49,10 +49,11 @@ gap_status gap_contract_simt_fixed(const double *phat, int D, int ldg, const int
                                    int n_rows, const double *X, const double *alpha, int M, double delta, int zeta,
                                    double *W, double *eps_part, double *g, double *eps, cudaStream_t st);
 
-// rows[] = atoms of species s in index order, *count = their number,
-// gp_of_atom[atom] = s and rank[atom] = its row for those atoms.
-gap_status gap_gp_rows(int n, const int *species, int s, int *flag, int *pos, int *scan_tmp, int *rows, int *count,
-                       int *gp_of_atom, int *rank, cudaStream_t st);
-gap_status gap_fill_int(int *a, int n, int v, cudaStream_t st);
+// rows[s][n] = atoms of species s in index order for every GP s < n_gp (at
+// most 8), counts[s] their number, gp_of_atom[atom] = s (-1: none), rank[atom]
+// = its row.  tmp: gap_gp_rows_tmp_ints ints.
+gap_status gap_gp_rows(int n, int n_gp, const int *species, int *tmp, int *rows, int *counts, int *gp_of_atom,
+                       int *rank, cudaStream_t st);
+size_t gap_gp_rows_tmp_ints(int n, int n_gp);
 gap_status gap_split_rows(const float *phat, int D, int D16, const int *rows, int nrows, const float *mu,
                           __nv_bfloat16 *Ahi, __nv_bfloat16 *Alo, __nv_bfloat16 *Amid, float *t_row, cudaStream_t st);

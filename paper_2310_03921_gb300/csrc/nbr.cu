@@ -39,12 +39,24 @@ __device__ __forceinline__ int config_of(const int *offsets, int n_configs, int 
     return lo;
 }
 
-__global__ void k_bin(int n, const double *__restrict__ pos, const int *__restrict__ offsets, int n_configs,
-                      const CellGeom *__restrict__ geo, D4 *__restrict__ cart, float4 *__restrict__ cart32,
-                      int *__restrict__ atom_cfg, int *__restrict__ atom_bin, int *__restrict__ bin_count)
+// What a build needs of the batch; err[1] is set for a species outside 0 .. S - 1.
+struct BinInputs {
+    int n, n_configs, S;
+    const double *pos;
+    const int *species, *offsets;
+    const CellGeom *geo;
+    int *err;
+};
+
+// Atom i: wrapped Cartesian coordinates, configuration and bin (returned).
+__device__ __forceinline__ int bin_atom(const BinInputs &in, int i, D4 *cart, float4 *cart32, int *atom_cfg,
+                                        int *atom_bin)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    const double *pos = in.pos;
+    const int *offsets = in.offsets;
+    const int n_configs = in.n_configs;
+    const CellGeom *geo = in.geo;
+    if (in.species && (in.species[i] < 0 || in.species[i] >= in.S)) atomicOr(in.err + 1, 1);
     int c = config_of(offsets, n_configs, i);
     const CellGeom &g = geo[c];
     double p[3] = {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]};
@@ -72,17 +84,90 @@ __global__ void k_bin(int n, const double *__restrict__ pos, const int *__restri
     cart32[i] = make_float4((float)x[0], (float)x[1], (float)x[2], near ? 1.f : 0.f);
     atom_cfg[i] = c;
     atom_bin[i] = gb;
-    atomicAdd(&bin_count[gb], 1);
+    return gb;
 }
 
+__global__ void k_bin(BinInputs in, D4 *__restrict__ cart, float4 *__restrict__ cart32, int *__restrict__ atom_cfg,
+                      int *__restrict__ atom_bin, int *__restrict__ bin_count)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < in.n) atomicAdd(&bin_count[bin_atom(in, i, cart, cart32, atom_cfg, atom_bin)], 1);
+}
+
+// The bins' places are taken from the end: bin_count goes back to zero.
 __global__ void k_scatter(int n, const int *__restrict__ atom_bin, const int *__restrict__ bin_start,
-                          int *__restrict__ bin_fill, int *__restrict__ bin_atoms)
+                          int *__restrict__ bin_count, int *__restrict__ bin_atoms)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     int gb = atom_bin[i];
-    int slot = atomicAdd(&bin_fill[gb], 1);
+    int slot = atomicSub(&bin_count[gb], 1) - 1;
     bin_atoms[bin_start[gb] + slot] = i;
+}
+
+// Exclusive prefix of v over the 1024 threads of a block; *total their sum.
+__device__ __forceinline__ int block_prefix(int v, int *warp_tot, int *total)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();  // warp_tot of an earlier call is read
+    if (lane == 31) warp_tot[w] = x;
+    __syncthreads();
+    int t = warp_tot[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, t, o);
+        if (lane >= o) t += y;
+    }
+    *total = __shfl_sync(0xffffffffu, t, 31);
+    const int before = __shfl_sync(0xffffffffu, t, w > 0 ? w - 1 : 0);
+    return (w > 0 ? before : 0) + x - v;
+}
+
+// The whole binning of a small batch (up to kSmallAtoms atoms and kSmallBins
+// bins) in one block: at these sizes a build is launch latency, and this is
+// one launch for a clear, the bins, a scan and the scatter (2 us each).  One
+// SM's FP64 pipe takes the ~40 FP64 instructions of 256 atoms in about 3 us;
+// beyond that the spread kernels are faster.
+constexpr int kSmallAtoms = 256, kSmallBins = 4096;
+__global__ void __launch_bounds__(1024)
+k_bin_small(BinInputs in, int n_bins, D4 *__restrict__ cart, float4 *__restrict__ cart32, int *__restrict__ atom_cfg,
+            int *__restrict__ atom_bin, int *__restrict__ bin_start, int *__restrict__ bin_atoms)
+{
+    __shared__ int cnt[kSmallBins], warp_tot[32];
+    const int i = threadIdx.x;
+    for (int b = i; b < n_bins; b += 1024) cnt[b] = 0;
+    __syncthreads();
+    int gb = 0;
+    if (i < in.n) {
+        gb = bin_atom(in, i, cart, cart32, atom_cfg, atom_bin);
+        atomicAdd(&cnt[gb], 1);
+    }
+    __syncthreads();
+    const int items = (n_bins + 1023) / 1024;  // consecutive bins of this thread
+    int sum = 0, total;
+    for (int k = 0; k < items; ++k) {
+        const int b = i * items + k;
+        if (b < n_bins) sum += cnt[b];
+    }
+    int at = block_prefix(sum, warp_tot, &total);
+    for (int k = 0; k < items; ++k) {
+        const int b = i * items + k;
+        if (b < n_bins) {
+            const int c = cnt[b];
+            bin_start[b] = at;
+            cnt[b] = at;  // becomes the bin's next free place
+            at += c;
+        }
+    }
+    if (i == 0) bin_start[n_bins] = total;
+    __syncthreads();
+    if (i < in.n) bin_atoms[atomicAdd(&cnt[gb], 1)] = i;
 }
 
 // floor(a / n) for n > 0.
@@ -370,24 +455,6 @@ k_fill_warp(int n, const D4 *__restrict__ cart, const float4 *__restrict__ cart3
     }
 }
 
-// Graph mode: a build with more pairs than the arrays hold empties every
-// neighbour list (so that no later kernel reads past the arrays) and flags it.
-__global__ void k_cap_offsets(int n, int cap, const int *__restrict__ total, int *__restrict__ offsets,
-                              int *__restrict__ used, int *__restrict__ err)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int t = *total;
-    if (t > cap) {
-        if (i <= n) offsets[i] = 0;
-        if (i == 0) {
-            *used = 0;
-            atomicOr(err, 1);
-        }
-    } else if (i == 0) {
-        *used = t;
-    }
-}
-
 __global__ void k_reverse(int n, const int *__restrict__ offsets, const long long *__restrict__ keys,
                           int *__restrict__ rev, int *__restrict__ err)
 {
@@ -412,82 +479,88 @@ __global__ void k_reverse(int n, const int *__restrict__ offsets, const long lon
 }
 
 // ------------------------------------------------- exclusive scan of ints
-__global__ void k_scan_blocks(const int *__restrict__ in, int n, int *__restrict__ out, int *__restrict__ sums)
+constexpr int kScanOne = 8192, kScanTile = 4096;  // ints of the one-block form; per block else
+
+// Sums of kScanTile ints each.
+__global__ void __launch_bounds__(1024) k_scan_sums(const int *__restrict__ in, int n, int *__restrict__ sums)
 {
     __shared__ int warp_tot[32];
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int v = i < n ? in[i] : 0;
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+    int v = 0, total;
+#pragma unroll
+    for (int k = 0; k < kScanTile / 1024; ++k) {
+        const int i = blockIdx.x * kScanTile + k * 1024 + threadIdx.x;
+        if (i < n) v += in[i];
     }
-    if (lane == 31) warp_tot[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        int t = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, t, o);
-            if (lane >= o) t += y;
-        }
-        warp_tot[lane] = t;
-    }
-    __syncthreads();
-    int base = w > 0 ? warp_tot[w - 1] : 0;
-    if (i < n) out[i] = base + x - v;
-    if (threadIdx.x == blockDim.x - 1) sums[blockIdx.x] = base + x;
+    block_prefix(v, warp_tot, &total);
+    if (threadIdx.x == 0) sums[blockIdx.x] = total;
 }
 
-__global__ void k_scan_add(int *__restrict__ out, int n, const int *__restrict__ block_off, int *__restrict__ total,
-                           const int *__restrict__ in)
+// out[0 .. n] of a block's `per` ints (a thread takes consecutive ones), after
+// the sums of the blocks before it (sums == NULL: one block).  With a cap
+// (graph mode): a total beyond it empties every list (out = 0), so that no
+// later kernel reads past the pair arrays, and sets err bit 0.
+__global__ void __launch_bounds__(1024)
+k_scan_out(const int *__restrict__ in, int n, int per, const int *__restrict__ sums, int *__restrict__ out,
+           int *__restrict__ total_out, ScanCap cap)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] += block_off[blockIdx.x];
-    if (i == n - 1) {
-        out[n] = out[i] + in[i];
-        if (total) *total = out[n];
+    __shared__ int warp_tot[32];
+    int base = 0, grand = 0;
+    if (sums) {
+        int before = 0, all = 0;
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += 1024) {
+            const int s = sums[b];
+            all += s;
+            if (b < (int)blockIdx.x) before += s;
+        }
+        block_prefix(before, warp_tot, &base);
+        block_prefix(all, warp_tot, &grand);
+    }
+    const int items = per / 1024, i0 = blockIdx.x * per + threadIdx.x * items;
+    int v = 0, total;
+    for (int k = 0; k < items; ++k)
+        if (i0 + k < n) v += in[i0 + k];
+    int at = base + block_prefix(v, warp_tot, &total);
+    if (!sums) grand = total;
+    const bool over = cap.used && grand > cap.cap;
+    for (int k = 0; k < items; ++k)
+        if (i0 + k < n) {
+            const int x = in[i0 + k];
+            out[i0 + k] = over ? 0 : at;
+            at += x;
+        }
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        out[n] = over ? 0 : grand;
+        if (total_out) *total_out = grand;
+        if (cap.used) {
+            *cap.used = over ? 0 : grand;
+            if (over) atomicOr(cap.err, 1);
+        }
     }
 }
 
 }  // namespace
 
-// Exclusive scan of n ints into out[0..n] (out[n] = total); uses tmp of size
-// 2 * ceil(n / 1024) + 2 ints.  Recursive over block sums.
-gap_status gap_scan(const int *in, int n, int *out, int *tmp, int *total, cudaStream_t st)
+// Exclusive scan of n ints into out[0..n] (out[n] = total): one launch up to
+// 8192 ints (the scans of a small step were six launches), else two, the
+// blocks of the second adding up the sums of those before them.
+gap_status gap_scan(const int *in, int n, int *out, int *tmp, int *total, cudaStream_t st, ScanCap cap)
 {
-    if (n <= 0) {
-        GAP_TRY_CUDA(cudaMemsetAsync(out, 0, sizeof(int), st));
-        if (total) GAP_TRY_CUDA(cudaMemsetAsync(total, 0, sizeof(int), st));
-        return GAP_OK;
+    if (n <= kScanOne) {
+        const int per = n <= 1024 ? 1024 : (n + 1023) / 1024 * 1024;
+        gap_count_launch();
+        k_scan_out<<<1, 1024, 0, st>>>(in, n, per, nullptr, out, total, cap);
+        return gap_cuda_status(cudaGetLastError(), "k_scan_out");
     }
-    const int B = 1024;
-    int nb = (n + B - 1) / B;
-    int *sums = tmp, *offs = tmp + nb + 1;
+    const int nb = (int)(((long)n + kScanTile - 1) / kScanTile);
     gap_count_launch();
-    k_scan_blocks<<<nb, B, 0, st>>>(in, n, out, sums);
+    k_scan_sums<<<nb, 1024, 0, st>>>(in, n, tmp);
     GAP_TRY_CUDA(cudaGetLastError());
-    if (nb > 1) {
-        GAP_TRY(gap_scan(sums, nb, offs, tmp + 2 * nb + 2, nullptr, st));
-    } else {
-        GAP_TRY_CUDA(cudaMemsetAsync(offs, 0, sizeof(int), st));
-    }
     gap_count_launch();
-    k_scan_add<<<nb, B, 0, st>>>(out, n, offs, total, in);
-    GAP_TRY_CUDA(cudaGetLastError());
-    return GAP_OK;
+    k_scan_out<<<nb, 1024, 0, st>>>(in, n, kScanTile, tmp, out, total, cap);
+    return gap_cuda_status(cudaGetLastError(), "k_scan_out");
 }
 
-size_t gap_scan_tmp_ints(int n)
-{
-    size_t t = 0;
-    while (n > 1) {
-        int nb = (n + 1023) / 1024;
-        t += 2 * (size_t)nb + 2;
-        n = nb;
-    }
-    return t + 4;
-}
+size_t gap_scan_tmp_ints(int n) { return n > 0 ? ((size_t)n + kScanTile - 1) / kScanTile + 4 : 4; }
 
 // Host-side geometry of each configuration's bin grid.
 gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom> &geo, int &n_bins)
@@ -547,48 +620,49 @@ gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom
     return GAP_OK;
 }
 
-gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, double rc, cudaStream_t st)
+gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, const int *d_species, int S, double rc,
+                          int *err, cudaStream_t st)
 {
     int n = b->n_atoms;
     std::vector<CellGeom> geo;
     int n_bins = 0;
     GAP_TRY(gap_cell_geometry(b, rc, geo, n_bins));
     GAP_TRY(w.reserve_atoms(n, b->n_configs, n_bins));
+    w.err = err + kNbrErr;
     if (!w.graph) {
         GAP_TRY_CUDA(cudaMemcpyAsync(w.geo, geo.data(), sizeof(CellGeom) * geo.size(), cudaMemcpyHostToDevice, st));
         GAP_TRY_CUDA(cudaMemcpyAsync(w.cfg_offsets, b->config_offsets, sizeof(int) * (b->n_configs + 1),
                                      cudaMemcpyHostToDevice, st));
     }
-    GAP_TRY_CUDA(cudaMemsetAsync(w.bin_count, 0, sizeof(int) * (n_bins + 1), st));
-    GAP_TRY_CUDA(cudaMemsetAsync(w.bin_fill, 0, sizeof(int) * (n_bins + 1), st));
-    GAP_TRY_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), st));
-    const int T = 128;
-    int gridN = (n + T - 1) / T;
-    if (n > 0) {
+    const BinInputs in{n, b->n_configs, S, d_pos, d_species, w.cfg_offsets, w.geo, err};
+    if (n > 0 && n <= kSmallAtoms && n_bins <= kSmallBins) {
         gap_count_launch();
-        k_bin<<<gridN, T, 0, st>>>(n, d_pos, w.cfg_offsets, b->n_configs, w.geo, w.cart, w.cart32, w.atom_cfg,
-                                   w.atom_bin, w.bin_count);
+        k_bin_small<<<1, 1024, 0, st>>>(in, n_bins, w.cart, w.cart32, w.atom_cfg, w.atom_bin, w.bin_start, w.bin_atoms);
+        GAP_TRY_CUDA(cudaGetLastError());
+    } else if (n > 0) {
+        const int T = 128, gridN = (n + T - 1) / T;
+        GAP_TRY_CUDA(cudaMemsetAsync(w.bin_count, 0, sizeof(int) * (n_bins + 1), st));
+        gap_count_launch();
+        k_bin<<<gridN, T, 0, st>>>(in, w.cart, w.cart32, w.atom_cfg, w.atom_bin, w.bin_count);
+        GAP_TRY_CUDA(cudaGetLastError());
+        GAP_TRY(gap_scan(w.bin_count, n_bins, w.bin_start, w.scan_tmp, nullptr, st));
+        gap_count_launch();
+        k_scatter<<<gridN, T, 0, st>>>(n, w.atom_bin, w.bin_start, w.bin_count, w.bin_atoms);
         GAP_TRY_CUDA(cudaGetLastError());
     }
-    GAP_TRY(gap_scan(w.bin_count, n_bins, w.bin_start, w.scan_tmp, nullptr, st));
     if (n > 0) {
-        gap_count_launch();
-        k_scatter<<<gridN, T, 0, st>>>(n, w.atom_bin, w.bin_start, w.bin_fill, w.bin_atoms);
-        GAP_TRY_CUDA(cudaGetLastError());
         gap_count_launch();
         const int gridW = (n + kNbrWarps - 1) / kNbrWarps;
         k_count_warp<<<gridW, 32 * kNbrWarps, 0, st>>>(n, w.cart, w.cart32, w.atom_cfg, w.atom_bin, w.geo,
                                                        w.bin_start, w.bin_atoms, w.counts);
         GAP_TRY_CUDA(cudaGetLastError());
     }
-    GAP_TRY(gap_scan(w.counts, n, w.pairs.offsets, w.scan_tmp, w.total, st));
+    GAP_TRY(gap_scan(w.counts, n, w.pairs.offsets, w.scan_tmp, w.total, st,
+                     w.graph ? ScanCap{w.pair_cap, w.total + 1, w.err} : ScanCap{}));
     int P = 0;
     if (w.graph) {
         P = w.pair_cap;
         GAP_TRY(w.reserve_pairs(P));
-        gap_count_launch();
-        k_cap_offsets<<<(n + 256) / 256, 256, 0, st>>>(n, P, w.total, w.pairs.offsets, w.total + 1, w.err);
-        GAP_TRY_CUDA(cudaGetLastError());
         w.pairs.count = w.total + 1;
     } else {
         GAP_TRY_CUDA(cudaMemcpyAsync(&P, w.total, sizeof(int), cudaMemcpyDeviceToHost, st));
@@ -610,11 +684,8 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, d
     return GAP_OK;
 }
 
-gap_status gap_neighbours_check(NbrWork &w, cudaStream_t st)
+gap_status gap_neighbours_status(const NbrWork &w, int e)
 {
-    int e = 0;
-    GAP_TRY_CUDA(cudaMemcpyAsync(&e, w.err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    GAP_TRY_CUDA(cudaStreamSynchronize(st));
     if (e & 1) {
         gap_set_error("more neighbour pairs than the pair capacity (" + std::to_string(w.pair_cap) +
                       ") of the captured step");
@@ -657,12 +728,10 @@ gap_status NbrWork::reserve_atoms(int n, int n_configs, int n_bins)
     GAP_TRY(grow((void **)&counts, cap_counts, sizeof(int) * (size_t)(n + 1)));
     GAP_TRY(grow((void **)&pairs.offsets, cap_offsets, sizeof(int) * (size_t)(n + 2)));
     GAP_TRY(grow((void **)&bin_count, cap_bcount, sizeof(int) * (size_t)(n_bins + 2)));
-    GAP_TRY(grow((void **)&bin_fill, cap_bfill, sizeof(int) * (size_t)(n_bins + 2)));
     GAP_TRY(grow((void **)&bin_start, cap_bstart, sizeof(int) * (size_t)(n_bins + 2)));
     size_t t = gap_scan_tmp_ints(n > n_bins ? n : n_bins);
     GAP_TRY(grow((void **)&scan_tmp, cap_scan, sizeof(int) * t));
     GAP_TRY(grow((void **)&total, cap_total, sizeof(int) * 4));
-    err = total + 2;
     return GAP_OK;
 }
 
@@ -681,7 +750,7 @@ gap_status NbrWork::reserve_pairs(int P)
 void NbrWork::release()
 {
     void *ps[] = {geo, cfg_offsets, cart, cart32, atom_cfg, atom_bin, bin_atoms, counts, pairs.offsets, bin_count,
-                  bin_fill, bin_start, scan_tmp, total, keys, pairs.i, pairs.j, pairs.rev, pairs.vec64, pairs.vec32};
+                  bin_start, scan_tmp, total, keys, pairs.i, pairs.j, pairs.rev, pairs.vec64, pairs.vec32};
     for (void *p : ps)
         if (p) cudaFree(p);
     *this = NbrWork();
