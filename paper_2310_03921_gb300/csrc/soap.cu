@@ -245,66 +245,104 @@ k_expand(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int *__rest
     if (lane == 0) pnorm[i] = nrm;
 }
 
+// N values to consecutive places, as 16- or 8-byte stores where N sizeof(T)
+// allows it (the rows start on multiples of N sizeof(T)).
+template <int N, typename T> __device__ __forceinline__ void store_n(T *__restrict__ p, const T (&v)[N])
+{
+    if constexpr ((N * sizeof(T)) % 16 == 0) {
+#pragma unroll
+        for (int k = 0; k < N * (int)sizeof(T) / 16; ++k)
+            reinterpret_cast<float4 *>(p)[k] = reinterpret_cast<const float4 *>(v)[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < N * (int)sizeof(T) / 8; ++k)
+            reinterpret_cast<float2 *>(p)[k] = reinterpret_cast<const float2 *>(v)[k];
+    }
+}
+
 // ------------------------------------------------------------ backward chain
-// Gam[i][z][n][lm] for every neighbour species z.
-template <int N, int L, int GA, typename T>
-__global__ void __launch_bounds__(32)
+// Gam[i][z][lm][n] for every neighbour species z; a warp per atom.  h =
+// (g - (g . p_hat) p_hat) / |p| goes to shared memory, then a lane takes the
+// (l, m) of its turn with all its channels in registers: the c_{a, lm} of the
+// Nc coupled channels once, then every h_{aa'l} (a broadcast or neighbouring
+// words: l is the fastest index) serves two FMAs, and Gamma^z is formed from
+// the lane's own gammas and stored as runs of N.  With a lane per (channel,
+// lm) entry (index arithmetic and two shared reads per FMA) a step of 512
+// four-species boxes took 0.9 ms longer, of 32768 atoms 0.11 ms.  MIXED: GA separate blocks of N channels (Eq. 25), else
+// one block of GA N channels.
+template <int N, int L, int GA, bool MIXED, typename T>
+__global__ void __launch_bounds__(128)
 k_chain(SoapGeom geo, int n_atoms, const T *__restrict__ gvec, const T *__restrict__ wsum,
         const T *__restrict__ mu, const int *__restrict__ gp_of_atom, const T *__restrict__ phat,
         const T *__restrict__ pnorm, const T *__restrict__ coef, T *__restrict__ Gam)
 {
-    constexpr int LM = (L + 1) * (L + 1);
+    constexpr int LM = (L + 1) * (L + 1), NB = MIXED ? GA : 1, NC = MIXED ? N : GA * N, PER = NC * (NC + 1) / 2 * (L + 1);
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int D = geo.D;
-    T *hsm = reinterpret_cast<T *>(smem_raw);
-    T *csm = hsm + D;
-    T *gsm = csm + GA * N * LM;  // gamma [GA][N][LM]
-    const int lane = threadIdx.x;
-    const int i = blockIdx.x;
+    const int D = geo.D, warps = blockDim.x >> 5;
+    T *hsm = reinterpret_cast<T *>(smem_raw) + (size_t)(threadIdx.x >> 5) * D;
+    const int lane = threadIdx.x & 31;
+    const int i = blockIdx.x * warps + (threadIdx.x >> 5);
     if (i >= n_atoms) return;
-    int s = gp_of_atom ? gp_of_atom[i] : 0;
+    const int s = gp_of_atom ? gp_of_atom[i] : 0;
     // g = G + wsum * mu (tensor-core path stores the centred product separately)
+    const bool centred = wsum && s >= 0;
+    const T ws = centred ? wsum[i] : T(0);
+    const T *mus = centred ? mu + (size_t)s * geo.D16 : nullptr;
+    const T *gi = gvec + (size_t)i * geo.D16, *pi = phat + (size_t)i * D;
     T gp = T(0);
+#pragma unroll 4
     for (int d = lane; d < D; d += 32) {
-        T g = gvec[(size_t)i * geo.D16 + d];
-        if (wsum && s >= 0) g += wsum[i] * mu[(size_t)s * geo.D16 + d];
+        T g = gi[d];
+        if (centred) g += ws * mus[d];
         hsm[d] = g;
-        gp += g * phat[(size_t)i * D + d];
+        gp += g * pi[d];
     }
     gp = warp_sum(gp);
-    T inv = T(1) / pnorm[i];
+    const T inv = T(1) / pnorm[i];
+#pragma unroll 4
+    for (int d = lane; d < D; d += 32) hsm[d] = (hsm[d] - gp * pi[d]) * inv;
     __syncwarp();
-    for (int d = lane; d < D; d += 32) hsm[d] = (hsm[d] - gp * phat[(size_t)i * D + d]) * inv;
-    for (int q = lane; q < GA * N * LM; q += 32) csm[q] = coef[(size_t)i * GA * N * LM + q];
-    __syncwarp();
-    const int per = geo.npair * (L + 1);
-    for (int q = lane; q < GA * N * LM; q += 32) {
-        int lm = q % LM, gn = q / LM, grp = gn / N, n = gn % N;
+    const T *ci = coef + (size_t)i * GA * N * LM;
+    for (int lm = lane; lm < LM; lm += 32) {
         const int l = (int)sqrtf((float)lm + 0.5f);  // floor(sqrt(lm)), lm < 121
-        int b, a;
-        if (geo.mixed) { b = grp; a = n; }
-        else { b = 0; a = grp * N + n; }
-        T acc = T(0);
-        for (int ap = 0; ap < geo.Nc; ++ap) {
-            int lo = a < ap ? a : ap, hi = a < ap ? ap : a;
-            T hv = hsm[b * per + pair_index(geo.Nc, lo, hi) * (L + 1) + l];
-            T fac = (a == ap) ? T(2) : T(1.41421356237309504880);
-            int g2, n2;
-            chan(geo, b, ap, N, g2, n2);
-            acc += fac * hv * csm[(g2 * N + n2) * LM + lm];
-        }
-        gsm[q] = acc;
-    }
-    __syncwarp();
-    // Gam[i][z][lm][n]: the pair-force kernel reads the n values of one lm
-    // as vectors
-    const int S = geo.S;
-    for (int q = lane; q < S * N * LM; q += 32) {
-        const int z = q / (N * LM), r = q % (N * LM), lm = r / N, n = r % N, src = n * LM + lm;
-        T acc = T(0);
+        T gam[NB * NC];
 #pragma unroll
-        for (int g = 0; g < GA; ++g) acc += wacc<T>(geo, g, z) * gsm[g * N * LM + src];
-        Gam[(size_t)i * S * N * LM + q] = acc;
+        for (int b = 0; b < NB; ++b) {
+            T c[NC], off[NC];
+#pragma unroll
+            for (int a = 0; a < NC; ++a) {
+                c[a] = ci[(b * NC + a) * LM + lm];
+                off[a] = T(0);
+            }
+            const T *h = hsm + b * PER + l;
+#pragma unroll
+            for (int a = 0, k = 0; a < NC; ++a) {
+                const T haa = h[(k++) * (L + 1)];
+#pragma unroll
+                for (int a2 = a + 1; a2 < NC; ++a2) {
+                    const T hv = h[(k++) * (L + 1)];
+                    off[a] += hv * c[a2];
+                    off[a2] += hv * c[a];
+                }
+                gam[b * NC + a] = T(2) * haa * c[a];
+            }
+#pragma unroll
+            for (int a = 0; a < NC; ++a) gam[b * NC + a] += T(1.41421356237309504880) * off[a];
+        }
+        // Gam[i][z][lm][n]: the pair-force kernel reads the n values of one lm
+        // as vectors
+        for (int z = 0; z < geo.S; ++z) {
+            T out[N];
+#pragma unroll
+            for (int n = 0; n < N; ++n) out[n] = T(0);
+#pragma unroll
+            for (int g = 0; g < GA; ++g) {
+                const T w = wacc<T>(geo, g, z);
+#pragma unroll
+                for (int n = 0; n < N; ++n) out[n] += w * gam[g * N + n];
+            }
+            store_n<N, T>(Gam + ((size_t)(i * (size_t)geo.S + z) * LM + lm) * N, out);
+        }
     }
 }
 
@@ -740,16 +778,17 @@ template <typename T> struct Launch {
     static gap_status chain(const SoapGeom &g, int n, const T *gvec, const T *wsum, const T *mu, const int *gp_of_atom,
                             const T *phat, const T *pnorm, const T *coef, T *Gam, cudaStream_t st)
     {
-        constexpr int LM = (L + 1) * (L + 1);
-        size_t shm = sizeof(T) * (g.D + 2 * GA * N * LM);
+        // four atoms per block once that fills the chip; one for few atoms
+        const int warps = n >= 2048 && 4 * sizeof(T) * (size_t)g.D <= kMaxSmem ? 4 : 1;
+        const size_t shm = sizeof(T) * (size_t)g.D * warps;
         if (shm > kMaxSmem) {
             gap_set_error("descriptor too large for the chain kernel's shared memory");
             return GAP_EUNSUPPORTED;
         }
-        auto kern = k_chain<N, L, GA, T>;
+        auto kern = GA > 1 && g.mixed ? k_chain<N, L, GA, (GA > 1), T> : k_chain<N, L, GA, false, T>;
         GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
         gap_count_launch();
-        kern<<<n, 32, shm, st>>>(g, n, gvec, wsum, mu, gp_of_atom, phat, pnorm, coef, Gam);
+        kern<<<(n + warps - 1) / warps, 32 * warps, shm, st>>>(g, n, gvec, wsum, mu, gp_of_atom, phat, pnorm, coef, Gam);
         return gap_cuda_status(cudaGetLastError(), "k_chain");
     }
     template <int N, int L, int GA>
