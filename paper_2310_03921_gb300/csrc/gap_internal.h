@@ -173,12 +173,14 @@ __device__ __forceinline__ T fcut_dev(T r, T rc, T d, T *df)
 }
 
 // Radial lookup.  The table holds, for every interval k of the uniform knot
-// grid r_k = k h and every (n, l), the coefficients (a0, a1, a2, a3) of the
+// grid r_k = k h, every l and n, the coefficients (a0, a1, a2, a3) of the
 // cubic Hermite interpolant in u = r/h - k, computed in FP64 from the knot
 // values and derivatives: I = a0 + u (a1 + u (a2 + u a3)),
 // dI/dr = (a1 + u (2 a2 + 3 u a3)) / h.  Evaluating the polynomial instead of
 // the Hermite basis avoids the (f_{k+1} - f_k)/h cancellation that would
-// amplify the rounding of an FP32 table by 1/h.
+// amplify the rounding of an FP32 table by 1/h.  The N entries of one (k, l)
+// are contiguous (128 bytes at N = 8 in FP32): a thread that walks l reads
+// whole lines.
 template <typename T> struct Coef4;
 template <> struct Coef4<float> { typedef float4 type; };
 template <> struct Coef4<double> { typedef D4 type; };
@@ -201,7 +203,7 @@ __device__ __forceinline__ RadialPos<T> radial_pos(T r, T inv_h, int G)
     return p;
 }
 
-// value and d/dr of entry q (= n (l_max+1) + l) at position p; NL entries per interval
+// value and d/dr of entry q (= l N + n) at position p; NL entries per interval
 template <typename T>
 __device__ __forceinline__ void radial_eval(const T *__restrict__ tab, int NL, int q, RadialPos<T> p, T inv_h, T &v,
                                             T &dv)
@@ -210,12 +212,4 @@ __device__ __forceinline__ void radial_eval(const T *__restrict__ tab, int NL, i
     T u = p.u;
     v = c.x + u * (c.y + u * (c.z + u * c.w));
     dv = (c.y + u * (T(2) * c.z + T(3) * u * c.w)) * inv_h;
-}
-
-template <typename T>
-__device__ __forceinline__ T radial_value(const T *__restrict__ tab, int NL, int q, RadialPos<T> p)
-{
-    typename Coef4<T>::type c = reinterpret_cast<const typename Coef4<T>::type *>(tab)[(size_t)p.k * NL + q];
-    T u = p.u;
-    return c.x + u * (c.y + u * (c.z + u * c.w));
 }

@@ -187,7 +187,7 @@ k_jacobian_rows(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int 
         const RadialPos<T> rp = radial_pos<T>(r, inv_h, geo.G);
         for (int q = lane; q < NL; q += 32) {
             T I, dI;
-            radial_eval<T>(tab, NL, q, rp, inv_h, I, dI);
+            radial_eval<T>(tab, NL, q % (L + 1) * N + q / (L + 1), rp, inv_h, I, dI);
             Rsm[q] = f * I;
             dRsm[q] = df * I + f * dI;
         }
@@ -489,9 +489,9 @@ k_jacobian_triples(SoapGeom geo, const float *__restrict__ tab, int n_atoms,
         }
         // w_g (f R, d(f R)/dr): a thread per (pair, n, l)
         for (int t = tid; t < nb * NL; t += nthr) {
-            const int b = t / NL, q = t - b * NL;
+            const int b = t / NL, e = t - b * NL, q = e % N * (L + 1) + e / N;
             float I, dI;
-            radial_eval<float>(tab, NL, q, RadialPos<float>{pr[b].k, pr[b].u}, inv_h, I, dI);
+            radial_eval<float>(tab, NL, e, RadialPos<float>{pr[b].k, pr[b].u}, inv_h, I, dI);
             const float R = pr[b].f * I, dR = pr[b].df * I + pr[b].f * dI;
 #pragma unroll
             for (int g = 0; g < GA; ++g) {

@@ -101,13 +101,14 @@ __global__ void k_radial_table(int N, int L, int G, double h, double sigma, int 
 }
 
 // Per-interval cubic coefficients from knot values/derivatives (FP64), and
-// their FP32 rounding.  knots: [G+1][NL][2]; coef: [G][NL][4].
-__global__ void k_knots_to_coef(const double *__restrict__ knots, int G, int NL, double h, double *__restrict__ c64,
-                                float *__restrict__ c32)
+// their FP32 rounding.  knots: [G+1][N][L+1][2]; coef: [G][L+1][N][4].
+__global__ void k_knots_to_coef(const double *__restrict__ knots, int G, int N, int L1, double h,
+                                double *__restrict__ c64, float *__restrict__ c32)
 {
+    const int NL = N * L1;
     size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (idx >= (size_t)G * NL) return;
-    size_t k = idx / NL, q = idx % NL;
+    const size_t k = idx / NL, e = idx % NL, q = (e % N) * L1 + e / N;
     double f0 = knots[(k * NL + q) * 2], d0 = h * knots[(k * NL + q) * 2 + 1];
     double f1 = knots[((k + 1) * NL + q) * 2], d1 = h * knots[((k + 1) * NL + q) * 2 + 1];
     double a[4] = {f0, d0, 3.0 * (f1 - f0) - 2.0 * d0 - d1, 2.0 * (f0 - f1) + d0 + d1};
@@ -192,8 +193,8 @@ gap_status gap_radial_table(const SoapGeom &g, double **tab64, double **coef64, 
     k_radial_table<<<g.G + 1, T, shm>>>(N, L, g.G, g.h, g.sigma, nq + 1, dx, dw, dg, *tab64);
     GAP_TRY_CUDA(cudaGetLastError());
     gap_count_launch();
-    k_knots_to_coef<<<(unsigned)(((size_t)g.G * N * (L + 1) + 255) / 256), 256>>>(*tab64, g.G, N * (L + 1), g.h,
-                                                                                  *coef64, *coef32);
+    k_knots_to_coef<<<(unsigned)(((size_t)g.G * N * (L + 1) + 255) / 256), 256>>>(*tab64, g.G, N, L + 1, g.h, *coef64,
+                                                                                  *coef32);
     GAP_TRY_CUDA(cudaGetLastError());
     GAP_TRY_CUDA(cudaDeviceSynchronize());
     cudaFree(dx);

@@ -50,6 +50,22 @@ __device__ __forceinline__ int pair_index(int Nc, int a, int ap)  // a <= ap
     return a * Nc - (a * (a - 1)) / 2 + (ap - a);
 }
 
+// N consecutive values (global or shared memory) as 16- or 8-byte vector
+// loads where N sizeof(T) allows it (the rows start on multiples of
+// N sizeof(T)).
+template <int N, typename T> __device__ __forceinline__ void load_n(const T *p, T (&out)[N])
+{
+    if constexpr ((N * sizeof(T)) % 16 == 0) {
+#pragma unroll
+        for (int k = 0; k < N * (int)sizeof(T) / 16; ++k)
+            reinterpret_cast<float4 *>(out)[k] = reinterpret_cast<const float4 *>(p)[k];
+    } else {
+#pragma unroll
+        for (int k = 0; k < N * (int)sizeof(T) / 8; ++k)
+            reinterpret_cast<float2 *>(out)[k] = reinterpret_cast<const float2 *>(p)[k];
+    }
+}
+
 // ------------------------------------------------------------ expansion
 // The accumulation c_{n lm} += w R_nl Y_lm gives each lane the m values of
 // one l, in runs of at most S (the smallest S with sum_l ceil((2l+1)/S) <= 32
@@ -96,6 +112,7 @@ k_expand(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int *__rest
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *base = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * STRIDE;
     constexpr int BP = kExpandBatch;
+    static_assert(N % 2 == 0 && (BP * LMS) % 4 == 0, "vector reads of the radial values");
     T *Ysm = base, *Rsm = base + BP * LMS, *Wsm = Rsm + BP * NL, *Psm = Wsm + BP * GA;  // Psm [3][BP]: k, u, f
     int *Ksm = reinterpret_cast<int *>(Psm);
     const int lane = threadIdx.x & 31;
@@ -137,7 +154,7 @@ k_expand(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int *__rest
 #pragma unroll
         for (int g = 0; g < GA; ++g)
 #pragma unroll
-            for (int n = 0; n < N; ++n) acc[0][g][n] += wacc<T>(geo, g, zi) * (T)geo.cw * tab[4 * (n * (L + 1))] * y00;
+            for (int n = 0; n < N; ++n) acc[0][g][n] += wacc<T>(geo, g, zi) * (T)geo.cw * tab[4 * n] * y00;
     }
 
     const int p0 = offsets[i], p1 = offsets[i + 1];
@@ -185,11 +202,9 @@ k_expand(SoapGeom geo, const T *__restrict__ tab, int n_atoms, const int *__rest
         }
         __syncwarp();
         for (int t = 0; t < cnt; ++t) {
-            const T *Rt = Rsm + t * NL + my_l;
             const T *Yt = Ysm + t * LMS + my_lm;
             T rv[N], yv[S];
-#pragma unroll
-            for (int n = 0; n < N; ++n) rv[n] = Rt[n * (L + 1)];
+            load_n<N, T>(Rsm + t * NL + my_l * N, rv);
 #pragma unroll
             for (int o = 0; o < S; ++o) yv[o] = o < my_cnt ? Yt[o] : T(0);
 #pragma unroll
@@ -346,33 +361,38 @@ k_chain(SoapGeom geo, int n_atoms, const T *__restrict__ gvec, const T *__restri
     }
 }
 
-// The n values Gam[..][lm][0 .. N-1] as 16- or 8-byte vector loads where
-// N sizeof(T) allows it (the rows start on multiples of N sizeof(T)).
-template <int N, typename T>
-__device__ __forceinline__ void load_n(const T *__restrict__ p, T (&out)[N])
-{
-    if constexpr ((N * sizeof(T)) % 16 == 0) {
-#pragma unroll
-        for (int k = 0; k < N * (int)sizeof(T) / 16; ++k) {
-            const float4 v = __ldg(reinterpret_cast<const float4 *>(p) + k);
-            reinterpret_cast<float4 *>(out)[k] = v;
-        }
-    } else if constexpr ((N * sizeof(T)) % 8 == 0) {
-#pragma unroll
-        for (int k = 0; k < N * (int)sizeof(T) / 8; ++k) {
-            const float2 v = __ldg(reinterpret_cast<const float2 *>(p) + k);
-            reinterpret_cast<float2 *>(out)[k] = v;
-        }
-    } else {
-#pragma unroll
-        for (int k = 0; k < N; ++k) out[k] = p[k];
-    }
-}
-
 // ------------------------------------------------------------ pair forces
-// fpair[p] = d eps_i / d r_ij for pair p = (i -> j).
+// The radial coefficients of entries n, n + 1 of one (interval, l): 32 bytes
+// in FP32 (one 256-bit load; N is even, so pairs start on 32 bytes).
+template <typename T> struct Coef2;
+template <> struct Coef2<float> {
+    float4 a, b;
+    __device__ __forceinline__ void load(const float *p)
+    {
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+            : "l"(p));
+    }
+};
+template <> struct Coef2<double> {
+    D4 a, b;
+    __device__ __forceinline__ void load(const double *p)
+    {
+        a = reinterpret_cast<const D4 *>(p)[0];
+        b = reinterpret_cast<const D4 *>(p)[1];
+    }
+};
+
+// fpair[p] = d eps_i / d r_ij for pair p = (i -> j), a thread per pair.  With
+// A_lm = sum_n Gamma_{n lm} R_nl and B_lm = sum_n Gamma_{n lm} dR_nl the force is
+// a sum over the polynomial forms Y_lm = K Q_l^|m|(z) {C_m, S_m}; its l sums are
+// taken first, per m, for the three factors they leave (x and y derivatives,
+// z derivative, value), so an (l, m) costs 2 N + 3 FMAs, and the C_m, S_m
+// enter once at the end.  The projection of the gradient onto the sphere
+// needs only the total.  The table rows bound it (1.2 KB per pair at n = l =
+// 8, from L2 where L1 misses): read as whole lines, 32 bytes per load.
 template <int N, int L, typename T>
-__global__ void __launch_bounds__(128, 6)
+__global__ void __launch_bounds__(128, sizeof(T) == 8 ? 2 : 4)
 k_pairforce(SoapGeom geo, const T *__restrict__ tab, int n_pairs, const int *__restrict__ n_valid,
             const int *__restrict__ pair_i, const int *__restrict__ nbr_j,
             const typename V4<T>::type *__restrict__ vec, const int *__restrict__ species,
@@ -380,6 +400,7 @@ k_pairforce(SoapGeom geo, const T *__restrict__ tab, int n_pairs, const int *__r
 {
     constexpr int LM = (L + 1) * (L + 1);
     constexpr int NL = N * (L + 1);
+    static_assert(N % 2 == 0, "entries are read in pairs");
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_pairs || p >= *n_valid) return;
     const int i = pair_i[p];
@@ -392,25 +413,27 @@ k_pairforce(SoapGeom geo, const T *__restrict__ tab, int n_pairs, const int *__r
     const T f = fcut_dev<T>(r, (T)geo.rc, (T)geo.d, &df);
     const T inv_h = T(1) / (T)geo.h;
     const RadialPos<T> rp = radial_pos<T>(r, inv_h, geo.G);
+    const T *row = tab + (size_t)rp.k * NL * 4;
+    const T fh = f * inv_h, u2 = T(2) * rp.u, u3 = T(3) * rp.u * rp.u;
 
-    T C[L + 1], Sn[L + 1];
-    C[0] = T(1); Sn[0] = T(0);
+    // per m >= 0 and its negative: sum_l A K Q_l^m, sum_l A K Q_l^{m+1}, sum_l B K Q_l^m
+    T P[L + 1], Pn[L + 1], Z[L + 1], Zn[L + 1], V[L + 1], Vn[L + 1];
 #pragma unroll
-    for (int m = 1; m <= L; ++m) {
-        C[m] = ux * C[m - 1] - uy * Sn[m - 1];
-        Sn[m] = ux * Sn[m - 1] + uy * C[m - 1];
-    }
+    for (int m = 0; m <= L; ++m) P[m] = Pn[m] = Z[m] = Zn[m] = V[m] = Vn[m] = T(0);
     T q1[L + 2], q2[L + 2];
-    T sU = T(0), sx = T(0), sy = T(0), sz = T(0);
 #pragma unroll
     for (int l = 0; l <= L; ++l) {
         T R[N], dR[N];
 #pragma unroll
-        for (int n = 0; n < N; ++n) {
-            T I, dI;
-            radial_eval<T>(tab, NL, n * (L + 1) + l, rp, inv_h, I, dI);
-            R[n] = f * I;
-            dR[n] = df * I + f * dI;
+        for (int n = 0; n < N; n += 2) {
+            Coef2<T> c;
+            c.load(row + 4 * (l * N + n));
+            const T I0 = c.a.x + rp.u * (c.a.y + rp.u * (c.a.z + rp.u * c.a.w));
+            const T I1 = c.b.x + rp.u * (c.b.y + rp.u * (c.b.z + rp.u * c.b.w));
+            R[n] = f * I0;
+            R[n + 1] = f * I1;
+            dR[n] = df * I0 + fh * (c.a.y + u2 * c.a.z + u3 * c.a.w);
+            dR[n + 1] = df * I1 + fh * (c.b.y + u2 * c.b.z + u3 * c.b.w);
         }
         T q[L + 2];
 #pragma unroll
@@ -418,46 +441,28 @@ k_pairforce(SoapGeom geo, const T *__restrict__ tab, int n_pairs, const int *__r
             if (m > l) { q[m] = T(0); continue; }
             if (m == l) q[m] = (l == 0) ? T(1) : T(2 * l - 1) * q1[l - 1];
             else if (m == l - 1) q[m] = T(2 * l - 1) * uz * q1[m];
-            else q[m] = (T(2 * l - 1) * uz * q1[m] - T(l + m - 1) * q2[m]) / T(l - m);
+            else q[m] = (T(2 * l - 1) * uz * q1[m] - T(l + m - 1) * q2[m]) * (T(1) / T(l - m));  // l, m unrolled: a constant
         }
 #pragma unroll
         for (int m = 0; m <= L; ++m) {
             if (m > l) continue;
-            const T k = ylm_k<T>(geo, l, m);
-            // (value, d/dx, d/dy, d/dz) of the polynomial extension, for +m and -m
-            T yp, gpx, gpy, gpz, yn = T(0), gnx = T(0), gny = T(0), gnz = T(0);
-            if (m == 0) {
-                yp = k * q[0];
-                gpx = T(0); gpy = T(0); gpz = k * q[1];
-            } else {
-                yp = k * q[m] * C[m];
-                gpx = k * q[m] * T(m) * C[m - 1];
-                gpy = -k * q[m] * T(m) * Sn[m - 1];
-                gpz = k * q[m + 1] * C[m];
-                yn = k * q[m] * Sn[m];
-                gnx = k * q[m] * T(m) * Sn[m - 1];
-                gny = k * q[m] * T(m) * C[m - 1];
-                gnz = k * q[m + 1] * Sn[m];
-            }
-            {
-                T G[N];
-                load_n<N, T>(Gm + (l * l + l + m) * N, G);
-                T A = T(0), B = T(0);
+            const T k = ylm_k<T>(geo, l, m), kq = k * q[m], kz = k * q[m + 1];
+            T G[N];
+            load_n<N, T>(Gm + (l * l + l + m) * N, G);
+            T A = T(0), B = T(0);
 #pragma unroll
-                for (int n = 0; n < N; ++n) { A += G[n] * R[n]; B += G[n] * dR[n]; }
-                T ud = ux * gpx + uy * gpy + uz * gpz;
-                sU += B * yp - A * ud * ir;
-                sx += A * gpx; sy += A * gpy; sz += A * gpz;
-            }
+            for (int n = 0; n < N; ++n) { A += G[n] * R[n]; B += G[n] * dR[n]; }
+            P[m] += A * kq;
+            Z[m] += A * kz;
+            V[m] += B * kq;
             if (m > 0) {
-                T G[N];
                 load_n<N, T>(Gm + (l * l + l - m) * N, G);
-                T A = T(0), B = T(0);
+                A = B = T(0);
 #pragma unroll
                 for (int n = 0; n < N; ++n) { A += G[n] * R[n]; B += G[n] * dR[n]; }
-                T ud = ux * gnx + uy * gny + uz * gnz;
-                sU += B * yn - A * ud * ir;
-                sx += A * gnx; sy += A * gny; sz += A * gnz;
+                Pn[m] += A * kq;
+                Zn[m] += A * kz;
+                Vn[m] += B * kq;
             }
         }
 #pragma unroll
@@ -467,6 +472,19 @@ k_pairforce(SoapGeom geo, const T *__restrict__ tab, int n_pairs, const int *__r
             q1[m] = q[m];
         }
     }
+    // (C_m, S_m) = (x + i y)^m; d/dx of C_m, S_m is m (C_{m-1}, S_{m-1}), d/dy m (-S_{m-1}, C_{m-1})
+    T sU = V[0], sx = T(0), sy = T(0), sz = Z[0], C = T(1), Sn = T(0);
+#pragma unroll
+    for (int m = 1; m <= L; ++m) {
+        sx += T(m) * (C * P[m] + Sn * Pn[m]);
+        sy += T(m) * (C * Pn[m] - Sn * P[m]);
+        const T c2 = ux * C - uy * Sn;
+        Sn = ux * Sn + uy * C;
+        C = c2;
+        sz += C * Z[m] + Sn * Zn[m];
+        sU += C * V[m] + Sn * Vn[m];
+    }
+    sU -= ir * (ux * sx + uy * sy + uz * sz);
     fpair[3 * (size_t)p] = sU * ux + sx * ir;
     fpair[3 * (size_t)p + 1] = sU * uy + sy * ir;
     fpair[3 * (size_t)p + 2] = sU * uz + sz * ir;
@@ -799,8 +817,12 @@ template <typename T> struct Launch {
         const typename V4<T>::type *vec;
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();
-        k_pairforce<N, L, T><<<(pl.n_pairs + 127) / 128, 128, 0, st>>>(g, tab, pl.n_pairs, pl.count, pl.i, pl.j,
-                                                                       vec, species, Gam, fpair);
+        // one warp per block while that spreads the warps over more SMs (the
+        // FP64 pipe and L1 are per SM); the FP64 form's registers allow no more
+        // warps per SM in larger blocks either
+        const int threads = sizeof(T) == 8 || pl.n_pairs <= 32 * 1024 ? 32 : 128;
+        k_pairforce<N, L, T><<<(pl.n_pairs + threads - 1) / threads, threads, 0, st>>>(
+            g, tab, pl.n_pairs, pl.count, pl.i, pl.j, vec, species, Gam, fpair);
         return gap_cuda_status(cudaGetLastError(), "k_pairforce");
     }
 };
