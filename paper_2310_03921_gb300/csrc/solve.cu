@@ -24,10 +24,6 @@
 #include "gap_internal.h"
 #include "solve.h"
 
-#ifndef GAP_CHOL_BLOCK
-#define GAP_CHOL_BLOCK 64
-#endif
-
 namespace {
 
 // Kmm[p][q] (column-major, ld M) = delta^2 (x_p . x_q)^zeta within a GP block, 0 across blocks.
@@ -446,8 +442,15 @@ __device__ __forceinline__ double rsqrt_newton(double x)
 // to ~66 bits before the final rounding.
 __device__ __forceinline__ double recip_newton(double x)
 {
-    int e;
-    const double f = frexp(x, &e);  // x = f 2^e, f in [0.5, 1)
+    const unsigned long long xb = (unsigned long long)__double_as_longlong(x);
+    const int ex = (int)(xb >> 52);  // x > 0: the biased exponent
+    // f = x with the exponent of [0.5, 1); the result is scaled back by its
+    // exponent field (plain bit fields where x and 1 / x are normal numbers:
+    // every FP64 instruction is ~64 cycles of the caller's critical path)
+    const bool plain = ex >= 2 && ex <= 2044;
+    int e = ex - 1022;
+    double f = __longlong_as_double((long long)((xb & 0x000FFFFFFFFFFFFFull) | 0x3FE0000000000000ull));
+    if (!plain) f = frexp(x, &e);
     const unsigned long long fb = (unsigned long long)__double_as_longlong(f);
     const float fs = __uint_as_float(0x3F000000u | (unsigned)((fb >> 29) & 0x7FFFFFu));  // f, truncated
     float rs;
@@ -456,6 +459,7 @@ __device__ __forceinline__ double recip_newton(double x)
     double y = __longlong_as_double((long long)(((unsigned long long)__float_as_uint(rs) + (896ull << 23)) << 29));
     const double d = fma(-f, y, 1.0);
     y = fma(y, fma(d, d, d), y);
+    if (plain) return __longlong_as_double(__double_as_longlong(y) - ((long long)e << 52));
     return ldexp(y, -e);
 }
 
@@ -473,86 +477,201 @@ __global__ void k_recip_check(int n, const double *__restrict__ x, double *__res
 }
 
 // Upper Cholesky factor R (G = R^T R) and its inverse X of an m x m block
-// (m <= kBlock) in one CTA of kBlock / 4 warps, FP64.  Elimination on M = [A | B]
-// (A = G, upper triangle; B = I): step k subtracts (M_ki / M_kk) times row k
-// from every row i > k, on the columns that stay live (A: j >= i; B: j <= k).
-// Rows are left unscaled, so each step needs only the reciprocal pivot; at
-// the end row k times M_kk^-1/2 gives row k of R (A part) and of R^-T (B
-// part, the product of the elimination matrices), so X = B^T.  Each row's
-// live columns are packed into 32-wide chunks (every FP64 instruction works
-// on whole warps), warp w takes the rows i = k + 1 + w (mod warps), and one
-// more warp forms the next pivot M_{k+1,k+1} and its reciprocal meanwhile (the
-// same expression the row update would use, so that long FP64 chain runs
-// beside the row updates rather than after one of them): one barrier per
-// step.  G column-major (ld ldg); R and X written column-major (ld ld) with
-// zero strict lower triangles.  A non-positive pivot sets *flag (the factor
-// is meaningless).
-constexpr int kBlock = GAP_CHOL_BLOCK;  // largest block factorised by one kernel
-constexpr int kBlockWarps = kBlock / 4;  // row warps of that kernel (plus one pivot warp)
-constexpr int kSplit = 32;               // granularity of the recursive split
-constexpr int kBlockLd = 2 * kBlock + 1;
-constexpr size_t kBlockSmem = sizeof(double) * (kBlock * kBlockLd + 2 * kBlock);
+// (m <= kBlock = 64) in a cluster of eight CTAs, FP64.  Elimination on M =
+// [A | B] (A = G, upper triangle; B = I): step k subtracts (M_ki / M_kk) times
+// row k from every row i > k, on the columns that stay live (A: j >= i; B: j
+// <= k).  Rows are left unscaled, so each step needs only the reciprocal
+// pivot; at the end row k times M_kk^-1/2 gives row k of R (A part) and of
+// R^-T (B part, the product of the elimination matrices), so X = B^T.
+//
+// A warp issues one FP64 instruction per ~64 cycles here and an SM one per
+// 19, so one CTA took ~4900 warp instructions and 72 us per block; this form
+// takes about 38 us (the 64 blocks of a 2000-column fit 4.6 -> 2.4 ms).  CTA c owns
+// the panel of rows 8 c .. 8 c + 7, whose live columns are always 72: A from
+// 8 c, B to 8 c + 7.  Panel by panel, the owner eliminates within its rows and
+// sends them to the CTAs after it (distributed shared memory, two buffers),
+// which subtract them from their own rows: one cluster barrier per panel.
+// In a CTA
+//   warp 0 (a scheduler of its own: warps 4 and 8 idle) keeps the upper
+//     triangle of the panel's 8 x 8 diagonal block, an entry per lane (28
+//     below its first row, 8 in it), brings it up to date first and then
+//     factorises it alone, shuffles only: the serial chain of pivots and
+//     reciprocals, five FP64 instructions a step;
+//   nine warps hold the 72 columns, four threads of two rows each; they
+//     subtract the earlier panel meanwhile, then follow warp 0's pivots.
+// Every row sees the same operations in the same order as a row-by-row
+// elimination.  G column-major (ld ldg); R and X written column-major (ld ld)
+// with zero strict lower triangles.  A non-positive pivot sets *flag (the
+// factor is meaningless).
+constexpr int kBlock = 64;     // largest block factorised by one kernel
+constexpr int kPanel = 8;      // rows per CTA
+constexpr int kBlockCtas = kBlock / kPanel;
+constexpr int kBlockThreads = 384;
+constexpr int kSplit = 32;     // granularity of the recursive split
 
-__global__ void __launch_bounds__(32 * (kBlockWarps + 1)) k_chol_inv_block(const double *__restrict__ G, long ldg, int m,
-                                                                     double *__restrict__ R, double *__restrict__ X,
-                                                                     long ld, int *__restrict__ flag)
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// Stores v at the place of p (this CTA's shared memory) in CTA `rank`'s.
+__device__ __forceinline__ void store_remote(double *p, int rank, double v)
 {
-    extern __shared__ double sm_block[];
-    double(*M)[kBlockLd] = reinterpret_cast<double(*)[kBlockLd]>(sm_block);
-    double *inv_s = sm_block + kBlock * kBlockLd;  // [kBlock] reciprocal pivots
-    double *ri_s = inv_s + kBlock;                 // [kBlock] pivot^-1/2
-    __shared__ int bad;
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    for (int idx = t; idx < m * m; idx += blockDim.x) {
-        const int i = idx % m, j = idx / m;
-        M[i][j] = G[i + (long)j * ldg];
-        M[i][kBlock + j] = i == j ? 1.0 : 0.0;
+    uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p)), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(r), "d"(v) : "memory");
+}
+
+__global__ void __cluster_dims__(kBlockCtas, 1, 1) __launch_bounds__(kBlockThreads)
+k_chol_inv_block(const double *__restrict__ G, long ldg, int m, double *__restrict__ R, double *__restrict__ X, long ld,
+                 int *__restrict__ flag)
+{
+    __shared__ double buf[2][kPanel][2 * kBlock];  // an earlier panel's rows: A columns, then B columns
+    __shared__ double binv[2][kPanel];             // and its reciprocal pivots
+    __shared__ double F[kPanel][kPanel];           // an earlier panel's multipliers of this CTA's rows ([panel row][row])
+    __shared__ double Fp[kPanel][kPanel];          // this panel's own
+    __shared__ double own[kPanel][9 * kPanel];     // this panel's final rows, live columns
+    __shared__ double own_inv[kPanel], own_piv[kPanel];
+    const int c = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const int np = (m + kPanel - 1) / kPanel, r0 = kPanel * c;
+    constexpr int kLive = 9 * kPanel, kBarThreads = 32 * 10;
+    // column threads: column col of 72, rows 2 g and 2 g + 1
+    const bool pivot_warp = warp == 0, idle = warp == 4 || warp == 8;
+    const int cw = warp - 1 - (warp > 4) - (warp > 8), ct = 32 * cw + lane, col = ct % kLive, g = ct / kLive;
+    const bool is_a = col < kBlock - r0;
+    const int j = is_a ? r0 + col : col - (kBlock - r0);  // A or B column
+    const int place = is_a ? j : kBlock + j;              // in a panel buffer
+    double v[2] = {0.0, 0.0};
+    // pivot warp: lane tri(a, b) holds D[a][b], 1 <= a <= b, of the diagonal
+    // block in d, and lane b < 8 D[0][b] in d0
+    int da = 1, db = lane + 1;
+#pragma unroll
+    for (int a = 1; a < kPanel - 1; ++a)
+        if (da == a && db >= kPanel) {  // past the end of row a
+            db = db - kPanel + a + 1;
+            da = a + 1;
+        }
+    const bool tri = db < kPanel;  // lanes 28 .. 31 hold no entry
+    if (!tri) da = db = kPanel - 1;
+    double d = 0.0, d0 = 0.0;
+    if (c < np) {
+        if (pivot_warp) {
+            if (r0 + db < m) d = G[r0 + da + (long)(r0 + db) * ldg];
+            if (lane < kPanel && r0 + lane < m) d0 = G[r0 + (long)(r0 + lane) * ldg];
+        } else if (!idle) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = r0 + 2 * g + h;
+                if (is_a) v[h] = i < m && j < m ? G[(i < j ? i : j) + (long)(i < j ? j : i) * ldg] : 0.0;
+                else v[h] = i == j ? 1.0 : 0.0;
+            }
+        }
     }
-    if (t == 0) bad = 0;
-    __syncthreads();
-    if (t == 0) {
-        const double piv = M[0][0];
-        if (!(piv > 0.0)) bad = 1;
-        inv_s[0] = piv > 0.0 ? recip_newton(piv) : 0.0;
-    }
-    __syncthreads();
-    for (int k = 0; k + 1 < m; ++k) {
-        const double inv = inv_s[k];
-        if (w < kBlockWarps) {
-            // this warp's rows and their multipliers M_ki / M_kk (lane q: row q)
-            const int nr = w + k + 1 < m ? (m - (k + 1 + w) + kBlockWarps - 1) / kBlockWarps : 0;
-            const int iq = k + 1 + w + kBlockWarps * lane;
-            const double fl = lane < nr ? M[k][iq] * inv : 0.0;
-            for (int q = 0; q < nr; ++q) {
-                const int i = k + 1 + w + kBlockWarps * q;
-                const double f = __shfl_sync(0xffffffffu, fl, q);
-                const int na = m - i, s_i = na + k + 1;  // live A columns [i, m), B columns [0, k]
-                const int cskip = i == k + 1 ? 0 : -1;  // the next pivot: the pivot warp's
-                for (int c0 = 0; c0 < s_i; c0 += 32) {
-                    const int c = c0 + lane;
-                    if (c < s_i && c != cskip) {
-                        const int col = c < na ? i + c : kBlock + (c - na);
-                        M[i][col] = fma(-f, M[k][col], M[i][col]);
+    bool bad = false;
+    cluster_arrive();  // every CTA of the cluster runs before its memory is written
+    cluster_wait();
+    for (int q = 0; q < np; ++q) {
+        if (c == q) {
+            if (pivot_warp) {
+#pragma unroll
+                for (int k = 0; k < kPanel; ++k) {
+                    // row k: in d0 of lane b, or (k >= 1) in d of lane tri(k, b) = base + b
+                    const int base = k * kPanel - k * (k + 1) / 2 - kPanel;
+                    const double row = k == 0 ? d0 : d;
+                    const double piv = __shfl_sync(0xffffffffu, row, k == 0 ? 0 : base + k);
+                    const bool in = r0 + k < m, ok = __double_as_longlong(piv) > 0 &&
+                                                     __double_as_longlong(piv) <= 0x7FF0000000000000ll;  // > 0, no NaN
+                    bad = bad || (in && !ok);
+                    const double inv = in && ok ? recip_newton(piv) : 0.0;
+                    const double ra = __shfl_sync(0xffffffffu, row, k == 0 ? da : (base + da) & 31),
+                                 rb = __shfl_sync(0xffffffffu, row, k == 0 ? db : (base + db) & 31);
+                    const double f = ra * inv;  // multiplier of row a
+                    if (da > k) d = fma(-f, rb, d);
+                    if (tri && db == kPanel - 1) Fp[k][da] = f;  // rows a > k are used
+                    if (lane == 0) {
+                        own_inv[k] = inv;
+                        own_piv[k] = piv;
+                    }
+                    if (k + 1 < kPanel) {
+                        __syncwarp();
+                        asm volatile("bar.arrive %0, %1;" ::"r"(1 + k), "r"(kBarThreads) : "memory");
+                    }
+                }
+            } else if (!idle) {
+#pragma unroll
+                for (int k = 0; k < kPanel; ++k) {
+                    if ((k >> 1) == g) own[k][col] = v[k & 1];
+                    if (k + 1 < kPanel) {
+                        asm volatile("bar.sync %0, %1;" ::"r"(1 + k), "r"(kBarThreads) : "memory");
+                        const double x = own[k][col];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            if (2 * g + h > k) v[h] = fma(-Fp[k][2 * g + h], x, v[h]);
+                    }
+                }
+                for (int r = q + 1; r < np; ++r)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) store_remote(&buf[q & 1][2 * g + h][place], r, v[h]);
+            }
+            if (pivot_warp) {
+                __syncwarp();
+                if (lane < kPanel) {
+                    const double x = own_inv[lane];
+                    for (int r = q + 1; r < np; ++r) store_remote(&binv[q & 1][lane], r, x);
+                }
+            }
+            __syncthreads();
+        }
+        __syncwarp();
+        cluster_arrive();
+        if (c == q) {
+            // outputs while the later panels go on
+            if (t == 0 && bad) atomicOr(flag, 1);
+            if (t < kPanel) own_inv[t] = own_piv[t] > 0.0 ? rsqrt_newton(own_piv[t]) : 0.0;
+            __syncthreads();
+            if (!pivot_warp && !idle) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int i = r0 + 2 * g + h;
+                    if (i >= m || j >= m) continue;
+                    const double ri = own_inv[2 * g + h];
+                    if (is_a) R[i + (long)j * ld] = j >= i ? v[h] * ri : 0.0;
+                    else X[j + (long)i * ld] = j <= i ? v[h] * ri : 0.0;
+                }
+            }
+            for (int e = t; e < kPanel * kBlock; e += kBlockThreads) {
+                const int i = r0 + (e & (kPanel - 1)), k = e / kPanel;
+                if (i < m && k < r0) R[i + (long)k * ld] = 0.0;
+                if (i < m && k >= r0 + kPanel && k < m) X[k + (long)i * ld] = 0.0;
+            }
+        }
+        __syncwarp();
+        cluster_wait();
+        if (c > q && c < np) {
+            const double(*bq)[2 * kBlock] = buf[q & 1];
+            if (pivot_warp) {
+                // multipliers of this CTA's rows, then the diagonal block
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = (lane >> 3) + 4 * h, r = lane & 7;
+                    F[k][r] = bq[k][r0 + r] * binv[q & 1][k];
+                }
+                __syncwarp();
+                asm volatile("bar.arrive %0, %1;" ::"r"(9), "r"(kBarThreads) : "memory");
+#pragma unroll
+                for (int k = 0; k < kPanel; ++k) {
+                    d = fma(-F[k][da], bq[k][r0 + db], d);
+                    d0 = fma(-F[k][0], bq[k][r0 + (lane & 7)], d0);
+                }
+            } else if (!idle) {
+                asm volatile("bar.sync %0, %1;" ::"r"(9), "r"(kBarThreads) : "memory");
+                if (is_a || j < kPanel * (q + 1)) {
+#pragma unroll
+                    for (int k = 0; k < kPanel; ++k) {
+                        const double x = bq[k][place];
+                        v[0] = fma(-F[k][2 * g], x, v[0]);
+                        v[1] = fma(-F[k][2 * g + 1], x, v[1]);
                     }
                 }
             }
-        } else if (lane == 0) {
-            // the next pivot, as the row update of row k + 1 would form it
-            const double f = M[k][k + 1] * inv;
-            const double v = fma(-f, M[k][k + 1], M[k + 1][k + 1]);
-            M[k + 1][k + 1] = v;
-            if (!(v > 0.0)) bad = 1;
-            inv_s[k + 1] = v > 0.0 ? recip_newton(v) : 0.0;
         }
-        __syncthreads();
-    }
-    if (t < m) ri_s[t] = M[t][t] > 0.0 ? rsqrt_newton(M[t][t]) : 0.0;
-    __syncthreads();
-    if (t == 0 && bad) atomicOr(flag, 1);
-    for (int idx = t; idx < m * m; idx += blockDim.x) {
-        const int i = idx % m, jj = idx / m;
-        R[i + (long)jj * ld] = i <= jj ? M[i][jj] * ri_s[i] : 0.0;
-        X[i + (long)jj * ld] = i <= jj ? M[jj][kBlock + i] * ri_s[jj] : 0.0;
     }
 }
 
@@ -701,18 +820,10 @@ struct CholInv {
     gap_status rec(const double *G, long ldg, int o, int m)
     {
         if (m <= kBlock) {
-            static bool smem_set[64] = {};  // the attribute is per device
-            int dev = 0;
-            GAP_TRY_CUDA(cudaGetDevice(&dev));
-            if (dev >= 64 || !smem_set[dev]) {
-                GAP_TRY_CUDA(cudaFuncSetAttribute(k_chol_inv_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                  (int)kBlockSmem));
-                if (dev < 64) smem_set[dev] = true;
-            }
             gap_count_launch();
             gap_prof_begin(ST_SOLVE_BLOCK, st);
-            k_chol_inv_block<<<1, 32 * (kBlockWarps + 1), kBlockSmem, st>>>(G, ldg, m, R + o + (long)o * n, X + o + (long)o * n, n,
-                                                         w.at<int>(W_ERR) + 1);
+            k_chol_inv_block<<<kBlockCtas, kBlockThreads, 0, st>>>(G, ldg, m, R + o + (long)o * n, X + o + (long)o * n, n,
+                                                                   w.at<int>(W_ERR) + 1);
             gap_prof_end(ST_SOLVE_BLOCK, st);
             return gap_cuda_status(cudaGetLastError(), "k_chol_inv_block");
         }

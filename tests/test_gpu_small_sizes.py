@@ -70,3 +70,25 @@ def test_knm_edges_four_species(G, prec, rel):
     K = model.assemble_knm(G.Batch.from_synth(S.make_batch(cells), device="cuda"), precision=prec).cpu().numpy()
     assert np.abs(K - ref).max() <= rel * np.abs(ref).max()
     assert np.all(K[ref == 0.0] == 0.0)
+
+
+@pytest.mark.parametrize("n", [1, 7, 8, 9, 31, 33, 63, 64, 65, 96, 129])
+def test_factor_and_inverse_edges(G, n):
+    """Cholesky factor and inverse at the edges of the 8-row panels and 64-row blocks: backward error of the factor
+    within 64 n u of the diagonal's scale, R X = I to 1e-10 (the tolerances of the solve's own tests)."""
+    rng = np.random.default_rng(n)
+    A = rng.normal(size=(n + 40, n)) * 10.0 ** rng.uniform(-2, 2, n)
+    Gm = A.T @ A
+    R, X = G.test_chol_inv(Gm)
+    d = np.sqrt(np.diag(Gm))
+    assert (np.abs(R.T @ R - Gm) / np.outer(d, d)).max() <= 64 * n * 2.0 ** -53
+    assert np.abs(R @ X - np.eye(n)).max() <= 1e-10
+    assert np.all(np.tril(R, -1) == 0.0) and np.all(np.tril(X, -1) == 0.0)
+
+
+def test_factor_of_an_indefinite_matrix_is_an_error(G):
+    for n in (9, 64, 100):
+        Gm = np.eye(n)
+        Gm[n - 2, n - 2] = -1.0
+        with pytest.raises(G.GapError):
+            G.test_chol_inv(Gm)
