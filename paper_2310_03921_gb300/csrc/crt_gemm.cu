@@ -1127,7 +1127,9 @@ gap_status gap_crt_prep_cols(const CrtVMat &V, int T, long kpad, __nv_bfloat16 *
         return GAP_EINVAL;
     }
     GAP_TRY_CUDA(cudaMemsetAsync(E, 0, sizeof(int) * V.cols, st));
-    const int rpb = 128;
+    // rows per block: 128, or 16 where that leaves SMs without a block (a
+    // thread walks its rows one batch of loads after another)
+    const int rpb = (V.rows + 127) / 128 * ((V.cols + 127) / 128) >= 608 ? 128 : 16;
     dim3 g1((V.cols + 127) / 128, (unsigned)(V.rows > 0 ? (V.rows + rpb - 1) / rpb : 1));
     gap_count_launch();
     k_col_exp<<<g1, 128, 0, st>>>(V, rpb, E, diag, ld_diag, n_diag);

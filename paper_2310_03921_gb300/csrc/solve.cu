@@ -741,29 +741,34 @@ __device__ __forceinline__ double op_at(const CrtVMat &V, bool cols_of, int r, i
 // fixed order), so that a small product spreads over as many SMs as it has
 // tiles and uses all four FP64 pipes of each (each SM's FP64 rate is low).
 // C may alias Cin element for element.
-constexpr int kSmallTile = 8;
+// Each quarter takes a fourth of every staged chunk of K, so a short or ragged
+// K is split evenly too (quarters of fixed 32-wide blocks left three idle at
+// K = 32 and doubled the time at K = 160: a 2648 x 300 solve 1.25 -> 1.12 ms,
+// the shorter exponent scan of the operand preparation included).
+constexpr int kSmallTile = 8, kSmallK = 128;
 __global__ void __launch_bounds__(256) k_gemm_f64_small(CrtVMat A, int a_cols, CrtVMat B, int b_cols, int rowsA,
                                                         int rowsB, int K, double alpha, const double *Cin, long ldcin,
                                                         double *C, long ldc)
 {
-    __shared__ double As[4][kSmallTile][33], Bs[4][kSmallTile][33];
+    __shared__ double As[kSmallTile][kSmallK + 1], Bs[kSmallTile][kSmallK + 1];
     __shared__ double part[4][kSmallTile * kSmallTile];
     const int kg = threadIdx.x >> 6, tid = threadIdx.x & 63;
     const int tr = tid >> 3, tc = tid & 7;
     const int r0 = blockIdx.y * kSmallTile, c0 = blockIdx.x * kSmallTile;
     double acc = 0.0;
-    // quarter kg takes the 32-wide K blocks kg, kg + 4, ... (the same trip
-    // count for every thread)
-    for (int k0 = 0; k0 < K; k0 += 4 * 32) {
-        const int kb = k0 + 32 * kg;
-        for (int e = tid; e < kSmallTile * 32; e += 64) {
-            const int rr = e >> 5, kk = e & 31, gk = kb + kk;
-            As[kg][rr][kk] = (r0 + rr < rowsA && gk < K) ? op_at(A, a_cols, r0 + rr, gk) : 0.0;
-            Bs[kg][rr][kk] = (c0 + rr < rowsB && gk < K) ? op_at(B, b_cols, c0 + rr, gk) : 0.0;
+    for (int k0 = 0; k0 < K; k0 += kSmallK) {
+        const int len = K - k0 < kSmallK ? K - k0 : kSmallK, quarter = (len + 3) >> 2;
+        for (int e = threadIdx.x; e < kSmallTile * kSmallK; e += 256) {
+            const int rr = e / kSmallK, kk = e % kSmallK, gk = k0 + kk;
+            if (kk < 4 * quarter) {
+                As[rr][kk] = (r0 + rr < rowsA && gk < K) ? op_at(A, a_cols, r0 + rr, gk) : 0.0;
+                Bs[rr][kk] = (c0 + rr < rowsB && gk < K) ? op_at(B, b_cols, c0 + rr, gk) : 0.0;
+            }
         }
         __syncthreads();
+        const double *as = &As[tr][kg * quarter], *bs = &Bs[tc][kg * quarter];
 #pragma unroll 8
-        for (int kk = 0; kk < 32; ++kk) acc = fma(As[kg][tr][kk], Bs[kg][tc][kk], acc);
+        for (int kk = 0; kk < quarter; ++kk) acc = fma(as[kk], bs[kk], acc);
         __syncthreads();
     }
     part[kg][tid] = acc;
