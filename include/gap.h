@@ -11,9 +11,10 @@
  *  - Structure metadata (config offsets, cells, periodicity) is always read
  *    from HOST memory.  Positions, species and every output array live on
  *    the device when gap_batch.device != 0 and on the host otherwise.
- *  - Device-pointer calls are asynchronous on `stream` (a cudaStream_t, or
- *    NULL for the legacy default stream) except for one 4-byte device-to-host
- *    read of the pair count after the neighbour search; host-pointer calls
+ *  - Device-pointer calls work on `stream` (a cudaStream_t, or NULL for the
+ *    legacy default stream) and read their error words (and the pair count,
+ *    after the neighbour search, where earlier calls on the handle do not
+ *    bound it) back before they return, unless stated otherwise; host-pointer calls
  *    copy in, run on `stream`, copy out and synchronise before returning.
  *  - The caller owns all input and output buffers.  Handles own their
  *    device tables and workspaces; a handle must not be used by two calls at

@@ -286,7 +286,7 @@ static float bf16_to_float(uint16_t h)
 
 struct Workspace {
     NbrWork nbr;
-    DBuf pos, spec, coef, phat, pnorm, gp_of_atom, scan_tmp, rows, counts, gvec, wsum, eps, eps2,
+    DBuf pos, spec, coef, phat, pnorm, gp_of_atom, scan_tmp, rows, gvec, wsum, eps, eps2,
         W, eps_part, Gam, fpair, fw2, forces, vir_atom, cfgpart, energy, virial, local, err, A_hi, A_lo, t_row, W_hi, W_lo,
         epart_f, wpart_f, Gs, outbuf, kA, kAhi, kAlo, ksrc, kseg, kdest, kmeta, kslot, kfirst, kcount, kbounds, rank, segstart, outrow, Wp, kq, P,
         Kbuf, A_mid, W_mid, kAmid, phatc, pnormc, hfull, kV;
@@ -294,11 +294,13 @@ struct Workspace {
     // rows of each GP are those of the last ordinary call (species are fixed).
     bool graph = false;
     std::vector<int> counts_fixed;
+    HostPinned words;  // host copy of the call's device words (err, see nbr.h)
     void release()
     {
         nbr.release();
+        words.release();
         DBuf *bs[] = {&pos, &spec, &coef, &phat, &pnorm, &gp_of_atom, &scan_tmp, &rows,
-                      &counts, &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &fw2, &forces, &vir_atom, &cfgpart, &energy,
+                      &gvec, &wsum, &eps, &eps2, &W, &eps_part, &Gam, &fpair, &fw2, &forces, &vir_atom, &cfgpart, &energy,
                       &virial, &local, &err, &A_hi, &A_lo, &t_row, &W_hi, &W_lo, &epart_f, &wpart_f, &Gs, &outbuf,
                       &kA, &kAhi, &kAlo, &ksrc, &kseg, &kdest, &kmeta, &kslot, &kfirst, &kcount, &kbounds, &rank, &segstart,
                       &outrow, &Wp, &kq, &P, &Kbuf, &A_mid, &W_mid, &kAmid, &phatc, &pnormc, &hfull, &kV};
@@ -549,8 +551,9 @@ static gap_status stage_inputs(Workspace &w, const gap_batch *b, int S, const do
                                cudaStream_t st)
 {
     int n = b->n_atoms;
-    GAP_TRY(w.err.ensure(16 * sizeof(int)));
-    GAP_TRY_CUDA(cudaMemsetAsync(w.err.p, 0, 16 * sizeof(int), st));
+    GAP_TRY(w.err.ensure(kWords * sizeof(int)));
+    GAP_TRY(w.words.ensure(kWords * sizeof(int)));
+    GAP_TRY_CUDA(cudaMemsetAsync(w.err.p, 0, kWords * sizeof(int), st));
     if (b->device) {
         *pos = b->pos;
         *spec = b->species;  // checked by the neighbour build
@@ -574,15 +577,16 @@ static gap_status stage_inputs(Workspace &w, const gap_batch *b, int S, const do
 
 static gap_status check_device_errors(Workspace &w, cudaStream_t st)
 {
-    int e[16];
-    GAP_TRY_CUDA(cudaMemcpyAsync(e, w.err.p, sizeof(e), cudaMemcpyDeviceToHost, st));
+    const int *e = static_cast<const int *>(w.words.p);
+    GAP_TRY_CUDA(cudaMemcpyAsync(w.words.p, w.err.p, kWords * sizeof(int), cudaMemcpyDeviceToHost, st));
     GAP_TRY_CUDA(cudaStreamSynchronize(st));
+    const gap_status nbr = gap_neighbours_done(w.nbr, e);
     if (e[1]) { gap_set_error("species index out of range"); return GAP_EINVAL; }
     if (e[2]) {
         gap_set_error("tensor-core GEMM wait expired (code " + std::to_string(e[2]) + ")");
         return GAP_ETIMEOUT;
     }
-    return gap_neighbours_status(w.nbr, e[kNbrErr]);
+    return nbr;
 }
 
 extern "C" gap_status gap_soap_set_compression(gap_soap *s, const gap_compression *c)
@@ -786,10 +790,19 @@ template <typename T> static const T *gp_phat(const gap_soap *s, const Workspace
     return s->comp ? w.phatc.as<T>() : w.phat.as<T>();
 }
 
-// Neighbours + expansion + power spectrum for a batch, in arithmetic T.
+static int m_gps(const gap_model *m);
+static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, const int *spec, cudaStream_t st);
+static bool counts_without_wait(const gap_model *m, const gap_batch *b, std::vector<int> &counts);
+
+// Neighbours + expansion + power spectrum for a batch, in arithmetic T; with a
+// model also the rows of every GP (launched first, so that their counts come
+// back with the pair count).  ahead: the caller handles GAP_ECAPACITY (see
+// gap_neighbours), taken where nothing has to be read back before the next
+// launches.
 template <typename T>
 static gap_status run_descriptor(gap_soap *soap, Workspace &w, const gap_batch *b, const int **spec_out,
-                                 cudaStream_t st)
+                                 cudaStream_t st, bool ahead, const gap_model *m = nullptr,
+                                 std::vector<int> *counts = nullptr)
 {
     const SoapGeom &g = soap->geo;
     int n = b->n_atoms;
@@ -797,7 +810,22 @@ static gap_status run_descriptor(gap_soap *soap, Workspace &w, const gap_batch *
     const int *spec;
     gap_prof_begin(ST_NEIGHBOURS, st);
     GAP_TRY(stage_inputs(w, b, g.S, &pos, &spec, st));
-    GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, g.S, g.rc, w.err.as<int>(), st));
+    bool known = true;
+    if (m) {
+        GAP_TRY(launch_gp_rows(m, w, n, spec, st));
+        known = !w.graph && counts_without_wait(m, b, *counts);
+    }
+    GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, g.S, g.rc, w.err.as<int>(), static_cast<int *>(w.words.p),
+                           ahead && known, st));
+    if (m && w.graph) {
+        *counts = w.counts_fixed;
+    } else if (m) {
+        if (!known) {
+            const int *c = static_cast<const int *>(w.words.p) + kGpCounts;
+            counts->assign(c, c + m_gps(m));
+        }
+        w.counts_fixed = *counts;
+    }
     const PairList &pl = w.nbr.pairs;
     gap_prof_end(ST_NEIGHBOURS, st);
     GAP_TRY(w.coef.ensure(sizeof(T) * (size_t)n * g.GA * g.N * g.LM));
@@ -839,7 +867,8 @@ extern "C" gap_status gap_descriptor_sizes(gap_soap *soap, const gap_batch *b, l
     const double *pos;
     const int *spec;
     GAP_TRY(stage_inputs(w, b, soap->geo.S, &pos, &spec, st));
-    GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, soap->geo.S, soap->geo.rc, w.err.as<int>(), st));
+    GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, soap->geo.S, soap->geo.rc, w.err.as<int>(),
+                           static_cast<int *>(w.words.p), false, st));
     GAP_TRY(check_device_errors(w, st));
     if (n_desc) *n_desc = b->n_atoms;
     if (n_pairs) *n_pairs = w.nbr.pairs.n_pairs;
@@ -869,22 +898,29 @@ extern "C" gap_status gap_descriptor(gap_soap *soap, const gap_batch *b, gap_pre
         GAP_TRY(w.outbuf.ensure(sizeof(double) * cnt));
         dst = w.outbuf.as<double>();
     }
-    if (prec == GAP_FP64) {
-        GAP_TRY(run_descriptor<double>(soap, w, b, &spec, st));
-        if (cnt)
-            GAP_TRY_CUDA(cudaMemcpyAsync(dst, gp_phat<double>(soap, w), sizeof(double) * cnt, cudaMemcpyDeviceToDevice, st));
-    } else {
-        GAP_TRY(run_descriptor<float>(soap, w, b, &spec, st));
-        if (cnt) {
-            gap_count_launch();
-            k_to_double<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(gp_phat<float>(soap, w), dst, cnt);
-            GAP_TRY_CUDA(cudaGetLastError());
+    gap_status rc = GAP_OK;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+        // ahead of the pair count first; again if the batch had more pairs
+        const bool ahead = attempt == 0;
+        if (prec == GAP_FP64) {
+            GAP_TRY(run_descriptor<double>(soap, w, b, &spec, st, ahead));
+            if (cnt)
+                GAP_TRY_CUDA(cudaMemcpyAsync(dst, gp_phat<double>(soap, w), sizeof(double) * cnt,
+                                             cudaMemcpyDeviceToDevice, st));
+        } else {
+            GAP_TRY(run_descriptor<float>(soap, w, b, &spec, st, ahead));
+            if (cnt) {
+                gap_count_launch();
+                k_to_double<<<(unsigned)((cnt + 255) / 256), 256, 0, st>>>(gp_phat<float>(soap, w), dst, cnt);
+                GAP_TRY_CUDA(cudaGetLastError());
+            }
         }
+        if (!b->device && cnt)
+            GAP_TRY_CUDA(cudaMemcpyAsync(p_out, dst, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
+        rc = check_device_errors(w, st);
+        if (rc != GAP_ECAPACITY) break;
     }
-    if (!b->device && cnt)
-        GAP_TRY_CUDA(cudaMemcpyAsync(p_out, dst, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
-    GAP_TRY(check_device_errors(w, st));
-    return GAP_OK;
+    return rc;
     GAP_API_END
 }
 
@@ -920,6 +956,8 @@ struct gap_model {
     std::mutex mu;
 };
 
+
+static int m_gps(const gap_model *m) { return m->n_gp; }
 
 static void release_model(gap_model *m)
 {
@@ -1164,45 +1202,45 @@ template <typename T> static const T *gp_alpha(const GPData &g);
 template <> const double *gp_alpha<double>(const GPData &g) { return g.a64.as<double>(); }
 template <> const float *gp_alpha<float>(const GPData &g) { return g.a32.as<float>(); }
 
-// Rows of every GP (atoms of species s); counts copied to host.
-static gap_status gp_rows_all(gap_model *m, Workspace &w, int n, const int *spec, std::vector<int> &counts,
-                              cudaStream_t st)
+// Rows of every GP (atoms of species s); their counts stay in the call's
+// device words.
+static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, const int *spec, cudaStream_t st)
 {
     int G = m->n_gp;
     GAP_TRY(w.gp_of_atom.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.rank.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_gp_rows_tmp_ints(n, G)));
     GAP_TRY(w.rows.ensure(sizeof(int) * (size_t)(G > 0 ? G : 1) * n));
-    GAP_TRY(w.counts.ensure(sizeof(int) * (size_t)(G + 1)));
-    GAP_TRY(gap_gp_rows(n, G, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.counts.as<int>(),
-                        w.gp_of_atom.as<int>(), w.rank.as<int>(), st));
-    if (w.graph) {
-        counts = w.counts_fixed;
-        return GAP_OK;
-    }
+    return gap_gp_rows(n, G, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.err.as<int>() + kGpCounts,
+                       w.gp_of_atom.as<int>(), w.rank.as<int>(), st);
+}
+
+// The counts where the host knows them: one species, or species on the host.
+static bool counts_without_wait(const gap_model *m, const gap_batch *b, std::vector<int> &counts)
+{
+    const int G = m->n_gp, n = b->n_atoms;
+    if (G > 0 && m->soap->geo.S > 1 && b->device) return false;
     counts.assign(G, 0);
-    if (G > 0) {
-        GAP_TRY_CUDA(cudaMemcpyAsync(counts.data(), w.counts.p, sizeof(int) * G, cudaMemcpyDeviceToHost, st));
-        GAP_TRY_CUDA(cudaStreamSynchronize(st));
+    if (G > 0 && m->soap->geo.S == 1) {
+        counts[0] = n;
+    } else if (G > 0) {
+        for (int i = 0; i < n; ++i)
+            if (b->species[i] < G) ++counts[b->species[i]];
     }
-    w.counts_fixed = counts;
-    return GAP_OK;
+    return true;
 }
 
 template <typename T>
-static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, gap_precision prec, double *energy,
-                               double *local_e, double *forces, double *virial, cudaStream_t st)
+static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, gap_precision prec, double *energy,
+                               double *local_e, double *forces, double *virial, bool ahead, cudaStream_t st)
 {
     gap_soap *soap = m->soap;
     const SoapGeom &g = soap->geo;
     const int n = b->n_atoms, C = b->n_configs;
     const int *spec;
-    GAP_TRY(run_descriptor<T>(soap, w, b, &spec, st));
-    const PairList &pl = w.nbr.pairs;
     std::vector<int> counts;
-    gap_prof_begin(ST_GP_ROWS, st);
-    GAP_TRY(gp_rows_all(m, w, n, spec, counts, st));
-    gap_prof_end(ST_GP_ROWS, st);
+    GAP_TRY(run_descriptor<T>(soap, w, b, &spec, st, ahead, m, &counts));
+    const PairList &pl = w.nbr.pairs;
 
     // Forces and virial need the backward pass (Eq. 3); energies alone do not.
     const bool grad = forces != nullptr || virial != nullptr;
@@ -1291,7 +1329,7 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
             const int nt = gap_contract_simt_parts(gp.M);
             GAP_TRY(w.W.ensure(sizeof(T) * (size_t)R * gp.M));
             GAP_TRY(w.eps_part.ensure(sizeof(double) * (size_t)R * nt));
-            GAP_TRY(gap_contract_simt<T>(phg, Dg, Dg16, rows, w.counts.as<int>() + s, R, gp_X<T>(gp),
+            GAP_TRY(gap_contract_simt<T>(phg, Dg, Dg16, rows, w.err.as<int>() + kGpCounts + s, R, gp_X<T>(gp),
                                          gp_alpha<T>(gp), gp.M, m->delta, m->zeta, w.W.as<T>(),
                                          w.eps_part.as<double>(), gvec, w.eps.as<double>(), st));
         } else {
@@ -1406,6 +1444,17 @@ static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, g
     }
     if (w.graph) return GAP_OK;  // errors are read by gap_step_graph_status
     return check_device_errors(w, st);
+}
+
+// Without a wait for the pair count first (gap_neighbours), and again with
+// one if the batch had more pairs per atom than this workspace has met.
+template <typename T>
+static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, gap_precision prec, double *energy,
+                               double *local_e, double *forces, double *virial, cudaStream_t st)
+{
+    const gap_status rc = predict_once<T>(m, w, b, prec, energy, local_e, forces, virial, true, st);
+    if (rc != GAP_ECAPACITY || w.graph) return rc;
+    return predict_once<T>(m, w, b, prec, energy, local_e, forces, virial, false, st);
 }
 
 extern "C" gap_status gap_predict(gap_model *m, const gap_batch *b, gap_precision prec, double *energy,
@@ -1789,9 +1838,8 @@ static gap_status knm_impl(gap_model *m, const gap_batch *b, gap_precision prec,
     if (krows * Mt && !(tc && m->soap->geo.S == 1 && m->n_gp == 1))
         GAP_TRY_CUDA(cudaMemsetAsync(K, 0, sizeof(double) * krows * Mt, st));
     const int *spec;
-    GAP_TRY(run_descriptor<T>(m->soap, w, b, &spec, st));
     std::vector<int> counts;
-    GAP_TRY(gp_rows_all(m, w, n, spec, counts, st));
+    GAP_TRY(run_descriptor<T>(m->soap, w, b, &spec, st, false, m, &counts));
     if (tc) {
         if constexpr (sizeof(T) == 4) {
             if (Mt > 0) GAP_TRY(knm_tc(m, w, b, prec == GAP_BF16X6 ? 3 : 2, spec, counts, K, Mt, st));
@@ -2093,9 +2141,8 @@ extern "C" gap_status gap_predict_variance(gap_model *m, const gap_batch *b, dou
     int Mt = 0;
     for (auto &g : m->gp) Mt += g.M;
     const int *spec;
-    GAP_TRY(run_descriptor<double>(m->soap, w, b, &spec, st));
     std::vector<int> counts;
-    GAP_TRY(gp_rows_all(m, w, n, spec, counts, st));
+    GAP_TRY(run_descriptor<double>(m->soap, w, b, &spec, st, false, m, &counts));
     double *dvar = var;
     if (!b->device) {
         GAP_TRY(m->var_out.ensure(sizeof(double) * (size_t)n));

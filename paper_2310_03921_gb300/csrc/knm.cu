@@ -829,7 +829,8 @@ struct JacLaunch {
             return GAP_EUNSUPPORTED;
         }
         auto kern = k_jacobian_rows<N, L, GA, T>;
-        GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        if (shm > 48 * 1024)
+            GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
         const typename V4<T>::type *vec;
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();

@@ -13,6 +13,7 @@
 #include "nbr.h"
 
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 namespace {
@@ -562,6 +563,9 @@ gap_status gap_scan(const int *in, int n, int *out, int *tmp, int *total, cudaSt
 
 size_t gap_scan_tmp_ints(int n) { return n > 0 ? ((size_t)n + kScanTile - 1) / kScanTile + 4 : 4; }
 
+// The cell geometries' part of the device buffer they share with the offsets.
+static size_t geo_bytes(int n_configs) { return (sizeof(CellGeom) * (size_t)(n_configs + 1) + 255) / 256 * 256; }
+
 // Host-side geometry of each configuration's bin grid.
 gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom> &geo, int &n_bins)
 {
@@ -621,18 +625,41 @@ gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom
 }
 
 gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, const int *d_species, int S, double rc,
-                          int *err, cudaStream_t st)
+                          int *words, int *host, bool ahead, cudaStream_t st)
 {
     int n = b->n_atoms;
     std::vector<CellGeom> geo;
     int n_bins = 0;
     GAP_TRY(gap_cell_geometry(b, rc, geo, n_bins));
     GAP_TRY(w.reserve_atoms(n, b->n_configs, n_bins));
-    w.err = err + kNbrErr;
+    int *err = words;
+    w.err = words + kNbrErr;
+    w.total = words + kNbrTotal;
+    w.n_atoms = n;
     if (!w.graph) {
-        GAP_TRY_CUDA(cudaMemcpyAsync(w.geo, geo.data(), sizeof(CellGeom) * geo.size(), cudaMemcpyHostToDevice, st));
-        GAP_TRY_CUDA(cudaMemcpyAsync(w.cfg_offsets, b->config_offsets, sizeof(int) * (b->n_configs + 1),
-                                     cudaMemcpyHostToDevice, st));
+        // geometry and offsets in one copy from pinned memory
+        const size_t og = geo_bytes(b->n_configs), bytes = og + sizeof(int) * (b->n_configs + 1);
+        if (w.in_flight) {  // an earlier call ended in an error before it synchronised
+            GAP_TRY_CUDA(cudaDeviceSynchronize());
+            w.in_flight = false;
+        }
+        if (bytes > w.cap_stage) {
+            if (w.stage) cudaFreeHost(w.stage);
+            w.stage = nullptr;
+            w.cap_stage = 0;
+            if (cudaMallocHost(&w.stage, bytes + bytes / 4) != cudaSuccess) {
+                cudaGetLastError();
+                w.stage = nullptr;
+                gap_set_error("pinned host allocation failed");
+                return GAP_ENOMEM;
+            }
+            w.cap_stage = bytes + bytes / 4;
+        }
+        if (!geo.empty()) std::memcpy(w.stage, geo.data(), sizeof(CellGeom) * geo.size());
+        if (b->n_configs > 0)
+            std::memcpy(static_cast<char *>(w.stage) + og, b->config_offsets, sizeof(int) * (b->n_configs + 1));
+        GAP_TRY_CUDA(cudaMemcpyAsync(w.geo, w.stage, bytes, cudaMemcpyHostToDevice, st));
+        w.in_flight = true;
     }
     const BinInputs in{n, b->n_configs, S, d_pos, d_species, w.cfg_offsets, w.geo, err};
     if (n > 0 && n <= kSmallAtoms && n_bins <= kSmallBins) {
@@ -657,19 +684,22 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, c
                                                        w.bin_start, w.bin_atoms, w.counts);
         GAP_TRY_CUDA(cudaGetLastError());
     }
+    // room for the pairs: a capacity, or (after a wait) their number
+    ahead = ahead && !w.graph && w.pairs_per_atom > 0.0;
+    const double room = std::ceil(1.05 * w.pairs_per_atom * n) + 64.0;
+    if (room > (double)(1 << 30)) ahead = false;
+    int P = w.graph ? w.pair_cap : ahead ? (int)room : 0;
+    const bool capped = w.graph || ahead;
     GAP_TRY(gap_scan(w.counts, n, w.pairs.offsets, w.scan_tmp, w.total, st,
-                     w.graph ? ScanCap{w.pair_cap, w.total + 1, w.err} : ScanCap{}));
-    int P = 0;
-    if (w.graph) {
-        P = w.pair_cap;
-        GAP_TRY(w.reserve_pairs(P));
-        w.pairs.count = w.total + 1;
-    } else {
-        GAP_TRY_CUDA(cudaMemcpyAsync(&P, w.total, sizeof(int), cudaMemcpyDeviceToHost, st));
+                     capped ? ScanCap{P, w.total + 1, w.err} : ScanCap{}));
+    w.pairs.count = capped ? w.total + 1 : w.total;
+    if (!capped) {
+        GAP_TRY_CUDA(cudaMemcpyAsync(host, words, sizeof(int) * kWords, cudaMemcpyDeviceToHost, st));
         GAP_TRY_CUDA(cudaStreamSynchronize(st));
-        GAP_TRY(w.reserve_pairs(P));
-        w.pairs.count = w.total;
+        w.in_flight = false;
+        P = host[kNbrTotal];
     }
+    GAP_TRY(w.reserve_pairs(P));
     w.pairs.n_pairs = P;
     if (n > 0) {
         gap_count_launch();
@@ -684,8 +714,14 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, c
     return GAP_OK;
 }
 
-gap_status gap_neighbours_status(const NbrWork &w, int e)
+gap_status gap_neighbours_done(NbrWork &w, const int *host)
 {
+    const int e = host[kNbrErr];
+    w.in_flight = false;
+    if (w.n_atoms > 0) {
+        const double ppa = (double)host[kNbrTotal] / w.n_atoms;
+        if (ppa > w.pairs_per_atom) w.pairs_per_atom = ppa;
+    }
     if (e & 1) {
         gap_set_error("more neighbour pairs than the pair capacity (" + std::to_string(w.pair_cap) +
                       ") of the captured step");
@@ -718,8 +754,8 @@ static gap_status grow(void **p, size_t &cap, size_t bytes)
 
 gap_status NbrWork::reserve_atoms(int n, int n_configs, int n_bins)
 {
-    GAP_TRY(grow((void **)&geo, cap_geo, sizeof(CellGeom) * (n_configs + 1)));
-    GAP_TRY(grow((void **)&cfg_offsets, cap_cfg, sizeof(int) * (n_configs + 2)));
+    GAP_TRY(grow((void **)&geo, cap_geo, geo_bytes(n_configs) + sizeof(int) * (n_configs + 2)));
+    cfg_offsets = reinterpret_cast<int *>(reinterpret_cast<char *>(geo) + geo_bytes(n_configs));
     GAP_TRY(grow((void **)&cart, cap_cart, sizeof(D4) * (size_t)(n + 1)));
     GAP_TRY(grow((void **)&cart32, cap_c32, sizeof(float4) * (size_t)(n + 1)));
     GAP_TRY(grow((void **)&atom_cfg, cap_acfg, sizeof(int) * (size_t)(n + 1)));
@@ -731,7 +767,6 @@ gap_status NbrWork::reserve_atoms(int n, int n_configs, int n_bins)
     GAP_TRY(grow((void **)&bin_start, cap_bstart, sizeof(int) * (size_t)(n_bins + 2)));
     size_t t = gap_scan_tmp_ints(n > n_bins ? n : n_bins);
     GAP_TRY(grow((void **)&scan_tmp, cap_scan, sizeof(int) * t));
-    GAP_TRY(grow((void **)&total, cap_total, sizeof(int) * 4));
     return GAP_OK;
 }
 
@@ -749,8 +784,9 @@ gap_status NbrWork::reserve_pairs(int P)
 
 void NbrWork::release()
 {
-    void *ps[] = {geo, cfg_offsets, cart, cart32, atom_cfg, atom_bin, bin_atoms, counts, pairs.offsets, bin_count,
-                  bin_start, scan_tmp, total, keys, pairs.i, pairs.j, pairs.rev, pairs.vec64, pairs.vec32};
+    if (stage) cudaFreeHost(stage);
+    void *ps[] = {geo, cart, cart32, atom_cfg, atom_bin, bin_atoms, counts, pairs.offsets, bin_count,
+                  bin_start, scan_tmp, keys, pairs.i, pairs.j, pairs.rev, pairs.vec64, pairs.vec32};
     for (void *p : ps)
         if (p) cudaFree(p);
     *this = NbrWork();

@@ -784,7 +784,8 @@ template <typename T> struct Launch {
             return GAP_EUNSUPPORTED;
         }
         auto kern = k_expand<N, L, GA, T, WARPS>;
-        GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        if (shm > 48 * 1024)
+            GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
         const typename V4<T>::type *vec;
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();
@@ -804,7 +805,8 @@ template <typename T> struct Launch {
             return GAP_EUNSUPPORTED;
         }
         auto kern = GA > 1 && g.mixed ? k_chain<N, L, GA, (GA > 1), T> : k_chain<N, L, GA, false, T>;
-        GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
+        if (shm > 48 * 1024)
+            GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
         gap_count_launch();
         kern<<<(n + warps - 1) / warps, 32 * warps, shm, st>>>(g, n, gvec, wsum, mu, gp_of_atom, phat, pnorm, coef, Gam);
         return gap_cuda_status(cudaGetLastError(), "k_chain");

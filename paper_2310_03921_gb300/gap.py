@@ -174,7 +174,7 @@ def _stream(stream):
     if stream is not None:
         return C.c_void_p(stream)
     import torch
-    if torch.cuda.is_available() and torch.cuda.is_initialized():
+    if torch.cuda.is_initialized():
         return C.c_void_p(torch.cuda.current_stream().cuda_stream)
     return None
 
@@ -467,8 +467,12 @@ def _energy_function():
             grad = ctx.needs_input_grad[0]
             out = model.predict(b, precision, local=False, forces=grad, virial=grad)
             if grad:
-                counts = torch.as_tensor(np.diff(b.offsets), dtype=torch.long, device=pos.device)
-                ctx.save_for_backward(out["forces"], counts)
+                # one configuration scales as a whole; several by their atoms' rows
+                if b.n_configs == 1:
+                    ctx.save_for_backward(out["forces"])
+                else:
+                    counts = torch.as_tensor(np.diff(b.offsets), dtype=torch.long, device=pos.device)
+                    ctx.save_for_backward(out["forces"], counts)
                 ctx.mark_non_differentiable(out["virial"])
                 return out["energy"], out["virial"]
             return out["energy"], None
@@ -476,9 +480,11 @@ def _energy_function():
         @staticmethod
         @once_differentiable
         def backward(ctx, g_energy, g_virial):
-            forces, counts = ctx.saved_tensors
-            per_atom = torch.repeat_interleave(g_energy, counts, output_size=forces.shape[0])
-            return -per_atom[:, None] * forces, None, None, None, None, None, None
+            forces, *counts = ctx.saved_tensors
+            g = -g_energy
+            if counts:
+                g = torch.repeat_interleave(g, counts[0], output_size=forces.shape[0])[:, None]
+            return g * forces, None, None, None, None, None, None
 
     _ENERGY_FN = GapEnergy
     return GapEnergy

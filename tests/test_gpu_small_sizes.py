@@ -92,3 +92,28 @@ def test_factor_of_an_indefinite_matrix_is_an_error(G):
         Gm[n - 2, n - 2] = -1.0
         with pytest.raises(G.GapError):
             G.test_chol_inv(Gm)
+
+
+def test_batches_denser_than_any_before(G):
+    """A call may size its pair arrays from earlier calls: denser batches, of more and of fewer atoms, give what a
+    fresh model gives, and so does a sparse one after them."""
+    _, _, sparse, alpha = oracle_model(0, 30, n_cells=1)
+    w = S.workload(0)
+
+    def model():
+        soap = G.Soap.from_spec(w.soap)
+        return soap, G.Model(soap, sparse, alpha, w.delta, w.zeta)
+
+    cells = [_cluster(9), S.displaced_diamond(0, 3, (2, 2, 2), 0.1), S.displaced_diamond(0, 4, (1, 1, 1), 0.1)]
+    squeezed = S.displaced_diamond(0, 5, (2, 2, 2), 0.05, a=4.2)
+    cells += [squeezed, _cluster(1), _cluster(9), squeezed]
+    soap, kept = model()
+    for s in cells:
+        b = G.Batch.from_synth(S.make_batch([s]), device="cuda")
+        fsoap, fresh = model()
+        for prec in ("fp64", "bf16x3"):
+            got, ref = kept.predict(b, prec), fresh.predict(b, prec)
+            for k in ref:
+                assert np.array_equal(got[k].cpu().numpy(), ref[k].cpu().numpy()), (k, s.n)
+            assert np.array_equal(soap.descriptor(b, prec).cpu().numpy(), fsoap.descriptor(b, prec).cpu().numpy())
+        assert soap.descriptor_sizes(b) == fsoap.descriptor_sizes(b)
