@@ -1268,10 +1268,17 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
             // several GPs: one persistent launch per GEMM stage over all of
             // them, each GP with its own slice of the scratch buffers
             grouped = true;
-            size_t ra = 0, rw = 0, rp = 0, rr = 0;
+            size_t ra = 0, rw = 0, rp = 0, rr = 0, rg = 0;
+            std::vector<int> nrs(m->n_gp), mpad(m->n_gp);
+            for (int s = 0; s < m->n_gp; ++s) {
+                nrs[s] = m->gp[s].M > 0 ? counts[s] : 0;
+                mpad[s] = m->gp[s].M_pad;
+            }
+            auto parts = [&](int s) { return gap_contract_parts(nrs.data(), mpad.data(), m->n_gp, Dg16, nsplit, s); };
             for (int s = 0; s < m->n_gp; ++s) {
                 const size_t R = counts[s];
                 ra += R * Dg16;
+                rg += R * Dg16 * parts(s);
                 rw += R * m->gp[s].M_pad;
                 rp += R * gap_tc_max_parts(m->gp[s].M_pad);
                 rr += R;
@@ -1287,22 +1294,20 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
             }
             GAP_TRY(w.epart_f.ensure(4 * rp));
             GAP_TRY(w.wpart_f.ensure(4 * rp));
-            GAP_TRY(w.Gs.ensure(4 * ra));
+            GAP_TRY(w.Gs.ensure(4 * rg));
             std::vector<TcScratch> scs(m->n_gp);
             std::vector<TcModelGP> mgs(m->n_gp);
             std::vector<const int *> rws(m->n_gp);
-            std::vector<int> nrs(m->n_gp);
-            size_t oa = 0, ow = 0, op = 0, orr = 0;
+            size_t oa = 0, ow = 0, op = 0, orr = 0, og = 0;
             const bool three = nsplit == 3;
             for (int s = 0; s < m->n_gp; ++s) {
                 const GPData &gp = m->gp[s];
                 const size_t R = counts[s];
-                nrs[s] = gp.M > 0 ? (int)R : 0;
                 rws[s] = w.rows.as<int>() + (size_t)s * n;
                 scs[s] = TcScratch{w.A_hi.as<__nv_bfloat16>() + oa, w.A_lo.as<__nv_bfloat16>() + oa,
                                    w.t_row.as<float>() + orr, w.W_hi.as<__nv_bfloat16>() + ow,
                                    w.W_lo.as<__nv_bfloat16>() + ow, w.epart_f.as<float>() + op,
-                                   w.wpart_f.as<float>() + op, w.Gs.as<float>() + oa,
+                                   w.wpart_f.as<float>() + op, w.Gs.as<float>() + og,
                                    three ? w.A_mid.as<__nv_bfloat16>() + oa : nullptr,
                                    three ? w.W_mid.as<__nv_bfloat16>() + ow : nullptr};
                 mgs[s] = TcModelGP{gp.M, gp.M_pad, m->mu_all.as<float>() + (size_t)s * Dg16, gp.s_col.as<float>(),
@@ -1311,6 +1316,7 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
                                    (three ? gp.BTlo3 : gp.BTlo).as<__nv_bfloat16>(), gp.Bmid.as<__nv_bfloat16>(),
                                    gp.BTmid.as<__nv_bfloat16>()};
                 oa += R * Dg16;
+                og += R * Dg16 * parts(s);
                 ow += R * gp.M_pad;
                 op += R * gap_tc_max_parts(gp.M_pad);
                 orr += R;
@@ -1346,7 +1352,7 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
                 }
                 GAP_TRY(w.epart_f.ensure(4 * (size_t)R * n_part));
                 GAP_TRY(w.wpart_f.ensure(4 * (size_t)R * n_part));
-                GAP_TRY(w.Gs.ensure(4 * (size_t)R * Dg16));
+                GAP_TRY(w.Gs.ensure(4 * (size_t)R * Dg16 * gap_contract_parts(&R, &gp.M_pad, 1, Dg16, nsplit, 0)));
                 TcScratch sc{w.A_hi.as<__nv_bfloat16>(), w.A_lo.as<__nv_bfloat16>(), w.t_row.as<float>(),
                              w.W_hi.as<__nv_bfloat16>(), w.W_lo.as<__nv_bfloat16>(), w.epart_f.as<float>(),
                              w.wpart_f.as<float>(), w.Gs.as<float>(), w.A_mid.as<__nv_bfloat16>(),

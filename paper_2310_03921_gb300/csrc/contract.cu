@@ -375,7 +375,8 @@ __global__ void k_split_rows(const float *__restrict__ phat, int D, int ld, cons
 __global__ void __launch_bounds__(128) k_tc_finalize(const int *__restrict__ rows, int nrows,
                                                      const float *__restrict__ eps_part,
                                                      const float *__restrict__ wsum_part, int n_part,
-                                                     const float *__restrict__ Gs, int D16, double *__restrict__ eps,
+                                                     const float *__restrict__ Gs, int parts, int D16,
+                                                     double *__restrict__ eps,
                                                      float *__restrict__ wsum, float *__restrict__ g)
 {
     const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
@@ -395,7 +396,11 @@ __global__ void __launch_bounds__(128) k_tc_finalize(const int *__restrict__ row
         wsum[atom] = (float)w;
     }
     if (g)
-        for (int d = lane; d < D16; d += 32) g[(size_t)atom * D16 + d] = Gs[(size_t)r * D16 + d];
+        for (int d = lane; d < D16; d += 32) {
+            float v = Gs[(size_t)r * D16 + d];
+            for (int p = 1; p < parts; ++p) v += Gs[((size_t)p * nrows + r) * D16 + d];
+            g[(size_t)atom * D16 + d] = v;
+        }
 }
 
 }  // namespace
@@ -508,6 +513,15 @@ gap_status gap_split_rows(const float *phat, int D, int D16, const int *rows, in
     return gap_cuda_status(cudaGetLastError(), "k_split_rows");
 }
 
+int gap_contract_parts(const int *rows, const int *M_pad, int n, int D16, int nsplit, int q)
+{
+    // column tile: a split product runs on 128 x 128 tiles, a group on its own
+    const int bn = n == 1 ? 128 : gap_tc_grouped_col_tile(nsplit);
+    long tiles = 0;
+    for (int k = 0; k < n; ++k) tiles += (long)((rows[k] + 127) / 128) * ((D16 + bn - 1) / bn);
+    return gap_tc_ksplit(tiles, M_pad[q]);
+}
+
 gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, int nrows, const TcModelGP &gp,
                            double delta, int zeta, int nsplit, TcScratch &sc, double *eps, float *wsum, float *g,
                            int *err, cudaStream_t st)
@@ -544,6 +558,7 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
     gap_prof_end(ST_GEMM_Q, st);
     TcOperands op2{sc.W_hi, sc.W_lo, gp.BT_hi, gp.BT_lo, nrows, D16, gp.M_pad, gp.M_pad, gp.M_pad, nsplit,
                    three ? sc.W_mid : nullptr, three ? gp.BT_mid : nullptr};
+    op2.ksplit = gap_contract_parts(&nrows, &gp.M_pad, 1, D16, nsplit, 0);
     TcEpilogue ep2{};
     ep2.C = sc.Gs;
     ep2.ldc = D16;
@@ -554,8 +569,8 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
     }
     gap_prof_begin(ST_FINALIZE, st);
     gap_count_launch();
-    k_tc_finalize<<<(nrows + 3) / 4, 128, 0, st>>>(rows, nrows, sc.eps_part, sc.wsum_part, n_part, sc.Gs, D16, eps,
-                                                     wsum, g);
+    k_tc_finalize<<<(nrows + 3) / 4, 128, 0, st>>>(rows, nrows, sc.eps_part, sc.wsum_part, n_part, sc.Gs, op2.ksplit,
+                                                     D16, eps, wsum, g);
     GAP_TRY_CUDA(cudaGetLastError());
     gap_prof_end(ST_FINALIZE, st);
     return GAP_OK;
@@ -569,6 +584,8 @@ gap_status gap_contract_tc_groups(const float *phat, int D, int D16, const int *
     const int bn = gap_tc_grouped_col_tile(nsplit);
     std::vector<TcOperands> op1(n), op2(n);
     std::vector<TcEpilogue> ep1(n), ep2(n);
+    std::vector<int> mpad(n);
+    for (int q = 0; q < n; ++q) mpad[q] = gps[q].M_pad;
     gap_prof_begin(ST_SPLIT, st);
     for (int q = 0; q < n; ++q) {
         const TcModelGP &gp = gps[q];
@@ -598,6 +615,7 @@ gap_status gap_contract_tc_groups(const float *phat, int D, int D16, const int *
         e.n_part = 2 * ((gp.M_pad + bn - 1) / bn);
         op2[q] = TcOperands{sc[q].W_hi, sc[q].W_lo, gp.BT_hi, gp.BT_lo, nrows[q], D16, gp.M_pad, gp.M_pad, gp.M_pad,
                             nsplit, three ? sc[q].W_mid : nullptr, three ? gp.BT_mid : nullptr};
+        op2[q].ksplit = gap_contract_parts(nrows, mpad.data(), n, D16, nsplit, q);
         ep2[q].C = sc[q].Gs;
         ep2[q].ldc = D16;
     }
@@ -615,7 +633,7 @@ gap_status gap_contract_tc_groups(const float *phat, int D, int D16, const int *
         if (nrows[q] <= 0 || gps[q].M <= 0) continue;
         gap_count_launch();
         k_tc_finalize<<<(nrows[q] + 3) / 4, 128, 0, st>>>(rows[q], nrows[q], sc[q].eps_part, sc[q].wsum_part,
-                                                          ep1[q].n_part, sc[q].Gs, D16, eps, wsum, g);
+                                                          ep1[q].n_part, sc[q].Gs, op2[q].ksplit, D16, eps, wsum, g);
         GAP_TRY_CUDA(cudaGetLastError());
     }
     gap_prof_end(ST_FINALIZE, st);

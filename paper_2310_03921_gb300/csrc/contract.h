@@ -22,7 +22,7 @@ struct TcScratch {
     float *t_row;                // [rows]
     __nv_bfloat16 *W_hi, *W_lo;  // [rows][M_pad]
     float *eps_part, *wsum_part; // [rows][2 * M_pad / column tile]
-    float *Gs;                   // [rows][D16]
+    float *Gs;                   // [parts of K][rows][D16] (gap_contract_parts)
     __nv_bfloat16 *A_mid, *W_mid;  // middle planes (three-plane split)
 };
 
@@ -35,6 +35,9 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
                            double delta, int zeta, int nsplit, TcScratch &sc, double *eps, float *wsum, float *g,
                            int *err, cudaStream_t st);
 
+// Parts of K of the gradient product of each GP (rows[q] x D16, K = M_pad[q])
+// in gap_contract_tc (n = 1) or gap_contract_tc_groups.
+int gap_contract_parts(const int *rows, const int *M_pad, int n, int D16, int nsplit, int q);
 // Capacity per row of gap_contract_simt's partial energies (eps_part).
 int gap_contract_simt_parts(int M);
 // Column tiles of gap_contract_simt_fixed for M sparse points: the row stride

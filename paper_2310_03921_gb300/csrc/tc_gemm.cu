@@ -72,6 +72,7 @@ __device__ __forceinline__ float powi_small(float q, int e)
 struct TcProblem {
     CUtensorMap mA[3], mB[3];
     int rows, cols, K, tile0;
+    int kpart, tiles_part;  // K blocks per part of K, tiles of one part
     TcEpilogue ep;
 };
 // G problems in one persistent launch (the GEMMs of a batch's GPs): tiles
@@ -112,13 +113,25 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
     // and the two TMEM accumulators continue across tiles, so the epilogue of
     // one tile overlaps the loads and MMAs of the next.
     const int n_tiles = P.n_tiles;
-    // tile -> (problem, tile within it)
-    auto locate = [&](int tile, int &gi, int &lt) {
+    // tile -> (problem, tile within it, K blocks [kb0, kb1) of its part of K);
+    // returns the part
+    auto locate = [&](int tile, int &gi, int &lt, int &kb0, int &kb1) {
         gi = 0;
 #pragma unroll
         for (int q = 1; q < G; ++q)
             if (q < P.n && tile >= P.p[q].tile0) gi = q;
         lt = tile - P.p[gi].tile0;
+        const int kblocks = (P.p[gi].K + BK - 1) / BK;
+        if (EPI != EPI_STORE) {
+            kb0 = 0;
+            kb1 = kblocks;
+            return 0;
+        }
+        const int part = lt / P.p[gi].tiles_part;
+        lt -= part * P.p[gi].tiles_part;
+        kb0 = part * P.p[gi].kpart;
+        kb1 = min(kb0 + P.p[gi].kpart, kblocks);
+        return part;
     };
 
     // K is consumed in chunks of KC blocks; each chunk accumulates in a fresh
@@ -156,12 +169,12 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
         if (lane == 0) {
             int g = 0;  // k blocks issued by this CTA
             for (int tile = blockIdx.x; tile < n_tiles && !*abort_flag; tile += gridDim.x) {
-                int gi, lt;
-                locate(tile, gi, lt);
+                int gi, lt, kb0, kb1;
+                locate(tile, gi, lt, kb0, kb1);
                 const TcProblem &pr = P.p[gi];
-                const int n_ct = (pr.cols + BN - 1) / BN, kblocks = (pr.K + BK - 1) / BK;
+                const int n_ct = (pr.cols + BN - 1) / BN;
                 const int row0 = (lt / n_ct) * BM, col0 = (lt % n_ct) * BN;
-                for (int kb = 0; kb < kblocks; ++kb, ++g) {
+                for (int kb = kb0; kb < kb1; ++kb, ++g) {
                     int s = g % STAGES, r = g / STAGES;
                     if (!mbar_wait(&tail->empty[s], (r & 1) ^ 1, abort_flag, wlim)) {
                         *abort_flag = 1;
@@ -191,10 +204,10 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
             int g = 0, gc = 0;  // k blocks and K chunks consumed by this CTA
             int nchunks = 0;
             for (int tile = blockIdx.x; tile < n_tiles && !*abort_flag; tile += gridDim.x, gc += nchunks) {
-                int gi, lt;
-                locate(tile, gi, lt);
+                int gi, lt, kb0, kb1;
+                locate(tile, gi, lt, kb0, kb1);
                 const int K = P.p[gi].K, cols = P.p[gi].cols;
-                const int n_ct = (cols + BN - 1) / BN, kblocks = (K + BK - 1) / BK;
+                const int n_ct = (cols + BN - 1) / BN, kblocks = kb1 - kb0;
                 nchunks = (kblocks + KC - 1) / KC;
                 int ncol = cols - (lt % n_ct) * BN;
                 if (ncol > BN) ncol = BN;
@@ -219,7 +232,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                     uint32_t pa[3] = {sa, sa + A_BYTES, sa + 2 * A_BYTES};
                     uint32_t sb = sa + NS * A_BYTES;
                     uint32_t pb[3] = {sb, sb + B_BYTES, sb + 2 * B_BYTES};
-                    int ksteps = (K - kb * BK) / 16;
+                    int ksteps = (K - (kb0 + kb) * BK) / 16;
                     if (ksteps > BK / 16) ksteps = BK / 16;
                     for (int kk = 0; kk < ksteps; ++kk) {
                         uint32_t off = kk * 32;
@@ -248,12 +261,12 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
         int gc = 0;                         // K chunks consumed by this CTA
         int nchunks = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, gc += nchunks) {
-            int gi, lt;
-            locate(tile, gi, lt);
+            int gi, lt, kb0, kb1;
+            const int part = locate(tile, gi, lt, kb0, kb1);
             const TcEpilogue &ep = P.p[gi].ep;
             const int rows = P.p[gi].rows, cols = P.p[gi].cols;
             const int n_ct = (cols + BN - 1) / BN;
-            nchunks = ((P.p[gi].K + BK - 1) / BK + KC - 1) / KC;
+            nchunks = (kb1 - kb0 + KC - 1) / KC;
             const int rt = lt / n_ct, ct = lt % n_ct;
             const int row0 = rt * BM, col0 = ct * BN;
             int ncol = cols - col0;
@@ -315,7 +328,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                     int c0 = col0 + cbase;
                     if (EPI == EPI_STORE) {
                         int orow = ep.row_map ? ep.row_map[r] : r;
-                        float *out = ep.C + (size_t)orow * ep.ldc + c0;
+                        float *out = ep.C + ((size_t)part * rows + orow) * ep.ldc + c0;
                         if (cbase + 32 <= ncol && (ep.ldc & 3) == 0) {
 #pragma unroll
                             for (int k = 0; k < 32; k += 4)
@@ -483,7 +496,16 @@ gap_status launch_g(const TcOperands *ops, const TcEpilogue *eps, int n, int *er
         pr.K = op.K;
         pr.tile0 = (int)tiles;
         pr.ep = eps[q];
-        tiles += (long)((op.cols + BN - 1) / BN) * ((op.rows + BM - 1) / BM);
+        const long per = (long)((op.cols + BN - 1) / BN) * ((op.rows + BM - 1) / BM);
+        const int kblocks = (op.K + BK - 1) / BK, parts = EPI == EPI_STORE && op.ksplit > 1 ? op.ksplit : 1;
+        const int chunks = (kblocks + 3) / 4;  // chunks of four K blocks (KC)
+        pr.kpart = (chunks + parts - 1) / parts * 4;
+        pr.tiles_part = (int)per;
+        if ((long)(parts - 1) * pr.kpart >= kblocks || (long)parts * pr.kpart < kblocks) {
+            gap_set_error("tensor-core GEMM: bad split of K");
+            return GAP_EINVAL;
+        }
+        tiles += per * parts;
         ++P.n;
     }
     if (P.n == 0) return GAP_OK;
@@ -612,6 +634,16 @@ TcEpilogue with_parts(const TcEpilogue &ep, int epi, const TcOperands &op, const
 
 int gap_tc_sm_count() { return sm_count(); }
 
+int gap_tc_ksplit(long tiles, int K)
+{
+    const int chunks = (K + 4 * BK - 1) / (4 * BK);
+    if (tiles <= 0 || chunks <= 1 || 2 * tiles > sm_count()) return 1;
+    int parts = (int)(sm_count() / tiles);
+    if (parts > chunks) parts = chunks;
+    const int per = (chunks + parts - 1) / parts;  // chunks per part
+    return (chunks + per - 1) / per;               // no empty part
+}
+
 gap_status gap_tc_make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows)
 {
     return make_map(m, ptr, rows, cols, ld, box_rows);
@@ -739,6 +771,7 @@ gap_status gap_tc_gemm(const TcOperands &op, const TcEpilogue &ep, int epi, int 
         }
         return launch_variant(op, ep, epi, 0, err, st);
     }
+    if (op.ksplit > 1) return launch_variant(op, ep, epi, 2, err, st);  // few 128 x 128 tiles
     if (const int fv = forced_variant(op, epi); fv >= 0)
         return launch_variant(op, with_parts(ep, epi, op, kVariants2[fv]), epi, fv, err, st);
     const int bn = gap_tc_plan(op, ep, epi, err, st);

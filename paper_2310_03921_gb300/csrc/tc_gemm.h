@@ -14,6 +14,8 @@ struct TcOperands {
     int rows, cols, K, lda, ldb;
     int nsplit;                              // 2: hi + lo planes, 3: hi + mid + lo
     const __nv_bfloat16 *A_mid, *B_mid;      // used when nsplit == 3
+    int ksplit;                              // EPI_STORE: parts of K, each its own partial C
+                                             // [part][rows][ldc] (0, 1: none; gap_tc_ksplit)
 };
 
 struct TcEpilogue {
@@ -60,6 +62,10 @@ bool gap_tc_tuned_entry(int k, int *fields, float *ms);
 // [rows][ld] (cols of them valid) loaded in boxes of box_rows x 64.
 int gap_tc_sm_count();
 gap_status gap_tc_make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows);
+// Parts of K (whole chunks of 256) that give a store-epilogue product of
+// `tiles` output tiles enough work for the SMs, at most one per chunk: a few
+// tiles with a long K are otherwise a serial chain on as many SMs.
+int gap_tc_ksplit(long tiles, int K);
 // *err (device int) receives a nonzero code if a bounded wait expired.
 gap_status gap_tc_gemm(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, cudaStream_t st);
 // Several problems (the GEMMs of a batch's GPs: same planes, epilogue

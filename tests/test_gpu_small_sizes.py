@@ -117,3 +117,18 @@ def test_batches_denser_than_any_before(G):
                 assert np.array_equal(got[k].cpu().numpy(), ref[k].cpu().numpy()), (k, s.n)
             assert np.array_equal(soap.descriptor(b, prec).cpu().numpy(), fsoap.descriptor(b, prec).cpu().numpy())
         assert soap.descriptor_sizes(b) == fsoap.descriptor_sizes(b)
+
+
+@pytest.mark.parametrize("prec", ["bf16x3", "bf16x6"])
+@pytest.mark.parametrize("atoms,M", [(1, 257), (64, 600), (9, 513)])
+def test_gradient_product_split_over_points(G, atoms, M, prec):
+    """Few atoms and many sparse points: the gradient product's sum over the points runs in parts."""
+    soap_o, model_o, sparse, alpha = oracle_model(1, M, n_cells=3)
+    w = S.workload(1)
+    s = _cluster(atoms)
+    E, le, F, V = O.predict(soap_o, model_o, s)
+    model = G.Model(G.Soap.from_spec(w.soap), sparse, alpha, w.delta, w.zeta)
+    out = model.predict(G.Batch.from_synth(S.make_batch([s]), device="cuda"), precision=prec)
+    assert np.abs(out["local_e"].cpu().numpy() - le).max() <= 1e-4
+    assert np.abs(out["forces"].cpu().numpy() - F).max() <= 1e-4
+    assert np.abs(out["virial"][0].cpu().numpy() - V).max() <= 1e-3 * max(1.0, np.abs(V).max())
