@@ -1211,7 +1211,7 @@ static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, const 
     GAP_TRY(w.rank.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_gp_rows_tmp_ints(n, G)));
     GAP_TRY(w.rows.ensure(sizeof(int) * (size_t)(G > 0 ? G : 1) * n));
-    return gap_gp_rows(n, G, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.err.as<int>() + kGpCounts,
+    return gap_gp_rows(n, G, m->soap->geo.S == 1, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.err.as<int>() + kGpCounts,
                        w.gp_of_atom.as<int>(), w.rank.as<int>(), st);
 }
 

@@ -250,15 +250,17 @@ template <typename T> bool small_tiles(int rows, int cols)
 constexpr int kRowsOne = 8192, kRowsTile = 1024;  // atoms of the one-block form; per block else
 constexpr int kMaxGPs = 8;
 
-// Atoms of each GP (species below n_gp) in kRowsTile consecutive atoms.
+// Atoms of each GP (species below n_gp) in kRowsTile consecutive atoms.  one:
+// a single species; the host takes its count as n without reading it back, so
+// every atom has a row whatever its species says (a wrong one fails the call).
 __global__ void __launch_bounds__(kRowsTile)
-k_gp_counts(int n, int n_gp, const int *__restrict__ species, int *__restrict__ block_counts)
+k_gp_counts(int n, int n_gp, bool one, const int *__restrict__ species, int *__restrict__ block_counts)
 {
     __shared__ int cnt[kMaxGPs];
     if (threadIdx.x < kMaxGPs) cnt[threadIdx.x] = 0;
     __syncthreads();
     const int i = blockIdx.x * kRowsTile + threadIdx.x;
-    const int z = i < n ? species[i] : -1;
+    const int z = i < n ? (one ? 0 : species[i]) : -1;
     for (int s = 0; s < n_gp; ++s) {
         const unsigned m = __ballot_sync(0xffffffffu, z == s);
         if ((threadIdx.x & 31) == 0 && m) atomicAdd(&cnt[s], __popc(m));
@@ -273,7 +275,7 @@ k_gp_counts(int n, int n_gp, const int *__restrict__ species, int *__restrict__ 
 // k_gp_counts, whose counts of the tiles before it each block adds up.  One
 // or two launches for all GPs; a flag, scan and compaction per GP were six.
 __global__ void __launch_bounds__(kRowsTile)
-k_gp_rows(int n, int n_gp, const int *__restrict__ species, const int *__restrict__ block_counts,
+k_gp_rows(int n, int n_gp, bool one, const int *__restrict__ species, const int *__restrict__ block_counts,
           int *__restrict__ rows, int *__restrict__ counts, int *__restrict__ gp_of_atom, int *__restrict__ rank)
 {
     __shared__ int wcnt[kMaxGPs][33], base[kMaxGPs];
@@ -302,7 +304,7 @@ k_gp_rows(int n, int n_gp, const int *__restrict__ species, const int *__restric
     const int t0 = block_counts ? blockIdx.x : 0, t1 = block_counts ? blockIdx.x + 1 : (n + kRowsTile - 1) / kRowsTile;
     for (int t = t0; t < t1; ++t) {
         const int i = t * kRowsTile + threadIdx.x;
-        const int z = i < n ? species[i] : -1;
+        const int z = i < n ? (one ? 0 : species[i]) : -1;
         int before = 0;
         for (int s = 0; s < n_gp; ++s) {
             const unsigned m = __ballot_sync(0xffffffffu, z == s);
@@ -474,8 +476,8 @@ gap_status gap_contract_simt_fixed(const double *phat, int D, int ldg, const int
     return gap_cuda_status(cudaGetLastError(), "k_eps_rows");
 }
 
-gap_status gap_gp_rows(int n, int n_gp, const int *species, int *tmp, int *rows, int *counts, int *gp_of_atom,
-                       int *rank, cudaStream_t st)
+gap_status gap_gp_rows(int n, int n_gp, bool one, const int *species, int *tmp, int *rows, int *counts,
+                       int *gp_of_atom, int *rank, cudaStream_t st)
 {
     if (n_gp > kMaxGPs) {
         gap_set_error("too many GPs");
@@ -487,15 +489,15 @@ gap_status gap_gp_rows(int n, int n_gp, const int *species, int *tmp, int *rows,
     }
     if (n <= kRowsOne) {
         gap_count_launch();
-        k_gp_rows<<<1, kRowsTile, 0, st>>>(n, n_gp, species, nullptr, rows, counts, gp_of_atom, rank);
+        k_gp_rows<<<1, kRowsTile, 0, st>>>(n, n_gp, one, species, nullptr, rows, counts, gp_of_atom, rank);
         return gap_cuda_status(cudaGetLastError(), "k_gp_rows");
     }
     const int nb = (n + kRowsTile - 1) / kRowsTile;
     gap_count_launch();
-    k_gp_counts<<<nb, kRowsTile, 0, st>>>(n, n_gp, species, tmp);
+    k_gp_counts<<<nb, kRowsTile, 0, st>>>(n, n_gp, one, species, tmp);
     GAP_TRY_CUDA(cudaGetLastError());
     gap_count_launch();
-    k_gp_rows<<<nb, kRowsTile, 0, st>>>(n, n_gp, species, tmp, rows, counts, gp_of_atom, rank);
+    k_gp_rows<<<nb, kRowsTile, 0, st>>>(n, n_gp, one, species, tmp, rows, counts, gp_of_atom, rank);
     return gap_cuda_status(cudaGetLastError(), "k_gp_rows");
 }
 

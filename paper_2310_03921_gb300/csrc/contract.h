@@ -54,9 +54,10 @@ gap_status gap_contract_simt_fixed(const double *phat, int D, int ldg, const int
 
 // rows[s][n] = atoms of species s in index order for every GP s < n_gp (at
 // most 8), counts[s] their number, gp_of_atom[atom] = s (-1: none), rank[atom]
-// = its row.  tmp: gap_gp_rows_tmp_ints ints.
-gap_status gap_gp_rows(int n, int n_gp, const int *species, int *tmp, int *rows, int *counts, int *gp_of_atom,
-                       int *rank, cudaStream_t st);
+// = its row; one: a single species, every atom is GP 0's.  tmp:
+// gap_gp_rows_tmp_ints ints.
+gap_status gap_gp_rows(int n, int n_gp, bool one, const int *species, int *tmp, int *rows, int *counts,
+                       int *gp_of_atom, int *rank, cudaStream_t st);
 size_t gap_gp_rows_tmp_ints(int n, int n_gp);
 gap_status gap_split_rows(const float *phat, int D, int D16, const int *rows, int nrows, const float *mu,
                           __nv_bfloat16 *Ahi, __nv_bfloat16 *Alo, __nv_bfloat16 *Amid, float *t_row, cudaStream_t st);

@@ -132,3 +132,21 @@ def test_gradient_product_split_over_points(G, atoms, M, prec):
     assert np.abs(out["local_e"].cpu().numpy() - le).max() <= 1e-4
     assert np.abs(out["forces"].cpu().numpy() - F).max() <= 1e-4
     assert np.abs(out["virial"][0].cpu().numpy() - V).max() <= 1e-3 * max(1.0, np.abs(V).max())
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32", "bf16x3"])
+def test_wrong_species_of_a_one_species_model(G, prec):
+    """The host takes n rows for a one-species model: a wrong species on the device leaves no row unset, the call ends
+    in an error and the next one is right."""
+    soap_o, model_o, sparse, alpha = oracle_model(0, 30, n_cells=1)
+    w = S.workload(0)
+    model = G.Model(G.Soap.from_spec(w.soap), sparse, alpha, w.delta, w.zeta)
+    s = _cluster(64)
+    E, le, F, V = O.predict(soap_o, model_o, s)
+    bad = S.make_batch([s])
+    bad.species[:] = 5
+    for call in (model.predict, model.assemble_knm):
+        with pytest.raises(G.GapError, match="species"):
+            call(G.Batch.from_synth(bad, device="cuda"), precision=prec)
+    out = model.predict(G.Batch.from_synth(S.make_batch([s]), device="cuda"), precision=prec)
+    assert np.abs(out["local_e"].cpu().numpy() - le).max() <= 1e-4
