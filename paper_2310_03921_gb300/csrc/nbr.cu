@@ -624,6 +624,12 @@ gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom
     return GAP_OK;
 }
 
+// Most pairs a build makes room for without waiting for their number: 2^20,
+// about 100 MB of pair arrays.  The wait costs ~20 us, 1% of a call with that
+// many pairs (1.5 ms and more); beyond, a workspace that once met a dense cell
+// would hold its density times the atoms of a large sparse one.
+constexpr int kAheadPairs = 1 << 20;
+
 gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, const int *d_species, int S, double rc,
                           int *words, int *host, bool ahead, cudaStream_t st)
 {
@@ -687,7 +693,7 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, c
     // room for the pairs: a capacity, or (after a wait) their number
     ahead = ahead && !w.graph && w.pairs_per_atom > 0.0;
     const double room = std::ceil(1.05 * w.pairs_per_atom * n) + 64.0;
-    if (room > (double)(1 << 30)) ahead = false;
+    if (room > (double)kAheadPairs) ahead = false;
     int P = w.graph ? w.pair_cap : ahead ? (int)room : 0;
     const bool capped = w.graph || ahead;
     GAP_TRY(gap_scan(w.counts, n, w.pairs.offsets, w.scan_tmp, w.total, st,

@@ -60,7 +60,8 @@ constexpr int kNbrErr = 8, kNbrTotal = 16, kGpCounts = 18, kWords = 32;
 // on the device).  Synchronises once to read the words (`host`) and with them
 // the pair count, except in graph mode and when `ahead` is allowed and the
 // workspace has finished a build before: the arrays then get room for the
-// most pairs per atom seen so far, and a batch with more empties every list
+// most pairs per atom seen so far (2^20 pairs in all at most, else it waits),
+// and a batch with more empties every list
 // and ends in GAP_ECAPACITY (gap_neighbours_done), to be run again without
 // `ahead`.
 gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, const int *d_species, int S, double rc,
