@@ -1332,7 +1332,7 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
         if (R == 0 || gp.M == 0) continue;
         const int *rows = w.rows.as<int>() + (size_t)s * n;
         if (!tc) {
-            const int nt = gap_contract_simt_parts(gp.M);
+            const int nt = gap_contract_simt_parts<T>(R, gp.M);
             GAP_TRY(w.W.ensure(sizeof(T) * (size_t)R * gp.M));
             GAP_TRY(w.eps_part.ensure(sizeof(double) * (size_t)R * nt));
             GAP_TRY(gap_contract_simt<T>(phg, Dg, Dg16, rows, w.err.as<int>() + kGpCounts + s, R, gp_X<T>(gp),

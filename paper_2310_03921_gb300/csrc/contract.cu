@@ -413,11 +413,10 @@ gap_status gap_contract_simt(const T *phat, int D, int D16, const int *rows, con
                              T *g, double *eps, cudaStream_t st)
 {
     if (max_rows <= 0 || M <= 0) return GAP_OK;
-    int n_tiles = (M + TN - 1) / TN;
+    const int n_tiles = gap_contract_simt_parts<T>(max_rows, M);
     gap_prof_begin(ST_GEMM_Q, st);
     gap_count_launch();
     if (small_tiles<T>(max_rows, M)) {
-        n_tiles = (M + kST - 1) / kST;
         k_small_qW<T><<<dim3(n_tiles, (max_rows + kST - 1) / kST), 256, 0, st>>>(
             phat, D, rows, nrows_dev, X, alpha, M, (T)(delta * delta), zeta, W, M, eps_part, n_tiles);
     } else {
@@ -452,7 +451,13 @@ template gap_status gap_contract_simt<float>(const float *, int, int, const int 
                                              cudaStream_t);
 
 int gap_contract_simt_tiles(int M) { return M > 0 ? (M + TN - 1) / TN : 0; }
-int gap_contract_simt_parts(int M) { return M > 0 ? (M + kST - 1) / kST : 0; }
+template <typename T> int gap_contract_simt_parts(int rows, int M)
+{
+    const int tile = small_tiles<T>(rows, M) ? kST : TN;
+    return M > 0 ? (M + tile - 1) / tile : 0;
+}
+template int gap_contract_simt_parts<double>(int, int);
+template int gap_contract_simt_parts<float>(int, int);
 
 // The same two GEMMs as gap_contract_simt<double> on the identity row list,
 // launched without stage profiling (used by the allocation-free entry point).

@@ -38,8 +38,8 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
 // Parts of K of the gradient product of each GP (rows[q] x D16, K = M_pad[q])
 // in gap_contract_tc (n = 1) or gap_contract_tc_groups.
 int gap_contract_parts(const int *rows, const int *M_pad, int n, int D16, int nsplit, int q);
-// Capacity per row of gap_contract_simt's partial energies (eps_part).
-int gap_contract_simt_parts(int M);
+// Partial energies per row of gap_contract_simt (eps_part) for that many rows.
+template <typename T> int gap_contract_simt_parts(int rows, int M);
 // Column tiles of gap_contract_simt_fixed for M sparse points: the row stride
 // of its partial energies (eps_part holds n_rows x tiles).
 int gap_contract_simt_tiles(int M);
