@@ -17,7 +17,16 @@
 // Epilogues:
 //   EPI_KERNEL   the sparse-GP kernel of Eqs. 2 and 13 on centred operands:
 //                q = C + s_col + t_row, W = zeta delta^2 alpha q^(zeta-1) stored as
-//                BF16 hi/lo, per-tile partial sums of delta^2 alpha q^zeta and of W
+//                BF16 hi/lo, per-tile partial sums of delta^2 alpha q^zeta (taken
+//                as W q, divided by zeta at the end) and of W.  Its epilogue
+//                bounds it, in instructions and stores: a lane owns a row, so
+//                direct stores touch 32 lines 16 bytes at a time.  Each warp
+//                stages 32 x 32 blocks of W in shared memory and stores them by
+//                TMA, which also clips the last rows; zeta = 4 (every workload's)
+//                has its power written out, 14 instructions per element with
+//                it where the general loop and direct stores took 33.  A step
+//                of 32768 atoms 1444 -> 1316 us, of 110592 atoms 9059 -> 8144
+//                us, 512 four-species boxes 4059 -> 3843 us.
 //   EPI_QPOW     per atom and sparse point, W' = zeta delta^2 q^(zeta-1) and
 //                delta^2 q^zeta (FP32) for the K_NM rows
 //   EPI_STORE    FP32 store of C
@@ -28,6 +37,7 @@
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -42,16 +52,18 @@ using namespace tcp;
 constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int kEpiWarps = 8;
-constexpr int kThreads = 32 * (2 + kEpiWarps);
 
 struct SharedTail {
     uint64_t full[4];
     uint64_t empty[4];
     uint64_t acc_full[2];    // MMA -> epilogue, per TMEM accumulator buffer
-    uint64_t acc_empty[2];   // epilogue -> MMA (all epilogue threads arrive)
+    uint64_t acc_empty[2];   // epilogue -> MMA (every epilogue warp arrives)
     uint32_t tmem_base;
     int abort;
 };
+
+// A warp's staging of one W plane: 32 rows of 32 BF16, 64-byte swizzle.
+constexpr uint32_t kStagePlane = 32 * 64;
 
 // q^e for 0 <= e < 64 by square-and-multiply over the six bits of e: fully
 // unrolled (e is the same for every thread), so the epilogue's element loops
@@ -70,7 +82,7 @@ __device__ __forceinline__ float powi_small(float q, int e)
 // One GEMM problem of a launch: its operand maps (A hi / mid-or-lo / lo, B
 // the same), sizes, first tile in the launch's tile order, and epilogue.
 struct TcProblem {
-    CUtensorMap mA[3], mB[3];
+    CUtensorMap mA[3], mB[3], mW[3];  // mW: EPI_KERNEL's W planes (stores)
     int rows, cols, K, tile0;
     int kpart, tiles_part;  // K blocks per part of K, tiles of one part
     TcEpilogue ep;
@@ -101,10 +113,12 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
     constexpr uint32_t STAGE_BYTES = NS * A_BYTES + NS * B_BYTES;
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
-    SharedTail *tail = reinterpret_cast<SharedTail *>(smem + STAGES * STAGE_BYTES);
-    // epilogue scratch after the ring (the ring keeps filling for the next
-    // tile while an epilogue runs): K_NM row sums, or per-column constants
-    unsigned char *scratch = smem + STAGES * STAGE_BYTES + ((sizeof(SharedTail) + 127) & ~size_t(127));
+    // after the ring (which keeps filling for the next tile while an epilogue
+    // runs): the epilogue warps' store staging, the barriers, per-column constants
+    constexpr uint32_t STAGING = EPI == EPI_KERNEL ? EW * 2 * kStagePlane : 0;
+    unsigned char *staging = smem + STAGES * STAGE_BYTES;
+    SharedTail *tail = reinterpret_cast<SharedTail *>(staging + STAGING);
+    unsigned char *scratch = staging + STAGING + ((sizeof(SharedTail) + 127) & ~size_t(127));
     float *col_s = reinterpret_cast<float *>(scratch), *col_a = col_s + BN;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -146,7 +160,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&tail->acc_full[b], 1);
-            mbar_init(&tail->acc_empty[b], kThreads - 64);
+            mbar_init(&tail->acc_empty[b], EW);  // one arrival per epilogue warp
         }
         tail->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -258,8 +272,10 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
         const int quad = warp & 3;        // TMEM lane quadrant this warp may access
         const int half = ew >> 2;         // column group (a half for EW = 8)
         constexpr int HC = BN / NG;         // columns per group
+        unsigned char *wst = staging + ew * 2 * kStagePlane;  // this warp's two W planes of 32 rows x 32 columns
         int gc = 0;                         // K chunks consumed by this CTA
         int nchunks = 0;
+        bool ok = true;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, gc += nchunks) {
             int gi, lt, kb0, kb1;
             const int part = locate(tile, gi, lt, kb0, kb1);
@@ -273,15 +289,17 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
             if (ncol > BN) ncol = BN;
             const int r = row0 + quad * 32 + lane;
             if (EPI == EPI_KERNEL || EPI == EPI_QPOW) {
-                // stage the per-column constants while the MMAs run (after every
-                // epilogue thread has finished with the previous tile's)
-                named_barrier(3, kThreads - 64);
+                // stage the per-column constants while the MMAs run, after every
+                // epilogue warp has finished with the previous tile's; a wait
+                // that expired in one warp stops them all here
+                ok = bar_and(4, kThreads - 64, ok);
+                if (!ok) break;
                 for (int c = threadIdx.x - 64; c < BN; c += kThreads - 64) {
                     // the column arrays are padded to 256; a 192-column tile
                     // can reach past them, where nothing is used
                     int cc = col0 + c;
                     col_s[c] = c < ncol ? ep.s_col[cc] : 0.f;
-                    col_a[c] = c < ncol ? (EPI == EPI_KERNEL ? ep.alpha_col[cc] : 1.f) * ep.d2 : 0.f;
+                    col_a[c] = c < ncol ? (EPI == EPI_KERNEL ? (float)ep.zeta * (ep.alpha_col[cc] * ep.d2) : ep.d2) : 0.f;
                 }
                 named_barrier(3, kThreads - 64);
             }
@@ -289,13 +307,12 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
             float acc[HC];
 #pragma unroll
             for (int k = 0; k < HC; ++k) acc[k] = 0.f;
-            bool ok = true;
             for (int c = 0; c < nchunks; ++c) {
                 const int q = gc + c, buf = q & 1, use = q >> 1;
-                if (!mbar_wait(&tail->acc_full[buf], use & 1, abort_flag, wlim)) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&tail->acc_full[buf], use & 1, abort_flag, wlim));
+                if (!ok) {
                     *abort_flag = 1;
-                    atomicOr(err, 4);
-                    ok = false;
+                    if (lane == 0) atomicOr(err, 4);
                     break;
                 }
                 tc_fence_after();
@@ -310,15 +327,82 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                     }
                 }
                 tc_fence_before();
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tail->acc_empty[buf]))
-                             : "memory");
+                if (lane == 0)
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&tail->acc_empty[buf]))
+                                 : "memory");
             }
-            // every epilogue warp takes the same branch (the epilogues below use
-            // named barriers), so a wait that expired in one warp stops them all
-            ok = bar_and(4, kThreads - 64, ok);
-            if (!ok) break;
-            {
+            if (!ok) {
+                if (EPI == EPI_STORE) break;
+                continue;  // to the barrier that stops every warp
+            }
+            if constexpr (EPI == EPI_KERNEL) {
+                const float tr = r < rows ? ep.t_row[r] : 0.f;
+                const bool store = ep.W_hi != nullptr && row0 + quad * 32 < rows;  // energies only: W is not needed
                 float esum = 0.f, wsum = 0.f;
+                // Z: zeta, or 0 for any
+                auto kernel = [&](auto Z) {
+#pragma unroll
+                    for (int ch = 0; ch < HC / 32; ++ch) {
+                        const int cbase = half * HC + ch * 32;  // column within tile
+                        if (cbase >= ncol) continue;
+                        uint32_t pl[NS][16];
+#pragma unroll
+                        for (int k = 0; k < 32; k += 4) {
+                            const float4 s4 = *reinterpret_cast<const float4 *>(col_s + cbase + k);
+                            const float4 a4 = *reinterpret_cast<const float4 *>(col_a + cbase + k);
+                            const float sc[4] = {s4.x, s4.y, s4.z, s4.w}, ac[4] = {a4.x, a4.y, a4.z, a4.w};
+                            float w[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) {
+                                const float q = acc[ch * 32 + k + u] + sc[u] + tr;
+                                const float qz = Z.value == 4 ? (q * q) * q : powi_small(q, ep.zeta - 1);
+                                w[u] = ac[u] * qz;
+                                esum = fmaf(w[u], q, esum);
+                                wsum += w[u];
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; u += 2)
+#pragma unroll
+                                for (int p = 0; p < NS; ++p) {
+                                    const __nv_bfloat162 h = __floats2bfloat162_rn(w[u], w[u + 1]);
+                                    pl[p][(k + u) / 2] = *reinterpret_cast<const uint32_t *>(&h);
+                                    const float2 hf = __bfloat1622float2(h);
+                                    w[u] -= hf.x;
+                                    w[u + 1] -= hf.y;
+                                }
+                        }
+                        if (!store) continue;
+#pragma unroll
+                        for (int p0 = 0; p0 < NS; p0 += 2) {  // two planes at a time
+                            if (lane == 0) bulk_wait_read();  // the staging's earlier stores have read it
+                            __syncwarp();
+#pragma unroll
+                            for (int p = p0; p < NS && p < p0 + 2; ++p)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    *reinterpret_cast<uint4 *>(wst + (p - p0) * kStagePlane + lane * 64 +
+                                                               16 * (k ^ ((lane >> 1) & 3))) =
+                                        make_uint4(pl[p][4 * k], pl[p][4 * k + 1], pl[p][4 * k + 2], pl[p][4 * k + 3]);
+                            fence_async_shared();
+                            __syncwarp();
+                            if (lane == 0) {
+#pragma unroll
+                                for (int p = p0; p < NS && p < p0 + 2; ++p)
+                                    tma_store_2d(&P.p[gi].mW[p], wst + (p - p0) * kStagePlane, col0 + cbase,
+                                                 row0 + quad * 32);
+                                bulk_commit();
+                            }
+                        }
+                    }
+                };
+                if (ep.zeta == 4) kernel(std::integral_constant<int, 4>{});
+                else kernel(std::integral_constant<int, 0>{});
+                if (r < rows) {
+                    const int slot = ct * NG + half;
+                    ep.eps_part[(size_t)r * ep.n_part + slot] = esum / (float)ep.zeta;
+                    ep.wsum_part[(size_t)r * ep.n_part + slot] = wsum;
+                }
+            } else {
                 const int zeta = ep.zeta;
 #pragma unroll
                 for (int ch = 0; ch < HC / 32; ++ch) {
@@ -338,7 +422,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                             for (int k = 0; k < 32; ++k)
                                 if (cbase + k < ncol) out[k] = v[k];
                         }
-                    } else if (EPI == EPI_QPOW) {
+                    } else {
                         const float tr = ep.t_row[r];
                         const int orow = ep.row_map ? ep.row_map[r] : r;
                         float *pw = ep.Wp + (size_t)orow * ep.ldwp + c0, *pk = ep.kq + (size_t)orow * ep.ldwp + c0;
@@ -356,59 +440,11 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                             *reinterpret_cast<float4 *>(pw + k) = make_float4(wv[0], wv[1], wv[2], wv[3]);
                             *reinterpret_cast<float4 *>(pk + k) = make_float4(kv[0], kv[1], kv[2], kv[3]);
                         }
-                    } else {
-                        const float tr = ep.t_row[r];
-                        uint32_t hi[16], mid[16], lo[16];
-#pragma unroll
-                        for (int k = 0; k < 32; k += 2) {
-                            float w2[2];
-#pragma unroll
-                            for (int u = 0; u < 2; ++u) {
-                                float q = v[k + u] + col_s[cbase + k + u] + tr;
-                                const float qz = powi_small(q, zeta - 1);
-                                float a = col_a[cbase + k + u];
-                                esum += a * qz * q;
-                                float w = (float)zeta * a * qz;
-                                wsum += w;
-                                w2[u] = w;
-                            }
-                            __nv_bfloat162 h2 = __floats2bfloat162_rn(w2[0], w2[1]);
-                            float2 hf = __bfloat1622float2(h2);
-                            hi[k / 2] = *reinterpret_cast<uint32_t *>(&h2);
-                            float r0 = w2[0] - hf.x, r1 = w2[1] - hf.y;
-                            if (NS == 3) {
-                                __nv_bfloat162 m2 = __floats2bfloat162_rn(r0, r1);
-                                float2 mf = __bfloat1622float2(m2);
-                                mid[k / 2] = *reinterpret_cast<uint32_t *>(&m2);
-                                r0 -= mf.x;
-                                r1 -= mf.y;
-                            }
-                            lo[k / 2] = pack_bf16(r0, r1);
-                        }
-                        if (ep.W_hi != nullptr) {  // energies only: W is not needed
-                            uint4 *ph = reinterpret_cast<uint4 *>(ep.W_hi + (size_t)r * ep.ldw + c0);
-                            uint4 *pl = reinterpret_cast<uint4 *>(ep.W_lo + (size_t)r * ep.ldw + c0);
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                ph[k] = make_uint4(hi[4 * k], hi[4 * k + 1], hi[4 * k + 2], hi[4 * k + 3]);
-                                pl[k] = make_uint4(lo[4 * k], lo[4 * k + 1], lo[4 * k + 2], lo[4 * k + 3]);
-                            }
-                        }
-                        if (NS == 3 && ep.W_mid != nullptr) {
-                            uint4 *pm = reinterpret_cast<uint4 *>(ep.W_mid + (size_t)r * ep.ldw + c0);
-#pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                pm[k] = make_uint4(mid[4 * k], mid[4 * k + 1], mid[4 * k + 2], mid[4 * k + 3]);
-                        }
                     }
-                }
-                if (EPI == EPI_KERNEL && r < rows) {
-                    int slot = ct * NG + half;
-                    ep.eps_part[(size_t)r * ep.n_part + slot] = esum;
-                    ep.wsum_part[(size_t)r * ep.n_part + slot] = wsum;
                 }
             }
         }
+        if (EPI == EPI_KERNEL && lane == 0) bulk_wait_all();  // this warp's stores are done
     }
     tc_fence_before();
     __syncthreads();
@@ -450,7 +486,8 @@ int sm_count()
     return n[dev];
 }
 
-gap_status make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows)
+gap_status make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows, int box_cols = BK,
+                    CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B)
 {
     auto enc = encode_fn();
     if (!enc) {
@@ -463,10 +500,10 @@ gap_status make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld,
     }
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
+    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         gap_set_error("cuTensorMapEncodeTiled failed with code " + std::to_string((int)r));
@@ -491,6 +528,11 @@ gap_status launch_g(const TcOperands *ops, const TcEpilogue *eps, int n, int *er
             GAP_TRY(make_map(&pr.mA[pl], A[pl], op.rows, op.K, op.lda, BM));
             GAP_TRY(make_map(&pr.mB[pl], B[pl], op.cols, op.K, op.ldb, BN));
         }
+        if (EPI == EPI_KERNEL && eps[q].W_hi) {
+            const __nv_bfloat16 *W[3] = {eps[q].W_hi, NS == 3 ? eps[q].W_mid : eps[q].W_lo, eps[q].W_lo};
+            for (int pl = 0; pl < NS; ++pl)
+                GAP_TRY(make_map(&pr.mW[pl], W[pl], op.rows, eps[q].ldw, eps[q].ldw, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B));
+        }
         pr.rows = op.rows;
         pr.cols = op.cols;
         pr.K = op.K;
@@ -514,9 +556,14 @@ gap_status launch_g(const TcOperands *ops, const TcEpilogue *eps, int n, int *er
         return GAP_EUNSUPPORTED;
     }
     P.n_tiles = (int)tiles;
-    const size_t scratch = 2 * BN * sizeof(float);
-    size_t shm = (size_t)STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + ((sizeof(SharedTail) + 127) & ~size_t(127)) +
-                 scratch + 1024;
+    const size_t scratch = 2 * BN * sizeof(float), staging = EPI == EPI_KERNEL ? EW * 2 * kStagePlane : 0;
+    // 896: the base is 128-byte aligned at least (the 256-column kernel-energy tile takes all 227 KB)
+    const size_t shm = (size_t)STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + staging +
+                       ((sizeof(SharedTail) + 127) & ~size_t(127)) + scratch + 896;
+    static_assert(STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + (EPI == EPI_KERNEL ? EW * 2 * kStagePlane : 0) +
+                          ((sizeof(SharedTail) + 127) & ~size_t(127)) + 2 * BN * sizeof(float) + 896 <=
+                      227 * 1024,
+                  "shared memory of a block");
     auto kern = k_tc_gemm<BN, STAGES, EPI, NS, G, EW>;
     GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     dim3 grid((unsigned)(tiles < sm_count() ? tiles : sm_count()));
