@@ -28,7 +28,9 @@
 //                of 32768 atoms 1444 -> 1316 us, of 110592 atoms 9059 -> 8144
 //                us, 512 four-species boxes 4059 -> 3843 us.
 //   EPI_QPOW     per atom and sparse point, W' = zeta delta^2 q^(zeta-1) and
-//                delta^2 q^zeta (FP32) for the K_NM rows
+//                delta^2 q^zeta (FP32) for the K_NM rows, bound by its 8 bytes
+//                per element, stored the same way (K_NM of 200 silicon cells
+//                7020 -> 6891 us)
 //   EPI_STORE    FP32 store of C
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -82,7 +84,7 @@ __device__ __forceinline__ float powi_small(float q, int e)
 // One GEMM problem of a launch: its operand maps (A hi / mid-or-lo / lo, B
 // the same), sizes, first tile in the launch's tile order, and epilogue.
 struct TcProblem {
-    CUtensorMap mA[3], mB[3], mW[3];  // mW: EPI_KERNEL's W planes (stores)
+    CUtensorMap mA[3], mB[3], mW[3];  // mW (stores): EPI_KERNEL's W planes, EPI_QPOW's W' and k
     int rows, cols, K, tile0;
     int kpart, tiles_part;  // K blocks per part of K, tiles of one part
     TcEpilogue ep;
@@ -115,7 +117,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
     // after the ring (which keeps filling for the next tile while an epilogue
     // runs): the epilogue warps' store staging, the barriers, per-column constants
-    constexpr uint32_t STAGING = EPI == EPI_KERNEL ? EW * 2 * kStagePlane : 0;
+    constexpr uint32_t STAGING = EPI != EPI_STORE ? EW * 2 * kStagePlane : 0;
     unsigned char *staging = smem + STAGES * STAGE_BYTES;
     SharedTail *tail = reinterpret_cast<SharedTail *>(staging + STAGING);
     unsigned char *scratch = staging + STAGING + ((sizeof(SharedTail) + 127) & ~size_t(127));
@@ -299,7 +301,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                     // can reach past them, where nothing is used
                     int cc = col0 + c;
                     col_s[c] = c < ncol ? ep.s_col[cc] : 0.f;
-                    col_a[c] = c < ncol ? (EPI == EPI_KERNEL ? (float)ep.zeta * (ep.alpha_col[cc] * ep.d2) : ep.d2) : 0.f;
+                    if (EPI == EPI_KERNEL) col_a[c] = c < ncol ? (float)ep.zeta * (ep.alpha_col[cc] * ep.d2) : 0.f;
                 }
                 named_barrier(3, kThreads - 64);
             }
@@ -402,49 +404,67 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                     ep.eps_part[(size_t)r * ep.n_part + slot] = esum / (float)ep.zeta;
                     ep.wsum_part[(size_t)r * ep.n_part + slot] = wsum;
                 }
+            } else if constexpr (EPI == EPI_QPOW) {
+                const float tr = r < rows ? ep.t_row[r] : 0.f;
+                const bool store = row0 + quad * 32 < rows;
+                const float d2 = ep.d2, zd2 = (float)ep.zeta * d2;
+                // Z: zeta, or 0 for any
+                auto powers = [&](auto Z) {
+#pragma unroll
+                    for (int ch = 0; ch < HC / 32; ++ch) {
+                        const int cbase = half * HC + ch * 32;  // column within tile
+                        if (cbase >= ncol || !store) continue;
+#pragma unroll
+                        for (int p = 0; p < 2; ++p) {  // W', then k: 128-byte rows, 128-byte swizzle
+                            if (lane == 0) bulk_wait_read();
+                            __syncwarp();
+#pragma unroll
+                            for (int k = 0; k < 32; k += 4) {
+                                const float4 s4 = *reinterpret_cast<const float4 *>(col_s + cbase + k);
+                                const float sc[4] = {s4.x, s4.y, s4.z, s4.w};
+                                float o[4];
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) {
+                                    const float q = acc[ch * 32 + k + u] + sc[u] + tr;
+                                    const float qz = Z.value == 4 ? (q * q) * q : powi_small(q, ep.zeta - 1);
+                                    o[u] = p == 0 ? zd2 * qz : d2 * qz * q;
+                                }
+                                *reinterpret_cast<float4 *>(wst + lane * 128 + 16 * ((k >> 2) ^ (lane & 7))) =
+                                    make_float4(o[0], o[1], o[2], o[3]);
+                            }
+                            fence_async_shared();
+                            __syncwarp();
+                            if (lane == 0) {
+                                tma_store_2d(&P.p[gi].mW[p], wst, col0 + cbase, row0 + quad * 32);
+                                bulk_commit();
+                            }
+                        }
+                    }
+                };
+                if (ep.zeta == 4) powers(std::integral_constant<int, 4>{});
+                else powers(std::integral_constant<int, 0>{});
             } else {
-                const int zeta = ep.zeta;
 #pragma unroll
                 for (int ch = 0; ch < HC / 32; ++ch) {
                     int cbase = half * HC + ch * 32;   // column within tile
                     if (cbase >= ncol || r >= rows) continue;
                     const float *v = acc + ch * 32;
                     int c0 = col0 + cbase;
-                    if (EPI == EPI_STORE) {
-                        int orow = ep.row_map ? ep.row_map[r] : r;
-                        float *out = ep.C + ((size_t)part * rows + orow) * ep.ldc + c0;
-                        if (cbase + 32 <= ncol && (ep.ldc & 3) == 0) {
+                    int orow = ep.row_map ? ep.row_map[r] : r;
+                    float *out = ep.C + ((size_t)part * rows + orow) * ep.ldc + c0;
+                    if (cbase + 32 <= ncol && (ep.ldc & 3) == 0) {
 #pragma unroll
-                            for (int k = 0; k < 32; k += 4)
-                                *reinterpret_cast<float4 *>(out + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 32; ++k)
-                                if (cbase + k < ncol) out[k] = v[k];
-                        }
+                        for (int k = 0; k < 32; k += 4)
+                            *reinterpret_cast<float4 *>(out + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
                     } else {
-                        const float tr = ep.t_row[r];
-                        const int orow = ep.row_map ? ep.row_map[r] : r;
-                        float *pw = ep.Wp + (size_t)orow * ep.ldwp + c0, *pk = ep.kq + (size_t)orow * ep.ldwp + c0;
 #pragma unroll
-                        for (int k = 0; k < 32; k += 4) {
-                            float wv[4], kv[4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                float q = v[k + u] + col_s[cbase + k + u] + tr;
-                                const float qz = powi_small(q, zeta - 1);
-                                float a = col_a[cbase + k + u];
-                                wv[u] = (float)zeta * a * qz;
-                                kv[u] = a * qz * q;
-                            }
-                            *reinterpret_cast<float4 *>(pw + k) = make_float4(wv[0], wv[1], wv[2], wv[3]);
-                            *reinterpret_cast<float4 *>(pk + k) = make_float4(kv[0], kv[1], kv[2], kv[3]);
-                        }
+                        for (int k = 0; k < 32; ++k)
+                            if (cbase + k < ncol) out[k] = v[k];
                     }
                 }
             }
         }
-        if (EPI == EPI_KERNEL && lane == 0) bulk_wait_all();  // this warp's stores are done
+        if (EPI != EPI_STORE && lane == 0) bulk_wait_all();  // this warp's stores are done
     }
     tc_fence_before();
     __syncthreads();
@@ -486,25 +506,28 @@ int sm_count()
     return n[dev];
 }
 
+// A row-major [rows][ld] array (cols of them valid) of BF16 or FP32, in boxes
+// of box_rows x box_cols.
 gap_status make_map(CUtensorMap *m, const void *ptr, int rows, int cols, int ld, int box_rows, int box_cols = BK,
-                    CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B)
+                    CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B, bool fp32 = false)
 {
     auto enc = encode_fn();
     if (!enc) {
         gap_set_error("cuTensorMapEncodeTiled is unavailable");
         return GAP_ECUDA;
     }
-    if ((reinterpret_cast<uintptr_t>(ptr) & 15) || (ld * 2) % 16) {
+    const int item = fp32 ? 4 : 2;
+    if ((reinterpret_cast<uintptr_t>(ptr) & 15) || ((long)ld * item) % 16) {
         gap_set_error("tensor map operand is not 16-byte aligned");
         return GAP_EINVAL;
     }
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+    cuuint64_t strides[1] = {(cuuint64_t)ld * item};
     cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(ptr), dims, strides, box, estr,
-                     CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    CUresult r = enc(m, fp32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                     const_cast<void *>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
         gap_set_error("cuTensorMapEncodeTiled failed with code " + std::to_string((int)r));
         return GAP_ECUDA;
@@ -533,6 +556,12 @@ gap_status launch_g(const TcOperands *ops, const TcEpilogue *eps, int n, int *er
             for (int pl = 0; pl < NS; ++pl)
                 GAP_TRY(make_map(&pr.mW[pl], W[pl], op.rows, eps[q].ldw, eps[q].ldw, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B));
         }
+        if (EPI == EPI_QPOW) {
+            float *out[2] = {eps[q].Wp, eps[q].kq};
+            for (int p = 0; p < 2; ++p)
+                GAP_TRY(make_map(&pr.mW[p], out[p], op.rows, eps[q].ldwp, eps[q].ldwp, 32, 32,
+                                 CU_TENSOR_MAP_SWIZZLE_128B, true));
+        }
         pr.rows = op.rows;
         pr.cols = op.cols;
         pr.K = op.K;
@@ -556,11 +585,11 @@ gap_status launch_g(const TcOperands *ops, const TcEpilogue *eps, int n, int *er
         return GAP_EUNSUPPORTED;
     }
     P.n_tiles = (int)tiles;
-    const size_t scratch = 2 * BN * sizeof(float), staging = EPI == EPI_KERNEL ? EW * 2 * kStagePlane : 0;
+    const size_t scratch = 2 * BN * sizeof(float), staging = EPI != EPI_STORE ? EW * 2 * kStagePlane : 0;
     // 896: the base is 128-byte aligned at least (the 256-column kernel-energy tile takes all 227 KB)
     const size_t shm = (size_t)STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + staging +
                        ((sizeof(SharedTail) + 127) & ~size_t(127)) + scratch + 896;
-    static_assert(STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + (EPI == EPI_KERNEL ? EW * 2 * kStagePlane : 0) +
+    static_assert(STAGES * (NS * BM * BK * 2 + NS * BN * BK * 2) + (EPI != EPI_STORE ? EW * 2 * kStagePlane : 0) +
                           ((sizeof(SharedTail) + 127) & ~size_t(127)) + 2 * BN * sizeof(float) + 896 <=
                       227 * 1024,
                   "shared memory of a block");
@@ -586,7 +615,9 @@ gap_status launch_grouped(const TcOperands *ops, const TcEpilogue *eps, int n, i
     constexpr int BN = NS == 3 ? 128 : 256;
     if (epi == EPI_KERNEL) return launch_g<BN, 2, EPI_KERNEL, NS, kMaxGroups>(ops, eps, n, err, st);
     if (epi == EPI_STORE) return launch_g<BN, 2, EPI_STORE, NS, kMaxGroups>(ops, eps, n, err, st);
-    if (epi == EPI_QPOW) return launch_g<BN, 2, EPI_QPOW, NS, kMaxGroups>(ops, eps, n, err, st);
+    // 128 columns: a training batch of several species has few rows of each
+    // (K_NM of 24 four-species boxes 804 -> 791 us, with the stores by TMA)
+    if (epi == EPI_QPOW) return launch_g<128, 2, EPI_QPOW, NS, kMaxGroups>(ops, eps, n, err, st);
     gap_set_error("grouped tensor-core GEMM: bad epilogue");
     return GAP_EINVAL;
 }

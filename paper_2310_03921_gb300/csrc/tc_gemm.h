@@ -31,7 +31,8 @@ struct TcEpilogue {
     int ldw;
     float *eps_part, *wsum_part;  // [rows][n_part]
     int n_part;                   // 2 * number of column tiles
-    // EPI_QPOW (row_map: optional): Wp[row][c] = zeta d2 q^(zeta-1), kq[row][c] = d2 q^zeta
+    // EPI_QPOW: Wp[row][c] = zeta d2 q^(zeta-1), kq[row][c] = d2 q^zeta; rows
+    // of ldwp (a multiple of 32) are written in blocks of 32 columns
     float *Wp, *kq;
     int ldwp;
     // Bounded waits: limit of each mbarrier wait in ns (0: the default 2 s).
@@ -70,7 +71,8 @@ int gap_tc_ksplit(long tiles, int K);
 gap_status gap_tc_gemm(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, cudaStream_t st);
 // Several problems (the GEMMs of a batch's GPs: same planes, epilogue
 // EPI_KERNEL, EPI_QPOW or EPI_STORE) in one persistent launch per four problems, tiles
-// numbered problem after problem; the default tile variant, whose column tile
-// gap_tc_grouped_col_tile gives (EPI_KERNEL's n_part must be 2 ceil(cols / it)).
+// numbered problem after problem; one tile variant, whose column tile for
+// EPI_KERNEL and EPI_STORE gap_tc_grouped_col_tile gives (EPI_KERNEL's n_part
+// must be 2 ceil(cols / it)).
 int gap_tc_grouped_col_tile(int nsplit);
 gap_status gap_tc_gemm_grouped(const TcOperands *ops, const TcEpilogue *eps, int n, int epi, int *err, cudaStream_t st);

@@ -150,3 +150,23 @@ def test_wrong_species_of_a_one_species_model(G, prec):
             call(G.Batch.from_synth(bad, device="cuda"), precision=prec)
     out = model.predict(G.Batch.from_synth(S.make_batch([s]), device="cuda"), precision=prec)
     assert np.abs(out["local_e"].cpu().numpy() - le).max() <= 1e-4
+
+
+@pytest.mark.parametrize("zeta", [1, 2, 3, 5])
+@pytest.mark.parametrize("prec", ["bf16x3", "bf16x6"])
+def test_tensor_core_powers(G, zeta, prec):
+    """Powers other than 4 take the general epilogue of the energy products: energies, forces and K_NM rows, at a
+    ragged number of rows and of points."""
+    soap_o, model_o, sparse, alpha = oracle_model(0, 130, n_cells=3)
+    w = S.workload(0)
+    mo = O.Model(sparse, alpha, w.delta, zeta)
+    s = _cluster(33)
+    E, le, F, V = O.predict(soap_o, mo, s)
+    ref = O.knm(soap_o, mo, s)
+    model = G.Model(G.Soap.from_spec(w.soap), sparse, alpha, w.delta, zeta)
+    batch = G.Batch.from_synth(S.make_batch([s]), device="cuda")
+    out = model.predict(batch, precision=prec)
+    assert np.abs(out["local_e"].cpu().numpy() - le).max() <= 1e-4
+    assert np.abs(out["forces"].cpu().numpy() - F).max() <= 1e-4
+    K = model.assemble_knm(batch, precision=prec).cpu().numpy()
+    assert np.abs(K - ref).max() <= (5e-5 if prec == "bf16x3" else 2e-5) * np.abs(ref).max()
