@@ -1278,7 +1278,7 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
             for (int s = 0; s < m->n_gp; ++s) {
                 const size_t R = counts[s];
                 ra += R * Dg16;
-                rg += R * Dg16 * parts(s);
+                rg += parts(s) > 1 ? R * Dg16 * parts(s) : 0;
                 rw += R * m->gp[s].M_pad;
                 rp += R * gap_tc_max_parts(m->gp[s].M_pad);
                 rr += R;
@@ -1316,7 +1316,7 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
                                    (three ? gp.BTlo3 : gp.BTlo).as<__nv_bfloat16>(), gp.Bmid.as<__nv_bfloat16>(),
                                    gp.BTmid.as<__nv_bfloat16>()};
                 oa += R * Dg16;
-                og += R * Dg16 * parts(s);
+                og += parts(s) > 1 ? R * Dg16 * parts(s) : 0;
                 ow += R * gp.M_pad;
                 op += R * gap_tc_max_parts(gp.M_pad);
                 orr += R;
@@ -1352,7 +1352,8 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
                 }
                 GAP_TRY(w.epart_f.ensure(4 * (size_t)R * n_part));
                 GAP_TRY(w.wpart_f.ensure(4 * (size_t)R * n_part));
-                GAP_TRY(w.Gs.ensure(4 * (size_t)R * Dg16 * gap_contract_parts(&R, &gp.M_pad, 1, Dg16, nsplit, 0)));
+                const int parts = gap_contract_parts(&R, &gp.M_pad, 1, Dg16, nsplit, 0);
+                GAP_TRY(w.Gs.ensure(parts > 1 ? 4 * (size_t)R * Dg16 * parts : 0));
                 TcScratch sc{w.A_hi.as<__nv_bfloat16>(), w.A_lo.as<__nv_bfloat16>(), w.t_row.as<float>(),
                              w.W_hi.as<__nv_bfloat16>(), w.W_lo.as<__nv_bfloat16>(), w.epart_f.as<float>(),
                              w.wpart_f.as<float>(), w.Gs.as<float>(), w.A_mid.as<__nv_bfloat16>(),

@@ -372,8 +372,11 @@ __global__ void k_split_rows(const float *__restrict__ phat, int D, int ld, cons
 
 // eps, wsum and g of the atoms of one GP from the tensor-core partials.
 // One warp per row: the column-tile partials of eps and sum_m W summed in
-// FP64 (lanes over partials, then a fixed shuffle tree), and g moved to the
-// row's atom.  Four rows per block.
+// FP64 (lanes over partials, then a fixed shuffle tree), and, where the
+// gradient product ran in parts of K (g not NULL), their sum in order to the
+// row's atom; else the product has written g itself (copying every row here
+// made a call of 512 four-species boxes 3843 us, 3749 now).  Four rows per
+// block.
 __global__ void __launch_bounds__(128) k_tc_finalize(const int *__restrict__ rows, int nrows,
                                                      const float *__restrict__ eps_part,
                                                      const float *__restrict__ wsum_part, int n_part,
@@ -567,7 +570,9 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
                    three ? sc.W_mid : nullptr, three ? gp.BT_mid : nullptr};
     op2.ksplit = gap_contract_parts(&nrows, &gp.M_pad, 1, D16, nsplit, 0);
     TcEpilogue ep2{};
-    ep2.C = sc.Gs;
+    const bool split = op2.ksplit > 1;
+    ep2.C = split ? sc.Gs : g;
+    ep2.row_map = split ? nullptr : rows;
     ep2.ldc = D16;
     if (g) {
         gap_prof_begin(ST_GEMM_G, st);
@@ -577,7 +582,7 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
     gap_prof_begin(ST_FINALIZE, st);
     gap_count_launch();
     k_tc_finalize<<<(nrows + 3) / 4, 128, 0, st>>>(rows, nrows, sc.eps_part, sc.wsum_part, n_part, sc.Gs, op2.ksplit,
-                                                     D16, eps, wsum, g);
+                                                     D16, eps, wsum, split ? g : nullptr);
     GAP_TRY_CUDA(cudaGetLastError());
     gap_prof_end(ST_FINALIZE, st);
     return GAP_OK;
@@ -623,7 +628,9 @@ gap_status gap_contract_tc_groups(const float *phat, int D, int D16, const int *
         op2[q] = TcOperands{sc[q].W_hi, sc[q].W_lo, gp.BT_hi, gp.BT_lo, nrows[q], D16, gp.M_pad, gp.M_pad, gp.M_pad,
                             nsplit, three ? sc[q].W_mid : nullptr, three ? gp.BT_mid : nullptr};
         op2[q].ksplit = gap_contract_parts(nrows, mpad.data(), n, D16, nsplit, q);
-        ep2[q].C = sc[q].Gs;
+        const bool split = op2[q].ksplit > 1;
+        ep2[q].C = split ? sc[q].Gs : g;
+        ep2[q].row_map = split ? nullptr : rows[q];
         ep2[q].ldc = D16;
     }
     gap_prof_end(ST_SPLIT, st);
@@ -640,7 +647,8 @@ gap_status gap_contract_tc_groups(const float *phat, int D, int D16, const int *
         if (nrows[q] <= 0 || gps[q].M <= 0) continue;
         gap_count_launch();
         k_tc_finalize<<<(nrows[q] + 3) / 4, 128, 0, st>>>(rows[q], nrows[q], sc[q].eps_part, sc[q].wsum_part,
-                                                          ep1[q].n_part, sc[q].Gs, op2[q].ksplit, D16, eps, wsum, g);
+                                                          ep1[q].n_part, sc[q].Gs, op2[q].ksplit, D16, eps, wsum,
+                                                          op2[q].ksplit > 1 ? g : nullptr);
         GAP_TRY_CUDA(cudaGetLastError());
     }
     gap_prof_end(ST_FINALIZE, st);

@@ -22,7 +22,7 @@ struct TcScratch {
     float *t_row;                // [rows]
     __nv_bfloat16 *W_hi, *W_lo;  // [rows][M_pad]
     float *eps_part, *wsum_part; // [rows][2 * M_pad / column tile]
-    float *Gs;                   // [parts of K][rows][D16] (gap_contract_parts)
+    float *Gs;                   // [parts of K][rows][D16] (gap_contract_parts), used when parts > 1
     __nv_bfloat16 *A_mid, *W_mid;  // middle planes (three-plane split)
 };
 
