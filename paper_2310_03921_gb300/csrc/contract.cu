@@ -371,12 +371,16 @@ __global__ void k_split_rows(const float *__restrict__ phat, int D, int ld, cons
 }
 
 // eps, wsum and g of the atoms of one GP from the tensor-core partials.
-// One warp per row: the column-tile partials of eps and sum_m W summed in
+// LANES lanes per row: the column-tile partials of eps and sum_m W summed in
 // FP64 (lanes over partials, then a fixed shuffle tree), and, where the
 // gradient product ran in parts of K (g not NULL), their sum in order to the
 // row's atom; else the product has written g itself (copying every row here
-// made a call of 512 four-species boxes 3843 us, 3749 now).  Four rows per
-// block.
+// made a call of 512 four-species boxes 3843 us, 3749 then).  The FP64 pipe
+// bounds the sums (two instructions per partial and per shuffle, ~19 cycles
+// each per SM): eight lanes per row halve them; a whole warp per row where a
+// few rows have g to copy.  32768 rows x 32 partials: 35 us with a warp per
+// row, 15 us with eight lanes.
+template <int LANES>
 __global__ void __launch_bounds__(128) k_tc_finalize(const int *__restrict__ rows, int nrows,
                                                      const float *__restrict__ eps_part,
                                                      const float *__restrict__ wsum_part, int n_part,
@@ -384,28 +388,43 @@ __global__ void __launch_bounds__(128) k_tc_finalize(const int *__restrict__ row
                                                      double *__restrict__ eps,
                                                      float *__restrict__ wsum, float *__restrict__ g)
 {
-    const int r = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (r >= nrows) return;
-    const int atom = rows[r];
+    const int r = blockIdx.x * (128 / LANES) + threadIdx.x / LANES, lane = threadIdx.x % LANES;
+    const bool in = r < nrows;
     double e = 0.0, w = 0.0;
-    for (int t = lane; t < n_part; t += 32) {
+    for (int t = in ? lane : n_part; t < n_part; t += LANES) {
         e += eps_part[(size_t)r * n_part + t];
         w += wsum_part[(size_t)r * n_part + t];
     }
-    for (int o = 16; o; o >>= 1) {
+#pragma unroll
+    for (int o = LANES / 2; o; o >>= 1) {
         e += __shfl_xor_sync(0xffffffffu, e, o);
         w += __shfl_xor_sync(0xffffffffu, w, o);
     }
+    if (!in) return;
+    const int atom = rows[r];
     if (lane == 0) {
         eps[atom] = e;
         wsum[atom] = (float)w;
     }
     if (g)
-        for (int d = lane; d < D16; d += 32) {
+        for (int d = lane; d < D16; d += LANES) {
             float v = Gs[(size_t)r * D16 + d];
             for (int p = 1; p < parts; ++p) v += Gs[((size_t)p * nrows + r) * D16 + d];
             g[(size_t)atom * D16 + d] = v;
         }
+}
+
+gap_status tc_finalize(const int *rows, int nrows, const TcScratch &sc, int n_part, int parts, int D16, double *eps,
+                       float *wsum, float *g, cudaStream_t st)
+{
+    gap_count_launch();
+    if (g && parts > 1)
+        k_tc_finalize<32><<<(nrows + 3) / 4, 128, 0, st>>>(rows, nrows, sc.eps_part, sc.wsum_part, n_part, sc.Gs, parts,
+                                                           D16, eps, wsum, g);
+    else
+        k_tc_finalize<8><<<(nrows + 15) / 16, 128, 0, st>>>(rows, nrows, sc.eps_part, sc.wsum_part, n_part, nullptr, 1,
+                                                            D16, eps, wsum, nullptr);
+    return gap_cuda_status(cudaGetLastError(), "k_tc_finalize");
 }
 
 }  // namespace
@@ -580,10 +599,7 @@ gap_status gap_contract_tc(const float *phat, int D, int D16, const int *rows, i
         gap_prof_end(ST_GEMM_G, st);
     }
     gap_prof_begin(ST_FINALIZE, st);
-    gap_count_launch();
-    k_tc_finalize<<<(nrows + 3) / 4, 128, 0, st>>>(rows, nrows, sc.eps_part, sc.wsum_part, n_part, sc.Gs, op2.ksplit,
-                                                     D16, eps, wsum, split ? g : nullptr);
-    GAP_TRY_CUDA(cudaGetLastError());
+    GAP_TRY(tc_finalize(rows, nrows, sc, n_part, op2.ksplit, D16, eps, wsum, g, st));
     gap_prof_end(ST_FINALIZE, st);
     return GAP_OK;
 }
@@ -645,11 +661,7 @@ gap_status gap_contract_tc_groups(const float *phat, int D, int D16, const int *
     gap_prof_begin(ST_FINALIZE, st);
     for (int q = 0; q < n; ++q) {
         if (nrows[q] <= 0 || gps[q].M <= 0) continue;
-        gap_count_launch();
-        k_tc_finalize<<<(nrows[q] + 3) / 4, 128, 0, st>>>(rows[q], nrows[q], sc[q].eps_part, sc[q].wsum_part,
-                                                          ep1[q].n_part, sc[q].Gs, op2[q].ksplit, D16, eps, wsum,
-                                                          op2[q].ksplit > 1 ? g : nullptr);
-        GAP_TRY_CUDA(cudaGetLastError());
+        GAP_TRY(tc_finalize(rows[q], nrows[q], sc[q], ep1[q].n_part, op2[q].ksplit, D16, eps, wsum, g, st));
     }
     gap_prof_end(ST_FINALIZE, st);
     return GAP_OK;
