@@ -134,15 +134,13 @@ CRT_MODULI = [256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 1
 
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one K_NM
-# force-row GEMM launch (k_tc_gemm, TMEM-resident K_NM epilogue), from one ncu
-# capture on the first 20 cells of the fit workload (194,934 Jacobian rows):
+# force-row GEMM launch (k_knm_gemm), from one ncu capture on the first 20
+# cells of the fit workload (194,934 Jacobian rows):
 #   ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none \
-#       --kernel-name-base demangled -k "regex:\(int\)192" -s 1 -c 1 \
-#       python -m paper_2310_03921_gb300.profile_run --fit 20 --steps 1
-# (the 128 x 192 tile with twelve epilogue warps that the autotuner picks)
+#       -k "regex:k_knm_gemm" -c 1 python -m paper_2310_03921_gb300.profile_run --fit 20 --steps 1
 # The operand rows, the W' rows and the K_NM rows all grow with the Jacobian
 # rows, so a full launch is scaled by 3 (N + P).
-KNM_TRAFFIC_READ, KNM_TRAFFIC_WRITE, KNM_TRAFFIC_JROWS = 223092736, 82601984, 194934
+KNM_TRAFFIC_READ, KNM_TRAFFIC_WRITE, KNM_TRAFFIC_JROWS = 240358912, 86377728, 194934
 
 
 def crt_moduli_counts(m: int, n_ext: int):
@@ -200,7 +198,8 @@ def alu_rooflines(per_launch, n_atoms, n_pairs, n_max, l_max, D, M, fp32_peak, f
                  rows written, 3 (N + P) rows x 2 BF16 planes x D16 x 2 B.
       solve_block the elimination on [A | I] of one diagonal block of the
                  factorisation (mean over the blocks of an M x M Gram
-                 matrix), on ONE SM: the peak is the chip's FP64 rate / SMs."""
+                 matrix), against ONE SM's rate (the chip's FP64 rate / SMs);
+                 a block runs on a cluster of eight, one panel at a time."""
     L1 = l_max + 1
     lam = L1 * L1
     npair = n_max * (n_max + 1) // 2
@@ -211,7 +210,7 @@ def alu_rooflines(per_launch, n_atoms, n_pairs, n_max, l_max, D, M, fp32_peak, f
                       24 * P + N * (4 * n_max * lam + 4 * D + 4), fp32_peak, "FP32"),
         "pairforce": ("k_pairforce", P * (4 * n_max * lam + 12 * n_max * L1 + 8 * lam),
                       36 * P + N * 4 * n_max * lam, fp32_peak, "FP32"),
-        "knm_jacobian": ("k_jacobian_rows", P * (8 * n_max * lam + 42 * D),
+        "knm_jacobian": ("k_jacobian_triples", P * (8 * n_max * lam + 42 * D),
                          3 * (N + P) * 2 * D16 * 2, fp32_peak, "FP32"),
     }
     out = {}
@@ -233,7 +232,7 @@ def alu_rooflines(per_launch, n_atoms, n_pairs, n_max, l_max, D, M, fp32_peak, f
         out["solve_block"] = {"kernel": "k_chol_inv_block", "bound": "alu", "ms_per_launch": per_launch["solve_block"],
                               "flops": fl, "blocks_per_factorisation": len(blocks), "factorisations": n_fact,
                               "achieved_tflops": a, "peak_tflops": sm_peak,
-                              "peak_source": f"FP64 FMA probe / {n_sm} SMs (one CTA)", "frac": a / sm_peak,
+                              "peak_source": f"FP64 FMA probe / {n_sm} SMs (one SM; a block runs on eight)", "frac": a / sm_peak,
                               "frac_of_chip": a / fp64_peak}
     return out
 
@@ -388,7 +387,7 @@ def run_ours(args, rank, world, local_rank):
     solve_flops = (T1 * m_ls * n_ext * (n_ext + 1)
                    + 2 * T2 * (n_ext ** 2 * (n_ext + 1) + n_ext * (n_ext + 1) * (n_ext + 2) / 3.0))
     tensor = {
-        "knm_gemm": ("k_tc_gemm (K_NM force rows, split BF16x3)",
+        "knm_gemm": ("k_knm_gemm (K_NM force rows, split BF16x3)",
                      2.0 * 3.0 * (n_atoms + n_pairs) * D * M,
                      "2 * 3 (N + P) * D * M: one D x M sweep per Jacobian row (3 own rows per atom, 3 per pair); "
                      "the energy rows are a separate launch; the split scheme issues 3x this on the tensor cores"),
