@@ -96,6 +96,14 @@ gap_status gap_test_fp64_recip(int n, const double *x, double *out);
  * contractions); other calls keep the tuned choice.  v < 0 restores the
  * autotuner.  For parity tests of every variant; process-wide. */
 gap_status gap_test_tc_force_variant(int v);
+/* The row lists of the GPs, as a prediction builds them: species host [n],
+ * GPs for species 0 .. n_gp - 1 (1 <= n_gp <= 8); one != 0 is the form of a
+ * one-species model, in which every atom is GP 0's.  Outputs (host): rows
+ * [n_gp][n], the atoms of each GP in index order (entries past the GP's
+ * count are -1), counts [n_gp], gp_of_atom [n] (-1: none) and rank [n], an
+ * atom's place among its GP's rows (-1: none).  Synchronous. */
+gap_status gap_test_gp_rows(int n, int n_gp, int one, const int *species, int *rows, int *counts, int *gp_of_atom,
+                            int *rank);
 
 #ifdef __cplusplus
 }

@@ -1,4 +1,5 @@
 // Host implementation of the C ABI declared in include/gap.h.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -2264,6 +2265,40 @@ extern "C" gap_status gap_test_bf16_gemm(int nsplit, int rows, int cols, int K, 
     if (st == GAP_OK)
         st = gap_cuda_status(cudaMemcpy(C, dc.p, sizeof(float) * (size_t)rows * cols, cudaMemcpyDeviceToHost), "copy");
     cleanup();
+    return st;
+    GAP_API_END
+}
+
+extern "C" gap_status gap_test_gp_rows(int n, int n_gp, int one, const int *species, int *rows, int *counts,
+                                       int *gp_of_atom, int *rank)
+{
+    GAP_API_BEGIN
+    if (n < 0 || n_gp < 1 || n_gp > 8 || (n > 0 && (!species || !rows || !gp_of_atom || !rank)) || !counts) {
+        gap_set_error("bad arguments");
+        return GAP_EINVAL;
+    }
+    const size_t sn = (size_t)n;
+    DBuf dspec, dtmp, dout;  // rows, gp_of_atom, rank, counts
+    const size_t n_out = sn * n_gp + 2 * sn + n_gp;
+    gap_status st = dspec.ensure(sizeof(int) * sn);
+    if (st == GAP_OK) st = dtmp.ensure(sizeof(int) * gap_gp_rows_tmp_ints(n, n_gp));
+    if (st == GAP_OK) st = dout.ensure(sizeof(int) * n_out);
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemset(dout.p, 0xff, sizeof(int) * n_out), "cudaMemset");
+    if (st == GAP_OK && n)
+        st = gap_cuda_status(cudaMemcpy(dspec.p, species, sizeof(int) * sn, cudaMemcpyHostToDevice), "copy");
+    int *d = dout.as<int>(), *d_gp = d + sn * n_gp, *d_rank = d_gp + n, *d_counts = d_rank + n;
+    if (st == GAP_OK) st = gap_gp_rows(n, n_gp, one != 0, dspec.as<int>(), dtmp.as<int>(), d, d_counts, d_gp, d_rank, 0);
+    std::vector<int> out(n_out);
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemcpy(out.data(), d, sizeof(int) * n_out, cudaMemcpyDeviceToHost), "copy");
+    if (st == GAP_OK) {
+        std::copy_n(out.data(), sn * n_gp, rows);
+        std::copy_n(out.data() + sn * n_gp, n, gp_of_atom);
+        std::copy_n(out.data() + sn * n_gp + n, n, rank);
+        std::copy_n(out.data() + sn * n_gp + 2 * sn, n_gp, counts);
+    }
+    dspec.release();
+    dtmp.release();
+    dout.release();
     return st;
     GAP_API_END
 }

@@ -280,7 +280,7 @@ k_gp_rows(int n, int n_gp, bool one, const int *__restrict__ species, const int 
 {
     __shared__ int wcnt[kMaxGPs][33], base[kMaxGPs];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (threadIdx.x < kMaxGPs) base[threadIdx.x] = 0;
+    // base[s]: GP s's rows before this block; one writer per entry before the barrier
     if (block_counts) {
         if (w < n_gp) {
             int sum = 0, all = 0;
@@ -299,6 +299,8 @@ k_gp_rows(int n, int n_gp, bool one, const int *__restrict__ species, const int 
                 if (blockIdx.x == 0) counts[w] = all;
             }
         }
+    } else if (threadIdx.x < kMaxGPs) {
+        base[threadIdx.x] = 0;
     }
     __syncthreads();
     const int t0 = block_counts ? blockIdx.x : 0, t1 = block_counts ? blockIdx.x + 1 : (n + kRowsTile - 1) / kRowsTile;

@@ -110,6 +110,7 @@ def lib():
             "gap_test_fail_alloc": [C.c_long],
             "gap_test_tc_force_variant": [C.c_int],
             "gap_test_fp64_recip": [C.c_int, _dp, _dp],
+            "gap_test_gp_rows": [C.c_int, C.c_int, C.c_int, _ip, _ip, _ip, _ip, _ip],
             "gap_model_set_alpha": [_vp, _vp, C.c_int, _vp],
             "gap_model_set_posterior": [_vp, C.c_long, _vp, _vp, C.c_double, C.c_int, _vp],
             "gap_predict_variance": [_vp, C.POINTER(BatchStruct), _vp, _vp],
@@ -659,6 +660,16 @@ def test_fp64_recip(x: np.ndarray) -> np.ndarray:
     out = np.zeros((x.size, 4))
     _check(lib().gap_test_fp64_recip(x.size, x.ctypes.data_as(_dp), out.ctypes.data_as(_dp)))
     return out
+
+
+def test_gp_rows(species: np.ndarray, n_gp: int, one: bool = False):
+    """(rows [n_gp][n], counts [n_gp], gp_of_atom [n], rank [n]) of the GPs' row lists (host int32)."""
+    z = np.ascontiguousarray(species, dtype=np.int32)
+    n = z.size
+    rows, counts = np.zeros((n_gp, n), np.int32), np.zeros(n_gp, np.int32)
+    gp, rank = np.zeros(n, np.int32), np.zeros(n, np.int32)
+    _check(lib().gap_test_gp_rows(n, n_gp, 1 if one else 0, *(a.ctypes.data_as(_ip) for a in (z, rows, counts, gp, rank))))
+    return rows, counts, gp, rank
 
 
 def exported_symbols() -> list[str]:
