@@ -74,6 +74,12 @@ gap_status gap_test_fma_peak(int fp64, double *tflops);
  * 4: epilogue).  Returns GAP_ETIMEOUT when a wait expired (the expected
  * outcome), GAP_OK if none did.  The device stays usable.  Synchronous. */
 gap_status gap_test_tc_timeout(unsigned long long wait_ns, int *code);
+/* The same in the middle of a product: 1024 x 1024 x 2048, of whose 32 blocks
+ * of K each CTA copies and multiplies the first `blocks` (0 ..) before its
+ * waits run out.  The CTA waits for what it has issued, frees its TMEM and
+ * exits.  Returns GAP_ETIMEOUT and the error bits, GAP_OK from 32 blocks on.
+ * The device stays usable.  Synchronous. */
+gap_status gap_test_tc_expiry(int blocks, unsigned long long wait_ns, int *code);
 /* Makes device allocations of the library's workspaces fail: after `after`
  * more successful allocations (0: the next one), every workspace allocation
  * returns cudaErrorMemoryAllocation without calling cudaMalloc, so the entry

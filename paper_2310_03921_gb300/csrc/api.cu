@@ -2303,18 +2303,15 @@ extern "C" gap_status gap_test_gp_rows(int n, int n_gp, int one, const int *spec
     GAP_API_END
 }
 
-// The bounded-wait path of the tcgen05 GEMM: one 128 x 256 x 64 tile whose
-// producer issues no copies (so no MMA is issued either) and whose waits
-// give up after wait_ns; every role's wait runs out with nothing in flight,
-// the CTA still frees its TMEM, and the call reports GAP_ETIMEOUT.
-extern "C" gap_status gap_test_tc_timeout(unsigned long long wait_ns, int *code)
+// The bounded-wait path of the tcgen05 GEMM on zero operands: every wait gives
+// up after wait_ns, with a producer that stops issuing copies after `blocks`
+// blocks of K.
+static gap_status tc_expiry(int rows, int cols, int K, int blocks, unsigned long long wait_ns, int *code)
 {
-    GAP_API_BEGIN
-    if (wait_ns == 0 || wait_ns > 1000000000ull || !code) {
-        gap_set_error("wait_ns must be in 1..1e9 and code non-NULL");
+    if (wait_ns == 0 || wait_ns > 1000000000ull || !code || blocks < 0) {
+        gap_set_error("wait_ns must be in 1..1e9, blocks >= 0 and code non-NULL");
         return GAP_EINVAL;
     }
-    const int rows = 128, cols = 256, K = 64;
     DBuf da, db, dc, derr;
     auto cleanup = [&]() { da.release(); db.release(); dc.release(); derr.release(); };
     gap_status st = da.ensure(2 * (size_t)rows * K);
@@ -2331,7 +2328,7 @@ extern "C" gap_status gap_test_tc_timeout(unsigned long long wait_ns, int *code)
         ep.C = dc.as<float>();
         ep.ldc = cols;
         ep.wait_ns = wait_ns;
-        ep.test_stall = 1;
+        ep.test_stall = blocks + 1;
         st = gap_tc_gemm(op, ep, EPI_STORE, derr.as<int>(), 0);
     }
     if (st == GAP_OK) st = gap_cuda_status(cudaDeviceSynchronize(), "tensor-core GEMM");
@@ -2344,6 +2341,19 @@ extern "C" gap_status gap_test_tc_timeout(unsigned long long wait_ns, int *code)
     }
     cleanup();
     return st;
+}
+
+extern "C" gap_status gap_test_tc_timeout(unsigned long long wait_ns, int *code)
+{
+    GAP_API_BEGIN
+    return tc_expiry(128, 256, 64, 0, wait_ns, code);
+    GAP_API_END
+}
+
+extern "C" gap_status gap_test_tc_expiry(int blocks, unsigned long long wait_ns, int *code)
+{
+    GAP_API_BEGIN
+    return tc_expiry(1024, 1024, 2048, blocks, wait_ns, code);
     GAP_API_END
 }
 

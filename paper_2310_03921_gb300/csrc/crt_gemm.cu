@@ -251,7 +251,7 @@ constexpr uint32_t A_BYTES = BM * BK * 2, B_BYTES = BN * BK * 2, STAGE_BYTES = A
 
 struct CrtTail {
     uint64_t full[STAGES], empty[STAGES];
-    uint64_t acc_full[2], acc_empty[2];
+    uint64_t acc_full[2], acc_empty[2], mma_done;
     uint32_t tmem_base;
     int abort;
 };
@@ -328,6 +328,7 @@ k_crt_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUten
             mbar_init(&tail->acc_full[b], 1);
             mbar_init(&tail->acc_empty[b], kThreads - 64);
         }
+        mbar_init(&tail->mma_done, 1);
         tail->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -369,6 +370,7 @@ k_crt_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUten
                 const int s = kb % STAGES, r = kb / STAGES;
                 if (!mbar_wait(&tail->empty[s], r & 1, abort_flag)) break;
             }
+            wait_copies(tail->full, g, STAGES);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -407,6 +409,7 @@ k_crt_gemm(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUten
                 if (!ok) break;
                 gc += c.nchunks;
             }
+            wait_mmas(&tail->mma_done);
         }
     } else {
         const int quad = warp & 3, half = (warp - 2) >> 2;

@@ -71,7 +71,7 @@ struct KnmParams {
 constexpr int kMaxRanges = 2048;
 
 struct KnmTail {
-    uint64_t full[4], empty[4], acc_full[2], acc_empty[2];
+    uint64_t full[4], empty[4], acc_full[2], acc_empty[2], mma_done;
     uint32_t tmem_base;
     int abort;
 };
@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
             mbar_init(&tail->acc_full[b], 1);
             mbar_init(&tail->acc_empty[b], 4 * NG);  // one arrival per epilogue warp
         }
+        mbar_init(&tail->mma_done, 1);
         tail->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -188,6 +189,7 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
             // drain: wait until the consumer has released every slot filled
             for (int k = it - STAGES < 0 ? 0 : it - STAGES; k < it && !*abort_flag; ++k)
                 if (!mbar_wait(&tail->empty[k % STAGES], (k / STAGES) & 1, abort_flag)) break;
+            wait_copies(tail->full, it, STAGES);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -234,6 +236,7 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
                     }
                 }
             }
+            wait_mmas(&tail->mma_done);
         }
     } else {
         const int quad = warp & 3, grp = (warp - 2) >> 2;  // TMEM lane quadrant, column group

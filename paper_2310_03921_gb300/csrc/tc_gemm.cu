@@ -60,6 +60,7 @@ struct SharedTail {
     uint64_t empty[4];
     uint64_t acc_full[2];    // MMA -> epilogue, per TMEM accumulator buffer
     uint64_t acc_empty[2];   // epilogue -> MMA (every epilogue warp arrives)
+    uint64_t mma_done;       // the issuer's last MMA
     uint32_t tmem_base;
     int abort;
 };
@@ -164,6 +165,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
             mbar_init(&tail->acc_full[b], 1);
             mbar_init(&tail->acc_empty[b], EW);  // one arrival per epilogue warp
         }
+        mbar_init(&tail->mma_done, 1);
         tail->abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -179,7 +181,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
     const uint32_t tmem = tail->tmem_base;
     volatile int *abort_flag = &tail->abort;
     const unsigned long long wlim = P.p[0].ep.wait_ns ? P.p[0].ep.wait_ns : kWaitNs;
-    const bool stall = P.p[0].ep.test_stall != 0;
+    const int stall = P.p[0].ep.test_stall;  // tests: copies of the first stall - 1 blocks only
 
     if (warp == 0) {
         if (lane == 0) {
@@ -197,7 +199,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                         atomicOr(err, 1);
                         break;
                     }
-                    if (stall) continue;
+                    if (stall && g >= stall - 1) continue;
                     unsigned char *st = smem + s * STAGE_BYTES;
                     mbar_expect_tx(&tail->full[s], STAGE_BYTES);
                     tma_load_2d(st, &pr.mA[0], &tail->full[s], kb * BK, row0);
@@ -214,6 +216,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                 int s = kb % STAGES, r = kb / STAGES;
                 if (!mbar_wait(&tail->empty[s], r & 1, abort_flag, wlim)) break;
             }
+            wait_copies(tail->full, stall && g > stall - 1 ? stall - 1 : g, STAGES);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -267,6 +270,7 @@ k_tc_gemm(const __grid_constant__ TcProblems<G> P, int *err)
                     if ((kb % KC) == KC - 1 || kb == kblocks - 1) umma_commit(&tail->acc_full[buf]);
                 }
             }
+            wait_mmas(&tail->mma_done);
         }
     } else {
         // epilogue warps
@@ -757,7 +761,7 @@ int gap_tc_plan(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, c
         return kVariants2[fv].bn;
     }
     if (op.nsplit == 3 || op.rows <= 0 || op.cols <= 0) return 128;
-    if (ep.test_stall) return kVariants2[0].bn;  // the timeout test: nothing to time
+    if (ep.wait_ns) return kVariants2[0].bn;  // the timeout tests: nothing to time
     int dev = 0;
     cudaGetDevice(&dev);
     const TuneKey key{dev, epi, op.nsplit, op.K, op.cols, rows_log2(op.rows)};

@@ -37,8 +37,8 @@ struct TcEpilogue {
     int ldwp;
     // Bounded waits: limit of each mbarrier wait in ns (0: the default 2 s).
     unsigned long long wait_ns;
-    // Test of the timeout path: the producer issues no copies (so no MMA is
-    // ever issued either); every role's wait runs out with nothing in flight.
+    // Tests of the timeout path: k > 0 lets a CTA's producer issue the copies
+    // of its first k - 1 blocks of K only, so that the waits after them run out.
     int test_stall;
 };
 

@@ -46,7 +46,7 @@ __device__ __forceinline__ bool mbar_try(uint64_t *bar, uint32_t parity)
 }
 
 // Bounded wait; false if the time limit (limit_ns of %globaltimer) passed or
-// another role aborted.
+// another role aborted (abort_flag NULL: the time limit alone ends it).
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag,
                                           unsigned long long limit_ns = kWaitNs)
 {
@@ -55,7 +55,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
     for (unsigned it = 1;; ++it) {
         if (mbar_try(bar, parity)) return true;
         if ((it & 63) == 0) {
-            if (*abort_flag) return false;
+            if (abort_flag && *abort_flag) return false;
             if (global_ns() - t0 > limit_ns) return false;
         }
     }
@@ -127,6 +127,23 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
+}
+
+// The last steps of a producer and of an MMA issuer, also after a wait of
+// theirs or another role's gave up: a block's shared memory and TMEM are given
+// back only when nothing in flight touches them.  wait_copies: the loads into
+// a ring of `stages` slots, `issued` so far (load k into slot k % stages).
+__device__ __forceinline__ void wait_copies(uint64_t *full, int issued, int stages)
+{
+    for (int k = issued > stages ? issued - stages : 0; k < issued; ++k)
+        mbar_wait(&full[k % stages], (k / stages) & 1, nullptr);
+}
+// wait_mmas: every MMA this thread has issued (done: a barrier of one arrival,
+// used for nothing else).
+__device__ __forceinline__ void wait_mmas(uint64_t *done)
+{
+    umma_commit(done);
+    mbar_wait(done, 0, nullptr);
 }
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

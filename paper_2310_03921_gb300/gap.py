@@ -107,6 +107,7 @@ def lib():
             "gap_test_congruence": [C.c_long, C.c_int, _dp, _dp, _dp, _dp, _dp, _dp, _dp],
             "gap_test_fma_peak": [C.c_int, _dp],
             "gap_test_tc_timeout": [C.c_ulonglong, _ip],
+            "gap_test_tc_expiry": [C.c_int, C.c_ulonglong, _ip],
             "gap_test_fail_alloc": [C.c_long],
             "gap_test_tc_force_variant": [C.c_int],
             "gap_test_fp64_recip": [C.c_int, _dp, _dp],
@@ -641,6 +642,13 @@ def test_tc_timeout(wait_ns: int = 20000):
     """(status, error bits) of the tensor-core GEMM's bounded-wait test."""
     code = C.c_int()
     st = lib().gap_test_tc_timeout(int(wait_ns), C.byref(code))
+    return st, code.value
+
+
+def test_tc_expiry(blocks: int, wait_ns: int = 1000000):
+    """(status, error bits) of a tensor-core GEMM whose waits run out after `blocks` blocks of K."""
+    code = C.c_int()
+    st = lib().gap_test_tc_expiry(int(blocks), int(wait_ns), C.byref(code))
     return st, code.value
 
 

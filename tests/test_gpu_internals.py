@@ -37,3 +37,15 @@ def test_rows_of_a_one_species_model(G):
         rows, counts, gp, rank = G.test_gp_rows(np.full(n, 5), 1, one=True)
         assert counts[0] == n and np.all(gp == 0)
         assert np.array_equal(rows[0], np.arange(n)) and np.array_equal(rank, np.arange(n))
+
+
+@pytest.mark.parametrize("blocks", [0, 1, 2, 3, 4, 5, 31, 32])
+def test_wait_expiry_in_the_middle_of_a_product(G, blocks):
+    """A CTA whose waits run out after some blocks of K waits for the copies and MMAs it has issued and ends in an error
+    status; the product after it is exact."""
+    rng = np.random.default_rng(3)
+    A = rng.integers(-8, 9, size=(500, 256)).astype(np.float32)
+    B = rng.integers(-8, 9, size=(700, 256)).astype(np.float32)
+    st, code = G.test_tc_expiry(blocks)
+    assert (st, code) == (0, 0) if blocks == 32 else (st == -4 and code), (st, code)
+    assert np.array_equal(G.test_bf16_gemm(A, B), A @ B.T)
