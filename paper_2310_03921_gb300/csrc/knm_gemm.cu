@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
                 // the next tile: its W' into flight, its data to shared memory; the one after: its data
                 float wn[kGT];
                 load_w(wn);
+                __syncwarp();  // every lane has read the tile before, whose place this is
                 if (lane < kGT) wmeta[((t + 1) & 1) * kGT + lane] = nm;
                 const int next_dest = nd;
                 load_meta(q + 2 * kGT);
