@@ -110,6 +110,13 @@ gap_status gap_test_tc_force_variant(int v);
  * atom's place among its GP's rows (-1: none).  Synchronous. */
 gap_status gap_test_gp_rows(int n, int n_gp, int one, const int *species, int *rows, int *counts, int *gp_of_atom,
                             int *rank);
+/* Forces and atomic virials from FP32 pair derivatives, as a reduced-precision
+ * prediction sums them: atom j's pairs are offsets[j] .. offsets[j + 1] - 1
+ * (host [n + 1], offsets[0] = 0), rev [P] the reverse pair of each, vec [P][4]
+ * (x, y, z, r) and fpair [P][3]; F_j = sum_p (f_p - f_rev(p)), W_j = -sum_p f_p
+ * (x) r_p.  forces host [n][3], virial host [n][9], FP64.  Synchronous. */
+gap_status gap_test_gather(int n, const int *offsets, const int *rev, const float *vec, const float *fpair,
+                           double *forces, double *virial);
 
 #ifdef __cplusplus
 }

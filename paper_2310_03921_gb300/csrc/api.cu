@@ -2303,6 +2303,46 @@ extern "C" gap_status gap_test_gp_rows(int n, int n_gp, int one, const int *spec
     GAP_API_END
 }
 
+extern "C" gap_status gap_test_gather(int n, const int *offsets, const int *rev, const float *vec, const float *fpair,
+                                      double *forces, double *virial)
+{
+    GAP_API_BEGIN
+    if (n < 1 || !offsets || !rev || !vec || !fpair || !forces || !virial || offsets[0] != 0) {
+        gap_set_error("bad arguments");
+        return GAP_EINVAL;
+    }
+    const int P = offsets[n];
+    bool ok = P > 0;
+    for (int j = 0; j < n; ++j) ok = ok && offsets[j] <= offsets[j + 1] && offsets[j + 1] <= P;
+    for (int p = 0; p < P && ok; ++p) ok = rev[p] >= 0 && rev[p] < P;
+    if (!ok) {
+        gap_set_error("offsets or reverse pairs out of range");
+        return GAP_EINVAL;
+    }
+    DBuf doff, drev, dvec, df, dF, dV;
+    gap_status st = upload(doff, std::vector<int>(offsets, offsets + n + 1));
+    if (st == GAP_OK) st = upload(drev, std::vector<int>(rev, rev + P));
+    if (st == GAP_OK) st = upload(dvec, std::vector<float>(vec, vec + 4 * (size_t)P));
+    if (st == GAP_OK) st = upload(df, std::vector<float>(fpair, fpair + 3 * (size_t)P));
+    if (st == GAP_OK) st = dF.ensure(sizeof(double) * 3 * (size_t)n);
+    if (st == GAP_OK) st = dV.ensure(sizeof(double) * 9 * (size_t)n);
+    if (st == GAP_OK) {
+        PairList pl{};
+        pl.n_pairs = P;
+        pl.offsets = doff.as<int>();
+        pl.rev = drev.as<int>();
+        pl.vec32 = dvec.as<float4>();
+        st = gap_gather<float>(n, pl, df.as<float>(), nullptr, dF.as<double>(), dV.as<double>(), 0);
+    }
+    if (st == GAP_OK)
+        st = gap_cuda_status(cudaMemcpy(forces, dF.p, sizeof(double) * 3 * (size_t)n, cudaMemcpyDeviceToHost), "copy");
+    if (st == GAP_OK)
+        st = gap_cuda_status(cudaMemcpy(virial, dV.p, sizeof(double) * 9 * (size_t)n, cudaMemcpyDeviceToHost), "copy");
+    for (DBuf *b : {&doff, &drev, &dvec, &df, &dF, &dV}) b->release();
+    return st;
+    GAP_API_END
+}
+
 // The bounded-wait path of the tcgen05 GEMM on zero operands: every wait gives
 // up after wait_ns, with a producer that stops issuing copies after `blocks`
 // blocks of K.

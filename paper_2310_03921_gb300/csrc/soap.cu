@@ -601,61 +601,90 @@ k_twobody(int n_atoms, const int *__restrict__ offsets, const D4 *__restrict__ v
 
 // ------------------------------------------------------ forces and virials
 // Running sums of the pair terms.  FP64 terms are summed in FP64; FP32 terms
-// (and the exact products of two of them) in a compensated FP32 pair (two-sum
-// and two-product, Ogita, Rump and Oishi 2005: ~48 bits), because one FP64
+// (and the exact products of two of them) in three FP32 words: two-sum and
+// two-product (Ogita, Rump and Oishi 2005) pass every rounding error on to the
+// next word, so the sum is good to more than FP64's 53 bits.  One FP64
 // instruction holds GB300's FP64 pipe for ~64 cycles per warp where the
-// seven FP32 ones of a two-sum take seven.
+// thirteen FP32 ones of a term take thirteen.  Every operation is rounded by
+// itself: contracted into a multiply-add, s + p would hold p's rounding error
+// already and sub_product count it twice.  (Products below 2^-102 keep an
+// absolute error of 2^-149.)
 template <typename T> struct PairSum;
 template <> struct PairSum<double> {
     double s = 0.0;
     __device__ __forceinline__ void add(double x) { s += x; }
     __device__ __forceinline__ void sub_product(double a, double b) { s -= a * b; }
-    __device__ __forceinline__ void reduce() { s = group_sum(s); }
+    // adds what the lane at distance o sends
+    __device__ __forceinline__ void receive(const PairSum &sent, int o) { s += __shfl_xor_sync(0xffffffffu, sent.s, o); }
     __device__ __forceinline__ double value() const { return s; }
 };
 template <> struct PairSum<float> {
-    float s = 0.f, c = 0.f;
+    float s = 0.f, c = 0.f, e = 0.f;
+    // a + x rounded; the error to r
+    static __device__ __forceinline__ float two_sum(float a, float x, float &r)
+    {
+        const float t = __fadd_rn(a, x), b = __fsub_rn(t, a);
+        r = __fadd_rn(__fsub_rn(a, __fsub_rn(t, b)), __fsub_rn(x, b));
+        return t;
+    }
+    __device__ __forceinline__ void carry(float x)
+    {
+        float r;
+        c = two_sum(c, x, r);
+        e = __fadd_rn(e, r);
+    }
     __device__ __forceinline__ void add(float x)
     {
-        const float t = s + x, b = t - s;
-        c += (s - (t - b)) + (x - b);
-        s = t;
+        float r;
+        s = two_sum(s, x, r);
+        carry(r);
     }
     __device__ __forceinline__ void sub_product(float a, float b)
     {
-        const float p = -(a * b);
-        c -= fmaf(a, b, p);
+        const float p = -__fmul_rn(a, b);
+        carry(-__fmaf_rn(a, b, p));
         add(p);
     }
-    __device__ __forceinline__ void reduce()
+    __device__ __forceinline__ void receive(const PairSum &sent, int o)
     {
-#pragma unroll
-        for (int o = kPairLanes / 2; o > 0; o >>= 1) {
-            const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
-            add(s2);
-            c += c2;
-        }
+        const float s2 = __shfl_xor_sync(0xffffffffu, sent.s, o), c2 = __shfl_xor_sync(0xffffffffu, sent.c, o),
+                    e2 = __shfl_xor_sync(0xffffffffu, sent.e, o);
+        add(s2);
+        carry(c2);
+        e = __fadd_rn(e, e2);
     }
-    // an infinite sum leaves a NaN correction, which is dropped
-    __device__ __forceinline__ double value() const { return c - c == 0.f ? (double)s + (double)c : (double)s; }
+    __device__ __forceinline__ double value() const { return (double)s + ((double)c + (double)e); }
 };
 
-// F_j = sum_{p in pairs(j)} (f[p] - f[rev p]);  W_j = -sum_{p in pairs(j)} f[p] (x) r_p,
-// plus the two-body force and virial of the atom (fw2, see k_twobody).
-// kPairLanes lanes per atom.  A captured step of 64 atoms takes 120 us with it
-// (151 us with one thread per atom), outputs bit for bit the same.
-template <typename T>
-__global__ void __launch_bounds__(128)
-k_gather(int n_atoms, const int *__restrict__ offsets, const int *__restrict__ rev,
-         const typename V4<T>::type *__restrict__ vec, const T *__restrict__ fpair, const double *__restrict__ fw2,
-         double *__restrict__ forces, double *__restrict__ vir_atom)
+// Halves the entries of two lanes at distance o: the upper half of them goes to
+// the lane with bit o set, each lane adding the other's share of its half.
+template <typename S, int N>
+__device__ __forceinline__ void share(const S (&all)[N], S (&mine)[N / 2], int o)
 {
-    const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kPairLanes, sub = threadIdx.x % kPairLanes;
-    PairSum<T> acc[12];  // F, then W row-major
-    const int p1 = j < n_atoms ? offsets[j + 1] : 0;
-    for (int p = j < n_atoms ? offsets[j] + sub : 0; p < p1; p += kPairLanes) {
+    const bool up = (threadIdx.x & o) != 0;
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+        const S sent = up ? all[k] : all[N / 2 + k];
+        mine[k] = up ? all[N / 2 + k] : all[k];
+        mine[k].receive(sent, o);
+    }
+}
+
+// The sums of one atom's pairs p0 + sub, p0 + sub + kPairLanes, ... over its
+// eight lanes.  Of the twelve (F, then W row-major, zero unless virial) lane
+// sub gets entries first_entry(sub) and, in even lanes, the next: the lanes
+// halve the entries three times (11 additions a lane where a butterfly over
+// all of them takes 36).
+__device__ __forceinline__ int first_entry(int sub) { return 6 * (sub >> 2) + 3 * ((sub >> 1) & 1) + 2 * (sub & 1); }
+
+template <typename S, typename T, typename V>
+__device__ __forceinline__ void sum_pairs(S (&mine)[2], int p0, int p1, int sub, const int *__restrict__ rev,
+                                          const V *__restrict__ vec, const T *__restrict__ fpair, bool virial)
+{
+    S acc[12], half[6], quarter[4];
+    for (int p = p0 + sub; p < p1; p += kPairLanes) {
         const size_t q = 3 * (size_t)rev[p];
-        const typename V4<T>::type v = vec[p];
+        const V v = vec[p];
         T fp[3], fq[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
@@ -667,7 +696,7 @@ k_gather(int n_atoms, const int *__restrict__ offsets, const int *__restrict__ r
             acc[a].add(fp[a]);
             acc[a].add(-fq[a]);
         }
-        if (vir_atom) {
+        if (virial) {
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 acc[3 + 3 * a].sub_product(fp[a], v.x);
@@ -676,21 +705,55 @@ k_gather(int n_atoms, const int *__restrict__ offsets, const int *__restrict__ r
             }
         }
     }
+    static_assert(kPairLanes == 8, "three halvings");
+    share(acc, half, 4);
+    S three[3];
+    share(half, three, 2);
 #pragma unroll
-    for (int q = 0; q < 12; ++q) acc[q].reduce();
+    for (int k = 0; k < 3; ++k) quarter[k] = three[k];
+    quarter[3] = S{};
+    share(quarter, mine, 1);
+}
+
+// F_j = sum_{p in pairs(j)} (f[p] - f[rev p]);  W_j = -sum_{p in pairs(j)} f[p] (x) r_p,
+// plus the two-body force and virial of the atom (fw2, see k_twobody).
+// kPairLanes lanes per atom: latency bounds it at few atoms (a captured step of
+// 64 atoms took 151 us with a thread per atom, 120 us with eight lanes).  Three
+// words per sum instead of two, with the halved entries in place of a butterfly:
+// a step of 64 atoms 73.8 -> 74.2 us, of 32768 1284 -> 1277 us.
+template <typename T>
+__global__ void __launch_bounds__(128)
+k_gather(int n_atoms, const int *__restrict__ offsets, const int *__restrict__ rev,
+         const typename V4<T>::type *__restrict__ vec, const T *__restrict__ fpair, const double *__restrict__ fw2,
+         double *__restrict__ forces, double *__restrict__ vir_atom)
+{
+    const int j = (blockIdx.x * blockDim.x + threadIdx.x) / kPairLanes, sub = threadIdx.x % kPairLanes;
+    const int p0 = j < n_atoms ? offsets[j] : 0, p1 = j < n_atoms ? offsets[j + 1] : 0;
+    PairSum<T> mine[2];
+    sum_pairs(mine, p0, p1, sub, rev, vec, fpair, vir_atom != nullptr);
+    double v[2] = {mine[0].value(), mine[1].value()};
+    if constexpr (sizeof(T) == 4) {
+        // beyond FP32's range (or infinite, or no number): the FP64 sum
+        const bool wide[2] = {!(fabsf(mine[0].s) <= 3.402823466e38f), !(fabsf(mine[1].s) <= 3.402823466e38f)};
+        if (__any_sync(0xffffffffu, wide[0] || wide[1])) {
+            PairSum<double> sums[2];
+            sum_pairs(sums, p0, p1, sub, rev, vec, fpair, vir_atom != nullptr);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) v[h] = wide[h] ? sums[h].s : v[h];
+        }
+    }
     if (j >= n_atoms) return;
-    // lane `sub` writes entries sub and sub + 8
 #pragma unroll
-    for (int q = 0; q < 12; ++q) {
-        if (q % kPairLanes != sub) continue;
-        double v = acc[q].value();
-        // the two-body term's symmetric virial is stored xx yy zz yz xz xy
-        constexpr int kSym[12] = {0, 1, 2, 3, 8, 7, 8, 4, 6, 7, 6, 5};
-        if (fw2) v += fw2[9 * (size_t)j + kSym[q]];
+    for (int h = 0; h < 2; ++h) {
+        const int q = first_entry(sub) + h;
+        if (h > (~sub & 1)) continue;  // odd lanes own one entry
+        // the two-body term's symmetric virial is stored xx yy zz yz xz xy: the
+        // place of entry q, four bits each
+        if (fw2) v[h] += fw2[9 * (size_t)j + ((0x567648783210ull >> (4 * q)) & 15)];
         if (q < 3) {
-            if (forces) forces[3 * (size_t)j + q] = v;
+            if (forces) forces[3 * (size_t)j + q] = v[h];
         } else if (vir_atom) {
-            vir_atom[9 * (size_t)j + q - 3] = v;
+            vir_atom[9 * (size_t)j + q - 3] = v[h];
         }
     }
 }

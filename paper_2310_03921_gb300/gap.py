@@ -111,6 +111,7 @@ def lib():
             "gap_test_fail_alloc": [C.c_long],
             "gap_test_tc_force_variant": [C.c_int],
             "gap_test_fp64_recip": [C.c_int, _dp, _dp],
+            "gap_test_gather": [C.c_int, _ip, _ip, C.POINTER(C.c_float), C.POINTER(C.c_float), _dp, _dp],
             "gap_test_gp_rows": [C.c_int, C.c_int, C.c_int, _ip, _ip, _ip, _ip, _ip],
             "gap_model_set_alpha": [_vp, _vp, C.c_int, _vp],
             "gap_model_set_posterior": [_vp, C.c_long, _vp, _vp, C.c_double, C.c_int, _vp],
@@ -678,6 +679,17 @@ def test_gp_rows(species: np.ndarray, n_gp: int, one: bool = False):
     gp, rank = np.zeros(n, np.int32), np.zeros(n, np.int32)
     _check(lib().gap_test_gp_rows(n, n_gp, 1 if one else 0, *(a.ctypes.data_as(_ip) for a in (z, rows, counts, gp, rank))))
     return rows, counts, gp, rank
+
+
+def test_gather(offsets: np.ndarray, rev: np.ndarray, vec: np.ndarray, fpair: np.ndarray):
+    """(forces [n][3], atomic virials [n][9]) summed from FP32 pair derivatives (host arrays)."""
+    off, rev = np.ascontiguousarray(offsets, np.int32), np.ascontiguousarray(rev, np.int32)
+    vec, f = np.ascontiguousarray(vec, np.float32), np.ascontiguousarray(fpair, np.float32)
+    n, fp = off.size - 1, C.POINTER(C.c_float)
+    F, W = np.zeros((n, 3)), np.zeros((n, 9))
+    _check(lib().gap_test_gather(n, off.ctypes.data_as(_ip), rev.ctypes.data_as(_ip), vec.ctypes.data_as(fp),
+                                 f.ctypes.data_as(fp), F.ctypes.data_as(_dp), W.ctypes.data_as(_dp)))
+    return F, W
 
 
 def exported_symbols() -> list[str]:

@@ -49,3 +49,85 @@ def test_wait_expiry_in_the_middle_of_a_product(G, blocks):
     st, code = G.test_tc_expiry(blocks)
     assert (st, code) == (0, 0) if blocks == 32 else (st == -4 and code), (st, code)
     assert np.array_equal(G.test_bf16_gemm(A, B), A @ B.T)
+
+
+def _pairs(counts, seed, span=3.0):
+    """Random pair derivatives and vectors of atoms with that many pairs, magnitudes over 10^(+-span), the last pair of
+    every atom nearly cancelling its first."""
+    rng = np.random.default_rng(seed)
+    off = np.concatenate([[0], np.cumsum(counts)]).astype(np.int32)
+    P = off[-1]
+    f = (rng.normal(size=(P, 3)) * 10.0 ** rng.uniform(-span, span, (P, 1))).astype(np.float32)
+    v = rng.normal(size=(P, 4)).astype(np.float32)
+    for a, b in zip(off[:-1], off[1:]):
+        if b - a > 1:
+            f[b - 1], v[b - 1] = -f[a], v[a] * np.float32(1 + 2.0 ** -20)
+    return off, rng.permutation(P).astype(np.int32), v, f
+
+
+def _gather_exact(off, rev, v, f):
+    """Sums in exact integer arithmetic by math.fsum of the exact FP64 products, and the sums of magnitudes."""
+    import math
+    n = off.size - 1
+    f, v = f.astype(np.float64), v.astype(np.float64)  # products of two FP32 numbers are exact in FP64
+    F, Fa, W, Wa = np.zeros((n, 3)), np.zeros((n, 3)), np.zeros((n, 9)), np.zeros((n, 9))
+    for j in range(n):
+        p = np.arange(off[j], off[j + 1])
+        for a in range(3):
+            t = np.concatenate([f[p, a], -f[rev[p], a]])
+            F[j, a], Fa[j, a] = math.fsum(t), np.abs(t).sum()
+            for b in range(3):
+                t = -f[p, a] * v[p, b]
+                W[j, 3 * a + b], Wa[j, 3 * a + b] = math.fsum(t), np.abs(t).sum()
+    return F, Fa, W, Wa
+
+
+PAIR_COUNTS = [[1], [3], [8], [0, 9, 0, 40], list(range(35)), [29] * 50, [500, 3, 120]]
+
+
+@pytest.mark.parametrize("counts", PAIR_COUNTS, ids=len)
+def test_pair_sums_of_fp32_terms(G, counts):
+    """Compensated sums with exact products: of n pairs the second word collects up to 4 n roundings of 2^-24 of the
+    terms and rounds as often itself, at most (4 n)^2 2^-48 of them (sums of FP32-rounded products are off by 2^-25)."""
+    off, rev, v, f = _pairs(counts, len(counts))
+    F, W = G.test_gather(off, rev, v, f)
+    Fx, Fa, Wx, Wa = _gather_exact(off, rev, v, f)
+    bound = (4.0 * np.array(counts)[:, None]) ** 2 * 2.0 ** -48
+    assert np.all(np.abs(F - Fx) <= bound * Fa)
+    assert np.all(np.abs(W - Wx) <= bound * Wa)
+    if max(counts) > 1:
+        print("largest error over the terms' magnitudes: F %.2e W %.2e" % (
+            (np.abs(F - Fx)[Fa > 0] / Fa[Fa > 0]).max(), (np.abs(W - Wx)[Wa > 0] / Wa[Wa > 0]).max()))
+
+
+@pytest.mark.parametrize("counts", PAIR_COUNTS, ids=len)
+def test_pair_sums_hold_no_less_than_fp64(G, counts):
+    """Three words per sum: the last one rounds at most (4 n)^3 2^-72 of the terms' magnitudes, the result once and its
+    lower words once, 2^-52 of it."""
+    off, rev, v, f = _pairs(counts, 7 + len(counts))
+    F, W = G.test_gather(off, rev, v, f)
+    Fx, Fa, Wx, Wa = _gather_exact(off, rev, v, f)
+    tail = (4.0 * np.array(counts)[:, None]) ** 3 * 2.0 ** -72
+    assert np.all(np.abs(F - Fx) <= 2.0 ** -52 * np.abs(Fx) + tail * Fa)
+    assert np.all(np.abs(W - Wx) <= 2.0 ** -52 * np.abs(Wx) + tail * Wa)
+
+
+def test_pair_sums_beyond_fp32(G):
+    """Sums that leave FP32's range, infinite terms and NaN: as the FP64 sums."""
+    off, rev, v, f = _pairs([4, 12, 3, 20, 0, 7], 3)
+    rev = np.arange(off[-1], dtype=np.int32)  # a pair's force against itself: F = 0 for finite terms
+    f[off[0]:off[1]] = 3e38
+    f[off[1]] = np.inf
+    f[off[3] + 9, 1] = np.nan
+    F, W = G.test_gather(off, rev, v, f)
+    f64, v64 = f.astype(np.float64), v.astype(np.float64)
+    with np.errstate(invalid="ignore"):
+        for j in range(6):
+            p = slice(off[j], off[j + 1])
+            t = f64[p, :, None] * v64[p, None, :3]
+            Wx, Wa, Fx = -t.sum(0).reshape(9), np.abs(t).sum(0).reshape(9), (f64[p] - f64[rev[p]]).sum(0)
+            ok = np.isfinite(Wx)
+            assert np.array_equal(np.isnan(W[j]), np.isnan(Wx))
+            assert np.array_equal(W[j][np.isinf(Wx)], Wx[np.isinf(Wx)])
+            assert np.all(np.abs(W[j] - Wx)[ok] <= 1e-13 * Wa[ok])
+            assert np.array_equal(F[j], Fx, equal_nan=True)
