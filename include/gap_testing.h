@@ -117,6 +117,14 @@ gap_status gap_test_gp_rows(int n, int n_gp, int one, const int *species, int *r
  * (x) r_p.  forces host [n][3], virial host [n][9], FP64.  Synchronous. */
 gap_status gap_test_gather(int n, const int *offsets, const int *rev, const float *vec, const float *fpair,
                            double *forces, double *virial);
+/* The K_NM force rows' product and its sums over a target's triples, in split
+ * BF16 (nsplit 2 or 3): out[3 j + a][m] = sum over the triples t of target j of
+ * W[src[t]][m] (J[3 t + a] . X[m]).  counts host [n]: triples of each target
+ * (0 allowed), in order; src host [T], each < R; J host [3 T][K], X host
+ * [M][K], W host [R][M], FP32 row-major; K a positive multiple of 16; out host
+ * [3 n][M] FP64.  Synchronous. */
+gap_status gap_test_knm_rows(int nsplit, int n, const int *counts, int R, const int *src, int K, const float *J, int M,
+                             const float *X, const float *W, double *out);
 
 #ifdef __cplusplus
 }

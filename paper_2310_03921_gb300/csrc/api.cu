@@ -2343,6 +2343,89 @@ extern "C" gap_status gap_test_gather(int n, const int *offsets, const int *rev,
     GAP_API_END
 }
 
+extern "C" gap_status gap_test_knm_rows(int nsplit, int n, const int *counts, int R, const int *src, int K,
+                                        const float *J, int M, const float *X, const float *W, double *out)
+{
+    GAP_API_BEGIN
+    bool ok = (nsplit == 2 || nsplit == 3) && n > 0 && counts && R > 0 && src && K > 0 && K % 16 == 0 && J && M > 0 && X &&
+              W && out;
+    long T = 0;
+    for (int j = 0; ok && j < n; ++j) {
+        ok = counts[j] >= 0;
+        T += counts[j];
+    }
+    ok = ok && T > 0 && T < (1 << 24);
+    for (long t = 0; ok && t < T; ++t) ok = src[t] >= 0 && src[t] < R;
+    if (!ok) {
+        gap_set_error("bad arguments");
+        return GAP_EINVAL;
+    }
+    const int M_pad = (M + 255) / 256 * 256;
+    // BF16 planes [rows_pad][K] of x [rows][K]: hi, lo or hi, mid, lo
+    auto planes = [&](const float *x, size_t rows, size_t rows_pad, std::vector<uint16_t> (&p)[3]) {
+        for (int k = 0; k < nsplit; ++k) p[k].assign(rows_pad * K, 0);
+        for (size_t e = 0; e < rows * K; ++e) {
+            float rest = x[e];
+            for (int k = 0; k < nsplit; ++k) {
+                p[k][e] = bf16_rne(rest);
+                rest -= bf16_to_float(p[k][e]);
+            }
+        }
+    };
+    std::vector<uint16_t> jp[3], xp[3];
+    planes(J, 3 * (size_t)T, 3 * (size_t)T, jp);
+    planes(X, M, M_pad, xp);
+    std::vector<float> wp((size_t)R * M_pad, 0.f), meta(4 * (size_t)T, 0.f);
+    for (int r = 0; r < R; ++r) std::copy_n(W + (size_t)r * M, M, wp.data() + (size_t)r * M_pad);
+    std::vector<int> first(n + 1, 0), dest(T, -1);
+    for (int j = 0; j < n; ++j) {
+        first[j + 1] = first[j] + counts[j];
+        if (counts[j] > 0) dest[first[j + 1] - 1] = 3 * j;
+    }
+    for (long t = 0; t < T; ++t) std::memcpy(&meta[4 * t + 3], &src[t], sizeof(int));
+    DBuf dj[3], dx[3], dw, dmeta, ddest, dfirst, dbounds, dout, derr;
+    gap_status st = GAP_OK;
+    for (int k = 0; k < nsplit && st == GAP_OK; ++k) {
+        st = upload(dj[k], jp[k]);
+        if (st == GAP_OK) st = upload(dx[k], xp[k]);
+    }
+    const size_t n_out = 3 * (size_t)n * M;
+    if (st == GAP_OK) st = upload(dw, wp);
+    if (st == GAP_OK) st = upload(dmeta, meta);
+    if (st == GAP_OK) st = upload(ddest, dest);
+    if (st == GAP_OK) st = upload(dfirst, first);
+    if (st == GAP_OK) st = dbounds.ensure(sizeof(int) * gap_knm_bounds_ints(1));
+    if (st == GAP_OK) st = dout.ensure(sizeof(double) * n_out);
+    if (st == GAP_OK) st = derr.ensure(sizeof(int) * 4);
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemset(dout.p, 0, sizeof(double) * n_out), "cudaMemset");
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemset(derr.p, 0, sizeof(int) * 4), "cudaMemset");
+    int e = 0;
+    if (st == GAP_OK) {
+        const bool three = nsplit == 3;
+        KnmTriples tri{};
+        tri.hi = dj[0].as<__nv_bfloat16>();
+        tri.mid = three ? dj[1].as<__nv_bfloat16>() : nullptr;
+        tri.lo = dj[nsplit - 1].as<__nv_bfloat16>();
+        tri.meta = dmeta.as<float4>();
+        tri.dest = ddest.as<int>();
+        tri.first = dfirst.as<int>();
+        const KnmGP gp{M, M_pad, R, dx[0].as<__nv_bfloat16>(), dx[nsplit - 1].as<__nv_bfloat16>(),
+                       three ? dx[1].as<__nv_bfloat16>() : nullptr, dw.as<float>(), nullptr, nullptr, 0};
+        st = gap_knm_force_tc(tri, T, n, K, nsplit, &gp, 1, dbounds.as<int>(), dout.as<double>(), M, derr.as<int>(), 0);
+    }
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemcpy(&e, derr.p, sizeof(int), cudaMemcpyDeviceToHost), "K_NM force rows");
+    if (st == GAP_OK && e) {
+        gap_set_error("tensor-core GEMM wait expired (code " + std::to_string(e) + ")");
+        st = GAP_ETIMEOUT;
+    }
+    if (st == GAP_OK)
+        st = gap_cuda_status(cudaMemcpy(out, dout.p, sizeof(double) * n_out, cudaMemcpyDeviceToHost), "copy");
+    for (DBuf *b : {&dj[0], &dj[1], &dj[2], &dx[0], &dx[1], &dx[2], &dw, &dmeta, &ddest, &dfirst, &dbounds, &dout, &derr})
+        b->release();
+    return st;
+    GAP_API_END
+}
+
 // The bounded-wait path of the tcgen05 GEMM on zero operands: every wait gives
 // up after wait_ns, with a producer that stops issuing copies after `blocks`
 // blocks of K.

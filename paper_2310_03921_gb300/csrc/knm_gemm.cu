@@ -15,9 +15,10 @@
 // The N side of a tile is NG groups of 48 rows (16 triples), each from its own
 // stream: the triples of a range of targets.  Four epilogue warps serve a
 // group (one per TMEM lane quadrant).  A CTA takes a work unit, one 128-point
-// tile against NG ranges; ranges end between targets, so the running sums
-// carry from tile to tile in registers, no group needs another's sums, and
-// every K entry is written once, complete.  Units that share ranges differ in
+// tile against NG ranges; ranges end between targets, so no group needs
+// another's sums and every K entry is written once, complete.  A target's sum
+// is FP32 over the triples of one tile (sixteen at most) and FP64 over its
+// tiles, in shared memory (0.4% of K_NM of 200 silicon cells).  Units that share ranges differ in
 // the point tile and run side by side, so a Jacobian row is read from HBM
 // once and otherwise from L2.
 //
@@ -110,8 +111,11 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
     KnmTail *tail = reinterpret_cast<KnmTail *>(smem + STAGES * STAGE_BYTES);
-    // J . mu of the triples of two tiles, per epilogue warp
+    // J . mu of the triples of two tiles, per epilogue warp; after them every
+    // epilogue thread's sums of its current target over earlier tiles
     float4 *meta_s = reinterpret_cast<float4 *>(smem + STAGES * STAGE_BYTES + 256);
+    constexpr int kEpi = 128 * NG;
+    double *carry_s = reinterpret_cast<double *>(meta_s + 4 * NG * 2 * kGT);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
@@ -242,6 +246,7 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
         const int quad = warp & 3, grp = (warp - 2) >> 2;  // TMEM lane quadrant, column group
         const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(grp * kGC);
         float4 *wmeta = meta_s + (warp - 2) * 2 * kGT;
+        double *carry = carry_s + (threadIdx.x - 64);  // [three rows][kEpi]
         int gc = 0;  // K chunks consumed
         bool ok = true;
         for (int u = blockIdx.x; u < n_units && ok; u += gridDim.x) {
@@ -254,7 +259,11 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
             const bool mine = m < pr.M;
             const float *Wm = pr.Wp + m;  // m < M_pad: inside the padded row
             double *Kc = P.K + pr.col0 + m;
-            float s0 = 0.f, s1 = 0.f, s2 = 0.f;  // the current target's sums
+            // the current target's sums: FP32 over a tile's triples (sixteen at
+            // most), FP64 over the tiles
+            float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+            bool carried = false;  // earlier tiles of the target are in carry
+            auto total = [&](int a, float s) { return carried ? carry[a * kEpi] + (double)s : (double)s; };
             float w[kGT];
             int dest = -1;
             // lane k < 16 holds triple k of a tile; past the range's end zeros
@@ -308,11 +317,12 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
                                 const int d = __shfl_sync(0xffffffffu, dest, 8 * h + k);
                                 if (mine) {
                                     double *o = Kc + (size_t)d * P.ldk;
-                                    o[0] = (double)s0;
-                                    o[P.ldk] = (double)s1;
-                                    o[2 * P.ldk] = (double)s2;
+                                    o[0] = total(0, s0);
+                                    o[P.ldk] = total(1, s1);
+                                    o[2 * P.ldk] = total(2, s2);
                                 }
                                 s0 = s1 = s2 = 0.f;
+                                carried = false;
                             }
                         }
                     }
@@ -355,6 +365,13 @@ __global__ void __launch_bounds__(64 + 128 * NG, 1) k_knm_gemm(const __grid_cons
                     if (!ok) break;
                     sum_half(0, v);
                     sum_half(1, v + 24);
+                }
+                if (!(ends >> (kGT - 1) & 1u)) {  // the target goes on in the next tile
+                    carry[0] = total(0, s0);
+                    carry[kEpi] = total(1, s1);
+                    carry[2 * kEpi] = total(2, s2);
+                    s0 = s1 = s2 = 0.f;
+                    carried = true;
                 }
 #pragma unroll
                 for (int k = 0; k < kGT; ++k) w[k] = wn[k];
@@ -479,7 +496,8 @@ gap_status launch_knm(KnmParams &P, const KnmTriples &t, const KnmGP *gps, const
     gap_count_launch();
     k_knm_ranges<<<P.n, 256, 0, st>>>(n, t.first, plan, bounds);
     GAP_TRY_CUDA(cudaGetLastError());
-    const size_t shm = (size_t)STAGES * NS * (BM + NG * kGC) * BK * 2 + 256 + 4 * NG * 2 * kGT * sizeof(float4) + 1024;
+    const size_t shm = (size_t)STAGES * NS * (BM + NG * kGC) * BK * 2 + 256 +
+                       4 * NG * 2 * kGT * sizeof(float4) + 3 * 128 * NG * sizeof(double) + 1024;
     auto kern = k_knm_gemm<NG, NS, STAGES, ONE>;
     GAP_TRY_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
     const int sms = gap_tc_sm_count();

@@ -112,6 +112,8 @@ def lib():
             "gap_test_tc_force_variant": [C.c_int],
             "gap_test_fp64_recip": [C.c_int, _dp, _dp],
             "gap_test_gather": [C.c_int, _ip, _ip, C.POINTER(C.c_float), C.POINTER(C.c_float), _dp, _dp],
+            "gap_test_knm_rows": [C.c_int, C.c_int, _ip, C.c_int, _ip, C.c_int, C.POINTER(C.c_float), C.c_int,
+                                  C.POINTER(C.c_float), C.POINTER(C.c_float), _dp],
             "gap_test_gp_rows": [C.c_int, C.c_int, C.c_int, _ip, _ip, _ip, _ip, _ip],
             "gap_model_set_alpha": [_vp, _vp, C.c_int, _vp],
             "gap_model_set_posterior": [_vp, C.c_long, _vp, _vp, C.c_double, C.c_int, _vp],
@@ -690,6 +692,17 @@ def test_gather(offsets: np.ndarray, rev: np.ndarray, vec: np.ndarray, fpair: np
     _check(lib().gap_test_gather(n, off.ctypes.data_as(_ip), rev.ctypes.data_as(_ip), vec.ctypes.data_as(fp),
                                  f.ctypes.data_as(fp), F.ctypes.data_as(_dp), W.ctypes.data_as(_dp)))
     return F, W
+
+
+def test_knm_rows(counts, src, J: np.ndarray, X: np.ndarray, W: np.ndarray, nsplit: int = 2) -> np.ndarray:
+    """[3 n][M]: K_NM force rows of given Jacobian triples (host arrays)."""
+    counts, src = np.ascontiguousarray(counts, np.int32), np.ascontiguousarray(src, np.int32)
+    J, X, W = (np.ascontiguousarray(a, np.float32) for a in (J, X, W))
+    out, fp = np.zeros((3 * counts.size, X.shape[0])), C.POINTER(C.c_float)
+    _check(lib().gap_test_knm_rows(nsplit, counts.size, counts.ctypes.data_as(_ip), W.shape[0], src.ctypes.data_as(_ip),
+                                   X.shape[1], J.ctypes.data_as(fp), X.shape[0], X.ctypes.data_as(fp),
+                                   W.ctypes.data_as(fp), out.ctypes.data_as(_dp)))
+    return out
 
 
 def exported_symbols() -> list[str]:

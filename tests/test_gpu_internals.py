@@ -131,3 +131,32 @@ def test_pair_sums_beyond_fp32(G):
             assert np.array_equal(W[j][np.isinf(Wx)], Wx[np.isinf(Wx)])
             assert np.all(np.abs(W[j] - Wx)[ok] <= 1e-13 * Wa[ok])
             assert np.array_equal(F[j], Fx, equal_nan=True)
+
+
+@pytest.mark.parametrize("K,nsplit", [(16, 2), (256, 2), (320, 2), (48, 3)])
+@pytest.mark.parametrize("counts", [[48], [0, 70, 1, 16, 15, 17, 0], [400, 33, 5], [31] * 40], ids=["one", "ragged", "long", "many"])
+def test_knm_target_sums(G, counts, K, nsplit):
+    """A target's sum over its triples: FP32 over at most sixteen of them, FP64 beyond.  Every J . X is a product of
+    small whole numbers, exact on the tensor cores.  A target's first triple is 2^26 times the others and its own tile
+    holds nothing else of the target, so that tile is exact, the others are off by sixteen roundings of 2^-24 of their
+    terms at most and the FP64 sum by 2^-50 of the whole; a longer FP32 sum would lose the small terms altogether."""
+    rng = np.random.default_rng(K + len(counts))
+    T, M, R = sum(counts), 130, 37
+    src = rng.integers(0, R, T)
+    J = rng.integers(1, 4, (3 * T, K)).astype(np.float32) * (rng.random((3 * T, K)) < 8 / K)
+    X = rng.integers(1, 4, (M, K)).astype(np.float32)
+    W = rng.uniform(0.5, 1.5, (R, M)).astype(np.float32)
+    W[0] = 1.0
+    J = J.reshape(T, 3, K)
+    off = np.concatenate([[0], np.cumsum(counts)])
+    for a, c in zip(off, counts):
+        if c:
+            src[a] = 0
+            J[a] *= 2.0 ** 26
+            J[a + 1:a + min(c, 16)] = 0.0
+    out = G.test_knm_rows(counts, src, J.reshape(3 * T, K), X, W, nsplit)
+    P = (J.astype(np.float64) @ X.T.astype(np.float64)) * W[src].astype(np.float64)[:, None, :]
+    for j, (a, c) in enumerate(zip(off, counts)):
+        exact, rest = P[a:a + c].sum(0), P[a + 1:a + c].sum(0)
+        bound = 16 * 2.0 ** -24 * rest + 2.0 ** -50 * np.abs(exact)
+        assert np.all(np.abs(out[3 * j:3 * j + 3] - exact) <= bound), j
