@@ -93,6 +93,10 @@ gap_status gap_test_fail_alloc(long after);
  * x host [n] (positive), out host [n][4] = (recip, rsqrt, CUDA 1/x, CUDA
  * rsqrt).  Synchronous. */
 gap_status gap_test_fp64_recip(int n, const double *x, double *out);
+/* The FP64 square root of the pair distances and the FP64 quotient of the
+ * two-body derivative (Newton corrections of an FP32 estimate): out host
+ * [n][2] = (sqrt(a), a / b) for a, b host [n].  Synchronous. */
+gap_status gap_test_fp64_pair(int n, const double *a, const double *b, double *out);
 /* Forces the tensor-core contractions' tile variant (the tile autotuner's
  * candidates, in its order: 0 = 128 x 256 with two TMA stages, 1 = 128 x 128
  * with two, 2 = 128 x 128 with three, 3 = 128 x 192 with twelve epilogue

@@ -174,19 +174,6 @@ k_bin_small(BinInputs in, int n_bins, D4 *__restrict__ cart, float4 *__restrict_
 // floor(a / n) for n > 0.
 __device__ __forceinline__ int floor_div(int a, int n) { return a >= 0 ? a / n : -((n - 1 - a) / n); }
 
-// sqrt(x) to the last bit or so for 0 < x < rc^2: the FP32 reciprocal square
-// root and two Newton steps on the root (errors 2^-22, 2^-43, 2^-64 before
-// rounding); CUDA's FP64 square root takes about three times the FP64
-// instructions.
-__device__ __forceinline__ double sqrt_newton(double x)
-{
-    if (!(x > 1e-30)) return sqrt(x);
-    const double y = (double)rsqrtf((float)x), h = 0.5 * y;
-    double r = x * y;
-    r = fma(fma(-r, r, x), h, r);
-    return fma(fma(-r, r, x), h, r);
-}
-
 // Per warp: the non-empty bins of the current chunk of 32 bins around the
 // atom (their lattice shifts in FP64 and FP32, the offset taking a candidate's
 // number to its slot of bin_atoms, the packed shift) and the candidates that
@@ -396,7 +383,7 @@ k_fill_warp(int n, const D4 *__restrict__ cart, const float4 *__restrict__ cart3
                             const int pos = w + __popc(m & ((1u << lane) - 1u));
                             if (pos < np) {
                                 const long long key = pair_key(j, code);
-                                const D4 d{v[0], v[1], v[2], sqrt_newton(r2)};
+                                const D4 d{v[0], v[1], v[2], sqrt64(r2)};
                                 if (local) {
                                     skey[wi][pos] = key;
                                     svec[wi][pos] = d;

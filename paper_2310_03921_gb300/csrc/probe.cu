@@ -54,7 +54,37 @@ template <typename T> gap_status probe(int iters, double *tflops)
     return GAP_OK;
 }
 
+__global__ void k_pair_arithmetic(int n, const double *__restrict__ a, const double *__restrict__ b,
+                                  double *__restrict__ out)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    out[2 * (size_t)i] = sqrt64(a[i]);
+    out[2 * (size_t)i + 1] = divide64(a[i], b[i]);
+}
+
 }  // namespace
+
+extern "C" gap_status gap_test_fp64_pair(int n, const double *a, const double *b, double *out)
+{
+    if (n < 1 || n > (1 << 26) || !a || !b || !out) {
+        gap_set_error("bad arguments");
+        return GAP_EINVAL;
+    }
+    const size_t bytes = sizeof(double) * (size_t)n;
+    double *d = nullptr;  // a, b, out
+    gap_status st = gap_cuda_status(gap_dev_malloc((void **)&d, 4 * bytes), "cudaMalloc");
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemcpy(d, a, bytes, cudaMemcpyHostToDevice), "copy");
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemcpy(d + n, b, bytes, cudaMemcpyHostToDevice), "copy");
+    if (st == GAP_OK) {
+        gap_count_launch();
+        k_pair_arithmetic<<<(n + 255) / 256, 256>>>(n, d, d + n, d + 2 * (size_t)n);
+        st = gap_cuda_status(cudaGetLastError(), "k_pair_arithmetic");
+    }
+    if (st == GAP_OK) st = gap_cuda_status(cudaMemcpy(out, d + 2 * (size_t)n, 2 * bytes, cudaMemcpyDeviceToHost), "copy");
+    if (d) cudaFree(d);
+    return st;
+}
 
 extern "C" gap_status gap_test_fma_peak(int fp64, double *tflops)
 {

@@ -521,16 +521,6 @@ __global__ void k_twobody_table(TwoBodyDev tb, D4 *__restrict__ tab)
     tab[k] = D4{e0, h * d0, 3.0 * (e1 - e0) - h * (2.0 * d0 + d1), 2.0 * (e0 - e1) + h * (d0 + d1)};
 }
 
-// 1 / r to the last bit or so: the FP32 reciprocal and two Newton steps
-// (errors 2^-23, 2^-46, 2^-92 before rounding).  CUDA's FP64 division takes
-// several times the FP64 instructions, each ~64 cycles per warp here.
-__device__ __forceinline__ double recip_newton(double r)
-{
-    double y = (double)(1.0f / (float)r);
-    y = fma(y, fma(-r, y, 1.0), y);
-    return fma(y, fma(-r, y, 1.0), y);
-}
-
 // Lanes that share one atom's pairs in the per-atom sums below.  An atom has
 // 25-40 pairs: eight lanes leave a chain of four or five dependent loads (one
 // thread per atom walked all of them: 30 us of latency at 64 atoms), and a
@@ -570,7 +560,7 @@ k_twobody(int n_atoms, const int *__restrict__ offsets, const D4 *__restrict__ v
         const D4 a = tb.tab[in ? k : tb.g_in + k];
         e += a.x + u * (a.y + u * (a.z + u * a.w));
         if (fw2) {
-            const double c = (a.y + u * (2.0 * a.z + 3.0 * u * a.w)) * inv * recip_newton(r);
+            const double c = divide64((a.y + u * (2.0 * a.z + 3.0 * u * a.w)) * inv, r);
             const double fx = c * v.x, fy = c * v.y, fz = c * v.z;
             F[0] += fx;
             F[1] += fy;

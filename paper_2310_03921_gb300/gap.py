@@ -114,6 +114,7 @@ def lib():
             "gap_test_gather": [C.c_int, _ip, _ip, C.POINTER(C.c_float), C.POINTER(C.c_float), _dp, _dp],
             "gap_test_knm_rows": [C.c_int, C.c_int, _ip, C.c_int, _ip, C.c_int, C.POINTER(C.c_float), C.c_int,
                                   C.POINTER(C.c_float), C.POINTER(C.c_float), _dp],
+            "gap_test_fp64_pair": [C.c_int, _dp, _dp, _dp],
             "gap_test_gp_rows": [C.c_int, C.c_int, C.c_int, _ip, _ip, _ip, _ip, _ip],
             "gap_model_set_alpha": [_vp, _vp, C.c_int, _vp],
             "gap_model_set_posterior": [_vp, C.c_long, _vp, _vp, C.c_double, C.c_int, _vp],
@@ -703,6 +704,14 @@ def test_knm_rows(counts, src, J: np.ndarray, X: np.ndarray, W: np.ndarray, nspl
                                    X.shape[1], J.ctypes.data_as(fp), X.shape[0], X.ctypes.data_as(fp),
                                    W.ctypes.data_as(fp), out.ctypes.data_as(_dp)))
     return out
+
+
+def test_fp64_pair(a: np.ndarray, b: np.ndarray):
+    """(sqrt(a), a / b) as the pair kernels form them in FP64 (host float64)."""
+    a, b = np.ascontiguousarray(a, np.float64), np.ascontiguousarray(b, np.float64)
+    out = np.zeros((a.size, 2))
+    _check(lib().gap_test_fp64_pair(a.size, a.ctypes.data_as(_dp), b.ctypes.data_as(_dp), out.ctypes.data_as(_dp)))
+    return out[:, 0], out[:, 1]
 
 
 def exported_symbols() -> list[str]:

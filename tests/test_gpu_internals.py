@@ -160,3 +160,29 @@ def test_knm_target_sums(G, counts, K, nsplit):
         exact, rest = P[a:a + c].sum(0), P[a + 1:a + c].sum(0)
         bound = 16 * 2.0 ** -24 * rest + 2.0 ** -50 * np.abs(exact)
         assert np.all(np.abs(out[3 * j:3 * j + 3] - exact) <= bound), j
+
+
+def test_pair_root_and_quotient(G):
+    """Correctly rounded but for one result in 2^32 (the error before the last rounding is 2^-33 of the last place), so
+    at most one of these three million may be the neighbouring number."""
+    rng = np.random.default_rng(5)
+    n = 1 << 20
+    r2 = np.concatenate([rng.uniform(1e-6, 30.0, n), np.ldexp(rng.uniform(1, 2, n), rng.integers(-110, 110, n)),
+                         30.25 * (1 - np.ldexp(1.0, -rng.integers(1, 53, 1000))),  # at a cutoff
+                         1e-30 * rng.uniform(0.1, 10, 1000), np.ldexp(rng.integers(1, 1 << 52, 1000).astype(float), -30)])
+    r = np.sqrt(r2[rng.permutation(r2.size)])
+    a = r2 * np.where(rng.random(r2.size) < 0.5, -1.0, 1.0)
+    root, _ = G.test_fp64_pair(r2, r)
+    _, quot = G.test_fp64_pair(a, r)
+    for got, ref in ((root, np.sqrt(r2)), (quot, a / r)):
+        off = got != ref
+        assert off.sum() <= 1 and np.all(np.abs(got - ref) <= np.spacing(np.abs(ref)))
+
+
+def test_pair_root_and_quotient_of_other_arguments(G):
+    a = np.array([0.0, -0.0, np.inf, -np.inf, np.nan, 1e-320, 1e308, -1.0, 5e-324, 1e-200, 1.0, 1.0, 0.0, 1.0])
+    b = np.array([2.0, 3.0, 2.0, 2.0, 2.0, 2.0, 1e-10, 2.0, 3.0, 1e200, 0.0, np.inf, 0.0, np.nan])
+    with np.errstate(all="ignore"):
+        root, quot = G.test_fp64_pair(a, b)
+        assert np.array_equal(root, np.sqrt(a), equal_nan=True)
+        assert np.array_equal(quot, a / b, equal_nan=True)
