@@ -101,11 +101,16 @@ gap_status gap_test_fp64_pair(int n, const double *a, const double *b, double *o
  * candidates, in its order: 0 = 128 x 256 with two TMA stages, 1 = 128 x 128
  * with two, 2 = 128 x 128 with three, 3 = 128 x 192 with twelve epilogue
  * warps) for every later single-problem two-plane call where the variant
- * applies (the grouped launch of several GPs keeps its own tile; variant
- * 3: the K_NM force rows with K <= 256, the kernel-energy and the gradient
- * contractions); other calls keep the tuned choice.  v < 0 restores the
- * autotuner.  For parity tests of every variant; process-wide. */
+ * applies (the grouped launch of several GPs keeps its own tile; variant 3:
+ * the kernel-energy and the gradient contractions); other calls keep the
+ * tuned choice.  A forced gradient contraction runs in one part of K.  The
+ * K_NM force rows have one tile per (inner size, planes) and are not touched;
+ * K_NM's W' and k are (variants 0 to 2).  v < 0 restores the autotuner.  For
+ * parity tests of every variant; process-wide. */
 gap_status gap_test_tc_force_variant(int v);
+/* Parts of K in which one GP's gradient contraction of rows x D16 over M_pad
+ * padded sparse points runs (1: whole). */
+int gap_test_contract_parts(int rows, int M_pad, int D16, int nsplit);
 /* The row lists of the GPs, as a prediction builds them: species host [n],
  * GPs for species 0 .. n_gp - 1 (1 <= n_gp <= 8); one != 0 is the form of a
  * one-species model, in which every atom is GP 0's.  Outputs (host): rows

@@ -203,6 +203,11 @@ extern "C" gap_status gap_test_tc_force_variant(int v)
     return GAP_OK;
 }
 
+extern "C" int gap_test_contract_parts(int rows, int M_pad, int D16, int nsplit)
+{
+    return gap_contract_parts(&rows, &M_pad, 1, D16, nsplit, 0);
+}
+
 struct DBuf {
     void *p = nullptr;
     size_t cap = 0;

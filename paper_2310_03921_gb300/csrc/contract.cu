@@ -546,6 +546,7 @@ gap_status gap_split_rows(const float *phat, int D, int D16, const int *rows, in
 
 int gap_contract_parts(const int *rows, const int *M_pad, int n, int D16, int nsplit, int q)
 {
+    if (n == 1 && gap_tc_variant_forced(nsplit)) return 1;  // the forced tile, not the split's own
     // column tile: a split product runs on 128 x 128 tiles, a group on its own
     const int bn = n == 1 ? 128 : gap_tc_grouped_col_tile(nsplit);
     long tiles = 0;

@@ -752,6 +752,7 @@ int forced_variant(const TcOperands &op, int epi)
 }  // namespace
 
 void gap_tc_force_variant(int v) { g_force_variant.store(v < 0 ? -1 : v); }
+bool gap_tc_variant_forced(int nsplit) { return nsplit == 2 && g_force_variant.load() >= 0; }
 
 int gap_tc_plan(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, cudaStream_t st, int *groups)
 {

@@ -58,6 +58,7 @@ int gap_tc_plan(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, c
 int gap_tc_tuned_count();
 // Test hook: every later two-plane call where variant v applies uses it (v < 0: the tuner).
 void gap_tc_force_variant(int v);
+bool gap_tc_variant_forced(int nsplit);  // whether one is forced for products of that many planes
 bool gap_tc_tuned_entry(int k, int *fields, float *ms);
 // SMs of the current device, and the tensor map of a BF16 operand
 // [rows][ld] (cols of them valid) loaded in boxes of box_rows x 64.

@@ -115,6 +115,7 @@ def lib():
             "gap_test_knm_rows": [C.c_int, C.c_int, _ip, C.c_int, _ip, C.c_int, C.POINTER(C.c_float), C.c_int,
                                   C.POINTER(C.c_float), C.POINTER(C.c_float), _dp],
             "gap_test_fp64_pair": [C.c_int, _dp, _dp, _dp],
+            "gap_test_contract_parts": [C.c_int, C.c_int, C.c_int, C.c_int],
             "gap_test_gp_rows": [C.c_int, C.c_int, C.c_int, _ip, _ip, _ip, _ip, _ip],
             "gap_model_set_alpha": [_vp, _vp, C.c_int, _vp],
             "gap_model_set_posterior": [_vp, C.c_long, _vp, _vp, C.c_double, C.c_int, _vp],
