@@ -715,9 +715,10 @@ gap_status gap_neighbours_done(NbrWork &w, const int *host)
         const double ppa = (double)host[kNbrTotal] / w.n_atoms;
         if (ppa > w.pairs_per_atom) w.pairs_per_atom = ppa;
     }
-    if (e & 1) {
-        gap_set_error("more neighbour pairs than the pair capacity (" + std::to_string(w.pair_cap) +
-                      ") of the captured step");
+    if (e & 1) {  // without a graph the caller runs the call again, and sets an error if that fails
+        if (w.graph)
+            gap_set_error("more neighbour pairs than the pair capacity (" + std::to_string(w.pair_cap) +
+                          ") of the captured step");
         return GAP_ECAPACITY;
     }
     if (e) {
