@@ -87,6 +87,9 @@ gap_status gap_test_tc_expiry(int blocks, unsigned long long wait_ns, int *code)
  * the per-call workspaces (descriptor, predict, K_NM, solve, neighbours);
  * object creation (gap_soap_create's tables) is not covered. */
 gap_status gap_test_fail_alloc(long after);
+/* The same for every workspace allocation of more than `bytes` bytes (< 0:
+ * none). */
+gap_status gap_test_fail_alloc_above(long bytes);
 /* The FP64 reciprocal and reciprocal square root of the factorisation's
  * block kernel (an FP32 estimate refined by Newton steps, no FP64 division
  * or square root) beside CUDA's own double-precision 1.0 / x and rsqrt(x):

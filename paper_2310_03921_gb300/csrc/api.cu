@@ -173,9 +173,14 @@ void gap_fill_ylm_constants(SoapGeom &g)
 // Every device allocation of the library goes through gap_dev_malloc, which
 // a test hook can make fail (gap_test_fail_alloc) to exercise GAP_ENOMEM.
 static std::atomic<long> g_fail_alloc_after{-1};
+static std::atomic<size_t> g_fail_alloc_above{(size_t)-1};
 
 cudaError_t gap_dev_malloc(void **p, size_t bytes)
 {
+    if (bytes > g_fail_alloc_above.load()) {
+        *p = nullptr;
+        return cudaErrorMemoryAllocation;
+    }
     long left = g_fail_alloc_after.load();
     while (left >= 0) {
         if (left == 0) {
@@ -190,6 +195,12 @@ cudaError_t gap_dev_malloc(void **p, size_t bytes)
 extern "C" gap_status gap_test_fail_alloc(long after)
 {
     g_fail_alloc_after.store(after < 0 ? -1 : after);
+    return GAP_OK;
+}
+
+extern "C" gap_status gap_test_fail_alloc_above(long bytes)
+{
+    g_fail_alloc_above.store(bytes < 0 ? (size_t)-1 : (size_t)bytes);
     return GAP_OK;
 }
 
@@ -800,9 +811,23 @@ static int m_gps(const gap_model *m);
 static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, const int *spec, cudaStream_t st);
 static bool counts_without_wait(const gap_model *m, const gap_batch *b, std::vector<int> &counts);
 
+// A call that first does not wait for its pair count (once(true)), and is run
+// again with the wait where its batch had more pairs per atom than the
+// workspace has met, or where the room for that many could not be had (that for
+// its own may be).
+template <typename F> static gap_status run_ahead(F &&once)
+{
+    const std::string message = g_last_error;
+    gap_status rc = once(true);
+    if (rc != GAP_ECAPACITY && rc != GAP_ENOMEM) return rc;
+    rc = once(false);
+    if (rc == GAP_OK) g_last_error = message;
+    return rc;
+}
+
 // Neighbours + expansion + power spectrum for a batch, in arithmetic T; with a
 // model also the rows of every GP (launched first, so that their counts come
-// back with the pair count).  ahead: the caller handles GAP_ECAPACITY (see
+// back with the pair count).  ahead: the caller is run_ahead's (see
 // gap_neighbours), taken where nothing has to be read back before the next
 // launches.
 template <typename T>
@@ -904,10 +929,7 @@ extern "C" gap_status gap_descriptor(gap_soap *soap, const gap_batch *b, gap_pre
         GAP_TRY(w.outbuf.ensure(sizeof(double) * cnt));
         dst = w.outbuf.as<double>();
     }
-    gap_status rc = GAP_OK;
-    for (int attempt = 0; attempt < 2; ++attempt) {
-        // ahead of the pair count first; again if the batch had more pairs
-        const bool ahead = attempt == 0;
+    auto once = [&](bool ahead) {
         if (prec == GAP_FP64) {
             GAP_TRY(run_descriptor<double>(soap, w, b, &spec, st, ahead));
             if (cnt)
@@ -923,10 +945,9 @@ extern "C" gap_status gap_descriptor(gap_soap *soap, const gap_batch *b, gap_pre
         }
         if (!b->device && cnt)
             GAP_TRY_CUDA(cudaMemcpyAsync(p_out, dst, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
-        rc = check_device_errors(w, st);
-        if (rc != GAP_ECAPACITY) break;
-    }
-    return rc;
+        return check_device_errors(w, st);
+    };
+    return run_ahead(once);
     GAP_API_END
 }
 
@@ -1459,15 +1480,12 @@ static gap_status predict_once(gap_model *m, Workspace &w, const gap_batch *b, g
     return check_device_errors(w, st);
 }
 
-// Without a wait for the pair count first (gap_neighbours), and again with
-// one if the batch had more pairs per atom than this workspace has met.
 template <typename T>
 static gap_status predict_impl(gap_model *m, Workspace &w, const gap_batch *b, gap_precision prec, double *energy,
                                double *local_e, double *forces, double *virial, cudaStream_t st)
 {
-    const gap_status rc = predict_once<T>(m, w, b, prec, energy, local_e, forces, virial, true, st);
-    if (rc != GAP_ECAPACITY || w.graph) return rc;
-    return predict_once<T>(m, w, b, prec, energy, local_e, forces, virial, false, st);
+    auto once = [&](bool ahead) { return predict_once<T>(m, w, b, prec, energy, local_e, forces, virial, ahead, st); };
+    return w.graph ? once(false) : run_ahead(once);
 }
 
 extern "C" gap_status gap_predict(gap_model *m, const gap_batch *b, gap_precision prec, double *energy,

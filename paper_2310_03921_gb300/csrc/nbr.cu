@@ -739,6 +739,7 @@ static gap_status grow(void **p, size_t &cap, size_t bytes)
     cudaError_t e = gap_dev_malloc(p, b);
     if (e != cudaSuccess) {
         *p = nullptr;
+        cudaGetLastError();  // the caller may go on with a smaller request
         gap_set_error(std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
         return GAP_ENOMEM;
     }

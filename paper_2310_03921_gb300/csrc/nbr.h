@@ -63,7 +63,7 @@ constexpr int kNbrErr = 8, kNbrTotal = 16, kGpCounts = 18, kWords = 32;
 // most pairs per atom seen so far (2^20 pairs in all at most, else it waits),
 // and a batch with more empties every list
 // and ends in GAP_ECAPACITY (gap_neighbours_done), to be run again without
-// `ahead`.
+// `ahead`, as is a call whose room ahead could not be had (GAP_ENOMEM).
 gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, const int *d_species, int S, double rc,
                           int *words, int *host, bool ahead, cudaStream_t st);
 // The status of a build from its words on the host, the stream synchronised.

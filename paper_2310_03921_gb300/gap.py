@@ -109,6 +109,7 @@ def lib():
             "gap_test_tc_timeout": [C.c_ulonglong, _ip],
             "gap_test_tc_expiry": [C.c_int, C.c_ulonglong, _ip],
             "gap_test_fail_alloc": [C.c_long],
+            "gap_test_fail_alloc_above": [C.c_long],
             "gap_test_tc_force_variant": [C.c_int],
             "gap_test_fp64_recip": [C.c_int, _dp, _dp],
             "gap_test_gather": [C.c_int, _ip, _ip, C.POINTER(C.c_float), C.POINTER(C.c_float), _dp, _dp],
@@ -660,6 +661,11 @@ def test_tc_expiry(blocks: int, wait_ns: int = 1000000):
 def test_fail_alloc(after: int):
     """Make the library's workspace allocations fail after `after` more (-1: off)."""
     _check(lib().gap_test_fail_alloc(int(after)))
+
+
+def test_fail_alloc_above(nbytes: int):
+    """Make the library's workspace allocations of more than nbytes fail (-1: off)."""
+    _check(lib().gap_test_fail_alloc_above(int(nbytes)))
 
 
 def test_tc_force_variant(v: int):

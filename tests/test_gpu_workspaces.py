@@ -38,3 +38,22 @@ def test_a_denser_batch_leaves_no_error_message(G, handles):
         message = G.lib().gap_last_error()
         call(_batch(G, dense), "fp64")
         assert G.lib().gap_last_error() == message
+
+
+def test_room_ahead_that_cannot_be_had(G, handles):
+    """After a dense cell, 4000 atoms without a pair would get room for 195 thousand: where memory has no place for it
+    the call still succeeds, with room for its own pairs."""
+    soap, model = handles
+    dense = S.displaced_diamond(0, 5, (2, 2, 2), 0.05, a=4.2)
+    pos = 20.0 * np.stack(np.meshgrid(*[np.arange(16.0)] * 3, indexing="ij"), -1).reshape(-1, 3)[:4000]
+    gas = S.Structure(pos, np.zeros(4000, np.int32), np.eye(3) * 320.0, np.ones(3, np.int32))
+    for call, prec in ((soap.descriptor, "fp64"), (model.predict, "fp64")):
+        call(_batch(G, dense), prec)
+        G.test_fail_alloc_above(6500000)  # their FP64 vectors, 7.8 MB with the slack, do not fit; all that goes by atoms does
+        try:
+            got = call(_batch(G, gas), prec)
+        finally:
+            G.test_fail_alloc_above(-1)
+        assert b"cudaMalloc" not in G.lib().gap_last_error()
+        p = got["local_e"] if isinstance(got, dict) else got
+        assert np.allclose(p.cpu().numpy()[1:], p.cpu().numpy()[0], atol=1e-12)
