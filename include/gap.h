@@ -410,7 +410,8 @@ gap_status gap_profile_read(double *ms, int *count);
 long gap_launch_count(void);
 /* The tile autotuner of the tensor-core contractions (the batching pattern:
  * tile shapes picked per workload).  The first call of a shape class on a
- * device (epilogue, split, K, columns, ceil(log2 rows)) outside stream
+ * device (epilogue, split, K, columns, ceil(log2 rows); the kernel-energy
+ * epilogue of calls with forces and of energies alone apart) outside stream
  * capture times each tile variant on its own operands - 128 x 256 with two
  * TMA stages, 128 x 128 with two, 128 x 128 with three, and for the
  * kernel-energy and the gradient contractions 128 x 192 with twelve epilogue

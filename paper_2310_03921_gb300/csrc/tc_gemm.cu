@@ -669,19 +669,22 @@ gap_status launch_variant(const TcOperands &op, const TcEpilogue &ep, int epi, i
     }
 }
 
-// Tile autotuner.  A shape class is (device, epilogue, planes, K, columns,
-// ceil(log2(rows))).  The first call of a class outside stream capture times
+// Tile autotuner.  A shape class is (device, epilogue and whether it stores W,
+// planes, K, columns, ceil(log2(rows))).  (Without the stores, an energies-only
+// call, the kernel-energy epilogue is another load, and its tile decides how
+// the energy partials are grouped.)  The first call of a class outside stream capture times
 // every variant on that call's own operands and outputs (CUDA events on the
 // call's stream: one warm-up launch, then the best of two) and keeps the
 // fastest; every later call, and any call under capture, reuses the choice
 // (the default variant while none is known).  All variants compute the same
 // values; their outputs are rewritten by the call that follows.
 struct TuneKey {
-    int dev, epi, nsplit, K, cols, rlog;
+    int dev, epi, stores, nsplit, K, cols, rlog;
     bool operator<(const TuneKey &o) const
     {
         if (dev != o.dev) return dev < o.dev;
         if (epi != o.epi) return epi < o.epi;
+        if (stores != o.stores) return stores < o.stores;
         if (nsplit != o.nsplit) return nsplit < o.nsplit;
         if (K != o.K) return K < o.K;
         if (cols != o.cols) return cols < o.cols;
@@ -701,6 +704,13 @@ int rows_log2(int rows)
     int r = 0;
     while ((1 << r) < rows && r < 30) ++r;
     return r;
+}
+
+TuneKey tune_key(const TcOperands &op, const TcEpilogue &ep, int epi)
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return {dev, epi, epi != EPI_KERNEL || ep.W_hi ? 1 : 0, op.nsplit, op.K, op.cols, rows_log2(op.rows)};
 }
 
 // The column tile a variant uses for this call (the energy epilogue's
@@ -763,9 +773,7 @@ int gap_tc_plan(const TcOperands &op, const TcEpilogue &ep, int epi, int *err, c
     }
     if (op.nsplit == 3 || op.rows <= 0 || op.cols <= 0) return 128;
     if (ep.wait_ns) return kVariants2[0].bn;  // the timeout tests: nothing to time
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const TuneKey key{dev, epi, op.nsplit, op.K, op.cols, rows_log2(op.rows)};
+    const TuneKey key = tune_key(op, ep, epi);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune.find(key);
@@ -864,10 +872,8 @@ gap_status gap_tc_gemm(const TcOperands &op, const TcEpilogue &ep, int epi, int 
     {
         // the planned variant (the plan returns its column tile; look up the
         // full entry for the stage count)
-        int dev = 0;
-        cudaGetDevice(&dev);
         std::lock_guard<std::mutex> lk(g_tune_mu);
-        auto it = g_tune.find(TuneKey{dev, epi, op.nsplit, op.K, op.cols, rows_log2(op.rows)});
+        auto it = g_tune.find(tune_key(op, ep, epi));
         if (it != g_tune.end()) v = it->second.variant;
     }
     return launch_variant(op, with_parts(ep, epi, op, kVariants2[v]), epi, v, err, st);
