@@ -843,7 +843,11 @@ static gap_status run_descriptor(gap_soap *soap, Workspace &w, const gap_batch *
     GAP_TRY(stage_inputs(w, b, g.S, &pos, &spec, st));
     bool known = true;
     if (m) {
+        gap_prof_end(ST_NEIGHBOURS, st);
+        gap_prof_begin(ST_GP_ROWS, st);
         GAP_TRY(launch_gp_rows(m, w, n, spec, st));
+        gap_prof_end(ST_GP_ROWS, st);
+        gap_prof_begin(ST_NEIGHBOURS, st);
         known = !w.graph && counts_without_wait(m, b, *counts);
     }
     GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, g.S, g.rc, w.err.as<int>(), static_cast<int *>(w.words.p),

@@ -57,3 +57,18 @@ def test_room_ahead_that_cannot_be_had(G, handles):
         assert b"cudaMalloc" not in G.lib().gap_last_error()
         p = got["local_e"] if isinstance(got, dict) else got
         assert np.allclose(p.cpu().numpy()[1:], p.cpu().numpy()[0], atol=1e-12)
+
+
+def test_gp_rows_are_a_stage_of_their_own(G, handles):
+    """One interval per call, beside the neighbours' two (the inputs before the rows, the lists after them)."""
+    _, model = handles
+    b = _batch(G, S.displaced_diamond(0, 3, (2, 2, 2), 0.05))
+    G.profile_enable(True)
+    try:
+        for _ in range(3):
+            model.predict(b, "fp64")
+        stages = G.profile_read()
+    finally:
+        G.profile_enable(False)
+    assert stages["gp_rows"][1] == 3 and stages["gp_rows"][0] > 0.0
+    assert stages["neighbours"][1] == 6 and stages["neighbours"][0] > 0.0
