@@ -36,7 +36,7 @@ def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
     t = os.path.getmtime(obj)
-    deps = [src] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    deps = [src] + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     deps.append(os.path.join(HERE, "..", "include", "gap.h"))
     deps.append(os.path.join(HERE, "..", "include", "gap_testing.h"))
     return any(os.path.getmtime(d) > t for d in deps if os.path.exists(d))
