@@ -1130,9 +1130,12 @@ gap_status gap_crt_prep_cols(const CrtVMat &V, int T, long kpad, __nv_bfloat16 *
         return GAP_EINVAL;
     }
     GAP_TRY_CUDA(cudaMemsetAsync(E, 0, sizeof(int) * V.cols, st));
-    // rows per block: 128, or 16 where that leaves SMs without a block (a
-    // thread walks its rows one batch of loads after another)
-    const int rpb = (V.rows + 127) / 128 * ((V.cols + 127) / 128) >= 608 ? 128 : 16;
+    // 16 rows per block: a thread walks its rows one batch of loads after
+    // another, so latency bounds larger blocks.  All scans of one solve with 16
+    // and with 128 rows: 2648 x 300 21 and 82 us, 10000 x 1000 82 and 149 us,
+    // 75176 x 2000 539 and 657 us, 200000 x 2000 1243 and 1304 us.  128 where
+    // the grid's 65535 blocks in y would not reach the last row.
+    const int rpb = V.rows > 16L * 65535 ? 128 : 16;
     dim3 g1((V.cols + 127) / 128, (unsigned)(V.rows > 0 ? (V.rows + rpb - 1) / rpb : 1));
     gap_count_launch();
     k_col_exp<<<g1, 128, 0, st>>>(V, rpb, E, diag, ld_diag, n_diag);
