@@ -148,7 +148,13 @@ k_eps_rows(const int *__restrict__ rows, const int *__restrict__ nrows_p, const 
 // products whose 64 x 64 tiles would leave most SMs idle (small_tiles).
 // Whole predictions with 64 x 64 and 8 x 8 tiles, n_max 8, l_max 6: FP64 215
 // atoms x 4000 points 5371 and 1216 us, 4095 x 2000 9089 and 8392 us; FP32 215
-// x 4000 (252 tiles and 16) 905 and 461 us.
+// x 4000 (252 tiles and 16) 905 and 461 us.  One FP32 product by its number of
+// 64 x 64 tiles, 64 x 64 and 8 x 8, inner size 252: 8 tiles 41 and 10 us, 32
+// tiles 43 and 17, 64 tiles 43 and 31, 96 tiles 43 and 32, 128 tiles 43 and
+// 52, 512 tiles 73 and 177; inner size 2000: 4 tiles 276 and 27, 32 tiles 278
+// and 103, 64 tiles 277 and 183, 108 tiles 281 and 300.  They cross near 100
+// tiles whatever the inner size; the line lies at 48, well on the side where
+// the small tiles win.
 constexpr int kST = 8, kSK = 64, kSplit = 4;
 
 // acc = sum over this thread's quarter of K of A(r, k) B(k, c); load(e, kk, rr)

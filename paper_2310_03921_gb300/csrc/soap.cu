@@ -850,7 +850,13 @@ template <typename T> struct Launch {
     static gap_status chain(const SoapGeom &g, int n, const T *gvec, const T *wsum, const T *mu, const int *gp_of_atom,
                             const T *phat, const T *pnorm, const T *coef, T *Gam, cudaStream_t st)
     {
-        // four atoms per block once that fills the chip; one for few atoms
+        // Four atoms per block once that fills the chip, one for few atoms.  One
+        // and four: 32768 atoms, (n, l) = (6, 4) 34 and 25 us, (8, 8) 63 and 56,
+        // four species unmixed (8, 6) 2735 and 2283; 1728 atoms the same but for
+        // the unmixed ones (199 and 133); 144 atoms unmixed 45 and 53.  FP64, four
+        // mixed species: 1000 atoms 74 and 81, 1728 atoms 116 and 116, 3584 atoms
+        // 225 and 225.  (Unmixed descriptors alone would change over at about one
+        // atom per SM.)
         const int warps = n >= 2048 && 4 * sizeof(T) * (size_t)g.D <= kMaxSmem ? 4 : 1;
         const size_t shm = sizeof(T) * (size_t)g.D * warps;
         if (shm > kMaxSmem) {
@@ -872,9 +878,14 @@ template <typename T> struct Launch {
         const typename V4<T>::type *vec;
         if constexpr (sizeof(T) == 8) vec = pl.vec64; else vec = pl.vec32;
         gap_count_launch();
-        // one warp per block while that spreads the warps over more SMs (the
+        // One warp per block while that spreads the warps over more SMs (the
         // FP64 pipe and L1 are per SM); the FP64 form's registers allow no more
-        // warps per SM in larger blocks either
+        // warps per SM in larger blocks either.  FP32 with 32 and 128 threads, (n,
+        // l) = (8, 8): 1800 pairs 12.2 and 13.3 us, 28 thousand 16.3 and 17.1, 56
+        // thousand 22.5 and 25.6, 918 thousand 242 and 250; (2, 1): 28 thousand
+        // 6.8 and 6.5, 918 thousand 22.5 and 16.3.  Beyond 32 thousand the
+        // difference is 1 to 3% either way but for the smallest shape, which
+        // blocks of one warp would slow down.
         const int threads = sizeof(T) == 8 || pl.n_pairs <= 32 * 1024 ? 32 : 128;
         k_pairforce<N, L, T><<<(pl.n_pairs + threads - 1) / threads, threads, 0, st>>>(
             g, tab, pl.n_pairs, pl.count, pl.i, pl.j, vec, species, Gam, fpair);
