@@ -198,8 +198,9 @@ def alu_rooflines(per_launch, n_atoms, n_pairs, n_max, l_max, D, M, fp32_peak, f
                  rows written, 3 (N + P) rows x 2 BF16 planes x D16 x 2 B.
       solve_block the elimination on [A | I] of one diagonal block of the
                  factorisation (mean over the blocks of an M x M Gram
-                 matrix), against ONE SM's rate (the chip's FP64 rate / SMs);
-                 a block runs on a cluster of eight, one panel at a time."""
+                 matrix), against ONE SM's rate (the chip's FP64 rate / SMs)
+                 and, frac_of_sms, that of the eight its cluster occupies
+                 (one panel, so one SM, factorises at a time)."""
     L1 = l_max + 1
     lam = L1 * L1
     npair = n_max * (n_max + 1) // 2
@@ -233,7 +234,7 @@ def alu_rooflines(per_launch, n_atoms, n_pairs, n_max, l_max, D, M, fp32_peak, f
                               "flops": fl, "blocks_per_factorisation": len(blocks), "factorisations": n_fact,
                               "achieved_tflops": a, "peak_tflops": sm_peak,
                               "peak_source": f"FP64 FMA probe / {n_sm} SMs (one SM; a block runs on eight)", "frac": a / sm_peak,
-                              "frac_of_chip": a / fp64_peak}
+                              "frac_of_chip": a / fp64_peak, "sms": 8, "frac_of_sms": a / (8 * sm_peak)}
     return out
 
 
@@ -433,7 +434,8 @@ def run_ours(args, rank, world, local_rank):
                      "peak": burst, "peak_source": f"bf16_tflops burst ({src}): each launch is a few ms, "
                      "far shorter than the seconds-long loop of the sustained figure", "unit": "TFLOP/s",
                      "frac": achieved / burst, "traffic": knm_traffic if dom == "knm_gemm" else None,
-                     "traffic_unit": "bytes per K_NM GEMM launch (ncu capture, scaled by Jacobian rows)",
+                     "traffic_unit": "bytes per K_NM GEMM launch (ncu capture, scaled by Jacobian rows)"
+                     if dom == "knm_gemm" else None,
                      "note": rooflines[dom]["note"]},
         "tensor_rooflines": rooflines,
         "stages_ms_per_step": {k: round(v, 4) for k, v in per_step.items()},

@@ -95,7 +95,7 @@ __global__ void k_bin(BinInputs in, D4 *__restrict__ cart, float4 *__restrict__ 
     if (i < in.n) atomicAdd(&bin_count[bin_atom(in, i, cart, cart32, atom_cfg, atom_bin)], 1);
 }
 
-// The bins' places are taken from the end: bin_count goes back to zero.
+// A bin's places are taken from the end of its count.
 __global__ void k_scatter(int n, const int *__restrict__ atom_bin, const int *__restrict__ bin_start,
                           int *__restrict__ bin_count, int *__restrict__ bin_atoms)
 {

@@ -17,3 +17,10 @@ def test_a_forced_tile_variant_reaches_the_gradient_product(variant):
     finally:
         gap.test_tc_force_variant(-1)
     assert parts(240, 512, 256, 2) > 1
+
+
+def test_block_roofline_counts_the_clusters_sms():
+    import bench
+    r = bench.alu_rooflines({"solve_block": 0.04}, n_atoms=1000, n_pairs=30000, n_max=8, l_max=6, D=252, M=2000,
+                            fp32_peak=80.0, fp64_peak=1.2, hbm=6800.0, n_sm=152, n_fact=2)["solve_block"]
+    assert r["sms"] == 8 and r["frac_of_sms"] == pytest.approx(r["frac"] / 8)
