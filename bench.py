@@ -140,7 +140,7 @@ CRT_MODULI = [256, 255, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 1
 #       -k "regex:k_knm_gemm" -c 1 python -m paper_2310_03921_gb300.profile_run --fit 20 --steps 1
 # The operand rows, the W' rows and the K_NM rows all grow with the Jacobian
 # rows, so a full launch is scaled by 3 (N + P).
-KNM_TRAFFIC_READ, KNM_TRAFFIC_WRITE, KNM_TRAFFIC_JROWS = 240358912, 86377728, 194934
+KNM_TRAFFIC_READ, KNM_TRAFFIC_WRITE, KNM_TRAFFIC_JROWS = 240387328, 86584064, 194934
 
 
 def crt_moduli_counts(m: int, n_ext: int):

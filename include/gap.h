@@ -14,7 +14,8 @@
  *  - Device-pointer calls work on `stream` (a cudaStream_t, or NULL for the
  *    legacy default stream) and read their error words (and the pair count,
  *    after the neighbour search, where earlier calls on the handle do not
- *    bound it) back before they return, unless stated otherwise; host-pointer calls
+ *    bound it; a batch with more pairs per atom than any before on its handle
+ *    is run twice) back before they return, unless stated otherwise; host-pointer calls
  *    copy in, run on `stream`, copy out and synchronise before returning.
  *  - The caller owns all input and output buffers.  Handles own their
  *    device tables and workspaces; a handle must not be used by two calls at
@@ -415,9 +416,9 @@ long gap_launch_count(void);
  * capture times each tile variant on its own operands - 128 x 256 with two
  * TMA stages, 128 x 128 with two, 128 x 128 with three, and for the
  * kernel-energy and the gradient contractions 128 x 192 with twelve epilogue
- * warps - and keeps the fastest; captured calls reuse the choice (128 x 256 with two stages
- * for a class not yet tuned).  gap_tile_tuning_count gives
- * the number of tuned classes; entry k: fields[8] = (epilogue, planes, K,
+ * warps - and keeps the fastest; captured calls reuse the choice (128 x 256
+ * with two stages for a class not yet tuned).  gap_tile_tuning_count gives the
+ * number of tuned classes; entry k: fields[8] = (epilogue, planes, K,
  * columns, ceil(log2 rows), chosen column tile, chosen stages, device) and
  * ms[4] = each variant's best time in that order (-1: not a candidate). */
 int gap_tile_tuning_count(void);

@@ -18,17 +18,17 @@
 // tile against NG ranges; ranges end between targets, so no group needs
 // another's sums and every K entry is written once, complete.  A target's sum
 // is FP32 over the triples of one tile (sixteen at most) and FP64 over its
-// tiles, in shared memory (0.4% of K_NM of 200 silicon cells).  Units that share ranges differ in
-// the point tile and run side by side, so a Jacobian row is read from HBM
-// once and otherwise from L2.
+// tiles, in shared memory (0.4% of K_NM of 200 silicon cells).  Units that
+// share ranges differ in the point tile and run side by side, so a Jacobian row
+// is read from HBM once and otherwise from L2.
 //
 // What bounds it is latency in the epilogue: one group over the whole tile
 // (four warps, one per scheduler) takes 12 thousand cycles per tile where the
 // MMAs take 4.6 thousand; with four groups each scheduler has four warps.
 // W' rows and row data are loaded one and two tiles ahead.  K_NM of 200
-// silicon cells (2.14 million rows, 2000 points, D = 252): 4.2 ms here, 7.3 ms
+// silicon cells (2.17 million rows, 2000 points, D = 252): 4.75 ms here, 7.4 ms
 // with the rows on the M side, W' gathered per row and the target sums through
-// shared memory; the MMAs alone take about 3.7 ms.
+// shared memory; the MMAs and the TMEM reads alone take about 3.7 ms.
 //
 //   warp 0       TMA producer (one lane), K blocks of 64, STAGES-deep ring
 //   warp 1       TMEM allocation, MMA issue (one lane)
