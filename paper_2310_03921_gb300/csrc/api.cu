@@ -808,7 +808,7 @@ template <typename T> static const T *gp_phat(const gap_soap *s, const Workspace
 }
 
 static int m_gps(const gap_model *m);
-static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, const int *spec, cudaStream_t st);
+static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, bool one, const int *spec, cudaStream_t st);
 static bool counts_without_wait(const gap_model *m, const gap_batch *b, std::vector<int> &counts);
 
 // A call that first does not wait for its pair count (once(true)), and is run
@@ -845,10 +845,12 @@ static gap_status run_descriptor(gap_soap *soap, Workspace &w, const gap_batch *
     if (m) {
         gap_prof_end(ST_NEIGHBOURS, st);
         gap_prof_begin(ST_GP_ROWS, st);
-        GAP_TRY(launch_gp_rows(m, w, n, spec, st));
+        // one species and its count not read back: every atom is GP 0's, whatever
+        // its species word says (a wrong one fails such a call)
+        GAP_TRY(launch_gp_rows(m, w, n, g.S == 1 && (ahead || w.graph), spec, st));
         gap_prof_end(ST_GP_ROWS, st);
         gap_prof_begin(ST_NEIGHBOURS, st);
-        known = !w.graph && counts_without_wait(m, b, *counts);
+        known = ahead && !w.graph && counts_without_wait(m, b, *counts);
     }
     GAP_TRY(gap_neighbours(w.nbr, b, pos, spec, g.S, g.rc, w.err.as<int>(), static_cast<int *>(w.words.p),
                            ahead && known, st));
@@ -1235,14 +1237,14 @@ template <> const float *gp_alpha<float>(const GPData &g) { return g.a32.as<floa
 
 // Rows of every GP (atoms of species s); their counts stay in the call's
 // device words.
-static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, const int *spec, cudaStream_t st)
+static gap_status launch_gp_rows(const gap_model *m, Workspace &w, int n, bool one, const int *spec, cudaStream_t st)
 {
     int G = m->n_gp;
     GAP_TRY(w.gp_of_atom.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.rank.ensure(sizeof(int) * (size_t)n));
     GAP_TRY(w.scan_tmp.ensure(sizeof(int) * gap_gp_rows_tmp_ints(n, G)));
     GAP_TRY(w.rows.ensure(sizeof(int) * (size_t)(G > 0 ? G : 1) * n));
-    return gap_gp_rows(n, G, m->soap->geo.S == 1, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.err.as<int>() + kGpCounts,
+    return gap_gp_rows(n, G, one, spec, w.scan_tmp.as<int>(), w.rows.as<int>(), w.err.as<int>() + kGpCounts,
                        w.gp_of_atom.as<int>(), w.rank.as<int>(), st);
 }
 

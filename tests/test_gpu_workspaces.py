@@ -72,3 +72,19 @@ def test_gp_rows_are_a_stage_of_their_own(G, handles):
         G.profile_enable(False)
     assert stages["gp_rows"][1] == 3 and stages["gp_rows"][0] > 0.0
     assert stages["neighbours"][1] == 6 and stages["neighbours"][0] > 0.0
+
+
+def test_variance_of_atoms_of_no_gp(G, handles):
+    """Atoms whose species word names no GP have no local energy, and so no variance, in a one-species model too."""
+    import torch
+    soap, model = handles
+    w = S.workload(0)
+    cells = [S.displaced_diamond(0, 600 + c, (1, 1, 2), 0.15) for c in range(4)]
+    K = model.assemble_knm(G.Batch.from_synth(S.make_batch(cells), device="cuda"), precision="fp64")
+    model.set_posterior(K, torch.full((K.shape[0],), 0.1, dtype=torch.float64, device="cuda"))
+    good = S.displaced_diamond(0, 700, (2, 2, 2), 0.1)
+    bad = S.Structure(good.pos, np.full(good.n, 3, np.int32), good.cell, good.pbc)
+    ref = model.predict_variance(_batch(G, good)).cpu().numpy()
+    got = model.predict_variance(G.Batch.from_synth(S.make_batch([good, bad]), device="cuda")).cpu().numpy()
+    assert ref.max() > 0 and np.allclose(got[:good.n], ref, atol=1e-10 * w.delta ** 2)
+    assert np.all(got[good.n:] == 0.0)
