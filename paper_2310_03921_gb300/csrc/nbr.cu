@@ -616,6 +616,8 @@ gap_status gap_cell_geometry(const gap_batch *b, double rc, std::vector<CellGeom
 // many pairs (1.5 ms and more); beyond, a workspace that once met a dense cell
 // would hold its density times the atoms of a large sparse one.
 constexpr int kAheadPairs = 1 << 20;
+// Most geometry a handle keeps pinned: about 80 thousand configurations.
+constexpr size_t kMaxStage = 16 << 20;
 
 gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, const int *d_species, int S, double rc,
                           int *words, int *host, bool ahead, cudaStream_t st)
@@ -630,29 +632,36 @@ gap_status gap_neighbours(NbrWork &w, const gap_batch *b, const double *d_pos, c
     w.total = words + kNbrTotal;
     w.n_atoms = n;
     if (!w.graph) {
-        // geometry and offsets in one copy from pinned memory
+        // geometry and offsets in one copy from pinned memory, or, beyond what a
+        // handle should keep pinned (or where none is to be had), in two from
+        // the host's own, which wait for the stream
         const size_t og = geo_bytes(b->n_configs), bytes = og + sizeof(int) * (b->n_configs + 1);
         if (w.in_flight) {  // an earlier call ended in an error before it synchronised
             GAP_TRY_CUDA(cudaDeviceSynchronize());
             w.in_flight = false;
         }
-        if (bytes > w.cap_stage) {
+        if (bytes > w.cap_stage && bytes <= kMaxStage) {
             if (w.stage) cudaFreeHost(w.stage);
             w.stage = nullptr;
             w.cap_stage = 0;
-            if (cudaMallocHost(&w.stage, bytes + bytes / 4) != cudaSuccess) {
+            if (cudaMallocHost(&w.stage, bytes + bytes / 4) == cudaSuccess) {
+                w.cap_stage = bytes + bytes / 4;
+            } else {
                 cudaGetLastError();
                 w.stage = nullptr;
-                gap_set_error("pinned host allocation failed");
-                return GAP_ENOMEM;
             }
-            w.cap_stage = bytes + bytes / 4;
         }
-        if (!geo.empty()) std::memcpy(w.stage, geo.data(), sizeof(CellGeom) * geo.size());
-        if (b->n_configs > 0)
-            std::memcpy(static_cast<char *>(w.stage) + og, b->config_offsets, sizeof(int) * (b->n_configs + 1));
-        GAP_TRY_CUDA(cudaMemcpyAsync(w.geo, w.stage, bytes, cudaMemcpyHostToDevice, st));
-        w.in_flight = true;
+        if (bytes <= w.cap_stage) {
+            if (!geo.empty()) std::memcpy(w.stage, geo.data(), sizeof(CellGeom) * geo.size());
+            if (b->n_configs > 0)
+                std::memcpy(static_cast<char *>(w.stage) + og, b->config_offsets, sizeof(int) * (b->n_configs + 1));
+            GAP_TRY_CUDA(cudaMemcpyAsync(w.geo, w.stage, bytes, cudaMemcpyHostToDevice, st));
+            w.in_flight = true;
+        } else if (b->n_configs > 0) {
+            GAP_TRY_CUDA(cudaMemcpyAsync(w.geo, geo.data(), sizeof(CellGeom) * geo.size(), cudaMemcpyHostToDevice, st));
+            GAP_TRY_CUDA(cudaMemcpyAsync(w.cfg_offsets, b->config_offsets, sizeof(int) * (b->n_configs + 1),
+                                         cudaMemcpyHostToDevice, st));
+        }
     }
     const BinInputs in{n, b->n_configs, S, d_pos, d_species, w.cfg_offsets, w.geo, err};
     if (n > 0 && n <= kSmallAtoms && n_bins <= kSmallBins) {

@@ -88,3 +88,24 @@ def test_variance_of_atoms_of_no_gp(G, handles):
     got = model.predict_variance(G.Batch.from_synth(S.make_batch([good, bad]), device="cuda")).cpu().numpy()
     assert ref.max() > 0 and np.allclose(got[:good.n], ref, atol=1e-10 * w.delta ** 2)
     assert np.all(got[good.n:] == 0.0)
+
+
+@pytest.mark.parametrize("n", [3, 100000])
+def test_batches_of_many_configurations(G, handles, n):
+    """Isolated atoms, each a configuration of its own: beyond about 80 thousand the cells' geometry is not pinned.  All
+    energies are the first one's, a batch of one's."""
+    soap, model = handles
+    cell = np.repeat(12.0 * np.eye(3)[None], n, 0)
+    pos = np.random.default_rng(1).uniform(0.0, 12.0, (n, 3))
+    import torch
+    dev = lambda a, t: torch.as_tensor(a, dtype=t, device="cuda")  # noqa: E731
+    b = G.Batch(dev(pos, torch.float64), dev(np.zeros(n), torch.int32), cell, np.ones((n, 3), np.int32),
+                np.arange(n + 1, dtype=np.int32))
+    one = G.Batch(dev(pos[:1], torch.float64), dev(np.zeros(1), torch.int32), cell[:1], np.ones((1, 3), np.int32),
+                  np.array([0, 1], np.int32))
+    for _ in range(2):
+        out = model.predict(b, "bf16x3")
+        E = out["energy"].cpu().numpy()
+        ref = float(model.predict(one, "bf16x3")["energy"][0])
+        assert E.shape == (n,) and np.abs(E - ref).max() <= 1e-5 * max(1.0, abs(ref))
+        assert float(out["forces"].abs().max()) <= 1e-6
